@@ -3,6 +3,7 @@
 // radix sort, per-group ranks, transaction depths (k-set levels), regrouping
 // by (level, type), insert slots, partition ids.
 #include <algorithm>
+#include <atomic>
 #include <cooperative_groups.h>
 #include <cstdio>
 
@@ -621,19 +622,16 @@ __global__ void tpl_reset_kernel(const uint32_t *skeys, int64_t m, uint32_t *don
     if ((i == 0 || skeys[i - 1] != k) && k < n_objects) done[slot(k)] = 0;
 }
 
-template <class Mode>
-cudaError_t run_scan(gputx_bulk *b, const Mode &mode, int64_t count, int ctr_slot)
+template <class Mode> cudaError_t run_scan(gputx_bulk *b, const Mode &mode, int64_t count)
 {
     if (count <= 0) return cudaSuccess;
     const int64_t tiles = (count + SCAN_TILE - 1) / SCAN_TILE;
     if (tiles > b->sc.scan_tiles) return cudaErrorInvalidValue;
     cudaStream_t s = b->stream;
-    cudaError_t e = cudaMemsetAsync(b->sc.scan_status, 0, tiles * sizeof(uint64_t), s);
-    if (e) return e;
-    e = cudaMemsetAsync(b->sc.tile_ctr + ctr_slot, 0, sizeof(uint32_t), s);
+    cudaError_t e = cudaMemsetAsync(b->sc.scan_zero, 0, (1 + tiles) * sizeof(uint64_t), s);
     if (e) return e;
     dualseg_scan_kernel<Mode><<<(unsigned)tiles, SCAN_THREADS, 0, s>>>(
-        mode, count, b->sc.scan_status, b->sc.tile_ctr + ctr_slot, &b->ctl->err,
+        mode, count, b->sc.scan_zero + 1, (uint32_t *)b->sc.scan_zero, &b->ctl->err,
         (uint64_t)b->db->cfg.spin_limit_ns);
     count_launches(1);
     return cudaGetLastError();
@@ -887,14 +885,13 @@ cudaError_t launch_scan_exec(gputx_bulk *b, const uint32_t *sk, const uint32_t *
         mode.R = b->R;
         mode.o_acc = db->dev.o_acc;
         Seg64Status st;
-        st.word = (uint32_t *)b->sc.scan_status;
+        st.word = (uint32_t *)(b->sc.scan_zero + 1);
         st.agg = b->sc.scan_vals;
         st.inc = b->sc.scan_vals + tiles;
-        cudaError_t e = cudaMemsetAsync(st.word, 0, tiles * sizeof(uint32_t), s);
-        if (!e) e = cudaMemsetAsync(b->sc.tile_ctr + 12, 0, sizeof(uint32_t), s);
+        cudaError_t e = cudaMemsetAsync(b->sc.scan_zero, 0, sizeof(uint64_t) + tiles * sizeof(uint32_t), s);
         if (e) return e;
         seg64_scan_kernel<ScanExecMode><<<(unsigned)tiles, SCAN_THREADS, 0, s>>>(
-            mode, m, st, b->sc.tile_ctr + 12, &b->ctl->err, (uint64_t)db->cfg.spin_limit_ns);
+            mode, m, st, (uint32_t *)b->sc.scan_zero, &b->ctl->err, (uint64_t)db->cfg.spin_limit_ns);
         count_launches(1);
     }
     if (b->n > 0) {
@@ -1074,7 +1071,7 @@ cudaError_t launch_extract(gputx_bulk *b, int mode, int part_size, uint32_t *pid
         cudaError_t e = cudaGetLastError();
         if (e) return e;
         OffsetMode om{b->sc.level, b->sc.op_off, b->n};
-        e = run_scan(b, om, b->n, 0);
+        e = run_scan(b, om, b->n);
         if (e) return e;
         a.op_off = b->sc.op_off;
     }
@@ -1083,45 +1080,76 @@ cudaError_t launch_extract(gputx_bulk *b, int mode, int part_size, uint32_t *pid
     return cudaGetLastError();
 }
 
+// A sort's scratch: a tile counter per pass (8 words), the digit counts, each
+// pass's look-back words -- for any number of key bits and up to `count` pairs.
+int64_t sort_scratch_words(int64_t count)
+{
+    int64_t words = 0;
+    for (int bits : {10, 32})   // at most three passes of 10-bit digits, four of 8-bit ones
+        for (int64_t c : {std::min(count, SORT_WIDE_FROM), count}) {
+            const SortShape s = sort_shape(c, bits);
+            const int passes = s.digit_bits == 10 ? 3 : 4;
+            words = std::max(words, 8 + passes * (int64_t)s.digits() * (1 + s.tiles));
+        }
+    return words;
+}
+
+template <int RB, int ITEMS>
+static cudaError_t launch_radix_passes(gputx_bulk *b, uint32_t *&keys, uint32_t *&vals, uint32_t *&keys_alt,
+                                       uint32_t *&vals_alt, uint32_t count, const SortShape &sh)
+{
+    constexpr int D = 1 << RB;
+    cudaStream_t s = b->stream;
+    uint32_t *ctr = b->sc.sort_zero, *hist = ctr + 8, *status = hist + sh.passes * D;
+    static std::atomic<uint64_t> attr_set{0};   // a bit per device
+    const uint64_t dev = 1ull << (b->db->device & 63);
+    if (!(attr_set.load(std::memory_order_relaxed) & dev)) {
+        const cudaError_t e = cudaFuncSetAttribute(radix_pass_kernel<RB, ITEMS>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)radix_smem<RB, ITEMS>());
+        if (e) return e;
+        attr_set.fetch_or(dev, std::memory_order_relaxed);
+    }
+    int hist_blocks = b->db->num_sms * 4;
+    const int64_t need = ((int64_t)count + 255) / 256;
+    if (hist_blocks > need) hist_blocks = (int)need;
+    radix_hist_kernel<RB><<<hist_blocks, 256, 0, s>>>(keys, count, sh.passes, hist, &b->ctl->err);
+    count_launches(1);
+    for (int p = 0; p < sh.passes; p++) {
+        radix_pass_kernel<RB, ITEMS><<<(unsigned)sh.tiles, SORT_THREADS, radix_smem<RB, ITEMS>(), s>>>(
+            keys, vals, keys_alt, vals_alt, count, RB * p, hist + p * D, status + (size_t)p * sh.tiles * D, ctr + p,
+            &b->ctl->err, (uint64_t)b->db->cfg.spin_limit_ns);
+        count_launches(1);
+        std::swap(keys, keys_alt);
+        std::swap(vals, vals_alt);
+    }
+    return cudaGetLastError();
+}
+
 cudaError_t launch_sort(gputx_bulk *b, uint32_t *&keys, uint32_t *&vals, uint32_t *&keys_alt, uint32_t *&vals_alt,
                         int64_t count, int bits)
 {
     if (count <= 1 || bits <= 0) return cudaSuccess;
     cudaStream_t s = b->stream;
-    const int passes = (bits + 7) / 8;
-    const int64_t tiles = (count + SORT_TILE - 1) / SORT_TILE;
-    if (tiles > b->sc.sort_tiles || passes > 4) return cudaErrorInvalidValue;
-    cudaError_t e = cudaMemsetAsync(b->sc.sort_hist, 0, 4 * RADIX * sizeof(uint32_t), s);
-    if (e) return e;
-    e = cudaMemsetAsync(b->sc.sort_status, 0, (size_t)passes * tiles * RADIX * sizeof(uint32_t), s);
-    if (e) return e;
-    e = cudaMemsetAsync(b->sc.tile_ctr + 8, 0, 4 * sizeof(uint32_t), s);
-    if (e) return e;
-    static bool smem_set = false;
-    if (!smem_set) {
-        e = cudaFuncSetAttribute(radix_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SORT_SMEM);
-        if (e) return e;
-        smem_set = true;
-    }
-    int hist_blocks = b->db->num_sms * 4;
-    const int64_t need = (count + 255) / 256;
-    if (hist_blocks > need) hist_blocks = (int)need;
-    radix_hist_kernel<<<hist_blocks, 256, 0, s>>>(keys, count, passes, b->sc.sort_hist, &b->ctl->err);
-    count_launches(1);
-    radix_offsets_kernel<<<passes, RADIX, 0, s>>>(b->sc.sort_hist, b->sc.sort_offs);
-    count_launches(1);
-    for (int p = 0; p < passes; p++) {
-        radix_pass_kernel<<<(unsigned)tiles, SORT_THREADS, SORT_SMEM, s>>>(
-            keys, vals, keys_alt, vals_alt, count, 8 * p, b->sc.sort_offs + p * RADIX,
-            b->sc.sort_status + (size_t)p * tiles * RADIX, b->sc.tile_ctr + 8 + p, &b->ctl->err,
-            (uint64_t)b->db->cfg.spin_limit_ns);
+    if (count <= SMALL_SORT) {
+        radix_small_kernel<<<1, SMALL_SORT_THREADS, 0, s>>>(keys, vals, keys_alt, vals_alt, (uint32_t)count, bits,
+                                                            &b->ctl->err);
         count_launches(1);
-        e = cudaGetLastError();
-        if (e) return e;
-        uint32_t *t = keys; keys = keys_alt; keys_alt = t;
-        t = vals; vals = vals_alt; vals_alt = t;
+        std::swap(keys, keys_alt);
+        std::swap(vals, vals_alt);
+        return cudaGetLastError();
     }
-    return cudaSuccess;
+    const SortShape sh = sort_shape(count, bits);
+    const int64_t words = 8 + sh.passes * (int64_t)sh.digits() * (1 + sh.tiles);
+    if (words > b->sc.sort_words || bits > 32 || count >= (1ll << 30)) return cudaErrorInvalidValue;
+    cudaError_t e = cudaMemsetAsync(b->sc.sort_zero, 0, words * sizeof(uint32_t), s);
+    if (e) return e;
+    const uint32_t n = (uint32_t)count;
+    if (sh.digit_bits == 10)
+        return sh.items == 4 ? launch_radix_passes<10, 4>(b, keys, vals, keys_alt, vals_alt, n, sh)
+                             : launch_radix_passes<10, 16>(b, keys, vals, keys_alt, vals_alt, n, sh);
+    return sh.items == 4 ? launch_radix_passes<8, 4>(b, keys, vals, keys_alt, vals_alt, n, sh)
+                         : launch_radix_passes<8, 16>(b, keys, vals, keys_alt, vals_alt, n, sh);
 }
 
 cudaError_t launch_rank_scan(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m, bool want_rid)
@@ -1129,7 +1157,7 @@ cudaError_t launch_rank_scan(gputx_bulk *b, const uint32_t *sk, const uint32_t *
     cudaError_t e = cudaMemsetAsync(b->sc.level, 0, b->n * sizeof(uint32_t), b->stream);
     if (e) return e;
     RankMode rm{sk, sv, b->sc.level, want_rid ? b->sc.rid : nullptr};
-    return run_scan(b, rm, m, 1);
+    return run_scan(b, rm, m);
 }
 
 cudaError_t launch_ticket_scan(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m)
@@ -1146,7 +1174,7 @@ cudaError_t launch_ticket_scan(gputx_bulk *b, const uint32_t *sk, const uint32_t
                   (uint32_t)(hot > 0xffffffffll ? 0xffffffffll : hot), b->db->dev.n_objects, &b->ctl->err};
     cudaError_t e = cudaMemsetAsync(&b->ctl->hot, 0, sizeof(uint32_t), b->stream);
     if (e) return e;
-    return run_scan(b, tm, m, 2);
+    return run_scan(b, tm, m);
 }
 
 cudaError_t launch_depth_flow(gputx_bulk *b, const uint32_t *sv, int64_t m)
@@ -1223,7 +1251,7 @@ cudaError_t launch_level_tables(gputx_bulk *b, const uint32_t *skeys, int64_t de
     // graph bulks do not know their depth on the host: scan every possible level
     const int64_t levels = b->graph ? b->n : depth + 1;
     ChunkMode cm{b->sc.level_off, b->sc.chunk_off, (uint32_t)block, b->ctl, b->sc.type_cut};
-    cudaError_t e = run_scan(b, cm, levels, 3);
+    cudaError_t e = run_scan(b, cm, levels);
     if (e) return e;
     chunk_level_kernel<<<grid_for(b->sc.chunk_cap), TB, 0, s>>>(b->sc.chunk_off, b->ctl, b->sc.chunk_level,
                                                                 b->sc.chunk_cap, &b->ctl->err);
@@ -1253,7 +1281,7 @@ cudaError_t launch_insert_slots(gputx_bulk *b)
     if (b->n == 0) return cudaSuccess;
     if (b->sc.slot_hist) {
         HistSlotMode hm{b->type, b->n, b->sc.slot_hist, b->ctl};
-        cudaError_t e = run_scan(b, hm, b->n, 7);
+        cudaError_t e = run_scan(b, hm, b->n);
         if (e) return e;
     }
     const uint32_t reg = b->db->dev.registered;
@@ -1261,10 +1289,10 @@ cudaError_t launch_insert_slots(gputx_bulk *b)
     const bool oe_no = (reg >> GPUTX_T_OE_NEW_ORDER) & 1u;
     if (!sub_ins && !oe_no) return cudaSuccess;
     SlotMode m0{b->type, b->params, b->P, b->n, b->sc.slot_cf, b->sc.slot_ord, b->ctl, 0};
-    cudaError_t e = run_scan(b, m0, b->n, 5);
+    cudaError_t e = run_scan(b, m0, b->n);
     if (e || !oe_no) return e;
     SlotMode m1{b->type, b->params, b->P, b->n, nullptr, b->sc.slot_ol, b->ctl, 1};
-    return run_scan(b, m1, b->n, 6);
+    return run_scan(b, m1, b->n);
 }
 
 cudaError_t launch_part_heads(gputx_bulk *b, const uint32_t *skeys, int64_t n)
@@ -1276,7 +1304,7 @@ cudaError_t launch_part_heads(gputx_bulk *b, const uint32_t *skeys, int64_t n)
     hm.ctl = b->ctl;
     hm.n = n;
     hm.n_live = b->graph ? &b->ctl->n_live : nullptr;
-    return run_scan(b, hm, n, 4);
+    return run_scan(b, hm, n);
 }
 
 cudaError_t launch_tpl_reset(gputx_bulk *b, const uint32_t *skeys, int64_t m)

@@ -204,10 +204,11 @@ size_t carve_bulk(gputx_bulk *b, char *base, bool device_inputs)
     s.chunk_level = c.take<uint32_t>(s.chunk_cap);
     s.done = c.take<uint32_t>(nn + 1);
     s.part_start = c.take<uint32_t>(nn + 1);
-    s.pid_key = c.take<uint32_t>(nn);
-    s.pid_val = c.take<uint32_t>(nn);
-    s.pid_key2 = c.take<uint32_t>(nn);
-    s.pid_val2 = c.take<uint32_t>(nn);
+    // partitions are sorted instead of operations, never beside them
+    s.pid_key = s.keys_a;
+    s.pid_val = s.vals_a;
+    s.pid_key2 = s.keys_b;
+    s.pid_val2 = s.vals_b;
     s.rec_params = c.take<int64_t>(nn * b->P);
     s.rec_ts = c.take<int64_t>(nn);
     s.rec_type = c.take<int32_t>(nn);
@@ -218,14 +219,11 @@ size_t carve_bulk(gputx_bulk *b, char *base, bool device_inputs)
     s.slot_ord = slots ? c.take<uint32_t>(nn) : nullptr;
     s.slot_ol = slots ? c.take<uint32_t>(nn) : nullptr;
     s.slot_hist = db->hist_by_type ? c.take<uint32_t>(nn) : nullptr;
-    s.sort_hist = c.take<uint32_t>(4 * 256);
-    s.sort_offs = c.take<uint32_t>(4 * 256);
     const int64_t big = std::max(mm, nn + 2);
-    s.sort_tiles = (big + 8191) / 8192;
-    s.sort_status = c.take<uint32_t>(4 * s.sort_tiles * 256);
-    s.tile_ctr = c.take<uint32_t>(16);
+    s.sort_words = sort_scratch_words(big);
+    s.sort_zero = c.take<uint32_t>(s.sort_words);
     s.scan_tiles = (big + 2047) / 2048;
-    s.scan_status = c.take<uint64_t>(s.scan_tiles);
+    s.scan_zero = c.take<uint64_t>(1 + s.scan_tiles);
     s.scan_vals = c.take<uint64_t>(2 * s.scan_tiles);
     s.rec_dc = db->dev.registered == (1u << GPUTX_T_DC_DEBIT_CREDIT) ? c.take<DcRecord>(nn) : nullptr;
     s.seg_off = b->graph ? c.take<uint32_t>(kSegMax + 1) : nullptr;

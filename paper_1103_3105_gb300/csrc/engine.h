@@ -44,17 +44,14 @@ struct Scratch {
     uint32_t *chunk_level; // n + n/min_block + 2
     uint32_t *done;        // n+1 per-level completion counters
     uint32_t *part_start;  // n
-    uint32_t *pid_key, *pid_val, *pid_key2, *pid_val2;  // PART sort, n each
+    uint32_t *pid_key, *pid_val, *pid_key2, *pid_val2;  // PART sort, n each (the op buffers: PART sorts no ops)
     int64_t *rec_params, *rec_ts;  // signatures gathered into execution order
     int32_t *rec_type;
     uint32_t *rec_t;
     uint32_t *slot_cf, *slot_ord, *slot_ol;   // n each
     uint32_t *slot_hist;   // n: history rows of debit-credit transactions in mixed databases
-    uint32_t *sort_hist;   // 4 x 256
-    uint32_t *sort_offs;   // 4 x 256
-    uint32_t *sort_status; // 4 x tiles x 256
-    uint32_t *tile_ctr;    // 16 counters
-    uint64_t *scan_status; // tiles
+    uint32_t *sort_zero;   // a sort's tile counters, digit counts and look-back words, cleared by it at once
+    uint64_t *scan_zero;   // a scan's tile counter and look-back words, likewise
     uint64_t *scan_vals;   // 2 x tiles: per-tile values of 64-bit scans
     DcRecord *rec_dc;      // n packed debit-credit records (debit-credit-only databases)
     // graph bulks that carry a segment of several bulks
@@ -63,7 +60,7 @@ struct Scratch {
     uint32_t *seg_depth;   // kSegMax: largest level of each bulk
     uint32_t *seg_base;    // kSegMax + 1: first global level of each bulk
     int64_t m_cap;         // op capacity
-    int64_t sort_tiles, scan_tiles, chunk_cap;
+    int64_t sort_words, scan_tiles, chunk_cap;   // capacity of sort_zero (words), of the scans (tiles)
 };
 
 }  // namespace gtx
@@ -148,6 +145,7 @@ cudaError_t launch_seg_levels(gputx_bulk *b);
 // PART in a graph: flags a segment with cross-partition transactions (it
 // then runs nothing and is re-run with TPL)
 cudaError_t launch_part_fallback_check(gputx_bulk *b);
+int64_t sort_scratch_words(int64_t count);   // scratch of a sort of up to `count` pairs
 cudaError_t launch_sort(gputx_bulk *b, uint32_t *&keys, uint32_t *&vals, uint32_t *&keys_alt,
                         uint32_t *&vals_alt, int64_t count, int bits);
 cudaError_t launch_rank_scan(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m, bool want_rid);

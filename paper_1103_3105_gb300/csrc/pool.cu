@@ -224,16 +224,15 @@ __global__ void pool_head_kernel(const uint8_t *pending, int64_t head, int64_t c
 inline unsigned blocks_for(int64_t n, int t = 256) { return (unsigned)std::max<int64_t>(1, (n + t - 1) / t); }
 
 template <class Mode>
-cudaError_t pool_scan(gputx_bulk *b, const Mode &mode, int64_t count, int ctr_slot)
+cudaError_t pool_scan(gputx_bulk *b, const Mode &mode, int64_t count)
 {
     if (count <= 0) return cudaSuccess;
     const int64_t tiles = (count + SCAN_TILE - 1) / SCAN_TILE;
     if (tiles > b->sc.scan_tiles) return cudaErrorInvalidValue;
-    cudaError_t e = cudaMemsetAsync(b->sc.scan_status, 0, tiles * sizeof(uint64_t), b->stream);
-    if (!e) e = cudaMemsetAsync(b->sc.tile_ctr + ctr_slot, 0, sizeof(uint32_t), b->stream);
+    cudaError_t e = cudaMemsetAsync(b->sc.scan_zero, 0, (1 + tiles) * sizeof(uint64_t), b->stream);
     if (e) return e;
     dualseg_scan_kernel<Mode><<<(unsigned)tiles, SCAN_THREADS, 0, b->stream>>>(
-        mode, count, b->sc.scan_status, b->sc.tile_ctr + ctr_slot, &b->ctl->err,
+        mode, count, b->sc.scan_zero + 1, (uint32_t *)b->sc.scan_zero, &b->ctl->err,
         (uint64_t)b->db->cfg.spin_limit_ns);
     count_launches(1);
     return cudaGetLastError();
@@ -450,9 +449,9 @@ gputx_status gputx_pool_step(gputx_pool *p, size_t *executed)
     PCK(cudaMemsetAsync(b->ctl, 0, sizeof(BulkCtl), s), "step");
     // ranks over the pool's sorted operations: rank > 0 blocks the transaction
     ZeroMode zm{p->a_key, p->a_val, p->r_blocked, step};
-    PCK(pool_scan(b, zm, p->m_pool, 13), "ranks");
+    PCK(pool_scan(b, zm, p->m_pool), "ranks");
     SelectMode sm{p->r_pending, p->r_blocked, p->sel, p->cnt, p->head, p->cap, span, step};
-    PCK(pool_scan(b, sm, span, 14), "select");
+    PCK(pool_scan(b, sm, span), "select");
     gputx_status st = read_counters(p);
     if (st) return st;
     const int64_t n0 = p->h_cnt[C_ZERO];
@@ -476,7 +475,7 @@ gputx_status gputx_pool_step(gputx_pool *p, size_t *executed)
     // the executed transactions' operations leave the sorted array
     if (p->m_pool > 0) {
         KeepMode km{p->a_key, p->a_val, p->c_key, p->c_val, p->cnt, p->r_pending, p->m_pool};
-        PCK(pool_scan(b, km, p->m_pool, 15), "compact");
+        PCK(pool_scan(b, km, p->m_pool), "compact");
     }
     PCK(cudaMemsetAsync(p->cnt + C_HEAD, 0xff, sizeof(uint32_t), s), "head");
     pool_head_kernel<<<blocks_for(span), 256, 0, s>>>(p->r_pending, p->head, p->cap, span, p->cnt);

@@ -1,5 +1,5 @@
-// scan.cuh -- single-pass tile scans with decoupled look-back, and the
-// onesweep LSD radix sort used by the dependency analysis (Section 4.2 steps
+// scan.cuh -- single-pass tile scans with decoupled look-back, and the LSD
+// radix sort used by the dependency analysis (Section 4.2 steps
 // 1 and 4: "a sort operation to perform grouping").
 //
 // Both follow published designs: decoupled look-back (Merrill & Garland,
@@ -357,178 +357,348 @@ seg64_scan_kernel(Mode mode, int64_t count, Seg64Status st, uint32_t *tile_ctr, 
 }
 
 // ===========================================================================
-// onesweep LSD radix sort of (u32 key, u32 value) pairs, 8-bit digits
+// LSD radix sort of (u32 key, u32 value) pairs
 // ===========================================================================
+// Up to SMALL_SORT pairs: one CTA sorts them in shared memory, one launch.
+// Above: a histogram of every digit, then one onesweep pass per digit.
+//
+// What bounds a pass is the latency of a tile (claim, load, rank, look back,
+// reorder, store), not bandwidth: 2^22 pairs are 67 MB, 10 us at the copy
+// rate, and a pass takes 46 us; 200,000 pairs take 10 us.  Hence
+//   * tiles of 2,048 pairs up to 2^19 pairs, where they are what fills the
+//     chip (a pass over 200,000 pairs: 10.1 us, 14.9 with tiles of 8,192;
+//     over 20,000: 7.5 and 13.7), and of 8,192 above, where longer runs per
+//     digit make the stores cheaper (2^22: 46 us, 58 with tiles of 2,048);
+//   * 10-bit digits where they save a pass (9-10, 17-20, 25-30 key bits): a
+//     10-bit pass costs 1.4 to 1.6 of an 8-bit one (2^22: 67 us against two
+//     passes of 47, 200,000: 16 against 20), and it is a launch less;
+//   * each pass scans its digit counts itself instead of a launch between.
 // (internal linkage: each translation unit that includes this header gets
 // its own copy of these kernels)
 namespace {
 constexpr int SORT_THREADS = 512;
-constexpr int SORT_ITEMS = 16;
-constexpr int SORT_TILE = SORT_THREADS * SORT_ITEMS;
 constexpr int SORT_WARPS = SORT_THREADS / 32;
-constexpr int RADIX = 256;
+constexpr int64_t SORT_WIDE_FROM = 1 << 19;   // pairs above which a tile holds 16 per thread, not 4
+constexpr int SMALL_SORT_THREADS = 1024, SMALL_SORT_ITEMS = 4;
+constexpr int SMALL_SORT = SMALL_SORT_THREADS * SMALL_SORT_ITEMS;
 constexpr uint32_t ST_AGG = 1u << 30, ST_INC = 2u << 30, ST_VAL = (1u << 30) - 1;
-constexpr size_t SORT_SMEM = (size_t)SORT_TILE * 8 + (size_t)SORT_WARPS * RADIX * 4;
 
-// Histograms of every digit position in one pass over the keys.
-__global__ void __launch_bounds__(256) radix_hist_kernel(const uint32_t *__restrict__ keys, int64_t n,
-                                                         int passes, uint32_t *hist, const uint32_t *err)
+struct SortShape {
+    int digit_bits, passes, items;
+    int64_t tiles;
+    __host__ __device__ int digits() const { return 1 << digit_bits; }
+};
+inline SortShape sort_shape(int64_t count, int bits)
 {
-    __shared__ uint32_t sh[4][RADIX];
-    __shared__ uint32_t s_abort;
-    if (threadIdx.x == 0) s_abort = *(volatile const uint32_t *)err;
+    const int p8 = (bits + 7) / 8, p10 = (bits + 9) / 10;
+    SortShape s;
+    s.digit_bits = p10 < p8 ? 10 : 8;
+    s.passes = p10 < p8 ? p10 : p8;
+    s.items = count <= SORT_WIDE_FROM ? 4 : 16;
+    s.tiles = (count + (int64_t)SORT_THREADS * s.items - 1) / ((int64_t)SORT_THREADS * s.items);
+    return s;
+}
+
+// lanes of the warp whose digit is this lane's (`ok` lanes only)
+template <int RB> __device__ __forceinline__ uint32_t digit_peers(uint32_t d, bool ok)
+{
+    uint32_t peers = __ballot_sync(0xffffffffu, ok);
+#pragma unroll
+    for (int b = 0; b < RB; b++) {
+        const uint32_t m = __ballot_sync(0xffffffffu, (d >> b) & 1u);
+        peers &= ((d >> b) & 1u) ? m : ~m;
+    }
+    return peers;
+}
+
+// The stable rank of each of this lane's items among its warp's items of the
+// same digit; wh[digit] ends as the warp's count.  Items are striped over the
+// warp: item j of lane l is element 32 j + l.
+template <int RB, int ITEMS>
+__device__ __forceinline__ void warp_digit_ranks(const uint32_t (&key)[ITEMS], int shift, uint32_t wbase, uint32_t n,
+                                                 uint16_t *wh, uint16_t (&rank)[ITEMS])
+{
+    const uint32_t lt = lanemask_lt();
+#pragma unroll
+    for (int j = 0; j < ITEMS; j++) {
+        const bool ok = wbase + j * 32 < n;
+        const uint32_t d = (key[j] >> shift) & ((1u << RB) - 1u);
+        const uint32_t peers = digit_peers<RB>(d, ok);
+        uint32_t prior = 0;
+        if (ok) prior = wh[d];
+        __syncwarp();
+        rank[j] = (uint16_t)(prior + __popc(peers & lt));
+        if (ok && (peers & lt) == 0) wh[d] = (uint16_t)(prior + __popc(peers));
+        __syncwarp();
+    }
+}
+
+// every digit position of up to SMALL_SORT pairs in one CTA: the pairs live in
+// registers, each digit reorders them through shared memory
+__global__ void __launch_bounds__(SMALL_SORT_THREADS, 1)
+radix_small_kernel(const uint32_t *__restrict__ kin, const uint32_t *__restrict__ vin, uint32_t *__restrict__ kout,
+                   uint32_t *__restrict__ vout, uint32_t n, int bits, const uint32_t *err)
+{
+    constexpr int ITEMS = SMALL_SORT_ITEMS, D = 256, W = SMALL_SORT_THREADS / 32;
+    __shared__ uint32_t s_kv[SMALL_SORT];
+    __shared__ uint16_t s_whist[W * D];
+    __shared__ uint32_t s_start[D], s_w[D / 32], s_abort;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) s_abort = *(volatile const uint32_t *)err;
+    const uint32_t wbase = warp * 32 * ITEMS + lane;
+    uint32_t key[ITEMS], val[ITEMS];
+    uint16_t rank[ITEMS];
+#pragma unroll
+    for (int j = 0; j < ITEMS; j++) {
+        const uint32_t i = wbase + j * 32;
+        key[j] = i < n ? kin[i] : 0xffffffffu;
+        val[j] = i < n ? vin[i] : 0u;
+    }
     __syncthreads();
     if (s_abort) return;
-    for (int i = threadIdx.x; i < 4 * RADIX; i += blockDim.x) (&sh[0][0])[i] = 0;
+    uint16_t *wh = s_whist + warp * D;
+    for (int shift = 0; shift < bits; shift += 8) {
+        for (int i = lane; i < D / 2; i += 32) ((uint32_t *)wh)[i] = 0;
+        __syncwarp();
+        warp_digit_ranks<8, ITEMS>(key, shift, wbase, n, wh, rank);
+        __syncthreads();
+        uint32_t cnt = 0, x = 0;
+        if (tid < D) {
+            uint16_t c[W];
+#pragma unroll
+            for (int w = 0; w < W; w++) c[w] = s_whist[w * D + tid];
+#pragma unroll
+            for (int w = 0; w < W; w++) {
+                s_whist[w * D + tid] = (uint16_t)cnt;
+                cnt += c[w];
+            }
+            x = cnt;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const uint32_t o = __shfl_up_sync(0xffffffffu, x, off);
+                if (lane >= off) x += o;
+            }
+            if (lane == 31) s_w[warp] = x;
+        }
+        __syncthreads();
+        if (tid < D) {
+            uint32_t a = x - cnt;
+            for (int w = 0; w < warp; w++) a += s_w[w];
+            s_start[tid] = a;
+        }
+        __syncthreads();
+        uint32_t pos[ITEMS];
+#pragma unroll
+        for (int j = 0; j < ITEMS; j++) {
+            const uint32_t d = (key[j] >> shift) & (D - 1);
+            pos[j] = s_start[d] + wh[d] + rank[j];
+        }
+        // keys, then values, through one buffer
+#pragma unroll
+        for (int j = 0; j < ITEMS; j++)
+            if (wbase + j * 32 < n) s_kv[pos[j]] = key[j];
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < ITEMS; j++)
+            if (wbase + j * 32 < n) key[j] = s_kv[wbase + j * 32];
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < ITEMS; j++)
+            if (wbase + j * 32 < n) s_kv[pos[j]] = val[j];
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < ITEMS; j++)
+            if (wbase + j * 32 < n) val[j] = s_kv[wbase + j * 32];
+    }
+#pragma unroll
+    for (int j = 0; j < ITEMS; j++) {
+        const uint32_t i = wbase + j * 32;
+        if (i < n) {
+            kout[i] = key[j];
+            vout[i] = val[j];
+        }
+    }
+}
+
+// Histograms of every digit position in one pass over the keys.
+template <int RB>
+__global__ void __launch_bounds__(256) radix_hist_kernel(const uint32_t *__restrict__ keys, int64_t n, int passes,
+                                                         uint32_t *hist, const uint32_t *err)
+{
+    constexpr int D = 1 << RB, MAXP = (32 + RB - 1) / RB;
+    __shared__ uint32_t sh[MAXP * D];
+    __shared__ uint32_t s_abort;
+    if (threadIdx.x == 0) s_abort = *(volatile const uint32_t *)err;
+    for (int i = threadIdx.x; i < passes * D; i += blockDim.x) sh[i] = 0;
     __syncthreads();
+    if (s_abort) return;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t k = keys[i];
-        for (int p = 0; p < passes; p++) atomicAdd(&sh[p][(k >> (8 * p)) & 255u], 1u);
+        for (int p = 0; p < passes; p++) atomicAdd(&sh[p * D + ((k >> (RB * p)) & (D - 1))], 1u);
     }
     __syncthreads();
-    for (int p = 0; p < passes; p++)
-        for (int d = threadIdx.x; d < RADIX; d += blockDim.x)
-            if (sh[p][d]) atomicAdd(&hist[p * RADIX + d], sh[p][d]);
+    for (int i = threadIdx.x; i < passes * D; i += blockDim.x)
+        if (sh[i]) atomicAdd(&hist[i], sh[i]);
 }
 
-// Exclusive scan of each pass's 256 counts (one block per pass).
-__global__ void __launch_bounds__(RADIX) radix_offsets_kernel(const uint32_t *hist, uint32_t *offs)
+template <int RB, int ITEMS> constexpr size_t radix_smem()
 {
-    __shared__ uint32_t s[RADIX];
-    const uint32_t *h = hist + blockIdx.x * RADIX;
-    uint32_t v = h[threadIdx.x];
-    s[threadIdx.x] = v;
-    __syncthreads();
-    for (int off = 1; off < RADIX; off <<= 1) {
-        uint32_t o = threadIdx.x >= off ? s[threadIdx.x - off] : 0;
-        __syncthreads();
-        s[threadIdx.x] += o;
-        __syncthreads();
-    }
-    offs[blockIdx.x * RADIX + threadIdx.x] = s[threadIdx.x] - v;
+    return (size_t)SORT_THREADS * ITEMS * 8 + (size_t)SORT_WARPS * (1 << RB) * sizeof(uint16_t);
 }
 
-// One stable counting pass on digit (key >> shift) & 255.
+// One stable counting pass on digit (key >> shift); hist = the digit's counts
+// over all keys.
+template <int RB, int ITEMS>
 __global__ void __launch_bounds__(SORT_THREADS, 2)
 radix_pass_kernel(const uint32_t *__restrict__ kin, const uint32_t *__restrict__ vin, uint32_t *__restrict__ kout,
-                  uint32_t *__restrict__ vout, int64_t n, int shift, const uint32_t *__restrict__ digit_off,
+                  uint32_t *__restrict__ vout, uint32_t n, int shift, const uint32_t *__restrict__ hist,
                   uint32_t *status, uint32_t *tile_ctr, uint32_t *err, uint64_t spin_limit_ns)
 {
-    extern __shared__ uint32_t smem[];
+    constexpr int D = 1 << RB, TILE = SORT_THREADS * ITEMS;
+    constexpr int DPT = (D + SORT_THREADS - 1) / SORT_THREADS;   // digits per thread
+    constexpr int LOOK = 4;                                      // predecessors per look
+    extern __shared__ __align__(16) uint32_t smem[];
     uint32_t *s_keys = smem;
-    uint32_t *s_vals = smem + SORT_TILE;
-    uint32_t *s_whist = s_vals + SORT_TILE;  // [SORT_WARPS][RADIX]
-    __shared__ uint32_t s_tile;
-    __shared__ uint32_t s_start[RADIX];      // tile-local start of each digit
-    __shared__ int64_t s_gbase[RADIX];       // global position of the digit's first tile element
-    __shared__ uint32_t s_scan[RADIX / 32];
-
-    __shared__ uint32_t s_abort;
+    uint32_t *s_vals = smem + TILE;
+    uint16_t *s_whist = (uint16_t *)(smem + 2 * TILE);  // [SORT_WARPS][D]: at most 32 ITEMS a warp
+    __shared__ uint32_t s_tile, s_abort;
+    __shared__ uint32_t s_start[D];          // tile-local start of each digit
+    __shared__ uint32_t s_gbase[D];          // its global position minus that start (modulo 2^32)
+    __shared__ uint32_t s_wt[SORT_WARPS], s_wg[SORT_WARPS];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {   // block-uniform abort decision, see dualseg_scan_kernel
         s_abort = *(volatile uint32_t *)err;
         if (!s_abort) s_tile = atomicAdd(tile_ctr, 1u);
     }
-    for (int i = tid; i < SORT_WARPS * RADIX; i += SORT_THREADS) s_whist[i] = 0;
+    for (int i = tid; i < SORT_WARPS * D / 2; i += SORT_THREADS) ((uint32_t *)s_whist)[i] = 0;
     __syncthreads();
     if (s_abort) return;
     const uint32_t tile = s_tile;
-    const int64_t base = (int64_t)tile * SORT_TILE;
-    const int64_t wbase = base + (int64_t)warp * 32 * SORT_ITEMS;
-
-    uint32_t key[SORT_ITEMS], val[SORT_ITEMS], rank[SORT_ITEMS];
+    const uint32_t base = tile * TILE;
+    const uint32_t wbase = base + (uint32_t)warp * 32 * ITEMS + lane;
+    uint32_t key[ITEMS], val[ITEMS];
+    uint16_t rank[ITEMS];
 #pragma unroll
-    for (int j = 0; j < SORT_ITEMS; j++) {
-        const int64_t i = wbase + j * 32 + lane;
+    for (int j = 0; j < ITEMS; j++) {
+        const uint32_t i = wbase + j * 32;
         const bool ok = i < n;
         key[j] = ok ? kin[i] : 0xffffffffu;
         val[j] = ok ? vin[i] : 0u;
     }
-    uint32_t *wh = s_whist + warp * RADIX;
-    const uint32_t lt = lanemask_lt();
+    uint32_t all[DPT];                       // the digit counts over all keys
 #pragma unroll
-    for (int j = 0; j < SORT_ITEMS; j++) {
-        const int64_t i = wbase + j * 32 + lane;
-        const bool ok = i < n;
-        const uint32_t d = (key[j] >> shift) & 255u;
-        uint32_t peers = __ballot_sync(0xffffffffu, ok);
-#pragma unroll
-        for (int b = 0; b < 8; b++) {
-            const uint32_t m = __ballot_sync(0xffffffffu, (d >> b) & 1u);
-            peers &= ((d >> b) & 1u) ? m : ~m;
-        }
-        uint32_t prior = 0;
-        if (ok) prior = wh[d];
-        __syncwarp();
-        if (ok) {
-            rank[j] = prior + __popc(peers & lt);
-            if ((peers & lt) == 0) wh[d] = prior + __popc(peers);
-        }
-        __syncwarp();
-    }
+    for (int q = 0; q < DPT; q++) all[q] = tid * DPT < D ? __ldg(&hist[tid * DPT + q]) : 0u;
+    uint16_t *wh = s_whist + warp * D;
+    warp_digit_ranks<RB, ITEMS>(key, shift, wbase, n, wh, rank);
     __syncthreads();
 
     // per digit: exclusive prefix over warps, tile count, look-back
-    uint32_t cnt = 0;
-    if (tid < RADIX) {
-        for (int w = 0; w < SORT_WARPS; w++) {
-            const uint32_t c = s_whist[w * RADIX + tid];
-            s_whist[w * RADIX + tid] = cnt;
-            cnt += c;
+    uint32_t cnt[DPT], excl[DPT], tsum = 0, gsum = 0;
+#pragma unroll
+    for (int q = 0; q < DPT; q++) cnt[q] = excl[q] = 0;
+    if (tid * DPT < D) {
+#pragma unroll
+        for (int q = 0; q < DPT; q++) {
+            const int d = tid * DPT + q;
+            uint16_t c[SORT_WARPS];
+#pragma unroll
+            for (int w = 0; w < SORT_WARPS; w++) c[w] = s_whist[w * D + d];
+            uint32_t a = 0;
+#pragma unroll
+            for (int w = 0; w < SORT_WARPS; w++) {
+                s_whist[w * D + d] = (uint16_t)a;
+                a += c[w];
+            }
+            cnt[q] = a;
+            st_relaxed_u32(status + (size_t)tile * D + d, (tile == 0 ? ST_INC : ST_AGG) | a);
+            tsum += a;
+            gsum += all[q];
         }
-        uint32_t *st = status + (int64_t)tile * RADIX + tid;
-        uint32_t excl = 0;
-        if (tile == 0) {
-            st_relaxed_u32(st, ST_INC | cnt);
-        } else {
-            st_relaxed_u32(st, ST_AGG | cnt);
+    }
+    // exclusive scans over the digits: the tile's counts and those of all keys
+    uint32_t xt = tsum, xg = gsum;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t ot = __shfl_up_sync(0xffffffffu, xt, off), og = __shfl_up_sync(0xffffffffu, xg, off);
+        if (lane >= off) {
+            xt += ot;
+            xg += og;
+        }
+    }
+    if (lane == 31) {
+        s_wt[warp] = xt;
+        s_wg[warp] = xg;
+    }
+    if (tid * DPT < D && tile > 0) {
+#pragma unroll
+        for (int q = 0; q < DPT; q++) {
+            const int d = tid * DPT + q;
             int64_t t = (int64_t)tile - 1;
             const uint64_t t0 = globaltimer();
-            while (t >= 0) {
-                const uint32_t s = ld_relaxed_u32(status + t * RADIX + tid);
-                if (s & ST_INC) { excl += s & ST_VAL; break; }
-                if (s & ST_AGG) { excl += s & ST_VAL; t--; continue; }
-                if (globaltimer() - t0 > spin_limit_ns) { set_err(err, ERR_TIMEOUT); break; }
+            bool done = false;
+            while (!done) {
+                uint32_t s[LOOK];
+#pragma unroll
+                for (int u = 0; u < LOOK; u++)
+                    s[u] = t - u >= 0 ? ld_relaxed_u32(status + (size_t)(t - u) * D + d) : ST_INC;
+                int used = 0;                // nearest first, up to the first not yet published
+#pragma unroll
+                for (int u = 0; u < LOOK; u++) {
+                    if (done || used < u || !(s[u] & (ST_INC | ST_AGG))) continue;
+                    excl[q] += s[u] & ST_VAL;
+                    used = u + 1;
+                    done = (s[u] & ST_INC) != 0;
+                }
+                t -= used;
+                if (!done && !used && globaltimer() - t0 > spin_limit_ns) {
+                    set_err(err, ERR_TIMEOUT);
+                    done = true;
+                }
             }
-            st_relaxed_u32(st, ST_INC | (excl + cnt));
+            st_relaxed_u32(status + (size_t)tile * D + d, ST_INC | (excl[q] + cnt[q]));
         }
-        // exclusive scan of the tile counts over digits (8 warps of 32)
-        uint32_t x = cnt;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            uint32_t o = __shfl_up_sync(0xffffffffu, x, off);
-            if (lane >= off) x += o;
-        }
-        if (lane == 31) s_scan[warp] = x;
-        s_start[tid] = x - cnt;  // within-warp exclusive for now
-        s_gbase[tid] = (int64_t)digit_off[tid] + excl;
     }
     __syncthreads();
-    if (tid < RADIX) {
-        uint32_t add = 0;
-        for (int w = 0; w < warp; w++) add += s_scan[w];
-        s_start[tid] += add;
+    if (tid * DPT < D) {
+        uint32_t at = xt - tsum, ag = xg - gsum;
+        for (int w = 0; w < warp; w++) {
+            at += s_wt[w];
+            ag += s_wg[w];
+        }
+#pragma unroll
+        for (int q = 0; q < DPT; q++) {
+            const int d = tid * DPT + q;
+            s_start[d] = at;
+            s_gbase[d] = ag + excl[q] - at;
+            at += cnt[q];
+            ag += all[q];
+        }
     }
     __syncthreads();
 #pragma unroll
-    for (int j = 0; j < SORT_ITEMS; j++) {
-        const int64_t i = wbase + j * 32 + lane;
-        if (i < n) {
-            const uint32_t d = (key[j] >> shift) & 255u;
-            const uint32_t pos = s_start[d] + s_whist[warp * RADIX + d] + rank[j];
+    for (int j = 0; j < ITEMS; j++) {
+        if (wbase + j * 32 < n) {
+            const uint32_t d = (key[j] >> shift) & (D - 1);
+            const uint32_t pos = s_start[d] + wh[d] + rank[j];
             s_keys[pos] = key[j];
             s_vals[pos] = val[j];
         }
     }
     __syncthreads();
-    const int64_t tile_n = (n - base) < SORT_TILE ? (n - base) : SORT_TILE;
-    for (int i = tid; i < tile_n; i += SORT_THREADS) {
-        const uint32_t k = s_keys[i];
-        const uint32_t d = (k >> shift) & 255u;
-        const int64_t g = s_gbase[d] + (i - (int64_t)s_start[d]);
-        if (g < 0 || g >= n) { set_err(err, ERR_BOUNDS); continue; }  // only after a timeout
-        kout[g] = k;
-        vout[g] = s_vals[i];
+    const uint32_t tile_n = (n - base) < TILE ? (n - base) : TILE;
+#pragma unroll
+    for (int j = 0; j < ITEMS; j++) {
+        const uint32_t i = tid + j * SORT_THREADS;
+        if (i < tile_n) {
+            const uint32_t k = s_keys[i];
+            const uint32_t g = s_gbase[(k >> shift) & (D - 1)] + i;
+            if (g < n) {
+                kout[g] = k;
+                vout[g] = s_vals[i];
+            } else {
+                set_err(err, ERR_BOUNDS);   // only after a timeout
+            }
+        }
     }
 }
 
