@@ -26,11 +26,14 @@ inline unsigned grid_for(int64_t n, int block = TB)
 // ---------------------------------------------------------------------------
 // bulk begin / finish: insert bases from the device cursors
 // ---------------------------------------------------------------------------
-// hist_rows < 0: the history rows were counted by the insert-slot scan
-__global__ void begin_kernel(const InsertBase *cursor, BulkCtl *ctl, int64_t hist_rows, bool live_rows)
+// hist_rows < 0: the history rows were counted by the insert-slot scan;
+// hist_cap >= 0: the bulk's history rows all fit, or nothing of it runs
+__global__ void begin_kernel(const InsertBase *cursor, BulkCtl *ctl, int64_t hist_rows, bool live_rows,
+                             int64_t hist_cap)
 {
     ctl->base = *cursor;
     if (hist_rows >= 0) ctl->total.hist = live_rows ? (int64_t)ctl->n_live : hist_rows;
+    if (hist_cap >= 0 && ctl->base.hist + ctl->total.hist > hist_cap) set_err(&ctl->err, ERR_CAPACITY);
 }
 
 __global__ void finish_kernel(InsertBase *cursor, const BulkCtl *ctl)
@@ -134,6 +137,69 @@ __global__ void extract_kernel(ExtractArgs a)
     if ((threadIdx.x & 31) == 0 && cross_mask) atomicAdd(&a.ctl->cross, (uint32_t)__popc(cross_mask));
 }
 
+// Extraction of a bulk whose registered types have one operation each, with
+// the digit counts of the sort that follows (`hist`, RB-bit digits; null: that
+// sort counts for itself).  Without the general kernel's per-transaction
+// arrays it streams: 2^22 debit-credit transactions take 40 us, extraction and
+// counting in two kernels took 67.
+struct ExtractOneArgs {
+    DevDB db;
+    DevBulk b;
+    BulkCtl *ctl;
+    uint32_t *keys, *vals, *hist;
+    int64_t *deltas;               // debit-credit-only bulks: each transaction's delta side by side (or null)
+    int mode, part_size, passes;
+    bool by_part;                  // key = partition, payload = transaction (else the item and launch_extract's payload)
+};
+
+template <int RB> __global__ void __launch_bounds__(256) extract_one_kernel(ExtractOneArgs a)
+{
+    constexpr int D = 1 << RB, MAXP = (32 + RB - 1) / RB;
+    __shared__ uint32_t sh[MAXP * D];
+    if (a.hist) {
+        for (int i = threadIdx.x; i < a.passes * D; i += blockDim.x) sh[i] = 0;
+        __syncthreads();
+    }
+    // kTxns transactions of a thread at once, their loads in flight together
+    constexpr int kTxns = 4;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t0 < a.b.n; t0 += kTxns * step) {
+        int32_t type[kTxns];
+        int64_t p0[kTxns], ts[kTxns], before[kTxns];
+#pragma unroll
+        for (int u = 0; u < kTxns; u++) {
+            const int64_t t = t0 + u * step;
+            if (t >= a.b.n) continue;
+            type[u] = __ldg(&a.b.type[t]);
+            p0[u] = __ldg(&a.b.params[t * a.b.P]);
+            ts[u] = __ldg(&a.b.ts[t]);
+            before[u] = t ? __ldg(&a.b.ts[t - 1]) : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < kTxns; u++) {
+            const int64_t t = t0 + u * step;
+            if (t >= a.b.n) continue;
+            // an invalid transaction (the bulk will not execute) reads item 0
+            uint32_t obj = 0, cls = CLS_R, root = 0;
+            if (valid_txn(a.db, type[u], a.b.params + t * a.b.P, a.b.P) && (t == 0 || ts[u] > before[u]))
+                single_op(a.db, type[u], p0[u], a.mode, obj, cls, root);
+            else
+                set_err(&a.ctl->err, ERR_INVAL);
+            const uint32_t key = a.by_part ? root / (uint32_t)a.part_size : obj;
+            a.keys[t] = key;
+            a.vals[t] = a.by_part ? (uint32_t)t : ((uint32_t)t << 7) | cls;
+            if (a.deltas) a.deltas[t] = a.b.P > 1 ? __ldg(&a.b.params[t * a.b.P + 1]) : 0;
+            if (a.hist)
+                for (int q = 0; q < a.passes; q++) atomicAdd(&sh[q * D + ((key >> (RB * q)) & (D - 1))], 1u);
+        }
+    }
+    if (a.hist) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < a.passes * D; i += blockDim.x)
+            if (sh[i]) atomicAdd(&a.hist[i], sh[i]);
+    }
+}
+
 // exclusive op offsets from per-transaction counts
 struct OffsetMode {
     const uint32_t *cnt;
@@ -166,7 +232,9 @@ struct RankMode {
             const uint32_t c = v & 3u, pc = sv[i - 1] & 3u;
             runhead = !(c == pc && c != CLS_W);
         }
-        return DualSeg::make(head, head ? 0u : runhead, 0, runhead);
+        // the run ids run on over all groups; without them both fields start
+        // again at each group (cutting the scan's look-back)
+        return DualSeg::make(head, head ? 0u : runhead, rid ? 0u : head, runhead);
     }
     __device__ void output(int64_t i, uint64_t s) const
     {
@@ -594,25 +662,6 @@ struct HeadMode {
     }
 };
 
-// records of a debit-credit bulk packed in execution order (32 B: two
-// 16-byte loads), teller and branch precomputed
-__global__ void gather_dc_kernel(DevDB db, DevBulk b, const uint32_t *order, DcRecord *rec, const uint32_t *err)
-{
-    const int64_t pos = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (pos >= b.n || *err) return;
-    const uint32_t t = order[pos];
-    if (!dbg_in(t, b.n, b.err)) return;
-    const uint32_t a = (uint32_t)b.params[(int64_t)t * b.P];
-    DcRecord r;
-    r.delta = b.params[(int64_t)t * b.P + 1];
-    r.ts = b.ts[t];
-    r.a = a;
-    r.t = t;
-    r.tl = db.div_tel.div(a);
-    r.br = db.div_br.div(a);
-    rec[pos] = r;
-}
-
 __global__ void tpl_reset_kernel(const uint32_t *skeys, int64_t m, uint32_t *done, uint32_t n_objects,
                                  LockSlots slot)
 {
@@ -776,40 +825,138 @@ __global__ void part_scatter_kernel(int64_t n, const uint32_t *off, const uint32
 // Teller and branch balances only receive sums, and wrapping addition is
 // associative and commutative, so atomic adds give the serial result.
 // ---------------------------------------------------------------------------
-struct ScanExecMode {
+struct AcctScanArgs {
     const uint32_t *sk, *sv;     // operations grouped by account object id
-    const int64_t *params;
+    const int64_t *deltas;       // by transaction, side by side
     int64_t *acc_bal, *out;
-    int32_t *status;
-    int64_t m;
-    int P, R;
+    uint32_t m;
+    int R;
     uint32_t o_acc;
-    __device__ Seg64 element(int64_t i) const
-    {
-        const uint32_t k = sk[i], t = sv[i] >> 7;
-        const bool head = i == 0 || sk[i - 1] != k;
-        const uint64_t d = (uint64_t)__ldg(&params[(int64_t)t * P + 1]);
-        // the balance before the bulk matters only at the first operation on
-        // the account; loading it for every operation keeps the loads free of
-        // branches, so the tile's loads all overlap
-        const uint64_t bal = (uint64_t)__ldcg(&acc_bal[k - o_acc]);
-        return Seg64::make(head ? 1u : 0u, head ? bal + d : d);
-    }
-    __device__ void output(int64_t i, const Seg64 &s) const
-    {
-        const uint32_t k = sk[i], t = sv[i] >> 7;
-        out[(int64_t)t * R] = (int64_t)s.v;
-        // last operation on the account: its balance after the bulk (every
-        // tile reading this account's balance published its aggregate
-        // before this tile finished its look-back)
-        if (i == m - 1 || sk[i + 1] != k) __stcg(&acc_bal[k - o_acc], (int64_t)s.v);
-    }
+    BulkCtl *stats;              // K-SET: accounts are the graph's paths, d and w0 are recorded (or null)
+    Seg64Status st;
+    uint32_t *tile_ctr, *err;
+    uint64_t spin_limit_ns;
 };
 
-// the whole bulk's history rows fit, or nothing of it runs
-__global__ void scan_capacity_kernel(BulkCtl *ctl, int64_t n, int64_t hist_cap)
+// element i of a tile in shared memory: a thread's SCAN_ITEMS consecutive
+// elements lie 9 words of 8 bytes apart, so a warp's reads spread over the banks
+__device__ __forceinline__ uint32_t tile_at(uint32_t i) { return i + i / SCAN_ITEMS; }
+
+// A tile's keys, transactions, deltas and balances are loaded, and its results
+// stored, element by element across the CTA (thread t takes elements t, t + 256,
+// ...); the scan itself wants consecutive elements per thread, so the values
+// change places through shared memory.  What bounds it is the sectors touched
+// one by one: per element the signature's, the account's (read at a group's
+// head, written at its end) and the output's; with consecutive elements per
+// thread in global memory too, every load of keys and payloads (six an element)
+// touched 32 sectors a warp as well: 2^22 uniform accounts 125 us against 201.
+__global__ void __launch_bounds__(SCAN_THREADS, 6) acct_scan_kernel(AcctScanArgs a)
 {
-    if (ctl->base.hist + n > hist_cap) set_err(&ctl->err, ERR_CAPACITY);
+    __shared__ uint32_t s_tile, s_abort;
+    __shared__ Seg64 s_warp[SCAN_THREADS / 32];
+    __shared__ Seg64 s_prefix;
+    __shared__ uint64_t s_v[SCAN_TILE + SCAN_TILE / SCAN_ITEMS];
+    __shared__ uint32_t s_fc[SCAN_TILE + SCAN_TILE / SCAN_ITEMS];
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) {
+        s_abort = *(volatile uint32_t *)a.err;
+        if (!s_abort) s_tile = atomicAdd(a.tile_ctr, 1u);
+    }
+    __syncthreads();
+    if (s_abort) return;
+    const uint32_t tile = s_tile, base = tile * SCAN_TILE;
+    uint32_t t[SCAN_ITEMS];
+    uint32_t heads = 0, lasts = 0;         // bit j: element j begins, ends its account's group
+#pragma unroll
+    for (int j = 0; j < SCAN_ITEMS; j++) {
+        const uint32_t i = base + j * SCAN_THREADS + tid;
+        t[j] = 0;
+        if (i < a.m) {
+            const uint32_t k = __ldcs(&a.sk[i]);
+            t[j] = __ldcs(&a.sv[i]) >> 7;
+            if (i == 0 || __ldg(&a.sk[i - 1]) != k) heads |= 1u << j;
+            if (i == a.m - 1 || __ldg(&a.sk[i + 1]) != k) lasts |= 1u << j;
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < SCAN_ITEMS; j++) {
+        const uint32_t i = j * SCAN_THREADS + tid;
+        uint64_t v = 0;
+        uint32_t fc = 0;
+        if (base + i < a.m) {
+            v = (uint64_t)__ldg(&a.deltas[t[j]]);
+            // the balance before the bulk joins at the account's first operation
+            if (heads >> j & 1u) v += (uint64_t)__ldcs(&a.acc_bal[__ldg(&a.sk[base + i]) - a.o_acc]);
+            fc = 2u | (heads >> j & 1u);
+        }
+        s_v[tile_at(i)] = v;
+        s_fc[tile_at(i)] = fc;
+    }
+    __syncthreads();
+    Seg64 acc = Seg64::identity();
+#pragma unroll
+    for (int j = 0; j < SCAN_ITEMS; j++) {
+        const uint32_t i = tile_at(tid * SCAN_ITEMS + j);
+        acc = Seg64::combine(acc, Seg64{s_fc[i], s_v[i]});
+    }
+    Seg64 x = acc;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const Seg64 o = shfl_up_seg(x, off);
+        if (lane >= (uint32_t)off) x = Seg64::combine(o, x);
+    }
+    if (lane == 31) s_warp[warp] = x;
+    Seg64 thread_excl = shfl_up_seg(x, 1);
+    if (lane == 0) thread_excl = Seg64::identity();
+    __syncthreads();
+    if (warp == 0) {
+        Seg64 w = (lane < SCAN_THREADS / 32) ? s_warp[lane] : Seg64::identity();
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const Seg64 o = shfl_up_seg(w, off);
+            if (lane >= (uint32_t)off) w = Seg64::combine(o, w);
+        }
+        const Seg64 tile_agg = shfl_seg(w, SCAN_THREADS / 32 - 1);
+        Seg64 wexcl = shfl_up_seg(w, 1);
+        if (lane == 0) wexcl = Seg64::identity();
+        if (lane < SCAN_THREADS / 32) s_warp[lane] = wexcl;
+        const Seg64 pre = lookback_seg64(a.st, tile, tile_agg, a.err, a.spin_limit_ns);
+        if (lane == 0) s_prefix = pre;
+    }
+    __syncthreads();
+    acc = Seg64::combine(Seg64::combine(s_prefix, s_warp[warp]), thread_excl);
+#pragma unroll
+    for (int j = 0; j < SCAN_ITEMS; j++) {
+        const uint32_t i = tile_at(tid * SCAN_ITEMS + j);
+        acc = Seg64::combine(acc, Seg64{s_fc[i], s_v[i]});
+        s_v[i] = acc.v;
+        s_fc[i] = acc.fc;
+    }
+    __syncthreads();
+    uint32_t longest = 0;
+#pragma unroll
+    for (int j = 0; j < SCAN_ITEMS; j++) {
+        const uint32_t i = j * SCAN_THREADS + tid;
+        if (base + i < a.m) {
+            const int64_t v = (int64_t)s_v[tile_at(i)];
+            a.out[(int64_t)t[j] * a.R] = v;
+            // the account's balance after the bulk (every tile reading it
+            // published its aggregate before this tile finished its look-back)
+            if (lasts >> j & 1u) {
+                __stcs(&a.acc_bal[__ldg(&a.sk[base + i]) - a.o_acc], v);
+                const uint32_t len = s_fc[tile_at(i)] >> 1;   // the path's length
+                longest = len > longest ? len : longest;
+            }
+        }
+    }
+    if (a.stats) {
+        longest = __reduce_max_sync(0xffffffffu, longest);
+        const uint32_t paths = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(lasts));
+        if (lane == 0) {
+            if (longest > 1) atomicMax(&a.stats->depth, longest - 1);
+            if (paths) atomicAdd(&a.stats->w0, paths);
+        }
+    }
 }
 
 // history rows in timestamp order (slot = base + t) and the teller and branch
@@ -817,7 +964,7 @@ __global__ void scan_capacity_kernel(BulkCtl *ctl, int64_t n, int64_t hist_cap)
 // shared memory first (one slot per teller and branch) and each block adds
 // its non-zero sums once: the same-address atomics on the few branch rows
 // would otherwise serialise in L2.
-__global__ void scan_dc_rows_kernel(DevDB db, DevBulk b, const BulkCtl *ctl, bool local)
+__global__ void dc_rows_kernel(DevDB db, DevBulk b, const BulkCtl *ctl, bool local)
 {
     extern __shared__ unsigned long long sums[];   // [n_tel] tellers, then [n_br] branches
     const bool stop = ctl->err != 0;               // uniform: set before this launch
@@ -828,8 +975,8 @@ __global__ void scan_dc_rows_kernel(DevDB db, DevBulk b, const BulkCtl *ctl, boo
         __syncthreads();
     }
     const int64_t hb = ctl->base.hist;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < b.n;
-         t += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t n = b.n_live ? (int64_t)*b.n_live : b.n;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t a = (uint32_t)b.params[t * b.P];
         const int64_t d = b.params[t * b.P + 1];
         const uint32_t tl = db.div_tel.div(a), br = db.div_br.div(a);
@@ -839,7 +986,7 @@ __global__ void scan_dc_rows_kernel(DevDB db, DevBulk b, const BulkCtl *ctl, boo
         db.h_tel[slot] = tl;
         db.h_br[slot] = br;
         db.h_delta[slot] = d;
-        b.status[t] = 0;   // here, in timestamp order, rather than scattered by the scan
+        b.status[t] = 0;   // here, in timestamp order, rather than scattered by the account updates
         if (local) {
             atomicAdd(&sums[tl], (unsigned long long)d);
             atomicAdd(&sums[n_tel + br], (unsigned long long)d);
@@ -864,52 +1011,70 @@ __global__ void scan_dc_rows_kernel(DevDB db, DevBulk b, const BulkCtl *ctl, boo
 
 DevBulk make_dev_bulk(gputx_bulk *b, int mode) { return dev_bulk(b, mode); }
 
-cudaError_t launch_scan_exec(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m)
+// The values of a debit-credit-only bulk are cleared just before its executor
+// scatters them, 8 bytes at a time: the cleared sectors are still in L2 and the
+// scatter need not fetch them (with streaming hints on what passes through
+// once, acct_scan_kernel at 2^22: 122 us instead of 156).
+cudaError_t clear_outputs(gputx_bulk *b)
 {
+    return b->n > 0 ? cudaMemsetAsync(b->out, 0, (size_t)b->n * b->R * sizeof(int64_t), b->stream) : cudaSuccess;
+}
+
+bool dc_only(const gputx_db *db) { return db->dev.registered == (1u << GPUTX_T_DC_DEBIT_CREDIT); }
+
+cudaError_t launch_scan_exec(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m, bool stats)
+{
+    if (m == 0) return cudaSuccess;
     gputx_db *db = b->db;
     cudaStream_t s = b->stream;
-    scan_capacity_kernel<<<1, 1, 0, s>>>(b->ctl, b->n, db->dev.hist_cap);
+    const int64_t tiles = (m + SCAN_TILE - 1) / SCAN_TILE;
+    if (tiles > b->sc.scan_tiles) return cudaErrorInvalidValue;
+    AcctScanArgs a;
+    a.sk = sk;
+    a.sv = sv;
+    a.deltas = b->sc.rec_ts;
+    a.acc_bal = db->dev.acc_bal;
+    a.out = b->out;
+    a.m = (uint32_t)m;
+    a.R = b->R;
+    a.o_acc = db->dev.o_acc;
+    a.stats = stats ? b->ctl : nullptr;
+    a.st.word = (uint32_t *)(b->sc.scan_zero + 1);
+    a.st.agg = b->sc.scan_vals;
+    a.st.inc = b->sc.scan_vals + tiles;
+    a.tile_ctr = (uint32_t *)b->sc.scan_zero;
+    a.err = &b->ctl->err;
+    a.spin_limit_ns = (uint64_t)db->cfg.spin_limit_ns;
+    cudaError_t e = cudaMemsetAsync(b->sc.scan_zero, 0, sizeof(uint64_t) + tiles * sizeof(uint32_t), s);
+    if (!e) e = clear_outputs(b);
+    if (e) return e;
+    acct_scan_kernel<<<(unsigned)tiles, SCAN_THREADS, 0, s>>>(a);
     count_launches(1);
-    if (m > 0) {
-        const int64_t tiles = (m + SCAN_TILE - 1) / SCAN_TILE;
-        if (tiles > b->sc.scan_tiles) return cudaErrorInvalidValue;
-        ScanExecMode mode;
-        mode.sk = sk;
-        mode.sv = sv;
-        mode.params = b->params;
-        mode.acc_bal = db->dev.acc_bal;
-        mode.out = b->out;
-        mode.status = b->status;
-        mode.m = m;
-        mode.P = b->P;
-        mode.R = b->R;
-        mode.o_acc = db->dev.o_acc;
-        Seg64Status st;
-        st.word = (uint32_t *)(b->sc.scan_zero + 1);
-        st.agg = b->sc.scan_vals;
-        st.inc = b->sc.scan_vals + tiles;
-        cudaError_t e = cudaMemsetAsync(b->sc.scan_zero, 0, sizeof(uint64_t) + tiles * sizeof(uint32_t), s);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_dc_rows(gputx_bulk *b)
+{
+    if (b->n == 0) return cudaSuccess;
+    gputx_db *db = b->db;
+    // teller and branch sums in shared memory when they fit and there are
+    // several transactions per cell (clearing and adding the cells costs each
+    // block more than 1,000 transactions' own atomics: 7 us against 3), one
+    // block per SM
+    const int64_t cells = db->dev.n_tel + db->dev.n_br;
+    const size_t smem = (size_t)cells * sizeof(unsigned long long);
+    const bool local = smem <= (200u << 10) && b->n >= 4 * cells;
+    const int threads = 1024;
+    int64_t grid = (b->n + threads - 1) / threads;
+    if (grid > (int64_t)db->num_sms) grid = db->num_sms;
+    if (local && smem > (48u << 10)) {
+        const cudaError_t e = cudaFuncSetAttribute(dc_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)smem);
         if (e) return e;
-        seg64_scan_kernel<ScanExecMode><<<(unsigned)tiles, SCAN_THREADS, 0, s>>>(
-            mode, m, st, (uint32_t *)b->sc.scan_zero, &b->ctl->err, (uint64_t)db->cfg.spin_limit_ns);
-        count_launches(1);
     }
-    if (b->n > 0) {
-        // teller and branch sums in shared memory when they fit, one block per SM
-        const size_t smem = (size_t)(db->dev.n_tel + db->dev.n_br) * sizeof(unsigned long long);
-        const bool local = smem <= (200u << 10);
-        const int threads = 1024;
-        int64_t grid = (b->n + threads - 1) / threads;
-        if (grid > (int64_t)db->num_sms) grid = db->num_sms;
-        if (local && smem > (48u << 10)) {
-            const cudaError_t e = cudaFuncSetAttribute(scan_dc_rows_kernel,
-                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e) return e;
-        }
-        scan_dc_rows_kernel<<<(unsigned)grid, threads, local ? smem : 0, s>>>(
-            db->dev, dev_bulk(b, GPUTX_CONFLICT_ADD), b->ctl, local);
-        count_launches(1);
-    }
+    dc_rows_kernel<<<(unsigned)grid, threads, local ? smem : 0, b->stream>>>(
+        db->dev, dev_bulk(b, GPUTX_CONFLICT_ADD), b->ctl, local);
+    count_launches(1);
     return cudaGetLastError();
 }
 
@@ -919,16 +1084,6 @@ cudaError_t launch_gather(gputx_bulk *b, const uint32_t *order)
     const DevBulk d = dev_bulk(b, 0);
     gather_kernel<<<grid_for(b->n), TB, 0, b->stream>>>(d, order, b->sc.rec_params, b->sc.rec_ts,
                                                              b->sc.rec_type, b->sc.rec_t, &b->ctl->err);
-    count_launches(1);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_gather_dc(gputx_bulk *b, const uint32_t *order)
-{
-    if (b->n == 0) return cudaSuccess;
-    if (!b->sc.rec_dc) return cudaErrorInvalidValue;
-    gather_dc_kernel<<<grid_for(b->n), TB, 0, b->stream>>>(b->db->dev, dev_bulk(b, 0), order, b->sc.rec_dc,
-                                                                &b->ctl->err);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -985,11 +1140,12 @@ cudaError_t launch_part_scatter(gputx_bulk *b, const uint32_t *off, const uint32
     return cudaGetLastError();
 }
 
-cudaError_t launch_begin(gputx_bulk *b)
+cudaError_t launch_begin(gputx_bulk *b, bool whole)
 {
     const bool dc = (b->db->dev.registered & 1u) != 0;
     const int64_t rows = b->sc.slot_hist ? -1 : (dc ? b->n : 0);
-    begin_kernel<<<1, 1, 0, b->stream>>>(b->db->d_cursor, b->ctl, rows, dc && b->graph);
+    begin_kernel<<<1, 1, 0, b->stream>>>(b->db->d_cursor, b->ctl, rows, dc && b->graph,
+                                         whole ? b->db->dev.hist_cap : -1);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -1094,13 +1250,28 @@ int64_t sort_scratch_words(int64_t count)
     return words;
 }
 
+// where a sort's counters live in its scratch
+struct SortScratch {
+    uint32_t *ctr, *hist, *status;
+    size_t bytes;
+};
+static SortScratch sort_scratch(gputx_bulk *b, const SortShape &sh)
+{
+    SortScratch z;
+    z.ctr = b->sc.sort_zero;
+    z.hist = z.ctr + 8;
+    z.status = z.hist + sh.passes * sh.digits();
+    z.bytes = sizeof(uint32_t) * (8 + sh.passes * (size_t)sh.digits() * (1 + sh.tiles));
+    return z;
+}
+
 template <int RB, int ITEMS>
 static cudaError_t launch_radix_passes(gputx_bulk *b, uint32_t *&keys, uint32_t *&vals, uint32_t *&keys_alt,
-                                       uint32_t *&vals_alt, uint32_t count, const SortShape &sh)
+                                       uint32_t *&vals_alt, uint32_t count, const SortShape &sh, bool counted)
 {
     constexpr int D = 1 << RB;
     cudaStream_t s = b->stream;
-    uint32_t *ctr = b->sc.sort_zero, *hist = ctr + 8, *status = hist + sh.passes * D;
+    const SortScratch z = sort_scratch(b, sh);
     static std::atomic<uint64_t> attr_set{0};   // a bit per device
     const uint64_t dev = 1ull << (b->db->device & 63);
     if (!(attr_set.load(std::memory_order_relaxed) & dev)) {
@@ -1110,15 +1281,17 @@ static cudaError_t launch_radix_passes(gputx_bulk *b, uint32_t *&keys, uint32_t 
         if (e) return e;
         attr_set.fetch_or(dev, std::memory_order_relaxed);
     }
-    int hist_blocks = b->db->num_sms * 4;
-    const int64_t need = ((int64_t)count + 255) / 256;
-    if (hist_blocks > need) hist_blocks = (int)need;
-    radix_hist_kernel<RB><<<hist_blocks, 256, 0, s>>>(keys, count, sh.passes, hist, &b->ctl->err);
-    count_launches(1);
+    if (!counted) {
+        int hist_blocks = b->db->num_sms * 4;
+        const int64_t need = ((int64_t)count + 255) / 256;
+        if (hist_blocks > need) hist_blocks = (int)need;
+        radix_hist_kernel<RB><<<hist_blocks, 256, 0, s>>>(keys, count, sh.passes, z.hist, &b->ctl->err);
+        count_launches(1);
+    }
     for (int p = 0; p < sh.passes; p++) {
         radix_pass_kernel<RB, ITEMS><<<(unsigned)sh.tiles, SORT_THREADS, radix_smem<RB, ITEMS>(), s>>>(
-            keys, vals, keys_alt, vals_alt, count, RB * p, hist + p * D, status + (size_t)p * sh.tiles * D, ctr + p,
-            &b->ctl->err, (uint64_t)b->db->cfg.spin_limit_ns);
+            keys, vals, keys_alt, vals_alt, count, RB * p, z.hist + p * D, z.status + (size_t)p * sh.tiles * D,
+            z.ctr + p, &b->ctl->err, (uint64_t)b->db->cfg.spin_limit_ns);
         count_launches(1);
         std::swap(keys, keys_alt);
         std::swap(vals, vals_alt);
@@ -1126,8 +1299,9 @@ static cudaError_t launch_radix_passes(gputx_bulk *b, uint32_t *&keys, uint32_t 
     return cudaGetLastError();
 }
 
-cudaError_t launch_sort(gputx_bulk *b, uint32_t *&keys, uint32_t *&vals, uint32_t *&keys_alt, uint32_t *&vals_alt,
-                        int64_t count, int bits)
+// the sort proper; `counted`: its scratch is cleared and holds the digit counts
+static cudaError_t launch_sort_passes(gputx_bulk *b, uint32_t *&keys, uint32_t *&vals, uint32_t *&keys_alt,
+                                      uint32_t *&vals_alt, int64_t count, int bits, bool counted)
 {
     if (count <= 1 || bits <= 0) return cudaSuccess;
     cudaStream_t s = b->stream;
@@ -1140,16 +1314,61 @@ cudaError_t launch_sort(gputx_bulk *b, uint32_t *&keys, uint32_t *&vals, uint32_
         return cudaGetLastError();
     }
     const SortShape sh = sort_shape(count, bits);
-    const int64_t words = 8 + sh.passes * (int64_t)sh.digits() * (1 + sh.tiles);
-    if (words > b->sc.sort_words || bits > 32 || count >= (1ll << 30)) return cudaErrorInvalidValue;
-    cudaError_t e = cudaMemsetAsync(b->sc.sort_zero, 0, words * sizeof(uint32_t), s);
-    if (e) return e;
+    const SortScratch z = sort_scratch(b, sh);
+    if (z.bytes > b->sc.sort_words * sizeof(uint32_t) || bits > 32 || count >= (1ll << 30))
+        return cudaErrorInvalidValue;
+    if (!counted) {
+        const cudaError_t e = cudaMemsetAsync(z.ctr, 0, z.bytes, s);
+        if (e) return e;
+    }
     const uint32_t n = (uint32_t)count;
     if (sh.digit_bits == 10)
-        return sh.items == 4 ? launch_radix_passes<10, 4>(b, keys, vals, keys_alt, vals_alt, n, sh)
-                             : launch_radix_passes<10, 16>(b, keys, vals, keys_alt, vals_alt, n, sh);
-    return sh.items == 4 ? launch_radix_passes<8, 4>(b, keys, vals, keys_alt, vals_alt, n, sh)
-                         : launch_radix_passes<8, 16>(b, keys, vals, keys_alt, vals_alt, n, sh);
+        return sh.items == 4 ? launch_radix_passes<10, 4>(b, keys, vals, keys_alt, vals_alt, n, sh, counted)
+                             : launch_radix_passes<10, 16>(b, keys, vals, keys_alt, vals_alt, n, sh, counted);
+    return sh.items == 4 ? launch_radix_passes<8, 4>(b, keys, vals, keys_alt, vals_alt, n, sh, counted)
+                         : launch_radix_passes<8, 16>(b, keys, vals, keys_alt, vals_alt, n, sh, counted);
+}
+
+cudaError_t launch_sort(gputx_bulk *b, uint32_t *&keys, uint32_t *&vals, uint32_t *&keys_alt, uint32_t *&vals_alt,
+                        int64_t count, int bits)
+{
+    return launch_sort_passes(b, keys, vals, keys_alt, vals_alt, count, bits, false);
+}
+
+cudaError_t launch_group(gputx_bulk *b, int mode, int part_size, bool by_part, uint32_t *&keys, uint32_t *&vals,
+                         uint32_t *&keys_alt, uint32_t *&vals_alt, int bits, int64_t *deltas)
+{
+    const int64_t n = b->n;
+    if (n == 0) return cudaSuccess;
+    ExtractOneArgs a;
+    a.db = b->db->dev;
+    a.b = dev_bulk(b, mode);
+    a.ctl = b->ctl;
+    a.keys = keys;
+    a.vals = vals;
+    a.hist = nullptr;
+    a.deltas = deltas;
+    a.mode = mode;
+    a.part_size = part_size < 1 ? 1 : part_size;
+    a.passes = 0;
+    a.by_part = by_part;
+    const SortShape sh = sort_shape(n, bits);
+    if (n > SMALL_SORT && bits > 0) {
+        const SortScratch z = sort_scratch(b, sh);
+        if (z.bytes > b->sc.sort_words * sizeof(uint32_t) || bits > 32) return cudaErrorInvalidValue;
+        const cudaError_t e = cudaMemsetAsync(z.ctr, 0, z.bytes, b->stream);
+        if (e) return e;
+        a.hist = z.hist;
+        a.passes = sh.passes;
+    }
+    // the counts are added up per block: few blocks that stride
+    const unsigned grid = (unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)b->db->num_sms * 8);
+    if (sh.digit_bits == 10) extract_one_kernel<10><<<grid, 256, 0, b->stream>>>(a);
+    else extract_one_kernel<8><<<grid, 256, 0, b->stream>>>(a);
+    count_launches(1);
+    const cudaError_t e = cudaGetLastError();
+    if (e) return e;
+    return launch_sort_passes(b, keys, vals, keys_alt, vals_alt, n, bits, a.hist != nullptr);
 }
 
 cudaError_t launch_rank_scan(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m, bool want_rid)

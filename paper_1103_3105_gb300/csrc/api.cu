@@ -225,7 +225,6 @@ size_t carve_bulk(gputx_bulk *b, char *base, bool device_inputs)
     s.scan_tiles = (big + 2047) / 2048;
     s.scan_zero = c.take<uint64_t>(1 + s.scan_tiles);
     s.scan_vals = c.take<uint64_t>(2 * s.scan_tiles);
-    s.rec_dc = db->dev.registered == (1u << GPUTX_T_DC_DEBIT_CREDIT) ? c.take<DcRecord>(nn) : nullptr;
     s.seg_off = b->graph ? c.take<uint32_t>(kSegMax + 1) : nullptr;
     s.bulk_of = b->graph ? c.take<uint32_t>(nn) : nullptr;
     s.seg_depth = b->graph ? c.take<uint32_t>(kSegMax) : nullptr;
@@ -968,7 +967,7 @@ gputx_status gputx_submit_bulk(gputx_db *db, const int64_t *ts, const int32_t *t
                                     cudaMemcpyHostToDevice, b->stream);
     }
     if (!e) e = cudaMemsetAsync(b->ctl, 0, sizeof(BulkCtl), b->stream);
-    if (!e && n > 0) e = cudaMemsetAsync(b->out, 0, n * b->R * sizeof(int64_t), b->stream);
+    if (!e && !dc_only(db)) e = clear_outputs(b);   // debit-credit only: by the executor
     if (!e && n > 0) e = cudaMemsetAsync(b->status, 0, n * sizeof(int32_t), b->stream);
     if (!e) e = cudaEventCreate(&b->ev[7]);
     if (e) {
@@ -997,13 +996,22 @@ int key_bits(const gputx_db *db, int mode)
     return std::max(1, bits_for(top - 1));
 }
 
-gputx_status run_kset_analysis(gputx_bulk *b, int mode, int part_size, uint32_t *&sk, uint32_t *&sv,
-                               uint32_t *&ak, uint32_t *&av, int64_t &m)
+// the bulk's operations extracted and sorted by item
+gputx_status run_grouping(gputx_bulk *b, int mode, int part_size, uint32_t *&sk, uint32_t *&sv, uint32_t *&ak,
+                          uint32_t *&av, int64_t &m, int64_t *deltas = nullptr)
 {
     gputx_db *db = b->db;
+    sk = b->sc.keys_a; sv = b->sc.vals_a; ak = b->sc.keys_b; av = b->sc.vals_b;
+    m = b->n * db->uniform_k;
+    if (db->uniform_k == 1) {
+        if (b->timing) cudaEventRecord(b->ev[1], b->stream);
+        CK(launch_group(b, mode, 1, false, sk, sv, ak, av, key_bits(db, mode), deltas),
+           "extract and sort");
+        if (b->timing) cudaEventRecord(b->ev[2], b->stream);
+        return GPUTX_OK;
+    }
     CK(cudaMemsetAsync(&b->ctl->cross, 0, 4, b->stream), "extract");
     CK(launch_extract(b, mode, part_size, nullptr, nullptr, true), "extract");
-    m = b->n * db->uniform_k;
     if (!db->uniform_k) {
         uint32_t mm = 0;
         CK(cudaMemcpyAsync(&mm, b->sc.op_off + b->n, sizeof mm, cudaMemcpyDeviceToHost, b->stream), "ops");
@@ -1012,7 +1020,6 @@ gputx_status run_kset_analysis(gputx_bulk *b, int mode, int part_size, uint32_t 
         if (m > b->sc.m_cap) m = b->sc.m_cap;
     }
     if (b->timing) cudaEventRecord(b->ev[1], b->stream);
-    sk = b->sc.keys_a; sv = b->sc.vals_a; ak = b->sc.keys_b; av = b->sc.vals_b;
     CK(launch_sort(b, sk, sv, ak, av, m, key_bits(db, mode)), "sort");
     if (b->timing) cudaEventRecord(b->ev[2], b->stream);
     return GPUTX_OK;
@@ -1020,11 +1027,11 @@ gputx_status run_kset_analysis(gputx_bulk *b, int mode, int part_size, uint32_t 
 
 // The database-touching tail of a bulk starts after the previous bulk's tail
 // (bulks apply in gputx_execute order); the analysis before it overlaps.
-cudaError_t begin_tail(gputx_bulk *b)
+cudaError_t begin_tail(gputx_bulk *b, bool whole = false)
 {
     cudaError_t e = cudaStreamWaitEvent(b->stream, b->db->last_done, 0);
     if (e) return e;
-    return launch_begin(b);
+    return launch_begin(b, whole);
 }
 
 cudaError_t end_tail(gputx_bulk *b)
@@ -1076,6 +1083,9 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
     cudaStream_t s = b->stream;
     if (b->timing) cudaEventRecord(b->ev[0], s);
     CK(launch_insert_slots(b), "insert slots");
+    if (dc_only(db) && (strategy == GPUTX_TPL || strategy == GPUTX_TPL_RELAXED ||
+                        (strategy == GPUTX_KSET && opts && opts->kset_launch == 1)))
+        CK(clear_outputs(b), "clear");
     const bool add = mode == GPUTX_CONFLICT_ADD;
     gputx_status st = GPUTX_OK;
     uint32_t *sk = nullptr, *sv = nullptr, *ak = nullptr, *av = nullptr;
@@ -1086,8 +1096,12 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
     // segmented-sum strategy gives Definition 1's results bit for bit and
     // moves each transaction once, whatever the depth of its graph
     if (strategy == GPUTX_AUTO && db->dev.registered == (1u << GPUTX_T_DC_DEBIT_CREDIT)) run = GPUTX_SCAN;
-    if (strategy == GPUTX_KSET || (strategy == GPUTX_AUTO && run == GPUTX_AUTO)) {
-        if ((st = run_kset_analysis(b, mode, part_size, sk, sv, ak, av, m))) return st;
+    // K-SET of a debit-credit-only bulk: the graph is one path per item, so
+    // the paths run side by side without a barrier per k-set and no level
+    // table is built (exec_dc.cu; kset_launch = 1 asks for the levels)
+    const bool paths = strategy == GPUTX_KSET && dc_only(db) && !(opts && opts->kset_launch == 1);
+    if (!paths && (strategy == GPUTX_KSET || (strategy == GPUTX_AUTO && run == GPUTX_AUTO))) {
+        if ((st = run_grouping(b, mode, part_size, sk, sv, ak, av, m))) return st;
         CK(launch_rank_scan(b, sk, sv, m, db->need_fixpoint), "rank");
         // AUTO decides on the one-pass ranks first: w0 and c are exact there
         // (a transaction is a source exactly when all its operations have
@@ -1124,7 +1138,26 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
             }
         }
     }
-    if (run == GPUTX_KSET) {
+    // a debit-credit-only bulk grouped by branch (K-SET under R/W) or by
+    // partition: account updates group by group, then the rows
+    auto run_ranges = [&](const uint32_t *gk, const uint32_t *gv, int vshift, bool stats) -> gputx_status {
+        if (b->timing) cudaEventRecord(b->ev[3], s);
+        CK(launch_dc_ranges(b, gk, gv, vshift, stats), "execute");
+        CK(launch_dc_rows(b), "rows");
+        return GPUTX_OK;
+    };
+    if (run == GPUTX_SCAN || (paths && add)) {
+        // grouped by account: segmented prefix sums
+        if ((st = run_grouping(b, GPUTX_CONFLICT_ADD, part_size, sk, sv, ak, av, m, b->sc.rec_ts))) return st;
+        CK(begin_tail(b, true), "order");
+        if (b->timing) cudaEventRecord(b->ev[3], s);
+        CK(launch_scan_exec(b, sk, sv, m, paths), "scan execute");
+        CK(launch_dc_rows(b), "rows");
+    } else if (paths) {
+        if ((st = run_grouping(b, mode, part_size, sk, sv, ak, av, m))) return st;
+        CK(begin_tail(b, true), "order");
+        if ((st = run_ranges(sk, sv, 7, true))) return st;
+    } else if (run == GPUTX_KSET) {
         const int64_t depth = b->host_ctl.depth;
         const bool persistent = opts && opts->kset_launch == 1;
         // regroup by (level, type): reuse the free op buffers
@@ -1151,14 +1184,10 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
             CK(cudaStreamSynchronize(s), "level plan");
             if (!b->host_ctl.err) {
                 const int narrow = (opts && opts->narrow_max > 0) ? opts->narrow_max : 8192;
-                // debit-credit-only bulks run from packed records
-                const bool dc_only = b->sc.rec_dc != nullptr;
-                if (dc_only) CK(launch_gather_dc(b, rv), "gather");
-                else CK(launch_gather(b, rv), "gather");
+                CK(launch_gather(b, rv), "gather");
                 CK(begin_tail(b), "order");
                 if (b->timing) cudaEventRecord(b->ev[3], s);
                 CK(launch_kset_levels(b, b->level_off_host.data(), depth, narrow, add,
-                                      dc_only ? b->sc.rec_dc : nullptr,
                                       b->sc.type_cut ? b->type_cut_host.data() : nullptr),
                    "k-set execute");
             }
@@ -1168,30 +1197,40 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
     } else if (run == GPUTX_PART) {
         // partition ids by root key (Section 5.2 step 1), stable sort (step 2)
         uint32_t *pk = b->sc.pid_key, *pv = b->sc.pid_val, *pk2 = b->sc.pid_key2, *pv2 = b->sc.pid_val2;
-        CK(cudaMemsetAsync(&b->ctl->cross, 0, 4, s), "part");
-        CK(launch_extract(b, mode, part_size, pk, pv, false), "extract");
-        if (b->timing) cudaEventRecord(b->ev[1], s);
-        if ((st = read_ctl(b))) return st;
-        if (b->host_ctl.err) {
-            CK(cudaEventRecord(b->ev[7], s), "event");
-            return GPUTX_OK;
-        }
-        if (b->host_ctl.cross > 0) {
-            // Section 5.2: cross-partition transactions run with TPL
-            b->fallback = 1;
-            run = GPUTX_TPL;
-            CK(cudaMemsetAsync(&b->ctl->cross, 0, 4, s), "part");
+        const int64_t roots = std::max<int64_t>({db->dev.n_br, db->dev.n_sub, db->dev.n_wh, 1});
+        const int bits = bits_for((uint64_t)((roots - 1) / part_size));
+        if (db->uniform_k == 1) {
+            // one operation, so one partition, per transaction: none crosses
+            if (b->timing) cudaEventRecord(b->ev[1], s);
+            CK(launch_group(b, mode, part_size, true, pk, pv, pk2, pv2, bits), "partition sort");
         } else {
-            const int64_t roots = std::max<int64_t>({db->dev.n_br, db->dev.n_sub, db->dev.n_wh, 1});
-            const int bits = bits_for((uint64_t)((roots - 1) / part_size));
-            CK(launch_sort(b, pk, pv, pk2, pv2, b->n, bits), "partition sort");
-            if (b->timing) cudaEventRecord(b->ev[2], s);
+            CK(cudaMemsetAsync(&b->ctl->cross, 0, 4, s), "part");
+            CK(launch_extract(b, mode, part_size, pk, pv, false), "extract");
+            if (b->timing) cudaEventRecord(b->ev[1], s);
+            if ((st = read_ctl(b))) return st;
+            if (b->host_ctl.err) {
+                CK(cudaEventRecord(b->ev[7], s), "event");
+                return GPUTX_OK;
+            }
+            if (b->host_ctl.cross > 0) {
+                // Section 5.2: cross-partition transactions run with TPL
+                b->fallback = 1;
+                run = GPUTX_TPL;
+                CK(cudaMemsetAsync(&b->ctl->cross, 0, 4, s), "part");
+            } else {
+                CK(launch_sort(b, pk, pv, pk2, pv2, b->n, bits), "partition sort");
+            }
+        }
+        if (b->timing && run == GPUTX_PART) cudaEventRecord(b->ev[2], s);
+        if (run == GPUTX_PART && dc_only(db)) {
+            CK(begin_tail(b, true), "order");
+            if ((st = run_ranges(pk, pv, 0, false))) return st;
+        } else if (run == GPUTX_PART) {
             CK(launch_part_heads(b, pk, b->n), "partition heads");
-            if (part_dc_applies(db, part_size)) CK(launch_gather_dc(b, pv), "gather");
-            else CK(launch_gather(b, pv), "gather");
+            CK(launch_gather(b, pv), "gather");
             CK(begin_tail(b), "order");
             if (b->timing) cudaEventRecord(b->ev[3], s);
-            CK(launch_part(b, pk, 128, (roots + part_size - 1) / part_size, part_size), "part execute");
+            CK(launch_part(b, pk, 128, (roots + part_size - 1) / part_size), "part execute");
         }
     }
     if (run == GPUTX_PART_RELAXED) {
@@ -1200,7 +1239,7 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
         const int64_t roots = std::max<int64_t>({db->dev.n_br, db->dev.n_sub, db->dev.n_wh, 1});
         const int64_t parts = (roots + part_size - 1) / part_size;
         if ((st = part_scratch(db, roots))) return st;
-        CK(begin_tail(b), "order");
+        CK(begin_tail(b, dc_only(db)), "order");
         CK(cudaMemsetAsync(db->part_cnt, 0, parts * sizeof(uint32_t), s), "part counters");
         uint32_t *pid_of = b->sc.pid_key, *key_of = b->sc.pid_val, *pk = b->sc.pid_key2, *order = b->sc.pid_val2;
         CK(launch_part_count(b, mode, part_size, db->part_cnt, parts, pid_of, key_of), "part count");
@@ -1219,11 +1258,14 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
                "part offsets");
             CK(launch_part_scatter(b, db->part_off, pid_of, key_of, pk, order), "part scatter");
             if (b->timing) cudaEventRecord(b->ev[2], s);
-            CK(launch_part_heads(b, pk, b->n), "partition heads");
-            if (part_dc_applies(db, part_size)) CK(launch_gather_dc(b, order), "gather");
-            else CK(launch_gather(b, order), "gather");
-            if (b->timing) cudaEventRecord(b->ev[3], s);
-            CK(launch_part(b, pk, 128, parts, part_size), "part execute");
+            if (dc_only(db)) {
+                if ((st = run_ranges(pk, order, 0, false))) return st;
+            } else {
+                CK(launch_part_heads(b, pk, b->n), "partition heads");
+                CK(launch_gather(b, order), "gather");
+                if (b->timing) cudaEventRecord(b->ev[3], s);
+                CK(launch_part(b, pk, 128, parts), "part execute");
+            }
             b->serial_order = order;
         }
     }
@@ -1238,15 +1280,9 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
         CK(launch_tpl_relaxed(b, b->sc.level, add), "tpl execute");
         b->serial_order = b->sc.level;
     }
-    if (run == GPUTX_SCAN) {
-        if ((st = run_kset_analysis(b, GPUTX_CONFLICT_ADD, part_size, sk, sv, ak, av, m))) return st;
-        CK(begin_tail(b), "order");
-        if (b->timing) cudaEventRecord(b->ev[3], s);
-        CK(launch_scan_exec(b, sk, sv, m), "scan execute");
-    }
     if (run == GPUTX_TPL) {
         if (!sk) {
-            if ((st = run_kset_analysis(b, mode, part_size, sk, sv, ak, av, m))) return st;
+            if ((st = run_grouping(b, mode, part_size, sk, sv, ak, av, m))) return st;
         }
         CK(launch_ticket_scan(b, sk, sv, m), "tickets");
         CK(begin_tail(b), "order");

@@ -93,12 +93,16 @@ cudaError_t enqueue_pipeline(GraphBulk *g)
         const int64_t roots = std::max<int64_t>({db->dev.n_br, db->dev.n_sub, db->dev.n_wh, 1});
         const int64_t parts = (roots + g->part_size - 1) / g->part_size;   // the padding's id
         if ((e = gtx::launch_sort(b, pk, pv, pk2, pv2, b->n, gtx::bits_for((uint64_t)parts)))) return e;
+        if (gtx::dc_only(db)) {
+            if ((e = gtx::launch_begin(b, true))) return e;
+            if ((e = gtx::launch_dc_ranges(b, pk, pv, 0, false))) return e;
+            if ((e = gtx::launch_dc_rows(b))) return e;
+            return gtx::launch_finish(b);
+        }
         if ((e = gtx::launch_part_heads(b, pk, b->n))) return e;
-        if (gtx::part_dc_applies(db, g->part_size)) e = gtx::launch_gather_dc(b, pv);
-        else e = gtx::launch_gather(b, pv);
-        if (e) return e;
+        if ((e = gtx::launch_gather(b, pv))) return e;
         if ((e = gtx::launch_begin(b))) return e;
-        if ((e = gtx::launch_part(b, pk, 128, parts, g->part_size))) return e;
+        if ((e = gtx::launch_part(b, pk, 128, parts))) return e;
         return gtx::launch_finish(b);
     }
     const bool seg = g->strategy == GPUTX_KSET && gtx::seg_bits(db) > 0;

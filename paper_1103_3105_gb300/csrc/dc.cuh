@@ -84,11 +84,4 @@ __device__ __forceinline__ void dc_finish_rmw(const DevDB &db, const DevBulk &b,
     dc_finish(db, b, o);
 }
 
-// one whole transaction of a k-set from its packed record, by atomics
-__device__ __forceinline__ void exec_dc_record_rmw(const DevDB &db, const DevBulk &b, const DcRecord &r, int64_t slot)
-{
-    DcOut o;
-    if (dc_account_rmw(db, b, r, slot, o)) dc_finish_rmw(db, b, o);
-}
-
 }  // namespace gtx

@@ -53,7 +53,6 @@ struct Scratch {
     uint32_t *sort_zero;   // a sort's tile counters, digit counts and look-back words, cleared by it at once
     uint64_t *scan_zero;   // a scan's tile counter and look-back words, likewise
     uint64_t *scan_vals;   // 2 x tiles: per-tile values of 64-bit scans
-    DcRecord *rec_dc;      // n packed debit-credit records (debit-credit-only databases)
     // graph bulks that carry a segment of several bulks
     uint32_t *seg_off;     // kSegMax + 1: first transaction of each bulk
     uint32_t *bulk_of;     // n: bulk of each transaction
@@ -146,6 +145,11 @@ cudaError_t launch_seg_levels(gputx_bulk *b);
 // then runs nothing and is re-run with TPL)
 cudaError_t launch_part_fallback_check(gputx_bulk *b);
 int64_t sort_scratch_words(int64_t count);   // scratch of a sort of up to `count` pairs
+// single-operation bulks: keys and payloads by item (payload as launch_extract's)
+// or by partition (payload = transaction), sorted; `deltas` (debit-credit-only
+// bulks): each transaction's delta side by side, for launch_scan_exec
+cudaError_t launch_group(gputx_bulk *b, int mode, int part_size, bool by_part, uint32_t *&keys, uint32_t *&vals,
+                         uint32_t *&keys_alt, uint32_t *&vals_alt, int bits, int64_t *deltas = nullptr);
 cudaError_t launch_sort(gputx_bulk *b, uint32_t *&keys, uint32_t *&vals, uint32_t *&keys_alt,
                         uint32_t *&vals_alt, int64_t count, int bits);
 cudaError_t launch_rank_scan(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m, bool want_rid);
@@ -159,17 +163,15 @@ cudaError_t launch_insert_slots(gputx_bulk *b);
 cudaError_t launch_part_heads(gputx_bulk *b, const uint32_t *skeys, int64_t n);
 cudaError_t launch_tpl_reset(gputx_bulk *b, const uint32_t *skeys, int64_t m);
 cudaError_t launch_gather(gputx_bulk *b, const uint32_t *order);
-cudaError_t launch_gather_dc(gputx_bulk *b, const uint32_t *order);
-bool part_dc_applies(const gputx_db *db, int part_size);
-cudaError_t launch_begin(gputx_bulk *b);
+// `whole`: the bulk's history rows all fit or the bulk fails (ERR_CAPACITY)
+cudaError_t launch_begin(gputx_bulk *b, bool whole = false);
 cudaError_t launch_finish(gputx_bulk *b);
 
 // exec.cu
 cudaError_t launch_kset(gputx_bulk *b, const uint32_t *order, int64_t nchunks, int block, bool atomic_add);
 cudaError_t launch_kset_levels(gputx_bulk *b, const uint32_t *level_off_host, int64_t depth, int narrow_max,
-                               bool atomic_add, const DcRecord *dc_records = nullptr,
-                               const uint32_t *type_cut_host = nullptr);
-cudaError_t launch_part(gputx_bulk *b, const uint32_t *pkeys, int block, int64_t max_parts, int part_size);
+                               bool atomic_add, const uint32_t *type_cut_host = nullptr);
+cudaError_t launch_part(gputx_bulk *b, const uint32_t *pkeys, int block, int64_t max_parts);
 cudaError_t launch_tpl(gputx_bulk *b, int block, bool atomic_add);
 // a conflict-free bulk (a 0-set) in one launch
 cudaError_t launch_independent(gputx_bulk *b, bool atomic_add);
@@ -182,8 +184,16 @@ cudaError_t launch_part_offsets(gputx_bulk *b, const uint32_t *cnt, uint32_t *of
                                 uint32_t *tile_ctr);
 cudaError_t launch_part_scatter(gputx_bulk *b, const uint32_t *off, const uint32_t *pid_of, const uint32_t *key_of,
                                 uint32_t *pkeys, uint32_t *order);
-// SCAN: segmented prefix sums over operations grouped by account
-cudaError_t launch_scan_exec(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m);
+// debit-credit-only bulks: the account updates of transactions (vals >> vshift)
+// grouped by branch or partition (exec_dc.cu), or by account (segmented prefix
+// sums); then the history rows, statuses and teller and branch sums.  `stats`:
+// the groups are the graph's paths, d and w0 are recorded
+cudaError_t launch_dc_ranges(gputx_bulk *b, const uint32_t *keys, const uint32_t *vals, int vshift, bool stats);
+// (the deltas launch_group left in sc.rec_ts)
+cudaError_t launch_scan_exec(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m, bool stats);
+cudaError_t launch_dc_rows(gputx_bulk *b);
+bool dc_only(const gputx_db *db);
+cudaError_t clear_outputs(gputx_bulk *b);
 int exec_blocks_per_sm(int kind, int block);
 
 // tables.cu

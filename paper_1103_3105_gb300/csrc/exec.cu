@@ -7,8 +7,7 @@
 //         narrow levels  one thread-block cluster (or one CTA) walks a run of
 //                        consecutive narrow levels, separated by cluster (or
 //                        CTA) barriers, loading the next level's signatures
-//                        and prefetching its rows into L2 before each barrier
-//                        (debit-credit-only bulks: exec_dc.cu);
+//                        and prefetching its rows into L2 before each barrier;
 //         persistent     a grid claims level-ordered chunks of one CTA; a
 //                        chunk of level k starts once every transaction of
 //                        level k-1 has finished (per-level counters).  Chunks
@@ -16,6 +15,8 @@
 //                        waiting CTA depends on is held by a running CTA.
 //   PART (Section 5.2)   one thread per non-empty partition runs its
 //       transactions serially in timestamp order.
+//   (K-SET under the read/write model and PART of debit-credit-only bulks:
+//   exec_dc.cu; K-SET of blind increments and SCAN: analysis.cu.)
 //   TPL (Section 5.1)    ordered counter locks: an operation whose group has
 //       `ticket` earlier operations before its run waits until that many have
 //       released the item's counter, then the transaction runs and every
@@ -28,7 +29,6 @@
 #include <cooperative_groups.h>
 
 #include "engine.h"
-#include "levels.cuh"
 #include "procs.cuh"
 #include "cta_groups.cuh"
 
@@ -37,6 +37,16 @@ namespace cg = cooperative_groups;
 namespace gtx {
 
 namespace {
+
+struct LevelArgs {
+    DevDB db;
+    DevBulk b;
+    const BulkCtl *ctl;
+    const uint32_t *level_off;
+    const uint32_t *type_cut; // per level, where new-order, payment, order-status start (or null)
+    uint32_t k0, k1;          // levels [k0, k1)
+    bool atomic_add;
+};
 
 struct KsetArgs {
     DevDB db;
@@ -137,11 +147,6 @@ __global__ void __launch_bounds__(256) kset_level_kernel(LevelArgs a)
     if (a.ctl->err) return;
     const int64_t hb = a.ctl->base.hist;
     const uint32_t lo = __ldg(&a.level_off[a.k0]), hi = __ldg(&a.level_off[a.k0 + 1]);
-    if (a.rec_dc) {
-        for (uint32_t pos = lo + blockIdx.x * blockDim.x + threadIdx.x; pos < hi; pos += gridDim.x * blockDim.x)
-            exec_dc_record(a.db, a.b, a.rec_dc[pos], hb + pos, a.atomic_add);
-        return;
-    }
     LevelLanes L;
     L.make(lo, hi, a.type_cut ? a.type_cut + 3 * (int64_t)a.k0 : nullptr);
     for (uint32_t x = blockIdx.x * blockDim.x + threadIdx.x; x < L.v; x += gridDim.x * blockDim.x) {
@@ -318,9 +323,6 @@ __global__ void part_kernel(DevDB db, DevBulk b, const BulkCtl *ctl, const uint3
     }
 }
 
-constexpr int kPartDcTellers = 32;   // tellers per branch the PART runner keeps on chip
-
-
 constexpr uint32_t kFull = 0xffffffffu;
 
 // sum of `x` over the lanes of `m` (this lane's group) and its inclusive
@@ -352,99 +354,6 @@ __device__ __forceinline__ void warp_add(bool on, uint32_t key, unsigned long lo
         x = tot;
     }
     if (on && lane == (uint32_t)(__ffs(m) - 1)) atomicAdd(cell, (unsigned long long)x);
-}
-
-// PART for debit-credit bulks with one warp per partition (branch).  The
-// warp runs its partition's transactions in timestamp order, 32 at a time:
-// each step loads 32 records and their accounts at once, and lanes that
-// share an account within the step are grouped by __match_any_sync -- each
-// lane's new balance is the balance loaded for the step plus the inclusive
-// prefix of the group's deltas in lane (timestamp) order, and the group's
-// last lane writes the account back.  That is the result of running the
-// step's transactions one by one, so the partition still executes serially
-// in the sense of Section 5.2 (no other partition touches its rows, no
-// locks); the step only spreads the order-independent work (records,
-// history rows, outputs, teller and branch sums) over the lanes.  The
-// branch balance and its tellers stay on chip for the whole partition.
-// __syncwarp between steps orders one step's account stores before the
-// next step's loads.
-__global__ void __launch_bounds__(256) part_dc_warp_kernel(DevDB db, DevBulk b, const BulkCtl *ctl,
-                                                           const DcRecord *rec, const uint32_t *pkeys,
-                                                           const uint32_t *part_start)
-{
-    __shared__ int64_t s_tel[8][32];   // this warp's tellers (at most 32 per branch)
-    const uint32_t lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const uint32_t p = blockIdx.x * (blockDim.x >> 5) + wib;
-    if (p >= ctl->npart || ctl->err) return;   // whole warps; no block barrier below
-    const int64_t hb = ctl->base.hist;
-    const uint32_t lo = part_start[p], hi = part_start[p + 1];
-    if (kDebug && (lo >= hi || !dbg_in(hi, b.n + 1, b.err))) {   // warp-uniform
-        set_err(b.err, ERR_BOUNDS);
-        return;
-    }
-    const uint32_t br = __ldg(&pkeys[lo]);     // partition key = branch
-    const uint32_t tpb = (uint32_t)(db.acc_per_br / db.acc_per_tel);
-    const uint32_t tel0 = br * tpb;
-    if (kDebug && (tpb > 32 || !dbg_in((int64_t)tel0 + tpb, db.n_tel + 1, b.err))) {
-        set_err(b.err, ERR_BOUNDS);
-        return;
-    }
-    int64_t *tel = s_tel[wib];
-    tel[lane] = lane < tpb ? __ldcg(&db.tel_bal[tel0 + lane]) : 0;
-    int64_t bsum = 0;
-    __syncwarp();
-    // the first step's records and accounts on their way
-    DcRecord r{};
-    if (lo + lane < hi) r = rec[lo + lane];
-    for (uint32_t base = lo; base < hi; base += 32) {
-        const uint32_t i = base + lane;
-        bool act = i < hi;
-        if (kDebug && act && !(dbg_dc_rows(db, b, r.a, r.tl, r.br, r.t) && r.br == br && r.tl >= tel0 &&
-                               r.tl < tel0 + tpb)) {
-            set_err(b.err, ERR_BOUNDS);       // a record outside this partition's rows
-            act = false;
-        }
-        const int64_t slot = hb + i;
-        const bool run = act && slot < db.hist_cap;
-        if (act && !run) {                     // history full: not executed
-            set_err(b.err, ERR_CAPACITY);
-            b.status[r.t] = 3;
-        }
-        const int64_t old = run ? __ldcg(&db.acc_bal[r.a]) : 0;
-        // the next step's records, and its accounts into L2
-        DcRecord nr{};
-        if (base + 32 + lane < hi) {
-            nr = rec[base + 32 + lane];
-            if (!kDebug || nr.a < db.n_acc) prefetch_l2(&db.acc_bal[nr.a]);
-        }
-        const uint32_t am = __match_any_sync(kFull, run ? r.a : (0xFFFFFFE0u | lane));
-        int64_t pre = r.delta, tot = r.delta;
-        if (__any_sync(kFull, run && __popc(am) > 1)) group_sum(am, r.delta, pre, tot);
-        if (run) {
-            const int64_t na = wrap_add(old, pre);
-            if (lane == 31u - (uint32_t)__clz(am)) __stcg(&db.acc_bal[r.a], wrap_add(old, tot));
-            db.h_ts[slot] = r.ts;
-            db.h_acc[slot] = r.a;
-            db.h_tel[slot] = r.tl;
-            db.h_br[slot] = br;
-            db.h_delta[slot] = r.delta;
-            b.out[(int64_t)r.t * b.R] = na;
-            b.status[r.t] = 0;
-        }
-        // teller sums: one addition per teller by its group's first lane
-        const uint32_t tm = __match_any_sync(kFull, run ? r.tl : (0xFFFFFFE0u | lane));
-        int64_t tpre, ttot = r.delta;
-        if (__any_sync(kFull, run && __popc(tm) > 1)) group_sum(tm, r.delta, tpre, ttot);
-        if (run && lane == (uint32_t)(__ffs(tm) - 1)) tel[r.tl - tel0] = wrap_add(tel[r.tl - tel0], ttot);
-        bsum = wrap_add(bsum, run ? r.delta : 0);
-        __syncwarp();   // this step's account stores before the next step's loads
-        r = nr;
-    }
-    // the branch: the sum of every lane's deltas
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) bsum = wrap_add(bsum, __shfl_xor_sync(kFull, bsum, o));
-    if (lane == 0) __stcg(&db.br_bal[br], wrap_add(__ldcg(&db.br_bal[br]), bsum));
-    if (lane < tpb) __stcg(&db.tel_bal[tel0 + lane], tel[lane]);
 }
 
 struct TplArgs {
@@ -1018,7 +927,7 @@ cudaError_t launch_kset(gputx_bulk *b, const uint32_t *order, int64_t nchunks, i
 }
 
 cudaError_t launch_kset_levels(gputx_bulk *b, const uint32_t *level_off_host, int64_t depth, int narrow_max,
-                               bool atomic_add, const DcRecord *dc_records, const uint32_t *type_cut_host)
+                               bool atomic_add, const uint32_t *type_cut_host)
 {
     gputx_db *db = b->db;
     if (b->n == 0) return cudaSuccess;
@@ -1027,8 +936,7 @@ cudaError_t launch_kset_levels(gputx_bulk *b, const uint32_t *level_off_host, in
     a.b = make_dev_bulk(b, atomic_add ? GPUTX_CONFLICT_ADD : GPUTX_CONFLICT_PAPER);
     a.ctl = b->ctl;
     a.level_off = b->sc.level_off;
-    a.rec_dc = dc_records;
-    a.type_cut = (type_cut_host && !dc_records) ? b->sc.type_cut : nullptr;
+    a.type_cut = type_cut_host ? b->sc.type_cut : nullptr;
     a.atomic_add = atomic_add;
     const int64_t levels = depth + 1;
     // lanes per level: the launch shapes follow them
@@ -1076,11 +984,7 @@ cudaError_t launch_kset_levels(gputx_bulk *b, const uint32_t *level_off_host, in
         int threads = (int)((wmax + csize - 1) / csize);
         threads = ((threads + 31) / 32) * 32;
         threads = threads < 32 ? 32 : (threads > 1024 ? 1024 : threads);
-        if (a.rec_dc) {
-            // the records this bulk was gathered into decide the runner
-            cudaError_t e2 = launch_narrow_dc(a, csize, threads, b->stream);
-            if (e2) return e2;
-        } else if (csize <= 1) {
+        if (csize <= 1) {
             if (threads <= 256) kset_narrow_kernel<false, 256><<<1, threads, 0, b->stream>>>(a);
             else kset_narrow_kernel<false, 1024><<<1, threads, 0, b->stream>>>(a);
         } else {
@@ -1110,14 +1014,7 @@ cudaError_t launch_kset_levels(gputx_bulk *b, const uint32_t *level_off_host, in
     return cudaGetLastError();
 }
 
-bool part_dc_applies(const gputx_db *db, int part_size)
-{
-    const DevDB &d = db->dev;
-    return d.registered == (1u << GPUTX_T_DC_DEBIT_CREDIT) && part_size == 1 && d.n_br > 0 &&
-           d.acc_per_br / d.acc_per_tel <= kPartDcTellers;
-}
-
-cudaError_t launch_part(gputx_bulk *b, const uint32_t *pkeys, int block, int64_t max_parts, int part_size)
+cudaError_t launch_part(gputx_bulk *b, const uint32_t *pkeys, int block, int64_t max_parts)
 {
     gputx_db *db = b->db;
     if (b->n == 0) return cudaSuccess;
@@ -1129,15 +1026,8 @@ cudaError_t launch_part(gputx_bulk *b, const uint32_t *pkeys, int block, int64_t
     threads = ((threads + 7) / 8) * 8;
     threads = threads < 8 ? 8 : (threads > block ? block : threads);
     const int64_t grid = (parts + threads - 1) / threads;   // npart <= parts, read on the device
-    if (part_dc_applies(db, part_size)) {
-        // one warp per partition, 8 warps a CTA
-        const int64_t wgrid = (parts + 7) / 8;
-        part_dc_warp_kernel<<<(unsigned)wgrid, 256, 0, b->stream>>>(db->dev, d, b->ctl, b->sc.rec_dc, pkeys,
-                                                                    b->sc.part_start);
-    } else {
-        const size_t smem = (size_t)threads * 2 * CachedCells::kSlots * sizeof(unsigned long long);
-        part_kernel<<<(unsigned)grid, threads, smem, b->stream>>>(db->dev, d, b->ctl, pkeys, b->sc.part_start);
-    }
+    const size_t smem = (size_t)threads * 2 * CachedCells::kSlots * sizeof(unsigned long long);
+    part_kernel<<<(unsigned)grid, threads, smem, b->stream>>>(db->dev, d, b->ctl, pkeys, b->sc.part_start);
     count_launches(1);
     return cudaGetLastError();
 }

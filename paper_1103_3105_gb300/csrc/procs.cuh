@@ -143,6 +143,22 @@ __device__ __forceinline__ int access_set(const DevDB &db, int32_t type, const i
     return 0;
 }
 
+// the operation of a transaction of a single-operation type (debit-credit, the
+// subscriber types), as access_set gives it
+__device__ __forceinline__ void single_op(const DevDB &db, int32_t type, int64_t p0, int mode, uint32_t &obj,
+                                          uint32_t &cls, uint32_t &root)
+{
+    if (type == GPUTX_T_DC_DEBIT_CREDIT) {
+        root = db.div_br.div((uint32_t)p0);
+        obj = mode == GPUTX_CONFLICT_ADD ? db.o_acc + (uint32_t)p0 : db.o_br + root;
+        cls = CLS_W;
+    } else {
+        root = (uint32_t)p0;
+        obj = db.o_sub + root;
+        cls = type <= GPUTX_T_SUB_GET_NEW_DEST ? CLS_R : CLS_W;
+    }
+}
+
 // number of operations without materialising them
 __device__ __forceinline__ int op_count(const DevDB &db, int32_t type, const int64_t *p)
 {
@@ -448,16 +464,6 @@ __device__ __forceinline__ void exec_dc(const DevDB &db, const DevBulk &b, const
 {
     DcOut o;
     if (dc_state(db, b, v, atomic_add, cells, o)) dc_finish(db, b, o);
-}
-
-// one whole transaction of a wide k-set from its packed record, reading its
-// balances then writing them (atomic_add: teller and branch by atomics)
-__device__ __forceinline__ void exec_dc_record(const DevDB &db, const DevBulk &b, const DcRecord &r, int64_t slot,
-                                               bool atomic_add)
-{
-    GlobalCells g;
-    DcOut o;
-    if (dc_state_core(db, b, r.a, r.tl, r.br, r.delta, r.ts, r.t, slot, atomic_add, g, o)) dc_finish(db, b, o);
 }
 
 // subscriber-location procedures (stand-ins shaped like TM-1, Appendix E)
