@@ -222,7 +222,7 @@ struct OffsetMode {
 struct RankMode {
     const uint32_t *sk, *sv;
     uint32_t *level;
-    uint32_t *rid;   // optional: global run id, bit 31 = first run of its group
+    uint32_t *rid;   // optional: place within the run, bit 31 = first run of its group
     __device__ uint64_t element(int64_t i) const
     {
         const uint32_t k = sk[i], v = sv[i];
@@ -230,11 +230,9 @@ struct RankMode {
         uint32_t runhead = 1;
         if (!head) {
             const uint32_t c = v & 3u, pc = sv[i - 1] & 3u;
-            runhead = !(c == pc && c != CLS_W);
+            runhead = !(c == pc && cls_shares(c));
         }
-        // the run ids run on over all groups; without them both fields start
-        // again at each group (cutting the scan's look-back)
-        return DualSeg::make(head, head ? 0u : runhead, rid ? 0u : head, runhead);
+        return DualSeg::make(head, head ? 0u : runhead, runhead, 1);
     }
     __device__ void output(int64_t i, uint64_t s) const
     {
@@ -266,7 +264,7 @@ struct TicketMode {
         uint32_t runhead = 1;
         if (!head) {
             const uint32_t c = v & 3u, pc = sv[i - 1] & 3u;
-            runhead = !(c == pc && c != CLS_W);
+            runhead = !(c == pc && cls_shares(c));
         }
         return DualSeg::make(head, 1, runhead, 1);
     }
@@ -292,34 +290,68 @@ struct TicketMode {
 // the largest, over its operations outside their group's first run, of one
 // more than the deepest transaction of the run before -- the longest path of
 // the conflict graph, the depth the Jacobi refinement converges to.  Here each
-// transaction computes it once the runs before its operations are complete.
-// Run q keeps one 64-bit word: the number of its operations still to finish
-// (high half) and the largest depth among the finished ones (low half).  A
-// finishing operation replaces both at once by compare-and-swap, so a waiter
-// that reads a count of zero reads the run's maximum in the same word: no
-// fence and no second read.  Transactions run in timestamp order, a CTA's
-// chunk of consecutive ones at a time, so every run a transaction waits for
-// belongs to earlier transactions already running: the chain of waits always
-// ends.
+// transaction computes it once the transactions of the runs before its
+// operations have theirs.
+//
+// Two numbers come out of the same pass: the depth (d and w0 are taken from
+// it) and the level the transaction executes in, which leaves out the edges
+// between two blind increments of the read/write model (CLS_BW): K-SET applies
+// those by atomic additions, so they order nothing.  Order-entry's payments
+// then run beside each other although all of a warehouse's write its total.
+// A finished transaction publishes both in one 64-bit word, so a waiter needs
+// no fence and no second read; a run of several operations is read word by
+// word.
+//
+// What bounds the pass is the longest path, so its hops are made few and cheap.
+// A CTA holds 1,024 consecutive transactions and works in rounds.  In a round a
+// transaction looks at those of the chunk it still waits for, in shared memory,
+// and every kFlowOutside-th round at those of earlier chunks, in L2.  One that
+// waits for a single transaction p knows its depth as max(m, depth(p) + l); if p
+// does too, it takes over p's p (pointer jumping), so a chain through a chunk --
+// the payments of a warehouse -- is one step behind the chunk before in
+// logarithmically many rounds, and in one once that step is known.  (Lanes that
+// each poll by themselves, without rounds: 2,570 us where this takes 1,050;
+// rounds without the jumps: 1,180.)  CTAs far behind the front would only flood
+// L2 with polls: a CTA starts when all but kFlowAhead chunks before its own are
+// finished.  Chunks are claimed in timestamp order, so every transaction waited
+// for belongs to a running CTA: the chain of waits always ends.  Order-entry,
+// 200,003 transactions under R/W (d = 1,442): 1,050 us; one 64-bit word per
+// run, counted off by compare-and-swap by each of its operations, polls in L2
+// only: 2,950.
 
-// per operation: its run id into the transaction's slot, its run counted
+// per operation: the last operation of the run before its own
+// (kPredNone: none).  Several transactions in that run: kPredRun | the sorted
+// position of the last.  One: its index, and kPredBlind if both are blind
+// increments.
+constexpr uint32_t kPredNone = 0xffffffffu, kPredRun = 1u << 30, kPredVal = kPredRun - 1u;
+constexpr uint32_t kPredBlind = 1u << 31, kPredTxn = (1u << 25) - 1u;
+// levels from the predecessor to the transaction (0: it does not order the execution)
+__device__ __forceinline__ uint32_t pred_step(uint32_t p) { return !(p & kPredRun) && (p & kPredBlind) ? 0u : 1u; }
+
 __global__ void depth_prep_kernel(const uint32_t *sv, const uint32_t *rid, int64_t m, const uint32_t *op_off,
-                                  int kslots, uint32_t *txn_rid, unsigned long long *runword, const BulkCtl *ctl)
+                                  int kslots, uint32_t *pred, const BulkCtl *ctl)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= m || ctl->err) return;
     const uint32_t v = sv[i];
     if (v == OP_SENTINEL) return;
-    const uint32_t rr = rid[i];
+    const uint32_t r = rid[i];
     const uint32_t txn = v >> 7, j = (v >> 2) & 31u;
     const int64_t slot = (op_off ? (int64_t)op_off[txn] : (int64_t)txn * kslots) + j;
-    txn_rid[slot] = rr;
-    atomicAdd(&runword[rr & 0x7fffffffu], 1ull << 32);
+    uint32_t p = kPredNone;
+    if (!(r & 0x80000000u)) {
+        const int64_t q = i - r - 1;                       // the run before ends here
+        const uint32_t w = sv[q];
+        p = (rid[q] & 0x7fffffffu) ? (kPredRun | (uint32_t)q) : (w >> 7);
+        if (!(p & kPredRun) && (v & 3u) == CLS_BW && (w & 3u) == CLS_BW) p |= kPredBlind;
+    }
+    pred[slot] = p;
 }
 
-constexpr uint32_t kNoRun = 0xffffffffu;   // an operation slot with no operation
-constexpr uint32_t kFlowSleepMax = 512;     // longest back-off between polls, ns
-constexpr int kFlowBlocksPerSm = 1;         // resident CTAs of the pass per SM (fewer waiters poll less)
+constexpr int kFlowThreads = 1024;
+constexpr uint32_t kFlowAhead = 8;          // unfinished chunks before one that starts
+constexpr uint32_t kFlowOutside = 1;        // rounds from one look at earlier chunks to the next
+constexpr unsigned long long kNotYet = ~0ull;
 
 __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long *p)
 {
@@ -328,104 +360,205 @@ __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long
     return v;
 }
 
-__global__ void __launch_bounds__(256) depth_flow_kernel(const uint32_t *txn_rid, const uint32_t *op_off, int kslots,
-                                                        unsigned long long *runword, uint32_t *level, BulkCtl *ctl,
-                                                        int64_t n, uint64_t limit_ns)
+struct FlowArgs {
+    const uint32_t *pred, *op_off, *sv, *rid;
+    int kslots;
+    unsigned long long *depths;              // per transaction: depth << 32 | level, kNotYet before
+    uint32_t *level;
+    BulkCtl *ctl;
+    int64_t n;
+    bool graph;                              // transactions from n_live on are padding
+    uint64_t limit_ns;
+};
+
+// what a transaction that waits for one other, p, knows: its depth is
+// max(dep, depth(p) + dlen), its level max(lev, level(p) + llen), or lev if llen
+// is 0; p = kPredNone while it waits for several
+struct FlowNode {
+    uint32_t p, len, dep, lev;               // len: dlen << 16 | llen, at most kFlowThreads each
+};
+
+__global__ void __launch_bounds__(kFlowThreads, 1) depth_flow_kernel(FlowArgs a)
 {
-    __shared__ uint32_t s_c, s_stop;
-    if (ctl->err) return;   // set before this launch only: every block returns
-    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->rounds = 1;
+    extern __shared__ __align__(16) uint32_t s_pred[];   // [MAX_OPS][kFlowThreads], then the nodes
+    FlowNode *s_node = reinterpret_cast<FlowNode *>(s_pred + MAX_OPS * kFlowThreads);
+    __shared__ uint32_t s_c, s_stop, s_moved, s_late;
+    __shared__ unsigned long long s_depth[kFlowThreads];
+    BulkCtl *ctl = a.ctl;
+    const uint32_t tid = threadIdx.x;
+    if (blockIdx.x == 0 && tid == 0) ctl->rounds = 1;
+    const int64_t n = a.graph ? (int64_t)ctl->n_live : a.n;
+    uint32_t dmax = 0, lmax = 0, zero = 0;
     while (true) {
-        if (threadIdx.x == 0) {
+        if (tid == 0) {
             s_stop = *(volatile uint32_t *)&ctl->err ? 1u : 0u;
             s_c = atomicAdd(&ctl->claim, 1u);
+            s_moved = 1;
+            s_late = 0;
         }
+        s_depth[tid] = kNotYet;
+        s_node[tid].p = kPredNone;
         __syncthreads();
-        const int64_t start = (int64_t)s_c * blockDim.x;
-        if (s_stop || start >= n) break;
-        const int64_t t = start + threadIdx.x;
+        const uint32_t c = s_c;
+        const int64_t start_ = (int64_t)c * kFlowThreads;
+        if (s_stop || start_ >= a.n) break;
+        const uint32_t start = (uint32_t)start_;
+        const int64_t t = start_ + tid;
+        // bit j: the run before operation j's is not known complete, and is a
+        // transaction of this chunk / one of an earlier chunk, or several
+        uint32_t inside = 0, outside = 0;
         if (t < n) {
-            const int64_t s0 = op_off ? (int64_t)op_off[t] : t * kslots;
-            const int k = op_off ? (int)(op_off[t + 1] - op_off[t]) : kslots;
-            // every per-operation array below is indexed by unrolled loop
-            // counters only, so it lives in registers
-            uint32_t rr[MAX_OPS];
-            uint32_t waits = 0, own = 0;   // bit j: operation j follows an earlier run / has a run
+            const int64_t s0 = a.op_off ? (int64_t)a.op_off[t] : t * a.kslots;
+            const int k = a.op_off ? (int)(a.op_off[t + 1] - a.op_off[t]) : a.kslots;
 #pragma unroll
             for (int j = 0; j < MAX_OPS; j++) {
-                rr[j] = j < k ? txn_rid[s0 + j] : kNoRun;
-                if (rr[j] != kNoRun) {
-                    own |= 1u << j;
-                    if (!(rr[j] & 0x80000000u)) waits |= 1u << j;
-                }
+                const uint32_t p = j < k ? __ldg(&a.pred[s0 + j]) : kPredNone;
+                if (p == kPredNone) continue;
+                s_pred[j * kFlowThreads + tid] = p;
+                if (!(p & kPredRun) && (p & kPredTxn) >= start) inside |= 1u << j;
+                else outside |= 1u << j;
             }
-            // the preceding runs: all polled at once (first, and after any of
-            // them completes), else only the first incomplete one, so that
-            // waiters far down a chain do not flood L2 with polls
-            uint32_t pending = waits, lv = 0;
+        }
+        if (tid == 0 && c > kFlowAhead) {                  // not yet near the front
+            uint32_t f = ld_relaxed_gpu(&ctl->front);
             uint64_t t_prog = globaltimer();
-            uint32_t ns = 64;
-            bool all = true;
-            while (pending) {
-                // this look's runs: every pending one, or the first
-                const uint32_t look = all ? pending : pending & (0u - pending);
-                unsigned long long w[MAX_OPS];
-#pragma unroll
-                for (int j = 0; j < MAX_OPS; j++)   // all loads in flight at once
-                    w[j] = (look >> j & 1u) ? ld_relaxed_u64(&runword[(rr[j] & 0x7fffffffu) - 1u]) : 0ull;
-                uint32_t still = pending;
-#pragma unroll
-                for (int j = 0; j < MAX_OPS; j++) {
-                    if ((look >> j & 1u) && !(w[j] >> 32)) {   // complete: its maximum is final
-                        still &= ~(1u << j);
-                        if ((uint32_t)w[j] + 1u > lv) lv = (uint32_t)w[j] + 1u;
-                    }
-                }
-                if (still != pending) {
-                    pending = still;
-                    t_prog = globaltimer();
-                    ns = 64;
-                    all = true;
-                    continue;
-                }
-                all = false;
-                if (globaltimer() - t_prog > limit_ns) {
-                    set_err(&ctl->err, ERR_TIMEOUT);
-                    break;
-                }
-                __nanosleep(ns);
-                if (ns < kFlowSleepMax) ns <<= 1;
+            while (c > f && c - f > kFlowAhead) {
+                if (globaltimer() - t_prog > a.limit_ns || *(volatile uint32_t *)&ctl->err) break;
+                __nanosleep(100);
+                const uint32_t g = ld_relaxed_gpu(&ctl->front);
+                if (g != f) t_prog = globaltimer();
+                f = g;
             }
-            level[t] = lv;
-            // this transaction's depth into each of its runs, counted off in
-            // the same compare-and-swap
-            unsigned long long cur[MAX_OPS];
-#pragma unroll
-            for (int j = 0; j < MAX_OPS; j++) cur[j] = 1ull << 32;   // a guess: the run's only operation
-            uint32_t todo = own;
-            for (int attempt = 0; todo && attempt < (1 << 20); attempt++) {
-                unsigned long long prev[MAX_OPS];
-#pragma unroll
-                for (int j = 0; j < MAX_OPS; j++) {   // every swap in flight at once
-                    prev[j] = cur[j];
-                    if (!(todo >> j & 1u)) continue;
-                    const uint32_t mx = (uint32_t)cur[j] > lv ? (uint32_t)cur[j] : lv;
-                    const unsigned long long nv = (((cur[j] >> 32) - 1ull) << 32) | mx;
-                    prev[j] = atomicCAS(&runword[rr[j] & 0x7fffffffu], cur[j], nv);
-                }
-#pragma unroll
-                for (int j = 0; j < MAX_OPS; j++) {
-                    if (!(todo >> j & 1u)) continue;
-                    if (prev[j] == cur[j]) todo &= ~(1u << j);
-                    else cur[j] = prev[j];
-                }
-            }
-            if (todo) set_err(&ctl->err, ERR_TIMEOUT);
         }
         __syncthreads();
+        uint32_t dep = 0, lev = 0;
+        auto take = [&](uint32_t word, unsigned long long w) {
+            const uint32_t step = pred_step(word), d = (uint32_t)(w >> 32) + 1u, l = (uint32_t)w + step;
+            dep = d > dep ? d : dep;
+            if (step) lev = l > lev ? l : lev;
+        };
+        bool done = t >= n;
+        FlowNode me{kPredNone, 0, 0, 0};
+        uint64_t t_prog = globaltimer();                   // thread 0's
+        for (uint32_t round = 0;; round++) {
+            // reads of what the round before left
+            bool moved = false;
+            const bool far = round % kFlowOutside == 0;
+            if (me.p != kPredNone) {
+                unsigned long long w = kNotYet;
+                if (me.p >= start) {
+                    w = s_depth[me.p - start];
+                    const FlowNode o = s_node[me.p - start];
+                    if (w == kNotYet && o.p != kPredNone) {           // jump over p
+                        const uint32_t dl = me.len >> 16, ll = me.len & 0xffffu;
+                        const uint32_t ol = o.len & 0xffffu;
+                        me.dep = o.dep + dl > me.dep ? o.dep + dl : me.dep;
+                        if (ll) me.lev = o.lev + ll > me.lev ? o.lev + ll : me.lev;
+                        me.len = ((dl + (o.len >> 16)) << 16) | (ll && ol ? ll + ol : 0u);
+                        me.p = o.p;
+                        moved = true;
+                    }
+                } else if (far) {
+                    w = ld_relaxed_u64(&a.depths[me.p]);
+                }
+                if (w != kNotYet) {
+                    const uint32_t d = (uint32_t)(w >> 32) + (me.len >> 16), l = (uint32_t)w + (me.len & 0xffffu);
+                    dep = d > me.dep ? d : me.dep;
+                    lev = (me.len & 0xffffu) && l > me.lev ? l : me.lev;
+                    inside = outside = 0;
+                    moved = true;
+                }
+            } else {
+                for (uint32_t b = inside; b; b &= b - 1) {
+                    const int j = __ffs(b) - 1;
+                    const uint32_t p = s_pred[j * kFlowThreads + tid];
+                    const unsigned long long w = s_depth[(p & kPredTxn) - start];
+                    if (w == kNotYet) continue;
+                    take(p, w);
+                    inside &= ~(1u << j);
+                    moved = true;
+                }
+                // up to four at a time, their loads in flight together
+                for (uint32_t b = far ? outside : 0u; b;) {
+                    uint32_t p[4], bit[4];
+                    unsigned long long w[4];
+#pragma unroll
+                    for (int u = 0; u < 4; u++) {
+                        bit[u] = b & (0u - b);
+                        b &= b - 1;
+                        p[u] = bit[u] ? s_pred[(__ffs(bit[u]) - 1) * kFlowThreads + tid] : kPredNone;
+                        w[u] = bit[u] && !(p[u] & kPredRun) ? ld_relaxed_u64(&a.depths[p[u] & kPredTxn]) : kNotYet;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; u++) {
+                        if (!bit[u]) continue;
+                        if (p[u] & kPredRun) {             // a run of several operations: all of them
+                            const uint32_t q = p[u] & kPredVal, len = (__ldg(&a.rid[q]) & 0x7fffffffu) + 1u;
+                            uint32_t d = 0, l = 0, k = 0;
+                            for (; k < len; k++) {
+                                const uint32_t x = __ldg(&a.sv[q - k]) >> 7;
+                                const unsigned long long v = x >= start ? s_depth[x - start]
+                                                                        : ld_relaxed_u64(&a.depths[x]);
+                                if (v == kNotYet) break;
+                                d = (uint32_t)(v >> 32) > d ? (uint32_t)(v >> 32) : d;
+                                l = (uint32_t)v > l ? (uint32_t)v : l;
+                            }
+                            w[u] = k == len ? ((unsigned long long)d << 32) | l : kNotYet;
+                        }
+                        if (w[u] == kNotYet) continue;
+                        take(p[u], w[u]);
+                        outside &= ~bit[u];
+                        moved = true;
+                    }
+                }
+                const uint32_t left = inside | outside;
+                if (left && !(left & (left - 1))) {        // one left
+                    const uint32_t p = s_pred[(__ffs(left) - 1) * kFlowThreads + tid];
+                    if (!(p & kPredRun)) me = FlowNode{p & kPredTxn, 0x10000u | pred_step(p), dep, lev};
+                }
+            }
+            if (s_late) inside = outside = 0;              // gave up, but publishes: no later waiter hangs
+            __syncthreads();
+            // writes for the next round
+            if (!done && !(inside | outside)) {
+                const unsigned long long w = ((unsigned long long)dep << 32) | lev;
+                s_depth[tid] = w;
+                asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(&a.depths[t]), "l"(w) : "memory");
+                me.p = kPredNone;
+                done = true;
+            } else if (me.p != kPredNone) {
+                s_node[tid] = me;
+            }
+            if (moved) s_moved = 1;
+            if (!__syncthreads_or(!done)) break;
+            if (tid == 0 && round % 64 == 0) {
+                if (s_moved) {
+                    t_prog = globaltimer();
+                    s_moved = 0;
+                } else if (globaltimer() - t_prog > a.limit_ns) {
+                    set_err(&ctl->err, ERR_TIMEOUT);
+                    s_late = 1;
+                }
+            }
+        }
+        if (t < n) {
+            a.level[t] = lev;
+            dmax = dep > dmax ? dep : dmax;
+            lmax = lev > lmax ? lev : lmax;
+            zero += dep == 0;
+        }
+        if (tid == 0) atomicAdd(&ctl->front, 1u);
+        __syncthreads();                                   // s_c, s_late are read until here
+    }
+    dmax = __reduce_max_sync(0xffffffffu, dmax);
+    lmax = __reduce_max_sync(0xffffffffu, lmax);
+    zero = __reduce_add_sync(0xffffffffu, zero);
+    if ((tid & 31) == 0) {
+        if (dmax) atomicMax(&ctl->depth, dmax);
+        if (lmax) atomicMax(&ctl->last_level, lmax);
+        if (zero) atomicAdd(&ctl->w0, zero);
     }
 }
-
 
 // d and w0 (Appendix D structural parameters)
 __global__ void level_stats_kernel(const uint32_t *level, int64_t n, BulkCtl *ctl)
@@ -443,7 +576,11 @@ __global__ void level_stats_kernel(const uint32_t *level, int64_t n, BulkCtl *ct
     zero = __reduce_add_sync(0xffffffffu, zero);
     if ((threadIdx.x & 31) == 0) { atomicMax(&s_max, mx); atomicAdd(&s_zero, zero); }
     __syncthreads();
-    if (threadIdx.x == 0) { atomicMax(&ctl->depth, s_max); atomicAdd(&ctl->w0, s_zero); }
+    if (threadIdx.x == 0) {
+        atomicMax(&ctl->depth, s_max);
+        atomicMax(&ctl->last_level, s_max);
+        atomicAdd(&ctl->w0, s_zero);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -503,7 +640,7 @@ __global__ void seg_base_kernel(const uint32_t *seg_depth, BulkCtl *ctl, uint32_
         acc += seg_depth[i] + 1;
     }
     seg_base[nseg] = acc;
-    ctl->depth = acc - 1;
+    ctl->depth = ctl->last_level = acc - 1;
 }
 
 __global__ void part_fallback_kernel(BulkCtl *ctl)
@@ -512,19 +649,18 @@ __global__ void part_fallback_kernel(BulkCtl *ctl)
 }
 
 // Level boundaries from the keys sorted by (level << tbits | type); with
-// type_cut, also where each level's new-order, payment and order-status
-// transactions start (type_cut[3 k + j] = first position of level k whose
-// type is >= 8 + j), so the executors can give order-entry's line-parallel
-// types their lane groups.  A cut (k, type) lands on the first key at or
-// above k << tbits | type; levels are contiguous, so between two adjacent
-// keys at most two levels' cuts fall.
+// type_cut, also where each level's new-orders and payments start (type_cut[2 k
+// + j] = first position of level k whose type is >= 8 + j), so the executors
+// can give the new-orders their lane groups.  A cut (k, type) lands on the first
+// key at or above k << tbits | type; levels are contiguous, so between two
+// adjacent keys at most two levels' cuts fall.
 // a debug build's check of the level table the executors index by: the
 // bounds of levels 0..depth rise and stay within the bulk (an executor whose
 // bulk carries an error returns before its first gather)
 __global__ void check_level_off_kernel(const uint32_t *level_off, int64_t n, BulkCtl *ctl)
 {
     const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (ctl->err || k > (int64_t)ctl->depth || k >= n) return;
+    if (ctl->err || k > (int64_t)ctl->last_level || k >= n) return;
     const uint32_t lo = level_off[k], hi = level_off[k + 1];
     if (lo > hi || !dbg_in(hi, n + 1, &ctl->err)) set_err(&ctl->err, ERR_BOUNDS);
 }
@@ -536,7 +672,7 @@ __global__ void level_off_kernel(const uint32_t *skeys, int64_t n, int tbits, ui
     if (i >= n || *err) return;
     // real levels are 0..depth; a graph bulk's padding sorts after them as
     // level n, whose boundary is the only one needed past depth
-    const uint32_t top = ctl->depth + 1;
+    const uint32_t top = ctl->last_level + 1;
     const uint32_t key = skeys[i];
     const uint32_t lv = key >> tbits;
     const uint32_t lvc = lv < top ? lv : top;
@@ -551,15 +687,15 @@ __global__ void level_off_kernel(const uint32_t *skeys, int64_t n, int tbits, ui
         const uint64_t below = i ? (uint64_t)skeys[i - 1] + 1 : 0;   // cuts in (key[i-1], key[i]]
         const uint32_t kmax = lv < top ? lv : top - 1;
         for (uint32_t k = i ? prev : 0; k <= kmax; k++)
-            for (uint32_t j = 0; j < 3; j++) {
+            for (uint32_t j = 0; j < 2; j++) {
                 const uint64_t cut = ((uint64_t)k << tbits) | (GPUTX_T_OE_NEW_ORDER + j);
-                if (cut >= below && cut <= key) type_cut[3 * k + j] = (uint32_t)i;
+                if (cut >= below && cut <= key) type_cut[2 * k + j] = (uint32_t)i;
             }
     }
     if (type_cut && i == n - 1 && lv < top)
-        for (uint32_t j = 0; j < 3; j++) {
+        for (uint32_t j = 0; j < 2; j++) {
             const uint64_t cut = ((uint64_t)lv << tbits) | (GPUTX_T_OE_NEW_ORDER + j);
-            if (cut > key) type_cut[3 * lv + j] = (uint32_t)n;
+            if (cut > key) type_cut[2 * lv + j] = (uint32_t)n;
         }
 }
 
@@ -567,12 +703,12 @@ struct ChunkMode {
     const uint32_t *level_off;
     uint32_t *chunk_off;
     uint32_t block;
-    const BulkCtl *ctl;   // levels = depth + 1, read on the device
+    const BulkCtl *ctl;   // levels = last_level + 1, read on the device
     const uint32_t *type_cut;   // chunks count lanes (order-entry groups) when set
     __device__ uint64_t element(int64_t k) const
     {
-        if (k > (int64_t)ctl->depth) return 0;
-        const uint32_t w = level_lane_count(level_off[k], level_off[k + 1], type_cut ? type_cut + 3 * k : nullptr);
+        if (k > (int64_t)ctl->last_level) return 0;
+        const uint32_t w = level_lane_count(level_off[k], level_off[k + 1], type_cut ? type_cut + 2 * k : nullptr);
         return DualSeg::make(0, 0, 0, (w + block - 1) / block);
     }
     __device__ void output(int64_t k, uint64_t s) const
@@ -587,7 +723,7 @@ __global__ void chunk_level_kernel(const uint32_t *chunk_off, const BulkCtl *ctl
 {
     const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (*err) return;
-    const int64_t levels = (int64_t)ctl->depth + 1;
+    const int64_t levels = (int64_t)ctl->last_level + 1;
     const uint32_t nchunks = chunk_off[levels];
     if (c >= cap || c >= nchunks) return;
     // largest k with chunk_off[k] <= c
@@ -1396,40 +1532,43 @@ cudaError_t launch_ticket_scan(gputx_bulk *b, const uint32_t *sk, const uint32_t
     return run_scan(b, tm, m);
 }
 
-cudaError_t launch_depth_flow(gputx_bulk *b, const uint32_t *sv, int64_t m)
-{
-    if (m == 0 || b->n == 0) return cudaSuccess;
-    cudaStream_t s = b->stream;
-    const bool fixed = b->db->uniform_k || b->graph;
-    const uint32_t *op_off = fixed ? nullptr : b->sc.op_off;
-    const int kslots = b->graph ? b->db->kmax : b->db->uniform_k;
-    // the per-slot run ids reuse a TPL buffer (free during the analysis)
-    uint32_t *txn_rid = b->sc.lock_key;
-    unsigned long long *runword = reinterpret_cast<unsigned long long *>(b->sc.runmax);
-    cudaError_t e;
-    if ((e = cudaMemsetAsync(txn_rid, 0xff, (size_t)m * sizeof(uint32_t), s))) return e;
-    if ((e = cudaMemsetAsync(runword, 0, (size_t)m * sizeof(unsigned long long), s))) return e;
-    if ((e = cudaMemsetAsync(&b->ctl->claim, 0, sizeof(uint32_t), s))) return e;
-    depth_prep_kernel<<<grid_for(m), TB, 0, s>>>(sv, b->sc.rid, m, op_off, kslots, txn_rid, runword, b->ctl);
-    static int per_sm = 0;
-    if (!per_sm) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, depth_flow_kernel, 256, 0);
-        if (per_sm > kFlowBlocksPerSm) per_sm = kFlowBlocksPerSm;
-        if (per_sm < 1) per_sm = 1;
-    }
-    int64_t grid = (int64_t)b->db->num_sms * per_sm;
-    const int64_t chunks = (b->n + 255) / 256;
-    if (grid > chunks) grid = chunks;
-    depth_flow_kernel<<<(unsigned)grid, 256, 0, s>>>(txn_rid, op_off, kslots, runword, b->sc.level, b->ctl, b->n,
-                                                     (uint64_t)b->db->cfg.spin_limit_ns);
-    count_launches(2);
-    return cudaGetLastError();
-}
-
 // exact depths after the one-pass ranks (A1): the dataflow pass
 cudaError_t launch_exact_depth(gputx_bulk *b, const uint32_t *sv, int64_t m)
 {
-    return launch_depth_flow(b, sv, m);
+    if (b->n == 0) return cudaSuccess;
+    if (m >= (int64_t)kPredVal) return cudaErrorInvalidValue;
+    cudaStream_t s = b->stream;
+    const bool fixed = b->db->uniform_k || b->graph;
+    FlowArgs a;
+    a.op_off = fixed ? nullptr : b->sc.op_off;
+    a.kslots = b->graph ? b->db->kmax : b->db->uniform_k;
+    // the per-slot predecessors reuse a TPL buffer (free during the analysis)
+    uint32_t *pred = b->sc.lock_key;
+    a.pred = pred;
+    a.sv = sv;
+    a.rid = b->sc.rid;
+    a.depths = b->sc.depths;
+    a.level = b->sc.level;
+    a.ctl = b->ctl;
+    a.n = b->n;
+    a.graph = b->graph;
+    a.limit_ns = (uint64_t)b->db->cfg.spin_limit_ns;
+    cudaError_t e;
+    if (m > 0 && (e = cudaMemsetAsync(pred, 0xff, (size_t)m * sizeof(uint32_t), s))) return e;
+    if ((e = cudaMemsetAsync(a.depths, 0xff, (size_t)b->n * sizeof(unsigned long long), s))) return e;
+    if ((e = cudaMemsetAsync(&b->ctl->claim, 0, sizeof(uint32_t), s))) return e;
+    if ((e = cudaMemsetAsync(&b->ctl->front, 0, sizeof(uint32_t), s))) return e;
+    if (m > 0) {
+        depth_prep_kernel<<<grid_for(m), TB, 0, s>>>(sv, b->sc.rid, m, a.op_off, a.kslots, pred, b->ctl);
+        count_launches(1);
+    }
+    const int64_t chunks = (b->n + kFlowThreads - 1) / kFlowThreads;
+    const int64_t grid = std::min<int64_t>(b->db->num_sms, chunks);
+    const size_t smem = (sizeof(uint32_t) * MAX_OPS + sizeof(FlowNode)) * kFlowThreads;
+    if ((e = cudaFuncSetAttribute(depth_flow_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
+    depth_flow_kernel<<<(unsigned)grid, kFlowThreads, smem, s>>>(a);
+    count_launches(1);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_level_stats(gputx_bulk *b)

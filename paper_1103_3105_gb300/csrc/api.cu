@@ -150,7 +150,7 @@ int type_ops(int t, int *maxk)
     switch (t) {
     case GPUTX_T_DC_DEBIT_CREDIT: *maxk = 1; return 1;
     case GPUTX_T_OE_NEW_ORDER: *maxk = 2 + 15; return -1;
-    case GPUTX_T_OE_PAYMENT: *maxk = 3; return 3;
+    case GPUTX_T_OE_PAYMENT: *maxk = 2; return 2;
     case GPUTX_T_OE_ORDER_STATUS: *maxk = 2; return 2;
     default: *maxk = 1; return 1;
     }
@@ -192,11 +192,11 @@ size_t carve_bulk(gputx_bulk *b, char *base, bool device_inputs)
     s.op_off = c.take<uint32_t>(nn + 1);
     s.level = c.take<uint32_t>(nn);
     s.rid = db->need_fixpoint ? c.take<uint32_t>(mm) : nullptr;
-    s.runmax = db->need_fixpoint ? c.take<uint32_t>(2 * mm) : nullptr;
+    s.depths = db->need_fixpoint ? c.take<unsigned long long>(nn) : nullptr;
     s.lock_key = c.take<uint32_t>(mm);
     s.lock_ticket = c.take<uint32_t>(mm);
     s.level_off = c.take<uint32_t>(nn + 2);
-    s.type_cut = db->group_oe ? c.take<uint32_t>(3 * (nn + 2)) : nullptr;
+    s.type_cut = db->group_oe ? c.take<uint32_t>(2 * (nn + 2)) : nullptr;
     s.chunk_off = c.take<uint32_t>(nn + 2);
     // chunks count lanes: at most lanes / block + levels, and order-entry
     // groups take up to 16 lanes a transaction (+ half-warp padding)
@@ -431,6 +431,9 @@ gputx_status gputx_create_db(const gputx_schema_desc *schema, const gputx_config
         TRY(dalloc(db, &d.c_ytd, n_c, "customer"));
         TRY(dalloc(db, &d.c_payment_cnt, n_c, "customer"));
         TRY(dalloc(db, &d.c_last_o_id, n_c, "customer"));
+        TRY(dalloc(db, &d.c_last_slot, n_c, "customer"));
+        if (cudaMemsetAsync(d.c_last_slot, 0xff, (size_t)n_c * sizeof(uint32_t), db->stream))
+            TRY(fail(db, GPUTX_ECUDA, "fill"));
         TRY(dalloc(db, &d.i_price, d.n_items, "item"));
         const int64_t ns = d.n_wh * d.n_items;
         TRY(dalloc(db, &d.s_quantity, ns, "stock"));
@@ -505,9 +508,9 @@ gputx_status gputx_register_types(gputx_db *db, const int32_t *type_ids, int n)
     // a bulk that mixes debit-credit with other types takes history rows
     // for its debit-credit transactions only
     db->hist_by_type = (db->dev.registered & 1u) && db->dev.registered != 1u;
-    // levels sorted by (level, type) know where each order-entry type starts
-    db->group_oe = db->tbits > 0 && (db->dev.registered & ((1u << GPUTX_T_OE_NEW_ORDER) |
-                                                           (1u << GPUTX_T_OE_ORDER_STATUS)));
+    // levels sorted by (level, type) know where the new-orders are; K-SET then
+    // runs them on lane groups and completes orders after the levels
+    db->group_oe = db->tbits > 0 && (db->dev.registered >> GPUTX_T_OE_NEW_ORDER & 1u);
     return GPUTX_OK;
 }
 
@@ -615,6 +618,7 @@ gputx_status gputx_load_table(gputx_db *db, int table, const int64_t *rows, size
         if ((st = put_col(db, d.c_balance, col64(1)))) return st;
         if ((st = put_col(db, d.c_ytd, col64(2)))) return st;
         if ((st = put_col(db, d.c_payment_cnt, col64(3)))) return st;
+        CK(cudaMemsetAsync(d.c_last_slot, 0xff, (size_t)n * sizeof(uint32_t), db->stream), "load");
         return put_col(db, d.c_last_o_id, col64(4));
     case GPUTX_TBL_OE_ITEM:
         if ((st = need(d.n_items, "item"))) return st;
@@ -1108,7 +1112,7 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
         // rank 0), and the one-pass depth bounds the exact one from below.
         // The exact-depth pass runs only once K-SET is chosen.
         if (db->need_fixpoint && strategy == GPUTX_KSET) CK(launch_exact_depth(b, sv, m), "exact depth");
-        CK(launch_level_stats(b), "stats");
+        else CK(launch_level_stats(b), "stats");
         if ((st = read_ctl(b))) return st;
         if (b->host_ctl.err) {
             CK(cudaEventRecord(b->ev[7], s), "event");
@@ -1127,9 +1131,8 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
                 b->fallback = 1;
             if (run == GPUTX_KSET && db->need_fixpoint) {
                 // exact depths for the level schedule (Property 1)
+                CK(cudaMemsetAsync(&b->ctl->depth, 0, 3 * sizeof(uint32_t), s), "stats");
                 CK(launch_exact_depth(b, sv, m), "exact depth");
-                CK(cudaMemsetAsync(&b->ctl->depth, 0, 2 * sizeof(uint32_t), s), "stats");
-                CK(launch_level_stats(b), "stats");
                 if ((st = read_ctl(b))) return st;
                 if (b->host_ctl.err) {
                     CK(cudaEventRecord(b->ev[7], s), "event");
@@ -1158,7 +1161,7 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
         CK(begin_tail(b, true), "order");
         if ((st = run_ranges(sk, sv, 7, true))) return st;
     } else if (run == GPUTX_KSET) {
-        const int64_t depth = b->host_ctl.depth;
+        const int64_t depth = b->host_ctl.last_level;
         const bool persistent = opts && opts->kset_launch == 1;
         // regroup by (level, type): reuse the free op buffers
         uint32_t *rk = ak, *rv = av, *rk2 = sk, *rv2 = sv;
@@ -1169,15 +1172,16 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
             CK(launch_gather(b, rv), "gather");
             CK(begin_tail(b), "order");
             if (b->timing) cudaEventRecord(b->ev[3], s);
-            CK(launch_kset(b, rv, b->sc.chunk_cap, block, add), "k-set execute");
+            CK(launch_kset(b, rv, b->sc.chunk_cap, block, add || db->need_fixpoint), "k-set execute");
+            CK(launch_orders(b), "orders");
         } else if (b->n > 0) {
             // plan launches from the level widths
             b->level_off_host.resize((size_t)depth + 2);
             CK(cudaMemcpyAsync(b->level_off_host.data(), b->sc.level_off, (depth + 2) * sizeof(uint32_t),
                                cudaMemcpyDeviceToHost, s), "level plan");
             if (b->sc.type_cut) {
-                b->type_cut_host.resize(3 * ((size_t)depth + 1));
-                CK(cudaMemcpyAsync(b->type_cut_host.data(), b->sc.type_cut, 3 * (depth + 1) * sizeof(uint32_t),
+                b->type_cut_host.resize(2 * ((size_t)depth + 1));
+                CK(cudaMemcpyAsync(b->type_cut_host.data(), b->sc.type_cut, 2 * (depth + 1) * sizeof(uint32_t),
                                    cudaMemcpyDeviceToHost, s), "level plan");
             }
             CK(cudaMemcpyAsync(&b->host_ctl.err, &b->ctl->err, 4, cudaMemcpyDeviceToHost, s), "level plan");
@@ -1187,9 +1191,10 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
                 CK(launch_gather(b, rv), "gather");
                 CK(begin_tail(b), "order");
                 if (b->timing) cudaEventRecord(b->ev[3], s);
-                CK(launch_kset_levels(b, b->level_off_host.data(), depth, narrow, add,
+                CK(launch_kset_levels(b, b->level_off_host.data(), depth, narrow, add || db->need_fixpoint,
                                       b->sc.type_cut ? b->type_cut_host.data() : nullptr),
                    "k-set execute");
+                CK(launch_orders(b), "orders");
             }
         } else {
             CK(begin_tail(b), "order");   // empty bulk
@@ -1288,6 +1293,7 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
         CK(begin_tail(b), "order");
         if (b->timing) cudaEventRecord(b->ev[3], s);
         CK(launch_tpl(b, block, add), "tpl execute");
+        CK(launch_orders(b), "orders");
         if (b->timing) cudaEventRecord(b->ev[4], s);
         CK(launch_tpl_reset(b, sk, m), "tpl reset");
     }
@@ -1470,16 +1476,17 @@ extern "C" gputx_status gputx_execute_kset_noalloc(gputx_db *db, const int64_t *
     CK(launch_sort(&b, sk, sv, ak, av, m, key_bits(db, conflict_mode)), "sort");
     CK(launch_rank_scan(&b, sk, sv, m, db->need_fixpoint), "rank");
     if (db->need_fixpoint) CK(launch_exact_depth(&b, sv, m), "exact depth");
-    CK(launch_level_stats(&b), "stats");
+    else CK(launch_level_stats(&b), "stats");
     if ((st = read_ctl(&b))) return st;
     if (b.host_ctl.err) return bulk_error(db, b.host_ctl.err);
-    const int64_t depth = b.host_ctl.depth;
+    const int64_t depth = b.host_ctl.last_level;
     uint32_t *rk = ak, *rv = av, *rk2 = sk, *rv2 = sv;
     CK(launch_regroup_keys(&b, rk, rv), "regroup");
     CK(launch_sort(&b, rk, rv, rk2, rv2, b.n, bits_for((uint64_t)depth) + db->tbits), "regroup sort");
     CK(launch_level_tables(&b, rk, depth, block, true), "level tables");
     CK(launch_gather(&b, rv), "gather");
-    CK(launch_kset(&b, rv, b.sc.chunk_cap, block, add), "k-set execute");
+    CK(launch_kset(&b, rv, b.sc.chunk_cap, block, add || db->need_fixpoint), "k-set execute");
+    CK(launch_orders(&b), "orders");
     CK(launch_finish(&b), "finish");
     CK(cudaEventRecord(db->last_done, s), "order");
     if ((st = read_ctl(&b))) return st;

@@ -114,8 +114,8 @@ cudaError_t enqueue_pipeline(GraphBulk *g)
     if ((e = gtx::launch_sort(b, sk, sv, ak, av, m, kbits))) return e;
     if (g->strategy == GPUTX_KSET) {
         if ((e = gtx::launch_rank_scan(b, sk, sv, m, db->need_fixpoint))) return e;
-        if (db->need_fixpoint && (e = gtx::launch_exact_depth(b, sv, m))) return e;
-        if ((e = gtx::launch_level_stats(b))) return e;
+        e = db->need_fixpoint ? gtx::launch_exact_depth(b, sv, m) : gtx::launch_level_stats(b);
+        if (e) return e;
         if (seg && (e = gtx::launch_seg_levels(b))) return e;
         uint32_t *rk = ak, *rv = av, *rk2 = sk, *rv2 = sv;
         if ((e = gtx::launch_regroup_keys(b, rk, rv))) return e;
@@ -124,11 +124,13 @@ cudaError_t enqueue_pipeline(GraphBulk *g)
         if ((e = gtx::launch_level_tables(b, rk, 0, g->block, true))) return e;
         if ((e = gtx::launch_gather(b, rv))) return e;
         if ((e = gtx::launch_begin(b))) return e;
-        if ((e = gtx::launch_kset(b, rv, b->sc.chunk_cap, g->block, add))) return e;
+        if ((e = gtx::launch_kset(b, rv, b->sc.chunk_cap, g->block, add || db->need_fixpoint))) return e;
+        if ((e = gtx::launch_orders(b))) return e;
     } else {
         if ((e = gtx::launch_ticket_scan(b, sk, sv, m))) return e;
         if ((e = gtx::launch_begin(b))) return e;
         if ((e = gtx::launch_tpl(b, g->block, add))) return e;
+        if ((e = gtx::launch_orders(b))) return e;
         if ((e = gtx::launch_tpl_reset(b, sk, m))) return e;
     }
     return gtx::launch_finish(b);

@@ -21,7 +21,13 @@
 
 namespace gtx {
 
-enum : uint32_t { CLS_R = 0, CLS_W = 1, CLS_A = 2 };
+// class of a basic operation: a read, a write, a blind increment under
+// GPUTX_CONFLICT_ADD, and a blind increment under the read/write model, where
+// it is a write (its old value is never read, so additions in any order leave
+// the same value: it orders the graph but need not order the execution)
+enum : uint32_t { CLS_R = 0, CLS_W = 1, CLS_A = 2, CLS_BW = 3 };
+// operations of this class share a run with their neighbours of the same class
+__host__ __device__ __forceinline__ bool cls_shares(uint32_t c) { return !(c & 1u); }
 
 // device error word bits
 enum : uint32_t {
@@ -81,6 +87,7 @@ struct DevDB {
     int64_t *w_tax, *w_ytd;
     int64_t *d_tax, *d_ytd, *d_next_o_id;
     int64_t *c_discount, *c_balance, *c_ytd, *c_payment_cnt, *c_last_o_id;
+    uint32_t *c_last_slot;         // order slot of c_last_o_id (kNoSlot: unknown, look it up)
     int64_t *i_price;
     int32_t *s_quantity, *s_order_cnt;
     int64_t *s_ytd;
@@ -134,6 +141,7 @@ struct DevBulk {
     int conflict_mode;
 };
 
+constexpr uint32_t kNoSlot = 0xffffffffu;
 constexpr uint32_t OP_SENTINEL = 0xffffffffu;   // payload of a padding operation
 
 // ---------------------------------------------------------------------------

@@ -13,8 +13,9 @@ namespace gtx {
 // Per-bulk control block in device memory (zeroed at submit).
 struct BulkCtl {
     uint32_t err;          // ERR_* bits
-    uint32_t depth;        // d: largest level
+    uint32_t depth;        // d: depth of the T-dependency graph
     uint32_t w0;           // 0-set size
+    uint32_t last_level;   // largest entry of the level array (below d where blind increments do not order it)
     uint32_t cross;        // cross-partition transactions
     uint32_t npart;        // PART: non-empty partitions
     uint32_t claim;        // executors: next chunk to claim
@@ -25,6 +26,7 @@ struct BulkCtl {
     uint32_t n_seg;        // segmented graph bulks: bulks in this segment (0 = one)
     uint32_t hot;          // TPL: some counter has a chain of at least the hot ticket
     uint32_t chunk;        // relaxed TPL: next chunk to claim (claim counts commit tickets)
+    uint32_t front;        // exact depth: chunks of transactions finished
 };
 
 constexpr int kSegMax = 64;        // bulks in one segment of a graph bulk, at most
@@ -34,12 +36,12 @@ struct Scratch {
     uint32_t *keys_a, *vals_a, *keys_b, *vals_b;  // sort ping-pong, m entries each
     uint32_t *op_off;      // n+1 exclusive op offsets (non-uniform op counts)
     uint32_t *level;       // n
-    uint32_t *rid;         // m: global run id per sorted op (exact depth)
-    uint32_t *runmax;      // m: deepest finished transaction of each run (exact depth)
+    uint32_t *rid;         // m: place in its run per sorted op (exact depth)
+    unsigned long long *depths;   // n: a finished transaction's depth and level (exact depth)
     uint32_t *lock_key;    // m: TPL per-op object, indexed by op slot
     uint32_t *lock_ticket; // m
     uint32_t *level_off;   // n+2
-    uint32_t *type_cut;    // 3 (n+2): per level, where types >= new-order, payment, order-status start
+    uint32_t *type_cut;    // 2 (n+2): per level, where types >= new-order, payment start
     uint32_t *chunk_off;   // n+2
     uint32_t *chunk_level; // n + n/min_block + 2
     uint32_t *done;        // n+1 per-level completion counters
@@ -81,7 +83,7 @@ struct gputx_db {
     int uniform_k = 0;                     // every registered type has exactly this many ops (0 = no)
     bool need_fixpoint = false;            // a registered type's ops may leave one-pass ranks inexact
     int tbits = 0;                         // type bits in the level/type regroup key
-    bool group_oe = false;                 // K-SET runs new-order and order-status on 16-lane groups
+    bool group_oe = false;                 // K-SET runs new-orders on 16-lane groups, orders are completed after it
     bool hist_by_type = false;             // debit-credit and other types: history rows for debit-credit only
     int obj_bits = 1;                      // key bits of object ids
     // Each bulk runs on a stream of this pool, so the analysis of one bulk
@@ -127,7 +129,7 @@ struct gputx_bulk {
     cudaEvent_t ev[8] = {};
     gtx::BulkCtl host_ctl{};
     std::vector<uint32_t> level_off_host;   // K-SET level boundaries read back for launch planning
-    std::vector<uint32_t> type_cut_host;    // and where each order-entry type starts in each level
+    std::vector<uint32_t> type_cut_host;    // and where the new-orders and payments start in each level
 };
 
 namespace gtx {
@@ -154,8 +156,9 @@ cudaError_t launch_sort(gputx_bulk *b, uint32_t *&keys, uint32_t *&vals, uint32_
                         uint32_t *&vals_alt, int64_t count, int bits);
 cudaError_t launch_rank_scan(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m, bool want_rid);
 cudaError_t launch_ticket_scan(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m);
-cudaError_t launch_depth_flow(gputx_bulk *b, const uint32_t *sv, int64_t m);
+// d, w0 and the level array, exact; the rank scan's rid precedes it
 cudaError_t launch_exact_depth(gputx_bulk *b, const uint32_t *sv, int64_t m);
+// d, w0 of the one-pass ranks
 cudaError_t launch_level_stats(gputx_bulk *b);
 cudaError_t launch_regroup_keys(gputx_bulk *b, uint32_t *keys, uint32_t *vals);
 cudaError_t launch_level_tables(gputx_bulk *b, const uint32_t *skeys, int64_t depth, int block, bool chunks);
@@ -173,6 +176,8 @@ cudaError_t launch_kset_levels(gputx_bulk *b, const uint32_t *level_off_host, in
                                bool atomic_add, const uint32_t *type_cut_host = nullptr);
 cudaError_t launch_part(gputx_bulk *b, const uint32_t *pkeys, int block, int64_t max_parts);
 cudaError_t launch_tpl(gputx_bulk *b, int block, bool atomic_add);
+// after K-SET's levels, after TPL: the rows of the new orders, then what the order-statuses read of them
+cudaError_t launch_orders(gputx_bulk *b);
 // a conflict-free bulk (a 0-set) in one launch
 cudaError_t launch_independent(gputx_bulk *b, bool atomic_add);
 // relaxed timestamps (Appendix G)

@@ -43,8 +43,9 @@ struct LevelArgs {
     DevBulk b;
     const BulkCtl *ctl;
     const uint32_t *level_off;
-    const uint32_t *type_cut; // per level, where new-order, payment, order-status start (or null)
+    const uint32_t *type_cut; // per level, where the new-orders and payments start (or null)
     uint32_t k0, k1;          // levels [k0, k1)
+    bool orders;              // new-orders are registered (launch_orders follows)
     bool atomic_add;
 };
 
@@ -53,10 +54,11 @@ struct KsetArgs {
     DevBulk b;
     BulkCtl *ctl;
     const uint32_t *order, *level_off, *chunk_off, *chunk_level;
-    const uint32_t *type_cut;   // per level, where new-order, payment, order-status start (or null)
+    const uint32_t *type_cut;   // per level, where the new-orders and payments start (or null)
     uint32_t *done;
     int64_t levels;
     uint64_t spin_limit_ns;
+    bool orders;                // new-orders are registered (launch_orders follows)
     bool atomic_add;
 };
 
@@ -95,50 +97,86 @@ __global__ void __launch_bounds__(256) independent_kernel(DevDB db, DevBulk b, c
 
 // The lanes of one level.  Records are sorted by (level, type) (Appendix
 // D's grouping by type), so a level is a run of each type in turn.  With
-// type cuts, order-entry's new-orders and order-statuses take 16 lanes each
-// (their line-parallel procedures), every group starting on a half warp;
-// every other transaction takes one lane.  Lane x maps to the record at
-// `pos`; gl = its index in a group, or -1 for a one-lane transaction.
+// type cuts, order-entry's new-orders take 16 lanes each (their line-parallel
+// procedure), their run starting on a half warp; every other transaction takes
+// one lane.  Lane x maps to the record at `pos`; gl = its index in a group, or
+// -1 for a one-lane transaction.
 struct LevelLanes {
-    uint32_t lo, c8, c9, c10, a1, b1, a2, v;
+    uint32_t lo, c8, c9, a1, b1, v;
     __device__ __forceinline__ void make(uint32_t lo_, uint32_t hi, const uint32_t *cut)
     {
         lo = lo_;
         if (!cut) {
-            c8 = c9 = c10 = hi;
-            a1 = b1 = a2 = v = hi - lo;
+            c8 = c9 = hi;
+            a1 = b1 = v = hi - lo;
             return;
         }
         c8 = __ldg(&cut[0]);
         c9 = __ldg(&cut[1]);
-        c10 = __ldg(&cut[2]);
-        a1 = (c8 - lo + kGroup - 1) & ~(uint32_t)(kGroup - 1);      // new-order groups start here
-        b1 = a1 + kGroup * (c9 - c8);                               // payments
-        a2 = (b1 + (c10 - c9) + kGroup - 1) & ~(uint32_t)(kGroup - 1);   // order-status groups
-        v = a2 + kGroup * (hi - c10);
+        a1 = (c8 - lo + kGroup - 1) & ~(uint32_t)(kGroup - 1);   // new-order groups start here
+        b1 = a1 + kGroup * (c9 - c8);                            // the types after them
+        v = b1 + (hi - c9);
     }
-    // false for an idle lane (alignment padding before a group run)
+    // false for an idle lane (alignment padding before the groups)
     __device__ __forceinline__ bool at(uint32_t x, uint32_t &pos, int &gl) const
     {
         gl = -1;
         if (x < c8 - lo) { pos = lo + x; return true; }
         if (x < a1) return false;
         if (x < b1) { pos = c8 + (x - a1) / kGroup; gl = (int)((x - a1) % kGroup); return true; }
-        if (x < b1 + (c10 - c9)) { pos = c9 + (x - b1); return true; }
-        if (x < a2) return false;
-        pos = c10 + (x - a2) / kGroup;
-        gl = (int)((x - a2) % kGroup);
+        pos = c9 + (x - b1);
         return true;
     }
 };
 
-__device__ __forceinline__ void exec_lane(const DevDB &db, const DevBulk &b, const TxnView &v, int gl,
+// One lane of a level.  Order-entry's procedures run in their first parts
+// (launch_orders runs the second ones after the last level).
+__device__ __forceinline__ void exec_lane(const DevDB &db, const DevBulk &b, const TxnView &v, int gl, bool first,
                                           bool atomic_add)
 {
-    GlobalCells g;
-    if (gl < 0) exec_txn(db, b, v, atomic_add, g);
-    else if (v.type == GPUTX_T_OE_NEW_ORDER) exec_new_order_group(db, b, v, (uint32_t)gl, g);
-    else exec_order_status_group(db, b, v, (uint32_t)gl, g);
+    if (first && gl < 0 && v.type == GPUTX_T_OE_NEW_ORDER) {
+        new_order_first_lane(db, b, v);
+    } else if (gl >= 0) {
+        int64_t p2, p3;
+        const int64_t line = new_order_params(b, v, (uint32_t)gl, p2, p3);
+        new_order_first(db, b, v, (uint32_t)gl, p2, p3, line, b.slot_ord[v.t], b.slot_ol[v.t]);
+    } else if (first && v.type == GPUTX_T_OE_ORDER_STATUS) {
+        order_status_first(db, b, v, __ldg(&v.p[2]));
+    } else {
+        exec_txn(db, b, v, atomic_add);
+    }
+}
+
+// The second parts of a bulk's new-orders (orders = true: order rows, lines,
+// index entries, outputs), then of its order-statuses, 16 lanes a transaction
+// in timestamp order, so slots and outputs are written side by side.
+__global__ void __launch_bounds__(256) orders_kernel(DevDB db, DevBulk b, const BulkCtl *ctl, bool orders)
+{
+    if (ctl->err & ~(uint32_t)ERR_CAPACITY) return;
+    const int64_t n = b.n_live ? (int64_t)*b.n_live : b.n;
+    const uint32_t gl = threadIdx.x & (kGroup - 1);
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x / kGroup;
+    for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kGroup; t < n; t += stride) {
+        const int32_t type = __ldg(&b.type[t]);
+        if (type != (orders ? GPUTX_T_OE_NEW_ORDER : GPUTX_T_OE_ORDER_STATUS) || b.status[t] != 0) continue;
+        const TxnView v = view_of(b, (uint32_t)t, 0);
+        if (orders) {
+            NewOrderPart o;
+            int64_t p2, p3;
+            o.line = new_order_params(b, v, gl, p2, p3);
+            o.o_id = b.out[t * b.R];
+            o.w = v.p0;
+            o.d = v.p0 * OE_DIST + v.p1;
+            o.c = o.d * OE_CUST + p2;
+            o.oslot = b.base->ord + b.slot_ord[t];
+            o.lslot = b.base->ol + b.slot_ol[t];
+            o.cnt = (int)p3;
+            o.run = true;
+            new_order_finish(db, b, v, gl, o);
+        } else {
+            order_status_finish(db, b, v, gl);
+        }
+    }
 }
 
 // one wide level [level_off[k0], level_off[k0+1]) over the whole grid
@@ -148,17 +186,66 @@ __global__ void __launch_bounds__(256) kset_level_kernel(LevelArgs a)
     const int64_t hb = a.ctl->base.hist;
     const uint32_t lo = __ldg(&a.level_off[a.k0]), hi = __ldg(&a.level_off[a.k0 + 1]);
     LevelLanes L;
-    L.make(lo, hi, a.type_cut ? a.type_cut + 3 * (int64_t)a.k0 : nullptr);
+    L.make(lo, hi, a.type_cut ? a.type_cut + 2 * (int64_t)a.k0 : nullptr);
     for (uint32_t x = blockIdx.x * blockDim.x + threadIdx.x; x < L.v; x += gridDim.x * blockDim.x) {
         uint32_t pos;
         int gl;
-        if (L.at(x, pos, gl)) exec_lane(a.db, a.b, view_at(a.b, pos, hb), gl, a.atomic_add);
+        if (L.at(x, pos, gl)) exec_lane(a.db, a.b, view_at(a.b, pos, hb), gl, a.orders, a.atomic_add);
     }
 }
 
+// one lane's record of a level, in registers before the level runs
+struct LaneRecord {
+    TxnView v;
+    int64_t p2, p3, line;    // order-entry: parameters 2, 3 and 4 + gl
+    uint32_t os, ls;         // insert slots of a new-order
+    int gl;                  // index in the lane group, or -1
+    bool has;
+};
+
+// the record of lane `rank` of a level into L1
+__device__ __forceinline__ void lane_prefetch(const DevBulk &b, const LevelLanes &L, uint32_t rank)
+{
+    uint32_t pos = 0;
+    int gl;
+    if (!(rank < L.v && L.at(rank, pos, gl))) return;
+    if (kDebug && pos >= b.n) return;
+    prefetch_record_l1(b, pos);
+    if (gl > 0 && 4 + gl < b.P)
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(b.rec_params + (int64_t)pos * b.P + 4 + gl));
+}
+
+// the loads of lane `rank` of a level; none depends on another
+__device__ __forceinline__ LaneRecord lane_record(const DevBulk &b, const LevelLanes &L, uint32_t rank)
+{
+    LaneRecord r{};
+    uint32_t pos = 0;
+    r.gl = -1;
+    r.has = rank < L.v && L.at(rank, pos, r.gl);
+    if (!r.has) return r;
+    r.v = record_at(b, pos);
+    if (b.P > 3) {
+        r.p2 = __ldg(&r.v.p[2]);
+        r.p3 = __ldg(&r.v.p[3]);
+    } else if (b.P > 2) {
+        r.p2 = __ldg(&r.v.p[2]);
+    }
+    if (r.gl >= 0 && 4 + r.gl < b.P) r.line = __ldg(&r.v.p[4 + r.gl]);
+    return r;
+}
+
 // a run of narrow levels [k0, k1) on one thread-block cluster (CLUSTER) or
-// one CTA.  While level k executes, level k+1's records come into L1; after
-// it, level k+1's rows are prefetched into L2; then the barrier.
+// one CTA.
+//
+// What bounds it is the latency of a level, so whatever need not lie between
+// two barriers does not.  A level's bounds are loaded four levels ahead, its
+// records come into L1 three and into registers two levels ahead, its rows into
+// L2 and its insert slots into registers one level ahead; order rows, lines,
+// index entries and the order-statuses' sums are left to launch_orders, and the
+// payments' totals follow the barrier's arrival.  Order-entry, 200,003
+// transactions, 317 a level: 3.5 us a level; 7.3 when the records were
+// loaded during the level before and the procedures ran whole (of it 3.0
+// without any procedure, 1.2 the index entry's compare-and-swap).
 template <bool CLUSTER, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) kset_narrow_kernel(LevelArgs a)
 {
@@ -171,61 +258,67 @@ __global__ void __launch_bounds__(MAXT, 1) kset_narrow_kernel(LevelArgs a)
         rank = cl.thread_rank();
     }
     const uint32_t *cut = a.type_cut;
-    LevelLanes L;
-    L.make(__ldg(&a.level_off[a.k0]), __ldg(&a.level_off[a.k0 + 1]), cut ? cut + 3 * (int64_t)a.k0 : nullptr);
-    // this thread's first lane of the current level, loaded ahead
-    TxnView v{};
-    uint32_t pos;
-    int gl = -1;
-    bool has = rank < L.v && L.at(rank, pos, gl);
-    if (has) {
-        v = view_at(a.b, pos, hb);
-        if (gl < 0) prefetch_txn(a.db, v);
-        else prefetch_group(a.db, v, (uint32_t)gl);
-    }
-    for (uint32_t k = a.k0; k < a.k1; k++) {
-        LevelLanes N;
-        if (k + 1 < a.k1)
-            N.make(__ldg(&a.level_off[k + 1]), __ldg(&a.level_off[k + 2]), cut ? cut + 3 * (int64_t)(k + 1) : nullptr);
-        else N.make(0, 0, nullptr);
-        // the next level's first record for this thread: loads in flight
-        // while this level executes
-        TxnView nv{};
-        uint32_t npos;
-        int ngl = -1;
-        const bool has_next = rank < N.v && N.at(rank, npos, ngl);
-        if (has_next) {
-            nv = view_at(a.b, npos, hb);
-            // the parameters this lane reads beyond the first two (a group
-            // lane's order line) into L1 while this level runs
-            if (a.b.P > 2) {
-                asm volatile("prefetch.global.L1 [%0];" ::"l"(nv.p + 2));
-                if (ngl >= 0 && 4 + ngl < a.b.P) asm volatile("prefetch.global.L1 [%0];" ::"l"(nv.p + 4 + ngl));
-            }
+    const bool first = a.orders;
+    // the bounds of level j; levels from k1 on are empty
+    auto lanes_of = [&](uint32_t j) {
+        LevelLanes L;
+        if (j < a.k1) L.make(__ldg(&a.level_off[j]), __ldg(&a.level_off[j + 1]), cut ? cut + 2 * (int64_t)j : nullptr);
+        else L.make(0, 0, nullptr);
+        return L;
+    };
+    // what hangs on a record's contents: its insert slots, its rows in L2
+    auto slots = [&](LaneRecord &r) {
+        if (!r.has) return;
+        if (r.gl >= 0) {
+            r.os = __ldg(&a.b.slot_ord[r.v.t]);
+            r.ls = __ldg(&a.b.slot_ol[r.v.t]);
+            prefetch_new_order(a.db, r.v, (uint32_t)r.gl, r.p2, r.p3, r.line);
+        } else {
+            prefetch_txn(a.db, r.v);
         }
-        if (has) exec_lane(a.db, a.b, v, gl, a.atomic_add);
-        for (uint32_t x = rank + nthreads; x < L.v; x += nthreads) {
+        if (a.b.slot_hist) r.v.hist_slot = __ldg(&a.b.slot_hist[r.v.t]);
+    };
+    LevelLanes L0 = lanes_of(a.k0), L1 = lanes_of(a.k0 + 1), L2 = lanes_of(a.k0 + 2), L3 = lanes_of(a.k0 + 3);
+    LaneRecord r0 = lane_record(a.b, L0, rank), r1 = lane_record(a.b, L1, rank);
+    slots(r0);
+    lane_prefetch(a.b, L2, rank);
+    for (uint32_t k = a.k0; k < a.k1; k++) {
+        const LevelLanes L4 = lanes_of(k + 4);
+        slots(r1);
+        LaneRecord r2 = lane_record(a.b, L2, rank);
+        lane_prefetch(a.b, L3, rank);
+        const bool pay = r0.has && first && r0.v.type == GPUTX_T_OE_PAYMENT;
+        r0.v.hist_slot += hb;
+        if (r0.has) {
+            if (r0.gl >= 0)
+                new_order_first(a.db, a.b, r0.v, (uint32_t)r0.gl, r0.p2, r0.p3, r0.line, r0.os, r0.ls);
+            else if (pay) payment_first(a.db, a.b, r0.v, r0.p2, r0.p3);
+            else exec_lane(a.db, a.b, r0.v, -1, first, a.atomic_add);
+        }
+        for (uint32_t x = rank + nthreads; x < L0.v; x += nthreads) {
             uint32_t p2;
             int g2;
-            if (L.at(x, p2, g2)) exec_lane(a.db, a.b, view_at(a.b, p2, hb), g2, a.atomic_add);
+            if (L0.at(x, p2, g2)) exec_lane(a.db, a.b, view_at(a.b, p2, hb), g2, first, a.atomic_add);
         }
-        if (has_next) {                             // rows into L2 before the barrier
-            if (ngl < 0) prefetch_txn(a.db, nv);
-            else prefetch_group(a.db, nv, (uint32_t)ngl);
-        }
-        if (CLUSTER) cg::this_cluster().sync();   // release/acquire at cluster scope
+        __syncwarp();
+        if (CLUSTER) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        if (pay) payment_totals(a.db, r0.v, r0.p3);
+        __syncwarp();
+        if (CLUSTER) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
         else __syncthreads();
-        L = N;
-        v = nv;
-        has = has_next;
-        gl = ngl;
+        L0 = L1;
+        L1 = L2;
+        L2 = L3;
+        L3 = L4;
+        r0 = r1;
+        r1 = r2;
     }
 }
 
 __global__ void kset_kernel(KsetArgs a)
 {
     __shared__ uint32_t s_k, s_start, s_cnt, s_stop;
-    const int64_t levels = (int64_t)a.ctl->depth + 1;   // from the analysis, on the device
+    const int64_t levels = (int64_t)a.ctl->last_level + 1;   // from the analysis, on the device
     const uint32_t nchunks = a.chunk_off[levels];
     const int64_t hb = a.ctl->base.hist;
     const uint32_t *cut = a.type_cut;
@@ -236,7 +329,7 @@ __global__ void kset_kernel(KsetArgs a)
             if (c < nchunks) {
                 // a chunk is a run of blockDim lanes of one level
                 const uint32_t k = a.chunk_level[c];
-                const uint32_t w = level_lane_count(a.level_off[k], a.level_off[k + 1], cut ? cut + 3 * k : nullptr);
+                const uint32_t w = level_lane_count(a.level_off[k], a.level_off[k + 1], cut ? cut + 2 * (int64_t)k : nullptr);
                 const uint32_t start = (c - a.chunk_off[k]) * blockDim.x;
                 const uint32_t cnt = (w - start) < blockDim.x ? (w - start) : blockDim.x;
                 s_k = k;
@@ -250,7 +343,7 @@ __global__ void kset_kernel(KsetArgs a)
         __syncthreads();
         if (s_stop) break;
         LevelLanes L;
-        L.make(a.level_off[s_k], a.level_off[s_k + 1], cut ? cut + 3 * (int64_t)s_k : nullptr);
+        L.make(a.level_off[s_k], a.level_off[s_k + 1], cut ? cut + 2 * (int64_t)s_k : nullptr);
         // signatures are immutable: load them and prefetch the rows while the
         // previous level may still be running
         TxnView v{};
@@ -259,12 +352,17 @@ __global__ void kset_kernel(KsetArgs a)
         const bool mine = threadIdx.x < s_cnt && L.at(s_start + threadIdx.x, pos, gl);
         if (mine) {
             v = view_at(a.b, pos, hb);
-            if (gl < 0) prefetch_txn(a.db, v);
-            else prefetch_group(a.db, v, (uint32_t)gl);
+            if (gl < 0) {
+                prefetch_txn(a.db, v);
+            } else {
+                int64_t p2, p3;
+                const int64_t line = new_order_params(a.b, v, (uint32_t)gl, p2, p3);
+                prefetch_new_order(a.db, v, (uint32_t)gl, p2, p3, line);
+            }
         }
         if (threadIdx.x == 0 && s_k > 0) {
             const uint32_t k = s_k;
-            const uint32_t prev = level_lane_count(a.level_off[k - 1], a.level_off[k], cut ? cut + 3 * (k - 1) : nullptr);
+            const uint32_t prev = level_lane_count(a.level_off[k - 1], a.level_off[k], cut ? cut + 2 * (int64_t)(k - 1) : nullptr);
             if (!wait_at_least(&a.done[k - 1], prev, a.spin_limit_ns)) {
                 set_err(&a.ctl->err, ERR_TIMEOUT);
                 s_stop = 1;
@@ -273,7 +371,7 @@ __global__ void kset_kernel(KsetArgs a)
         __syncthreads();
         if (s_stop) break;
         if (mine) {
-            exec_lane(a.db, a.b, v, gl, a.atomic_add);
+            exec_lane(a.db, a.b, v, gl, a.orders, a.atomic_add);
             __threadfence();
         }
         __syncthreads();
@@ -367,6 +465,7 @@ struct TplArgs {
     bool atomic_add;
     bool graph;          // fixed-capacity bulk: K slots per transaction, only the
                          // first op_count are real; padding transactions skipped
+    bool orders;         // new-orders are registered: launch_orders completes them and the order-statuses
     LockSlots slot;      // item -> its counter in `done`
     int when_hot;        // debit-credit executors: -1 run, 1 run only if ctl->hot, 0 only if not
 };
@@ -410,7 +509,9 @@ __device__ __forceinline__ void warp_release(const TplArgs &a, bool rel, int64_t
 // Every lane whose locks are all granted takes one acquire fence and runs
 // its procedure: first the short ones, then the new-orders (up to four of
 // them on a half warp each, one lane per order line), each phase followed by
-// its releases.  Releases are warp-aggregated: lanes releasing the same
+// its releases.  Order-entry's procedures hold their locks for their first
+// parts only (launch_orders runs the second ones after this kernel; 200,003
+// transactions: 12.9 ms, 14.5 with the procedures whole under the locks).  Releases are warp-aggregated: lanes releasing the same
 // counter in a phase are grouped by __match_any_sync and their lowest lane
 // adds the group's size.  A round in which nothing is granted sleeps until
 // the first lane is due to poll, so a lane about to be granted never sleeps
@@ -513,10 +614,15 @@ __global__ void __launch_bounds__(512) tpl_kernel(TplArgs a)
             // the same warp.  Phase 1: every other granted transaction, one
             // lane each (and the releases of timed-out ones).
             const bool no = ready && !failed && v.type == GPUTX_T_OE_NEW_ORDER;
-            const bool r1 = ready && !no;
-            if (r1 && !failed) exec_txn(a.db, a.b, v, a.atomic_add);
+            const bool r1 = ready && !no, pay = r1 && !failed && v.type == GPUTX_T_OE_PAYMENT;
+            if (pay) payment_first(a.db, a.b, v, __ldg(&v.p[2]), __ldg(&v.p[3]));
+            else if (r1 && !failed && v.type == GPUTX_T_OE_ORDER_STATUS && a.orders)
+                order_status_first(a.db, a.b, v, __ldg(&v.p[2]));
+            else if (r1 && !failed) exec_txn(a.db, a.b, v, a.atomic_add);
             __syncwarp();   // every lane's writes precede the releases of its phase
             warp_release(a, r1, off, cnt);
+            // no transaction of the bulk reads the totals and additions commute
+            if (pay) payment_totals(a.db, v, __ldg(&v.p[3]));
             // Phase 2: the granted new-orders.  Up to four run on a half warp
             // each, two at a time (the line-parallel procedure: one lane per
             // order line, as in the K-SET runners); more run one lane each.
@@ -537,12 +643,13 @@ __global__ void __launch_bounds__(512) tpl_kernel(TplArgs a)
                     g.t = __shfl_sync(kFull, v.t, src);
                     g.type = __shfl_sync(kFull, v.type, src);
                     if (lane < 16 || l1 >= 0) {
-                        GlobalCells gc;
-                        exec_new_order_group(a.db, a.b, g, lane & 15u, gc);
+                        int64_t p2, p3;
+                        const int64_t line = new_order_params(a.b, g, lane & 15u, p2, p3);
+                        new_order_first(a.db, a.b, g, lane & 15u, p2, p3, line, a.b.slot_ord[g.t], a.b.slot_ol[g.t]);
                     }
                 }
             } else if (no) {
-                exec_txn(a.db, a.b, v, a.atomic_add);
+                new_order_first_lane(a.db, a.b, v);
             }
             __syncwarp();
             warp_release(a, no, off, cnt);
@@ -913,6 +1020,7 @@ cudaError_t launch_kset(gputx_bulk *b, const uint32_t *order, int64_t nchunks, i
     a.type_cut = b->sc.type_cut;
     a.done = b->sc.done;
     a.levels = 0;
+    a.orders = db->dev.registered >> GPUTX_T_OE_NEW_ORDER & 1u;
     a.spin_limit_ns = (uint64_t)db->cfg.spin_limit_ns;
     a.atomic_add = atomic_add;
     cudaError_t e = cudaMemsetAsync(b->sc.done, 0, (size_t)(b->n + 1) * sizeof(uint32_t), b->stream);
@@ -937,12 +1045,13 @@ cudaError_t launch_kset_levels(gputx_bulk *b, const uint32_t *level_off_host, in
     a.ctl = b->ctl;
     a.level_off = b->sc.level_off;
     a.type_cut = type_cut_host ? b->sc.type_cut : nullptr;
+    a.orders = db->dev.registered >> GPUTX_T_OE_NEW_ORDER & 1u;
     a.atomic_add = atomic_add;
     const int64_t levels = depth + 1;
     // lanes per level: the launch shapes follow them
     std::vector<uint32_t> width((size_t)levels);
     for (int64_t j = 0; j < levels; j++)
-        width[j] = level_lane_count(level_off_host[j], level_off_host[j + 1], a.type_cut ? type_cut_host + 3 * j : nullptr);
+        width[j] = level_lane_count(level_off_host[j], level_off_host[j + 1], a.type_cut ? type_cut_host + 2 * j : nullptr);
     static bool attr_set = false;
     if (!attr_set) {
         cudaFuncSetAttribute(kset_narrow_kernel<true, 256>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -1032,6 +1141,21 @@ cudaError_t launch_part(gputx_bulk *b, const uint32_t *pkeys, int block, int64_t
     return cudaGetLastError();
 }
 
+cudaError_t launch_orders(gputx_bulk *b)
+{
+    gputx_db *db = b->db;
+    if (b->n == 0 || !(db->dev.registered >> GPUTX_T_OE_NEW_ORDER & 1u)) return cudaSuccess;
+    const DevBulk d = make_dev_bulk(b, GPUTX_CONFLICT_PAPER);
+    const unsigned grid = (unsigned)std::min<int64_t>((b->n * kGroup + 255) / 256, (int64_t)db->num_sms * 8);
+    orders_kernel<<<grid, 256, 0, b->stream>>>(db->dev, d, b->ctl, true);
+    count_launches(1);
+    if (db->dev.registered >> GPUTX_T_OE_ORDER_STATUS & 1u) {
+        orders_kernel<<<grid, 256, 0, b->stream>>>(db->dev, d, b->ctl, false);
+        count_launches(1);
+    }
+    return cudaGetLastError();
+}
+
 cudaError_t launch_independent(gputx_bulk *b, bool atomic_add)
 {
     gputx_db *db = b->db;
@@ -1063,6 +1187,7 @@ cudaError_t launch_tpl(gputx_bulk *b, int block, bool atomic_add)
     cudaError_t e = cudaMemsetAsync(&b->ctl->claim, 0, sizeof(uint32_t), b->stream);
     if (e) return e;
     a.slot = db->lock_slots;
+    a.orders = db->dev.registered >> GPUTX_T_OE_NEW_ORDER & 1u;
     // debit-credit-only bulks of single-lock transactions
     const bool dc = db->dev.registered == (1u << GPUTX_T_DC_DEBIT_CREDIT) && !b->graph && db->uniform_k == 1;
     // the general kernel's registers allow CTAs of up to 512 threads; the

@@ -150,7 +150,7 @@ struct ZeroMode {
         uint32_t runhead = 0;
         if (!head) {
             const uint32_t c = sv[i] & 3u, pc = sv[i - 1] & 3u;
-            runhead = !(c == pc && c != CLS_W);
+            runhead = !(c == pc && cls_shares(c));
         }
         return DualSeg::make(head, runhead, 0, 0);
     }

@@ -76,7 +76,7 @@ __device__ __forceinline__ bool valid_txn(const DevDB &db, int32_t type, const i
 __device__ __forceinline__ int access_set(const DevDB &db, int32_t type, const int64_t *p, int mode,
                                           uint32_t *obj, uint8_t *cls, uint32_t *root)
 {
-    const uint8_t blind = (mode == GPUTX_CONFLICT_ADD) ? CLS_A : CLS_W;
+    const uint8_t blind = (mode == GPUTX_CONFLICT_ADD) ? CLS_A : CLS_BW;
     int k = 0;
     switch (type) {
     case GPUTX_T_DC_DEBIT_CREDIT: {
@@ -127,10 +127,12 @@ __device__ __forceinline__ int access_set(const DevDB &db, int32_t type, const i
     case GPUTX_T_OE_PAYMENT: {
         uint32_t w = (uint32_t)p[0], d = w * OE_DIST + (uint32_t)p[1];
         uint32_t c = d * OE_CUST + (uint32_t)p[2];
+        // the district's total is incremented too: two payments that conflict
+        // on it conflict on the warehouse's above it (or, with ADD, on neither),
+        // and nothing else touches either, so the warehouse stands for both
         obj[0] = db.o_wytd + w;  cls[0] = blind; root[0] = w;
-        obj[1] = db.o_dytd + d;  cls[1] = blind; root[1] = w;
-        obj[2] = db.o_cpay + c;  cls[2] = CLS_W; root[2] = w;
-        return 3;
+        obj[1] = db.o_cpay + c;  cls[1] = CLS_W; root[1] = w;
+        return 2;
     }
     case GPUTX_T_OE_ORDER_STATUS: {
         uint32_t w = (uint32_t)p[0], d = w * OE_DIST + (uint32_t)p[1];
@@ -169,7 +171,7 @@ __device__ __forceinline__ int op_count(const DevDB &db, int32_t type, const int
         for (int j = 0; j < cnt; j++) k += ((p[4 + j] & 0xFFFFFF) < db.n_items);
         return k;
     }
-    case GPUTX_T_OE_PAYMENT: return 3;
+    case GPUTX_T_OE_PAYMENT: return 2;
     case GPUTX_T_OE_ORDER_STATUS: return 2;
     default: return 1;
     }
@@ -299,6 +301,29 @@ __device__ __forceinline__ TxnView view_at(const DevBulk &b, uint32_t pos, int64
     return v;
 }
 
+// the record at position pos alone: hist_slot is its history row before the
+// bulk's base is added, or for the caller to look up (slot_hist), so no load
+// waits for another
+__device__ __forceinline__ TxnView record_at(const DevBulk &b, uint32_t pos)
+{
+    TxnView v;
+    bool bad = !dbg_in(pos, b.n, b.err);
+    if (kDebug && bad) pos = 0;
+    v.p = b.rec_params + (int64_t)pos * b.P;
+    v.p0 = __ldg(&v.p[0]);
+    v.p1 = b.P > 1 ? __ldg(&v.p[1]) : 0;
+    v.ts = __ldg(&b.rec_ts[pos]);
+    v.type = __ldg(&b.rec_type[pos]);
+    v.t = __ldg(&b.rec_t[pos]);
+    if (kDebug && !dbg_in(v.t, b.n, b.err)) {
+        bad = true;
+        v.t = 0;
+    }
+    if (kDebug && bad) v.type = -1;
+    v.hist_slot = pos;
+    return v;
+}
+
 // signature of transaction t straight from the bulk (timestamp order)
 __device__ __forceinline__ TxnView view_of(const DevBulk &b, uint32_t t, int64_t hist_base)
 {
@@ -345,6 +370,13 @@ __device__ __forceinline__ void prefetch_txn(const DevDB &db, const TxnView &v)
         prefetch_l2(&db.c_balance[c]);
         prefetch_l2(&db.c_ytd[c]);
         prefetch_l2(&db.c_payment_cnt[c]);
+        break;
+    }
+    case GPUTX_T_OE_ORDER_STATUS: {
+        const int64_t w = __ldg(&p[0]), d = w * OE_DIST + __ldg(&p[1]), c = d * OE_CUST + __ldg(&p[2]);
+        prefetch_l2(&db.c_last_o_id[c]);
+        prefetch_l2(&db.c_last_slot[c]);
+        prefetch_l2(&db.c_balance[c]);
         break;
     }
     case GPUTX_T_OE_NEW_ORDER: {
@@ -634,6 +666,7 @@ __device__ __forceinline__ void exec_oe(const DevDB &db, const DevBulk &b, const
             set_err(b.err, ERR_CAPACITY); st = 3; break;
         }
         cells.st(&db.c_last_o_id[c], o_id);
+        stg_cg(&db.c_last_slot[c], (uint32_t)oslot);
         out[0] = o_id;
         out[1] = total * (10000 - disc) * (10000 + w_tax + d_tax) / 100000000;
         out[2] = cnt;
@@ -668,7 +701,8 @@ __device__ __forceinline__ void exec_oe(const DevDB &db, const DevBulk &b, const
         out[0] = cells.ld(&db.c_balance[c]);
         out[1] = o;
         if (o == 0) { st = 1; break; }
-        const int64_t r = hash_find(db.ord_idx, ord_key(d, o));
+        const uint32_t last = ldg_cg(&db.c_last_slot[c]);
+        const int64_t r = last != kNoSlot ? (int64_t)last : hash_find(db.ord_idx, ord_key(d, o));
         if (r < 0) { set_err(b.err, ERR_BOUNDS); st = 1; break; }
         if (!dbg_in(r, db.ord_cap, b.err)) { st = 1; break; }
         const int cnt = ldg_cg(&db.o_cnt[r]);
@@ -685,28 +719,25 @@ __device__ __forceinline__ void exec_oe(const DevDB &db, const DevBulk &b, const
 }
 
 // ---------------------------------------------------------------------------
-// order-entry's line-parallel procedures: one transaction on a group of 16
-// lanes (a half warp).  A new-order's lines touch distinct stock rows (its
-// items are distinct), so they need no order among themselves: lane l runs
-// line l, and the reads of all lines go out in one round trip instead of one
-// per chunk of lines.  Lane 0 also runs the transaction's own part (district
-// counter, order row, index, customer, outputs).  The results equal
-// exec_oe's bit for bit.  Every lane of the group calls these together;
-// `gl` is the lane's index in its group.
+// order-entry's line-parallel procedures: one new-order on a group of 16 lanes
+// (a half warp).  Its lines touch distinct stock rows (its items are distinct),
+// so they need no order among themselves: lane l runs line l, and the reads of
+// all lines go out in one round trip instead of one per chunk of lines.  Lane 0
+// also runs the transaction's own part.  The results equal exec_oe's bit for
+// bit.  Every lane of the group calls these together; `gl` is the lane's index
+// in its group.
 // ---------------------------------------------------------------------------
 constexpr int kGroup = 16;
 
-// lanes a level [lo, hi) takes: one per transaction, 16 per new-order and
-// order-status, each run of groups starting on a half warp.  cut = where the
-// level's types >= new-order, payment, order-status start (null: no groups)
+// lanes a level [lo, hi) takes: one per transaction, 16 per new-order, their
+// run starting on a half warp.  cut = where the level's types >= new-order,
+// payment start (null: no groups)
 __host__ __device__ inline uint32_t level_lane_count(uint32_t lo, uint32_t hi, const uint32_t *cut)
 {
     if (!cut) return hi - lo;
-    const uint32_t c8 = cut[0], c9 = cut[1], c10 = cut[2];
+    const uint32_t c8 = cut[0], c9 = cut[1];
     const uint32_t a1 = (c8 - lo + kGroup - 1) & ~(uint32_t)(kGroup - 1);
-    const uint32_t b1 = a1 + kGroup * (c9 - c8);
-    const uint32_t a2 = (b1 + (c10 - c9) + kGroup - 1) & ~(uint32_t)(kGroup - 1);
-    return a2 + kGroup * (hi - c10);
+    return a1 + kGroup * (c9 - c8) + (hi - c9);
 }
 
 __device__ __forceinline__ uint32_t group_mask() { return 0xFFFFu << ((threadIdx.x & 31) & 16); }
@@ -739,81 +770,104 @@ __device__ __forceinline__ int64_t group_probe(uint32_t gm, uint32_t gl, const H
     return -1;
 }
 
-template <class Cells>
-__device__ __forceinline__ void exec_new_order_group(const DevDB &db, const DevBulk &b, const TxnView &v, uint32_t gl,
-                                                     Cells &cells)
+// A new-order in two parts.  new_order_state updates what later transactions
+// of the bulk read and write -- the lines' stock rows, the district's counter,
+// the customer's last order -- and new_order_finish writes the rest: order row,
+// lines, index entry, outputs.  Only an order-status of the customer reads
+// those, and its sum over the order's lines can wait as well, since an order
+// never changes (order_status_state, order_status_finish).  K-SET and TPL run
+// the first parts level by level, or under the locks, and all second parts
+// after that, side by side.
+struct NewOrderPart {
+    int64_t o_id, line;                      // (line: the lane's)
+    int64_t w, d, c, oslot, lslot;
+    int cnt;
+    bool run;                                // the order was not aborted
+};
+
+// p2, p3, line: parameters 2, 3 and 4 + gl (0 beyond the order's lines);
+// os, ls: the order's insert slots
+__device__ __forceinline__ void new_order_state(const DevDB &db, const DevBulk &b, const TxnView &v, uint32_t gl,
+                                                int64_t p2, int64_t p3, int64_t line, int64_t os, int64_t ls,
+                                                NewOrderPart &o)
 {
+    o.run = false;
     if (kDebug && (v.type != GPUTX_T_OE_NEW_ORDER || !valid_txn(db, v.type, v.p, b.P))) {
         if (gl == 0) set_err(b.err, ERR_BOUNDS);   // the group's lanes all leave here
         return;
     }
     const uint32_t gm = group_mask();
-    const int64_t *p = v.p;
-    const uint32_t t = v.t;
-    const int64_t w = v.p0, d = w * OE_DIST + v.p1;
-    const int64_t cw = __ldg(&p[2]);
-    const int64_t c = d * OE_CUST + cw;
-    const int cnt = (int)__ldg(&p[3]);
-    const bool mine = (int)gl < cnt;
-    int64_t line = 0, item = 0, sw = 0, qty = 0, s = 0;
-    if (mine) {
-        line = __ldg(&p[4 + gl]);
-        item = line & 0xFFFFFF;
-        sw = (line >> 24) & 0xFFFF;
-        qty = (line >> 40) & 0xFF;
-    }
-    // every read in one round trip, issued before the checks below so that
-    // the insert slots' loads overlap them: the district's counter and the
-    // rates on lane 0, each line's item and stock row on its lane (a line
-    // with an unknown item reads nothing)
-    const int64_t ob = b.base->ord, lb = b.base->ol;
-    const int64_t os = b.slot_ord[t], ls = b.slot_ol[t];
-    int64_t o_id = 0, disc = 0, w_tax = 0, d_tax = 0, price = 0, sy = 0;
+    o.w = v.p0;
+    o.d = v.p0 * OE_DIST + v.p1;
+    o.c = o.d * OE_CUST + p2;
+    o.cnt = (int)p3;
+    o.line = line;
+    o.oslot = b.base->ord + os;
+    o.lslot = b.base->ol + ls;
+    const bool mine = (int)gl < o.cnt;
+    const int64_t item = line & 0xFFFFFF, sw = (line >> 24) & 0xFFFF, qty = (line >> 40) & 0xFF;
+    // every read in one round trip: the district's counter on lane 0, each
+    // line's stock row on its lane (a line with an unknown item reads nothing)
+    o.o_id = 0;
+    int64_t s = 0, sy = 0;
     int32_t q = 0, so = 0;
-    if (gl == 0) {
-        o_id = cells.ld(&db.d_next_o_id[d]);
-        disc = __ldg(&db.c_discount[c]);
-        w_tax = __ldg(&db.w_tax[w]);
-        d_tax = __ldg(&db.d_tax[d]);
-    }
+    if (gl == 0) o.o_id = __ldcg(&db.d_next_o_id[o.d]);
     if (mine && item < db.n_items) {
         s = sw * db.n_items + item;
-        price = __ldg(&db.i_price[item]);
         q = ldg_cg(&db.s_quantity[s]);
-        sy = cells.ld(&db.s_ytd[s]);
+        sy = __ldcg(&db.s_ytd[s]);
         so = ldg_cg(&db.s_order_cnt[s]);
     }
     // read phase: an unknown item aborts the order (status 1, no writes)
     if (__any_sync(gm, mine && item >= db.n_items)) {
-        if (gl == 0) b.status[t] = 1;
+        if (gl == 0) b.status[v.t] = 1;
         return;
     }
-    const int64_t oslot = ob + os;
-    const int64_t lslot = lb + ls;
-    if (oslot >= db.ord_cap || lslot + cnt > db.ol_cap) {
+    if (o.oslot >= db.ord_cap || o.lslot + o.cnt > db.ol_cap) {
         if (gl == 0) {
             set_err(b.err, ERR_CAPACITY);
-            b.status[t] = 3;
+            b.status[v.t] = 3;
         }
         return;
     }
-    int64_t amount = 0;
     if (mine) {
-        amount = qty * price;
         const int32_t nq = (q >= qty + 10) ? (int32_t)(q - qty) : (int32_t)(q - qty + 91);
         stg_cg(&db.s_quantity[s], nq);
-        cells.st(&db.s_ytd[s], sy + qty);
+        __stcg(&db.s_ytd[s], sy + qty);
         stg_cg(&db.s_order_cnt[s], so + 1);
-        db.ol_item[lslot + gl] = (int32_t)item;
-        db.ol_sw[lslot + gl] = (int32_t)sw;
-        db.ol_qty[lslot + gl] = (int32_t)qty;
-        stg_cg(&db.ol_amount[lslot + gl], amount);
+    }
+    if (gl == 0) {
+        __stcg(&db.d_next_o_id[o.d], o.o_id + 1);
+        __stcg(&db.c_last_o_id[o.c], o.o_id);
+        stg_cg(&db.c_last_slot[o.c], (uint32_t)o.oslot);
+    }
+    o.run = true;
+}
+
+__device__ __forceinline__ void new_order_finish(const DevDB &db, const DevBulk &b, const TxnView &v, uint32_t gl,
+                                                 const NewOrderPart &o)
+{
+    if (!o.run) return;                      // the whole group
+    const uint32_t gm = group_mask();
+    const int64_t item = o.line & 0xFFFFFF, qty = (o.line >> 40) & 0xFF;
+    int64_t amount = 0, disc = 0, w_tax = 0, d_tax = 0;
+    if (gl == 0) {
+        disc = __ldg(&db.c_discount[o.c]);
+        w_tax = __ldg(&db.w_tax[o.w]);
+        d_tax = __ldg(&db.d_tax[o.d]);
+    }
+    if ((int)gl < o.cnt) {
+        amount = qty * __ldg(&db.i_price[item]);
+        db.ol_item[o.lslot + gl] = (int32_t)item;
+        db.ol_sw[o.lslot + gl] = (int32_t)((o.line >> 24) & 0xFFFF);
+        db.ol_qty[o.lslot + gl] = (int32_t)qty;
+        stg_cg(&db.ol_amount[o.lslot + gl], amount);
     }
     const int64_t total = group_sum16(gm, amount);
-    o_id = __shfl_sync(gm, o_id, 0, kGroup);
+    const int64_t o_id = __shfl_sync(gm, o.o_id, 0, kGroup);
     // the order index: the first free slot on the key's probe path, claimed
     // by compare-and-swap (other orders' inserts may race for it)
-    const unsigned long long key = ord_key(d, o_id);
+    const unsigned long long key = ord_key(o.d, o_id);
     bool inserted = false;
     {
         // an empty home slot is the slot the probe would find first: taken
@@ -824,7 +878,7 @@ __device__ __forceinline__ void exec_new_order_group(const DevDB &db, const DevB
         if (gl == 0) prev = atomicCAS(&db.ord_idx.keys[home], HKEY_EMPTY, key);
         prev = __shfl_sync(gm, prev, 0, kGroup);
         if (prev == HKEY_EMPTY) {
-            if (gl == 0) __stcg(&db.ord_idx.rows[home], (uint32_t)oslot);
+            if (gl == 0) __stcg(&db.ord_idx.rows[home], (uint32_t)o.oslot);
             inserted = true;
         }
     }
@@ -836,69 +890,144 @@ __device__ __forceinline__ void exec_new_order_group(const DevDB &db, const DevB
         if (gl == 0) prev = atomicCAS(&db.ord_idx.keys[slot], cur, key);
         prev = __shfl_sync(gm, prev, 0, kGroup);
         if (prev == cur) {
-            if (gl == 0) __stcg(&db.ord_idx.rows[slot], (uint32_t)oslot);
+            if (gl == 0) __stcg(&db.ord_idx.rows[slot], (uint32_t)o.oslot);
             inserted = true;
         }
     }
     if (gl == 0) {
-        cells.st(&db.d_next_o_id[d], o_id + 1);
-        db.o_w[oslot] = (int32_t)w;
-        db.o_d[oslot] = (int32_t)v.p1;
-        db.o_c[oslot] = (int32_t)cw;
-        stg_cg(&db.o_cnt[oslot], (int32_t)cnt);
-        stg_cg(&db.o_id[oslot], o_id);
-        stg_cg(&db.o_first[oslot], lslot);
-        stg_cg(&db.o_live[oslot], (uint8_t)1);
-        int64_t *out = b.out + (int64_t)t * b.R;
+        db.o_w[o.oslot] = (int32_t)o.w;
+        db.o_d[o.oslot] = (int32_t)v.p1;
+        db.o_c[o.oslot] = (int32_t)(o.c - o.d * OE_CUST);
+        stg_cg(&db.o_cnt[o.oslot], (int32_t)o.cnt);
+        stg_cg(&db.o_id[o.oslot], o_id);
+        stg_cg(&db.o_first[o.oslot], o.lslot);
+        stg_cg(&db.o_live[o.oslot], (uint8_t)1);
         if (!inserted) {
             set_err(b.err, ERR_CAPACITY);
-            b.status[t] = 3;
+            b.status[v.t] = 3;
             return;
         }
-        cells.st(&db.c_last_o_id[c], o_id);
+        int64_t *out = b.out + (int64_t)v.t * b.R;
         out[0] = o_id;
         out[1] = total * (10000 - disc) * (10000 + w_tax + d_tax) / 100000000;
-        out[2] = cnt;
-        b.status[t] = 0;
+        out[2] = o.cnt;
+        b.status[v.t] = 0;
     }
 }
 
-template <class Cells>
-__device__ __forceinline__ void exec_order_status_group(const DevDB &db, const DevBulk &b, const TxnView &v,
-                                                        uint32_t gl, Cells &cells)
+// a new-order's parameters 2, 3 and this lane's line (0 beyond the last)
+__device__ __forceinline__ int64_t new_order_params(const DevBulk &b, const TxnView &v, uint32_t gl, int64_t &p2,
+                                                    int64_t &p3)
 {
-    if (kDebug && (v.type != GPUTX_T_OE_ORDER_STATUS || !valid_txn(db, v.type, v.p, b.P))) {
-        if (gl == 0) set_err(b.err, ERR_BOUNDS);   // the group's lanes all leave here
+    p2 = __ldg(&v.p[2]);
+    p3 = __ldg(&v.p[3]);
+    return (int64_t)gl < p3 && 4 + (int)gl < b.P ? __ldg(&v.p[4 + gl]) : 0;
+}
+
+// the first part of a new-order whose second runs after the levels: it finds
+// the order's id in the first output (a status other than 0 tells it to stay
+// away)
+__device__ __forceinline__ void new_order_first(const DevDB &db, const DevBulk &b, const TxnView &v, uint32_t gl,
+                                                int64_t p2, int64_t p3, int64_t line, int64_t os, int64_t ls)
+{
+    NewOrderPart o;
+    new_order_state(db, b, v, gl, p2, p3, line, os, ls, o);
+    if (o.run && gl == 0) {
+        b.out[(int64_t)v.t * b.R] = o.o_id;
+        b.status[v.t] = 0;
+    }
+}
+
+// new_order_first by one lane (its lines in chunks, each chunk's loads in
+// flight together)
+__device__ __forceinline__ void new_order_first_lane(const DevDB &db, const DevBulk &b, const TxnView &v)
+{
+    if (kDebug && !valid_txn(db, v.type, v.p, b.P)) {
+        set_err(b.err, ERR_BOUNDS);
         return;
     }
-    const uint32_t gm = group_mask();
     const int64_t *p = v.p;
-    const uint32_t t = v.t;
-    const int64_t w = v.p0, d = w * OE_DIST + v.p1, c = d * OE_CUST + __ldg(&p[2]);
-    int64_t *out = b.out + (int64_t)t * b.R;
-    int64_t o = 0;
-    if (gl == 0) {
-        o = cells.ld(&db.c_last_o_id[c]);
-        const int64_t bal = cells.ld(&db.c_balance[c]);
-        out[0] = bal;
-        out[1] = o;
-    }
-    o = __shfl_sync(gm, o, 0, kGroup);
-    if (o == 0) {
-        if (gl == 0) b.status[t] = 1;
+    const int64_t d = v.p0 * OE_DIST + v.p1, c = d * OE_CUST + p[2];
+    const int cnt = (int)p[3];
+    for (int j = 0; j < cnt; j++)                                  // read phase
+        if ((p[4 + j] & 0xFFFFFF) >= db.n_items) {
+            b.status[v.t] = 1;
+            return;
+        }
+    const int64_t oslot = b.base->ord + b.slot_ord[v.t], lslot = b.base->ol + b.slot_ol[v.t];
+    if (oslot >= db.ord_cap || lslot + cnt > db.ol_cap) {
+        set_err(b.err, ERR_CAPACITY);
+        b.status[v.t] = 3;
         return;
     }
-    unsigned long long k = 0;
-    const int64_t slot = group_probe(gm, gl, db.ord_idx, ord_key(d, o), 1, &k);
-    if (slot < 0 || k != ord_key(d, o)) {
+    constexpr int kLineChunk = 5;
+    const int64_t o_id = __ldcg(&db.d_next_o_id[d]);
+    for (int j0 = 0; j0 < cnt; j0 += kLineChunk) {
+        int64_t sy[kLineChunk];
+        int32_t q[kLineChunk], so[kLineChunk];
+#pragma unroll
+        for (int u = 0; u < kLineChunk; u++) {
+            if (j0 + u < cnt) {
+                const int64_t line = p[4 + j0 + u];
+                const int64_t s = ((line >> 24) & 0xFFFF) * db.n_items + (line & 0xFFFFFF);
+                q[u] = ldg_cg(&db.s_quantity[s]);
+                sy[u] = __ldcg(&db.s_ytd[s]);
+                so[u] = ldg_cg(&db.s_order_cnt[s]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kLineChunk; u++) {
+            if (j0 + u < cnt) {
+                const int64_t line = p[4 + j0 + u];
+                const int64_t s = ((line >> 24) & 0xFFFF) * db.n_items + (line & 0xFFFFFF), qty = (line >> 40) & 0xFF;
+                stg_cg(&db.s_quantity[s], (int32_t)((q[u] >= qty + 10) ? q[u] - qty : q[u] - qty + 91));
+                __stcg(&db.s_ytd[s], sy[u] + qty);
+                stg_cg(&db.s_order_cnt[s], so[u] + 1);
+            }
+        }
+    }
+    __stcg(&db.d_next_o_id[d], o_id + 1);
+    __stcg(&db.c_last_o_id[c], o_id);
+    stg_cg(&db.c_last_slot[c], (uint32_t)oslot);
+    b.out[(int64_t)v.t * b.R] = o_id;
+    b.status[v.t] = 0;
+}
+
+// an order-status in two parts: the customer's balance and last order, then
+// the order's count and amounts (the order's slot waits in the third output)
+__device__ __forceinline__ void order_status_first(const DevDB &db, const DevBulk &b, const TxnView &v, int64_t p2)
+{
+    if (kDebug && !valid_txn(db, v.type, v.p, b.P)) {
+        set_err(b.err, ERR_BOUNDS);
+        return;
+    }
+    const int64_t c = (v.p0 * OE_DIST + v.p1) * OE_CUST + p2;
+    const int64_t o = __ldcg(&db.c_last_o_id[c]), bal = __ldcg(&db.c_balance[c]);
+    const uint32_t last = __ldcg(&db.c_last_slot[c]);
+    int64_t *out = b.out + (int64_t)v.t * b.R;
+    out[0] = bal;
+    out[1] = o;
+    out[2] = o == 0 ? 0 : (int64_t)last;
+    b.status[v.t] = o == 0 ? 1 : 0;
+}
+__device__ __forceinline__ void order_status_finish(const DevDB &db, const DevBulk &b, const TxnView &v, uint32_t gl)
+{
+    const uint32_t gm = group_mask();
+    int64_t *out = b.out + (int64_t)v.t * b.R;
+    int64_t r = 0;
+    if (gl == 0) {
+        r = out[2];
+        if ((uint32_t)r == kNoSlot) r = hash_find(db.ord_idx, ord_key(v.p0 * OE_DIST + v.p1, out[1]));
+        if (r >= 0 && !dbg_in(r, db.ord_cap, b.err)) r = -1;
+    }
+    r = __shfl_sync(gm, r, 0, kGroup);
+    if (r < 0) {
         if (gl == 0) {
             set_err(b.err, ERR_BOUNDS);
-            b.status[t] = 1;
+            b.status[v.t] = 1;
         }
         return;
     }
-    int64_t r = (int64_t)__ldcg(&db.ord_idx.rows[slot]);
-    if (kDebug && !dbg_in(r, db.ord_cap, b.err)) r = 0;
     int cnt = ldg_cg(&db.o_cnt[r]);
     const int64_t first = ldg_cg(&db.o_first[r]);
     if (kDebug && (cnt < 0 || cnt > kGroup || !dbg_in(first, db.ol_cap - cnt + 1, b.err))) cnt = 0;
@@ -907,30 +1036,54 @@ __device__ __forceinline__ void exec_order_status_group(const DevDB &db, const D
     if (gl == 0) {
         out[2] = cnt;
         out[3] = sum;
-        b.status[t] = 0;
     }
 }
 
-// L2 prefetch of the rows lane gl of a group will touch
-__device__ __forceinline__ void prefetch_group(const DevDB &db, const TxnView &v, uint32_t gl)
+// a payment in two parts, likewise: the customer's cells and the output, then
+// the warehouse's and district's totals (by atomic additions)
+__device__ __forceinline__ void payment_first(const DevDB &db, const DevBulk &b, const TxnView &v, int64_t p2,
+                                              int64_t amount)
+{
+    if (kDebug && !valid_txn(db, v.type, v.p, b.P)) {
+        set_err(b.err, ERR_BOUNDS);
+        return;
+    }
+    const int64_t c = (v.p0 * OE_DIST + v.p1) * OE_CUST + p2;
+    const int64_t cb = __ldcg(&db.c_balance[c]), cy = __ldcg(&db.c_ytd[c]), cn = __ldcg(&db.c_payment_cnt[c]);
+    const int64_t bal = wrap_add(cb, -amount);
+    __stcg(&db.c_balance[c], bal);
+    __stcg(&db.c_ytd[c], wrap_add(cy, amount));
+    __stcg(&db.c_payment_cnt[c], cn + 1);
+    b.out[(int64_t)v.t * b.R] = bal;
+    b.status[v.t] = 0;
+}
+__device__ __forceinline__ void payment_totals(const DevDB &db, const TxnView &v, int64_t amount)
+{
+    if (kDebug && (v.type < 0 || v.p0 < 0 || v.p0 >= db.n_wh || v.p1 < 0 || v.p1 >= OE_DIST)) return;
+    atomicAdd((unsigned long long *)&db.w_ytd[v.p0], (unsigned long long)amount);
+    atomicAdd((unsigned long long *)&db.d_ytd[v.p0 * OE_DIST + v.p1], (unsigned long long)amount);
+}
+
+// L2 prefetch of the rows lane gl of a new-order will touch; p2, p3 and line as
+// in new_order_state
+__device__ __forceinline__ void prefetch_new_order(const DevDB &db, const TxnView &v, uint32_t gl, int64_t p2,
+                                                   int64_t p3, int64_t line)
 {
     if (kDebug && v.type < 0) return;
-    const int64_t *p = v.p;
-    if (v.type == GPUTX_T_OE_NEW_ORDER) {
-        if (gl == 0) prefetch_l2(&db.d_next_o_id[v.p0 * OE_DIST + v.p1]);
-        const int cnt = (int)__ldg(&p[3]);
-        if ((int)gl < cnt) {
-            const int64_t line = __ldg(&p[4 + gl]);
-            const int64_t item = line & 0xFFFFFF, sw = (line >> 24) & 0xFFFF;
-            if (item < db.n_items) {
-                prefetch_l2(&db.s_quantity[sw * db.n_items + item]);
-                prefetch_l2(&db.s_ytd[sw * db.n_items + item]);
-            }
+    const int64_t d = v.p0 * OE_DIST + v.p1;
+    if (gl == 0) {
+        prefetch_l2(&db.d_next_o_id[d]);
+        prefetch_l2(&db.c_last_o_id[d * OE_CUST + p2]);
+        prefetch_l2(&db.c_last_slot[d * OE_CUST + p2]);
+    }
+    if ((int64_t)gl < p3) {
+        const int64_t item = line & 0xFFFFFF, sw = (line >> 24) & 0xFFFF;
+        if (item < db.n_items) {
+            const int64_t s = sw * db.n_items + item;
+            prefetch_l2(&db.s_quantity[s]);
+            prefetch_l2(&db.s_ytd[s]);
+            prefetch_l2(&db.s_order_cnt[s]);
         }
-    } else if (gl == 0) {
-        const int64_t c = (v.p0 * OE_DIST + v.p1) * OE_CUST + __ldg(&p[2]);
-        prefetch_l2(&db.c_last_o_id[c]);
-        prefetch_l2(&db.c_balance[c]);
     }
 }
 
