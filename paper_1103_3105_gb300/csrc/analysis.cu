@@ -247,7 +247,8 @@ struct RankMode {
 // TPL tickets: number of operations of the group before this operation's run
 // (Section 5.1 key values, read with ticket semantics).  A ticket of at least
 // `hot_ticket` raises `hot`: some counter carries a chain that long, which
-// picks the executor (the flag is written once, by the first such ticket seen).
+// picks the order the debit-credit executor hands transactions out in (the flag
+// is written once, by the first such ticket seen).
 struct TicketMode {
     const uint32_t *sk, *sv;
     uint32_t *lock_key, *lock_ticket;
@@ -1518,15 +1519,9 @@ cudaError_t launch_rank_scan(gputx_bulk *b, const uint32_t *sk, const uint32_t *
 cudaError_t launch_ticket_scan(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m)
 {
     const bool fixed = b->db->uniform_k || b->graph;
-    // CTA-wide lock groups pay off once a counter's chain reaches about
-    // n/512 operations: on debit-credit under R/W (one lock per branch) they
-    // run Zipf 0.7 accounts (a branch chain of about n/300) 15 % faster than
-    // warp groups, and uniform ones (1,000 chains of about n/1,000) 13 %
-    // slower
-    const int64_t hot = b->n / 512 > 32 ? b->n / 512 : 32;
     TicketMode tm{sk, sv, b->sc.lock_key, b->sc.lock_ticket, fixed ? nullptr : b->sc.op_off,
                   b->graph ? b->db->kmax : b->db->uniform_k, &b->ctl->hot,
-                  (uint32_t)(hot > 0xffffffffll ? 0xffffffffll : hot), b->db->dev.n_objects, &b->ctl->err};
+                  kTplHot, b->db->dev.n_objects, &b->ctl->err};
     cudaError_t e = cudaMemsetAsync(&b->ctl->hot, 0, sizeof(uint32_t), b->stream);
     if (e) return e;
     return run_scan(b, tm, m);

@@ -1292,7 +1292,7 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
         CK(launch_ticket_scan(b, sk, sv, m), "tickets");
         CK(begin_tail(b), "order");
         if (b->timing) cudaEventRecord(b->ev[3], s);
-        CK(launch_tpl(b, block, add), "tpl execute");
+        CK(launch_tpl(b, sk, sv, block, add), "tpl execute");
         CK(launch_orders(b), "orders");
         if (b->timing) cudaEventRecord(b->ev[4], s);
         CK(launch_tpl_reset(b, sk, m), "tpl reset");

@@ -129,7 +129,7 @@ cudaError_t enqueue_pipeline(GraphBulk *g)
     } else {
         if ((e = gtx::launch_ticket_scan(b, sk, sv, m))) return e;
         if ((e = gtx::launch_begin(b))) return e;
-        if ((e = gtx::launch_tpl(b, g->block, add))) return e;
+        if ((e = gtx::launch_tpl(b, sk, sv, g->block, add))) return e;
         if ((e = gtx::launch_orders(b))) return e;
         if ((e = gtx::launch_tpl_reset(b, sk, m))) return e;
     }

@@ -195,6 +195,26 @@ __device__ __forceinline__ int64_t wrap_add(int64_t a, int64_t b)
     return (int64_t)((unsigned long long)a + (unsigned long long)b);
 }
 
+constexpr uint32_t kFull = 0xffffffffu;   // every lane of a warp
+
+// inclusive prefix of `x` over the lanes of `peers` up to this lane, in lane
+// order, by pointer jumping along each group; every lane of the warp calls it
+__device__ __forceinline__ int64_t lanes_prefix(uint32_t peers, int64_t x)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t below = peers & ((1u << lane) - 1u);
+    uint32_t p = below ? 31 - __clz(below) : lane;   // the group's lane before this one (itself: none)
+#pragma unroll
+    for (int s = 0; s < 5; s++) {
+        const int64_t y = __shfl_sync(kFull, x, p);
+        const uint32_t q = __shfl_sync(kFull, p, p);
+        const bool more = p != lane;
+        if (more) x = wrap_add(x, y);
+        p = q == p || !more ? lane : q;              // the head of the list has been added: done
+    }
+    return x;
+}
+
 __device__ __forceinline__ void set_err(uint32_t *err, uint32_t bit) { atomicOr(err, bit); }
 
 // Debug builds (compiled with -DGPUTX_DEBUG into libgputx_debug.so) check,

@@ -1,6 +1,5 @@
-// cta_groups.cuh -- lock groups over a whole CTA, shared by the debit-credit
-// TPL executors (ordered counters in exec.cu, relaxed spin locks in
-// relaxed.cu).
+// cta_groups.cuh -- lock groups over a whole CTA, for the debit-credit relaxed
+// TPL executor (spin locks, relaxed.cu).
 //
 // A CTA holds a chunk of up to 256 consecutive transactions of the bulk.
 // Those that need the same lock form one group: a shared-memory hash table

@@ -24,10 +24,12 @@ struct BulkCtl {
     InsertBase total;      // inserts this bulk reserves
     uint32_t rounds;       // exact-depth passes run (the dataflow pass: 1)
     uint32_t n_seg;        // segmented graph bulks: bulks in this segment (0 = one)
-    uint32_t hot;          // TPL: some counter has a chain of at least the hot ticket
+    uint32_t hot;          // TPL: some counter has a chain of more than kTplHot operations
     uint32_t chunk;        // relaxed TPL: next chunk to claim (claim counts commit tickets)
     uint32_t front;        // exact depth: chunks of transactions finished
 };
+
+constexpr uint32_t kTplHot = 128;  // debit-credit TPL: a chain longer than this is served in lock order
 
 constexpr int kSegMax = 64;        // bulks in one segment of a graph bulk, at most
 
@@ -175,7 +177,7 @@ cudaError_t launch_kset(gputx_bulk *b, const uint32_t *order, int64_t nchunks, i
 cudaError_t launch_kset_levels(gputx_bulk *b, const uint32_t *level_off_host, int64_t depth, int narrow_max,
                                bool atomic_add, const uint32_t *type_cut_host = nullptr);
 cudaError_t launch_part(gputx_bulk *b, const uint32_t *pkeys, int block, int64_t max_parts);
-cudaError_t launch_tpl(gputx_bulk *b, int block, bool atomic_add);
+cudaError_t launch_tpl(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int block, bool atomic_add);
 // after K-SET's levels, after TPL: the rows of the new orders, then what the order-statuses read of them
 cudaError_t launch_orders(gputx_bulk *b);
 // a conflict-free bulk (a 0-set) in one launch

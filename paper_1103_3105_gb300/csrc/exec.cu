@@ -30,7 +30,6 @@
 
 #include "engine.h"
 #include "procs.cuh"
-#include "cta_groups.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -421,23 +420,12 @@ __global__ void part_kernel(DevDB db, DevBulk b, const BulkCtl *ctl, const uint3
     }
 }
 
-constexpr uint32_t kFull = 0xffffffffu;
-
 // sum of `x` over the lanes of `m` (this lane's group) and its inclusive
 // prefix up to this lane, in lane order; every lane of the warp calls it
 __device__ __forceinline__ void group_sum(uint32_t m, int64_t x, int64_t &pre, int64_t &tot)
 {
-    const uint32_t lane = threadIdx.x & 31;
-    pre = 0;
-    tot = 0;
-#pragma unroll 4
-    for (int L = 0; L < 32; L++) {
-        const int64_t d = __shfl_sync(kFull, x, L);
-        if ((m >> L) & 1u) {
-            tot += d;
-            if ((uint32_t)L <= lane) pre += d;
-        }
-    }
+    pre = lanes_prefix(m, x);
+    tot = __shfl_sync(kFull, pre, 31 - __clz(m));
 }
 
 // one addition per distinct cell among the lanes with `on`, by the lowest
@@ -467,17 +455,8 @@ struct TplArgs {
                          // first op_count are real; padding transactions skipped
     bool orders;         // new-orders are registered: launch_orders completes them and the order-statuses
     LockSlots slot;      // item -> its counter in `done`
-    int when_hot;        // debit-credit executors: -1 run, 1 run only if ctl->hot, 0 only if not
+    const uint32_t *sk, *sv;   // debit-credit: the operations sorted by lock
 };
-
-// whether a debit-credit TPL executor sits this bulk out (the other one runs)
-__device__ __forceinline__ bool tpl_skip(const TplArgs &a)
-{
-    if (a.when_hot < 0) return false;
-    const bool hot = *(volatile const uint32_t *)&a.ctl->hot != 0u;
-    return hot != (a.when_hot == 1);
-}
-
 
 // releases of the lanes with `rel` (every lane of the warp calls it): lanes
 // releasing the same counter are grouped by __match_any_sync and their
@@ -671,30 +650,40 @@ __global__ void __launch_bounds__(512) tpl_kernel(TplArgs a)
 // hand-off waits for one atomic round trip instead of a load, the stores and
 // their acknowledgement.
 //
-// A warp works on 32 consecutive transactions and resolves the conflicts
-// among them itself.  __match_any_sync groups the lanes that need the same
-// counter.  Every operation here is a write and the warp holds consecutive
-// timestamps, so no other transaction's operation on that item lies between
-// two lanes of a group: their tickets are consecutive, and the whole group
-// runs, in lane (timestamp) order, as soon as its first lane's ticket is
-// granted.  Only that lane polls the counter, and one addition of the group's
-// size releases it.  Within a group, lanes on the same account combine their
-// deltas (warp-aggregated atomics): one fetch-and-add of the sum, each lane's
-// new balance = the old value plus the inclusive prefix of the deltas in lane
-// order -- the serial result bit for bit.  Teller and branch additions are
-// aggregated the same way.  The warp polls in lockstep rounds: each group
-// polls again after about 500 ns per release it still misses, and the warp
-// sleeps until the first group is due, so a group whose counter is about to
-// be released never sleeps behind one far back in its chain.  A warp in
-// which no two lanes share a counter needs none of this: there each lane
-// waits on its own counter and runs as soon as it is granted.
+// A warp works on 32 transactions and resolves the conflicts among them
+// itself.  They are consecutive in timestamp order, or, once the ticket scan has
+// found a chain of more than kTplHot operations, consecutive in the operations
+// sorted by lock: a lock's queue then changes hands once per 32 transactions
+// instead of once per transaction.  Either way a transaction waits for ones
+// handed out before it only.  What bounds a long chain is its hand-offs, about
+// 2 us each through L2; in lock order the signatures and outputs are scattered,
+// which costs about 50 us per 2^20, hence the line.  1,000 branches, 2^20
+// transactions (chains of 1,050): 360 us, 1,900 in timestamp order; Zipf 0.99
+// accounts, 200,003: 490 us, 5,500 with CTA-wide groups in timestamp order.
+//
+// __match_any_sync groups the lanes that need the same counter.  Every
+// operation here is a write and no other transaction's operation on that item
+// lies between two lanes of a group (the warp holds consecutive timestamps, or
+// consecutive tickets): their tickets are consecutive, and the whole group runs,
+// in lane (timestamp) order, as soon as its first lane's ticket is granted.
+// Only that lane polls the counter, and one addition of the group's size
+// releases it.  Within a group, lanes on the same account combine their deltas
+// (warp-aggregated atomics): one fetch-and-add of the sum, each lane's new
+// balance = the old value plus the inclusive prefix of the deltas in lane order
+// -- the serial result bit for bit.  Teller and branch additions are aggregated
+// the same way.  The warp polls in lockstep rounds: each group polls again after
+// about 500 ns per release it still misses, and the warp sleeps until the first
+// group is due, so a group whose counter is about to be released never sleeps
+// behind one far back in its chain.  A warp in which no two lanes share a
+// counter needs none of this: there each lane waits on its own counter and runs
+// as soon as it is granted.
 __global__ void tpl_dc_kernel(TplArgs a)
 {
     __shared__ uint32_t s_c, s_stop;
-    if (tpl_skip(a)) return;
     const int64_t n = a.b.n;
     const int64_t hb = a.ctl->base.hist;
     const uint32_t lane = threadIdx.x & 31;
+    const bool by_lock = a.ctl->hot != 0;
     while (true) {
         if (threadIdx.x == 0) {
             s_stop = *(volatile uint32_t *)&a.ctl->err ? 1u : 0u;
@@ -703,8 +692,9 @@ __global__ void tpl_dc_kernel(TplArgs a)
         __syncthreads();
         const int64_t start = (int64_t)s_c * blockDim.x;
         if (s_stop || start >= n) break;
-        const int64_t t = start + threadIdx.x;
-        const bool live = t < n;
+        const int64_t i = start + threadIdx.x;
+        const bool live = i < n;
+        const int64_t t = live && by_lock ? (int64_t)(__ldg(&a.sv[i]) >> 7) : i;
         DcRecord r{};
         uint32_t key = 0xFFFFFFE0u | lane, tk = 0;   // a key of its own for an idle lane
         bool rows_ok = true;   // a debug build's check of the record's rows
@@ -717,7 +707,7 @@ __global__ void tpl_dc_kernel(TplArgs a)
             r.br = a.db.div_br.div(r.a);
             rows_ok = dbg_dc_rows(a.db, a.b, r.a, r.tl, r.br, r.t);
             if (rows_ok) prefetch_l2(&a.db.acc_bal[r.a]);
-            key = a.slot(a.lock_key[t]);
+            key = a.slot(by_lock ? __ldg(&a.sk[i]) : a.lock_key[t]);
             tk = a.lock_ticket[t];
         }
         const uint32_t grp = __match_any_sync(kFull, key);
@@ -744,7 +734,8 @@ __global__ void tpl_dc_kernel(TplArgs a)
                 if (pending && lane == leader && need && now >= t_next) {
                     v = seen = ld_acquire(&a.done[key]);
                     // missing `gap` releases take at least that many hand-offs
-                    const uint32_t gap = v < need ? need - v : 0;
+                    // (in lock order: a hand-off releases a warp's 32)
+                    const uint32_t gap = v >= need ? 0 : by_lock ? (need - v + 31) / 32 : need - v;
                     t_next = now + (gap > 1 ? (uint64_t)(gap > 64 ? 64 : gap) * 500 : 0);
                 }
                 v = __shfl_sync(kFull, v, leader);
@@ -807,116 +798,6 @@ __global__ void tpl_dc_kernel(TplArgs a)
                 idle = 0;
             }
         }
-        __syncthreads();
-    }
-}
-
-// TPL for debit-credit-only bulks with the lock groups formed over the whole
-// CTA (up to 256 consecutive transactions) instead of one warp
-// (cta_groups.cuh).  The chunk holds consecutive timestamps, so a group's
-// tickets are consecutive and the group runs as soon as its first member's
-// ticket is granted: that member waits on the counter and publishes the grant
-// in shared memory; once every member has its account balance it releases
-// the counter by the group's size.  On a hot item a whole chunk's operations
-// cost one hand-off through L2.
-__global__ void __launch_bounds__(kCtaMax) tpl_dc_block_kernel(TplArgs a)
-{
-    __shared__ uint32_t s_c, s_stop;
-    __shared__ CtaGroupTables g;
-    if (tpl_skip(a)) return;
-    const int64_t n = a.b.n;
-    const int64_t hb = a.ctl->base.hist;
-    const uint32_t tid = threadIdx.x;
-    while (true) {
-        if (tid == 0) {
-            s_stop = *(volatile uint32_t *)&a.ctl->err ? 1u : 0u;
-            s_c = atomicAdd(&a.ctl->claim, 1u);
-        }
-        cta_groups_reset(g, tid, blockDim.x);
-        __syncthreads();
-        const int64_t start = (int64_t)s_c * blockDim.x;
-        if (s_stop || start >= n) break;
-        const int64_t t = start + tid;
-        const bool live = t < n;
-        DcRecord r{};
-        bool rows_ok = true;   // a debug build's check of the record's rows
-        uint32_t key = 0, tk = 0, e = 0;
-        if (live) {
-            r.a = (uint32_t)__ldg(&a.b.params[t * a.b.P]);
-            r.delta = __ldg(&a.b.params[t * a.b.P + 1]);
-            r.ts = __ldg(&a.b.ts[t]);
-            r.t = (uint32_t)t;
-            r.tl = a.db.div_tel.div(r.a);
-            r.br = a.db.div_br.div(r.a);
-            rows_ok = dbg_dc_rows(a.db, a.b, r.a, r.tl, r.br, r.t);
-            if (rows_ok) prefetch_l2(&a.db.acc_bal[r.a]);
-            key = a.slot(a.lock_key[t]);
-            tk = a.lock_ticket[t];
-            e = cta_group_join(g, key, tid);
-        }
-        const int64_t slot = hb + t;
-        const bool run = live && rows_ok && slot < a.db.hist_cap;
-        g.delta[tid] = run ? r.delta : 0;
-        g.acct[tid] = r.a;
-        g.aflag[tid] = 0;
-        __syncthreads();
-        if (live) {
-            CtaMember c;
-            cta_member(g, e, tid, r.a, c);
-            if (c.size == 1) {
-                // the only transaction of the chunk on its counter: it waits
-                // on its own and runs as soon as it is granted
-                const bool ok1 = !tk || wait_at_least(&a.done[key], tk, a.spin_limit_ns, 500);
-                if (!ok1) set_err(&a.ctl->err, ERR_TIMEOUT);
-                DcOut o;
-                const bool pend = ok1 && dc_account_rmw(a.db, a.b, r, slot, o);
-                red_release_add(&a.done[key], 1u);
-                if (pend) dc_finish_rmw(a.db, a.b, o);
-                goto next_chunk;
-            }
-            volatile uint32_t *state = &g.state[e];
-            bool ok = true;
-            if (tid == c.leader) {
-                ok = !tk || wait_at_least(&a.done[key], tk, a.spin_limit_ns, 500);
-                if (!ok) set_err(&a.ctl->err, ERR_TIMEOUT);
-                __threadfence_block();
-                *state = ok ? 1u : 2u;
-            } else if (!wait_smem(state, a.spin_limit_ns) || *state != 1u) {
-                ok = false;
-                if (*state == 0u) set_err(&a.ctl->err, ERR_TIMEOUT);
-            }
-            __threadfence_block();   // the leader's acquire before this member's accesses
-            if (ok && !run && rows_ok) {           // history full: not executed
-                set_err(a.b.err, ERR_CAPACITY);
-                a.b.status[r.t] = 3;
-            }
-            int64_t old = 0;
-            const bool have = ok && run &&
-                              cta_account_update(g, c, tid, &a.db.acc_bal[r.a], a.spin_limit_ns, &a.ctl->err, old);
-            // every member counted once its account update is done (or it gave up)
-            __threadfence_block();
-            atomicAdd(&g.fin[e], 1u);
-            if (tid == c.leader) {
-                // the group's updates precede its one release
-                if (!cta_wait_members(g, e, c.size, a.spin_limit_ns)) set_err(&a.ctl->err, ERR_TIMEOUT);
-                red_release_add(&a.done[key], c.size);
-            }
-            if (have) {
-                atomicAdd((unsigned long long *)&a.db.tel_bal[r.tl], (unsigned long long)r.delta);
-                atomicAdd((unsigned long long *)&a.db.br_bal[r.br], (unsigned long long)r.delta);
-                DcOut o;
-                o.slot = slot;
-                o.ts = r.ts;
-                o.delta = r.delta;
-                o.na = wrap_add(old, c.pre);
-                o.a = r.a;
-                o.tl = r.tl;
-                o.br = r.br;
-                o.t = r.t;
-                dc_finish(a.db, a.b, o);
-            }
-        }
-    next_chunk:
         __syncthreads();
     }
 }
@@ -1000,7 +881,6 @@ int exec_blocks_per_sm(int kind, int block)
     int nb = 1;
     if (kind == 0) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kset_kernel, block, 0);
     else if (kind == 2) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, tpl_dc_kernel, block, 0);
-    else if (kind == 3) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, tpl_dc_block_kernel, block, 0);
     else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, tpl_kernel, block, 0);
     return nb < 1 ? 1 : nb;
 }
@@ -1168,7 +1048,7 @@ cudaError_t launch_independent(gputx_bulk *b, bool atomic_add)
     return cudaGetLastError();
 }
 
-cudaError_t launch_tpl(gputx_bulk *b, int block, bool atomic_add)
+cudaError_t launch_tpl(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int block, bool atomic_add)
 {
     gputx_db *db = b->db;
     if (b->n == 0) return cudaSuccess;
@@ -1196,26 +1076,11 @@ cudaError_t launch_tpl(gputx_bulk *b, int block, bool atomic_add)
     int64_t grid = (int64_t)db->num_sms * exec_blocks_per_sm(dc ? 2 : 1, block);
     const int64_t chunks = (b->n + block - 1) / block;
     if (grid > chunks) grid = chunks;
-    a.when_hot = -1;
-    if (dc && block <= kCtaMax) {
-        // CTAs of up to 256 threads can group over the whole CTA: the ticket
-        // scan's flag picks that executor when a counter's chain is long
-        // enough to put several of its operations in one chunk, else the
-        // warp groups (both are launched; the one not picked returns at once)
-        a.when_hot = 1;
-        int64_t grid_b = (int64_t)db->num_sms * exec_blocks_per_sm(3, block);
-        if (grid_b > chunks) grid_b = chunks;
-        tpl_dc_block_kernel<<<(unsigned)grid_b, block, 0, b->stream>>>(a);
-        a.when_hot = 0;
-        tpl_dc_kernel<<<(unsigned)grid, block, 0, b->stream>>>(a);
-        count_launches(2);
-    } else {
-        if (dc)
-            tpl_dc_kernel<<<(unsigned)grid, block, 0, b->stream>>>(a);
-        else
-            tpl_kernel<<<(unsigned)grid, block, 0, b->stream>>>(a);
-        count_launches(1);
-    }
+    a.sk = sk;
+    a.sv = sv;
+    if (dc) tpl_dc_kernel<<<(unsigned)grid, block, 0, b->stream>>>(a);
+    else tpl_kernel<<<(unsigned)grid, block, 0, b->stream>>>(a);
+    count_launches(1);
     return cudaGetLastError();
 }
 

@@ -18,7 +18,6 @@ namespace gtx {
 
 namespace {
 
-constexpr uint32_t kFull = 0xffffffffu;
 constexpr int kThreads = 256, kWarps = kThreads / 32;
 constexpr int kTab = 512;                    // hash slots, at most kThreads used
 constexpr uint32_t kFree = 0xffffffffu;      // an unused slot's account
@@ -74,24 +73,6 @@ __device__ uint32_t first_other(const uint32_t *keys, uint32_t lo, uint32_t hi, 
         span = 0;
     }
     return hi;
-}
-
-// inclusive prefix of `x` over the lanes of `peers` up to this lane, in lane
-// order, by pointer jumping along each group; every lane of the warp calls it
-__device__ __forceinline__ int64_t lanes_prefix(uint32_t peers, int64_t x)
-{
-    const uint32_t lane = threadIdx.x & 31;
-    const uint32_t below = peers & ((1u << lane) - 1u);
-    uint32_t p = below ? 31 - __clz(below) : lane;   // the group's lane before this one (itself: none)
-#pragma unroll
-    for (int s = 0; s < 5; s++) {
-        const int64_t y = __shfl_sync(kFull, x, p);
-        const uint32_t q = __shfl_sync(kFull, p, p);
-        const bool more = p != lane;
-        if (more) x = wrap_add(x, y);
-        p = q == p || !more ? lane : q;              // the head of the list has been added: done
-    }
-    return x;
 }
 
 // A CTA runs the groups that begin in its slice of the sorted positions, from

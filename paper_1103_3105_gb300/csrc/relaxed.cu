@@ -30,7 +30,6 @@ struct TplRelaxedArgs {
     bool atomic_add;
 };
 
-constexpr uint32_t kFull = 0xffffffffu;
 
 // The lock of Figure 10, extended to shared readers, with a version in the
 // word: bits 0..19 count the readers holding it, bit 20 is set while a writer

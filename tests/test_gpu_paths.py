@@ -80,3 +80,27 @@ def test_signature_widths_and_alignment(P, shift):
         b.free()
         assert np.array_equal(st, ost) and np.array_equal(out, oout), strategy
         g.close()
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("pattern", ["one account", "one branch", "hot and rest", "pairs"])
+@pytest.mark.parametrize("n", [127, 129, 130, 300, 8193])
+def test_tpl_in_lock_order(n, pattern, mode):
+    """Chains of up to 128 operations are served in timestamp order, longer
+    ones in lock order: queues cut at a warp's and a CTA's 32 and 256."""
+    rng = np.random.default_rng(n)
+    acct = accounts(pattern, n, rng)
+    bulk = {"ts": np.arange(n, dtype=np.int64), "type": np.zeros(n, np.int32), "P": 2,
+            "params": np.stack([acct, rng.integers(-(1 << 62), 1 << 62, n)], 1).astype(np.int64)}
+    ost, oout = oracle.OracleDB(dc=W.dc_tables(B, T, A), hist_cap=2 * n).execute(bulk, 1)
+    g = G.Database(dc=(B, T, A), history_capacity=n, max_bulk=n)
+    g.register(G.DC_TYPES)
+    b = g.submit_dict(bulk).execute("tpl", conflict_mode=mode)
+    st, out = b.results()
+    b.free()
+    assert np.array_equal(st, ost) and np.array_equal(out, oout)
+    with np.errstate(over="ignore"):
+        want = np.zeros(B, np.int64)
+        np.add.at(want, acct // 100, bulk["params"][:, 1])
+    assert np.array_equal(g.read(G.TBL_DC_BRANCH)[:, 0], want)
+    g.close()
