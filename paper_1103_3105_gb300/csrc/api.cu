@@ -1104,8 +1104,13 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
     // the paths run side by side without a barrier per k-set and no level
     // table is built (exec_dc.cu; kset_launch = 1 asks for the levels)
     const bool paths = strategy == GPUTX_KSET && dc_only(db) && !(opts && opts->kset_launch == 1);
+    // likewise any bulk of single-operation transactions (kset_rounds_kernel)
+    const bool single = db->uniform_k == 1 && !paths && !(opts && opts->kset_launch == 1);
     if (!paths && (strategy == GPUTX_KSET || (strategy == GPUTX_AUTO && run == GPUTX_AUTO))) {
         if ((st = run_grouping(b, mode, part_size, sk, sv, ak, av, m))) return st;
+    }
+    if (!paths && !(single && strategy == GPUTX_KSET) &&
+        (strategy == GPUTX_KSET || (strategy == GPUTX_AUTO && run == GPUTX_AUTO))) {
         CK(launch_rank_scan(b, sk, sv, m, db->need_fixpoint), "rank");
         // AUTO decides on the one-pass ranks first: w0 and c are exact there
         // (a transaction is a source exactly when all its operations have
@@ -1160,6 +1165,10 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
         if ((st = run_grouping(b, mode, part_size, sk, sv, ak, av, m))) return st;
         CK(begin_tail(b, true), "order");
         if ((st = run_ranges(sk, sv, 7, true))) return st;
+    } else if (run == GPUTX_KSET && single) {
+        CK(begin_tail(b), "order");
+        if (b->timing) cudaEventRecord(b->ev[3], s);
+        CK(launch_kset_rounds(b, sk, sv, strategy == GPUTX_KSET, add), "k-set execute");
     } else if (run == GPUTX_KSET) {
         const int64_t depth = b->host_ctl.last_level;
         const bool persistent = opts && opts->kset_launch == 1;

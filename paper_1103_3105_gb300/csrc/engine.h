@@ -176,6 +176,8 @@ cudaError_t launch_finish(gputx_bulk *b);
 cudaError_t launch_kset(gputx_bulk *b, const uint32_t *order, int64_t nchunks, int block, bool atomic_add);
 cudaError_t launch_kset_levels(gputx_bulk *b, const uint32_t *level_off_host, int64_t depth, int narrow_max,
                                bool atomic_add, const uint32_t *type_cut_host = nullptr);
+// single-operation bulks, from the sorted operations: item by item, run by run
+cudaError_t launch_kset_rounds(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, bool stats, bool atomic_add);
 cudaError_t launch_part(gputx_bulk *b, const uint32_t *pkeys, int block, int64_t max_parts);
 cudaError_t launch_tpl(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int block, bool atomic_add);
 // after K-SET's levels, after TPL: the rows of the new orders, then what the order-statuses read of them

@@ -13,6 +13,7 @@
 // the same thing without the k-set numbers.
 #include "dc.cuh"
 #include "engine.h"
+#include "ranges.cuh"
 
 namespace gtx {
 
@@ -43,38 +44,6 @@ struct RangeArgs {
 __device__ __forceinline__ uint32_t acct_hash(uint32_t a) { return (a * 2654435761u) >> 23; }
 static_assert(kTab == 512, "acct_hash yields 9 bits");
 
-// first position in [lo, hi) whose key is not `key` (hi if none; keys sorted);
-// the whole CTA calls it
-__device__ uint32_t first_other(const uint32_t *keys, uint32_t lo, uint32_t hi, uint32_t key, uint32_t *s_min)
-{
-    const uint32_t tid = threadIdx.x;
-    uint32_t span = kThreads;                // the next kThreads positions, then kThreads probes a round
-    while (lo < hi) {
-        const uint32_t len = hi - lo;
-        const uint32_t step = span == 0 ? (len + kThreads - 1) / kThreads : 1;
-        if (tid == 0) *s_min = kThreads;
-        __syncthreads();
-        const uint64_t at = (uint64_t)lo + (uint64_t)(tid + 1) * step - 1;
-        const uint32_t p = at < hi ? (uint32_t)at : hi - 1;
-        const uint32_t m = __ballot_sync(kFull, __ldg(&keys[p]) != key);
-        if ((tid & 31) == 0 && m) atomicMin(s_min, tid + (uint32_t)__ffs(m) - 1);
-        __syncthreads();
-        const uint32_t i = *s_min;
-        __syncthreads();
-        if (i == kThreads) {                 // none among the probes, the last of which was min(...) below
-            if (step > 1 || len <= (uint32_t)kThreads) return hi;
-            lo += kThreads;
-        } else {
-            const uint32_t a = lo + i * step;
-            if (step == 1) return a < hi ? a : hi - 1;
-            hi = a + step < hi ? a + step : hi;
-            lo = a;
-        }
-        span = 0;
-    }
-    return hi;
-}
-
 // A CTA runs the groups that begin in its slice of the sorted positions, from
 // the first group's head to the last group's end, 256 positions (a window) at
 // a time.  Groups share no account, so windows need not respect their bounds.
@@ -104,19 +73,10 @@ __global__ void __launch_bounds__(kThreads, 4) dc_range_kernel(RangeArgs a)
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const DevBulk &b = a.b;
     const uint32_t n = b.n_live ? *b.n_live : (uint32_t)b.n;
-    const uint64_t s0_ = (uint64_t)blockIdx.x * a.slice;
     if (tid == 0) s_stop = *(volatile uint32_t *)&a.ctl->err;
     __syncthreads();
-    if (s_stop || s0_ >= n) return;          // uniform
-    const uint32_t s0 = (uint32_t)s0_;
-    const uint32_t s1 = n - s0 < a.slice ? n : s0 + a.slice;
-    uint32_t lo = 0, hi = n;
-    if (s0 > 0) {
-        const uint32_t k = __ldg(&a.keys[s0 - 1]);
-        if (__ldg(&a.keys[s1 - 1]) == k) return;   // the slice lies inside an earlier slice's group
-        lo = first_other(a.keys, s0, s1, k, &s_min);
-    }
-    if (s1 < n) hi = first_other(a.keys, s1, n, __ldg(&a.keys[s1 - 1]), &s_min);
+    uint32_t lo, hi;
+    if (s_stop || !group_range<kThreads>(a.keys, n, a.slice, &s_min, lo, hi)) return;   // uniform
     for (uint32_t i = tid; i < kTab; i += kThreads)
         for (int w = 0; w < 2; w++) {
             s_win[w].acct[i] = kFree;

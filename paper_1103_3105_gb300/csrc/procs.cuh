@@ -349,6 +349,14 @@ __device__ __forceinline__ void prefetch_record_l1(const DevBulk &b, uint32_t po
     asm volatile("prefetch.global.L1 [%0];" ::"l"(b.rec_t + pos));
 }
 
+// the home slot of a key in an index
+__device__ __forceinline__ void prefetch_home(const HashIndex &h, unsigned long long key)
+{
+    const uint64_t i = hmix(key) & h.mask;
+    prefetch_l2(&h.keys[i]);
+    prefetch_l2(&h.rows[i]);
+}
+
 __device__ __forceinline__ void prefetch_txn(const DevDB &db, const TxnView &v)
 {
     const int64_t *p = v.p;
@@ -362,8 +370,27 @@ __device__ __forceinline__ void prefetch_txn(const DevDB &db, const TxnView &v)
     }
     case GPUTX_T_SUB_GET_SUBSCRIBER:
     case GPUTX_T_SUB_UPDATE_LOCATION:
+        prefetch_l2(db.sub_rows + v.p0 * SUB_FIELDS);
+        break;
     case GPUTX_T_SUB_UPDATE_FACILITY:
         prefetch_l2(db.sub_rows + v.p0 * SUB_FIELDS);
+        prefetch_home(db.sf_idx, sf_key(v.p0, v.p1));
+        break;
+    case GPUTX_T_SUB_GET_ACCESS:
+        prefetch_home(db.ai_idx, ai_key(v.p0, v.p1));
+        break;
+    case GPUTX_T_SUB_GET_NEW_DEST: {
+        prefetch_home(db.sf_idx, sf_key(v.p0, v.p1));
+        const int64_t start = __ldg(&p[2]);
+        for (int64_t st = 0; st <= 16 && st <= start; st += 8) prefetch_home(db.cf_idx, cf_key(v.p0, v.p1, st));
+        break;
+    }
+    case GPUTX_T_SUB_INSERT_CF:
+        prefetch_home(db.sf_idx, sf_key(v.p0, v.p1));
+        prefetch_home(db.cf_idx, cf_key(v.p0, v.p1, __ldg(&p[2])));
+        break;
+    case GPUTX_T_SUB_DELETE_CF:
+        prefetch_home(db.cf_idx, cf_key(v.p0, v.p1, __ldg(&p[2])));
         break;
     case GPUTX_T_OE_PAYMENT: {
         const int64_t w = __ldg(&p[0]), d = w * OE_DIST + __ldg(&p[1]), c = d * OE_CUST + __ldg(&p[2]);
