@@ -180,11 +180,19 @@ size_t carve_bulk(gputx_bulk *b, char *base, bool device_inputs)
         b->type = c.take<int32_t>(nn);
         b->params = c.take<int64_t>(nn * b->P);
     }
-    b->status = c.take<int32_t>(nn);
     b->out = c.take<int64_t>(nn * b->R);
-    b->ctl = c.take<BulkCtl>(1);
     Scratch &s = b->sc;
     s.m_cap = m;
+    // cleared together at submission: statuses, the control block, the first
+    // sort's and scans' counters and look-back words
+    b->status = c.take<int32_t>(nn);
+    b->ctl = c.take<BulkCtl>(1);
+    const int64_t big = std::max(mm, nn + 2);
+    s.sort_words = sort_scratch_words(big);
+    s.sort_zero = c.take<uint32_t>(s.sort_words);
+    s.scan_tiles = (big + 2047) / 2048;
+    s.scan_zero = c.take<uint64_t>(kScanAreas * (1 + s.scan_tiles));
+    s.cleared = c.base ? c.base + c.off : nullptr;
     s.keys_a = c.take<uint32_t>(mm);
     s.vals_a = c.take<uint32_t>(mm);
     s.keys_b = c.take<uint32_t>(mm);
@@ -219,11 +227,6 @@ size_t carve_bulk(gputx_bulk *b, char *base, bool device_inputs)
     s.slot_ord = slots ? c.take<uint32_t>(nn) : nullptr;
     s.slot_ol = slots ? c.take<uint32_t>(nn) : nullptr;
     s.slot_hist = db->hist_by_type ? c.take<uint32_t>(nn) : nullptr;
-    const int64_t big = std::max(mm, nn + 2);
-    s.sort_words = sort_scratch_words(big);
-    s.sort_zero = c.take<uint32_t>(s.sort_words);
-    s.scan_tiles = (big + 2047) / 2048;
-    s.scan_zero = c.take<uint64_t>(1 + s.scan_tiles);
     s.scan_vals = c.take<uint64_t>(2 * s.scan_tiles);
     s.seg_off = b->graph ? c.take<uint32_t>(kSegMax + 1) : nullptr;
     s.bulk_of = b->graph ? c.take<uint32_t>(nn) : nullptr;
@@ -242,11 +245,68 @@ gputx_status bulk_error(gputx_db *db, uint32_t err)
     return GPUTX_OK;
 }
 
+// Pinned homes for the control blocks of bulks in flight, so that reading one
+// back is a copy queued behind the bulk instead of a blocking one (20 us) after
+// it: one allocation of kPinnedCtls for the process, handed out under a lock.  A
+// bulk freed before its copy has landed leaves its event here, and the block is
+// handed out again once that has completed.  When all are taken, a bulk does
+// without.
+constexpr int kPinnedCtls = 256;
+
+struct PinnedCtls {
+    std::mutex mu;
+    bool tried = false;
+    std::vector<BulkCtl *> free;
+    std::vector<std::pair<BulkCtl *, cudaEvent_t>> busy;
+};
+PinnedCtls &pinned_ctls()
+{
+    static PinnedCtls *p = new PinnedCtls;   // lives as long as the process: bulks may be freed late
+    return *p;
+}
+
+BulkCtl *pinned_ctl_take()
+{
+    PinnedCtls &p = pinned_ctls();
+    std::lock_guard<std::mutex> lock(p.mu);
+    if (!p.tried) {
+        p.tried = true;
+        void *q = nullptr;
+        if (cudaHostAlloc(&q, kPinnedCtls * sizeof(BulkCtl), cudaHostAllocPortable) == cudaSuccess)
+            for (int i = 0; i < kPinnedCtls; i++) p.free.push_back((BulkCtl *)q + i);
+        else
+            cudaGetLastError();
+    }
+    for (size_t i = 0; p.free.empty() && i < p.busy.size(); i++)
+        if (cudaEventQuery(p.busy[i].second) == cudaSuccess) {
+            cudaEventDestroy(p.busy[i].second);
+            p.free.push_back(p.busy[i].first);
+            p.busy.erase(p.busy.begin() + (long)i);
+        }
+    if (p.free.empty()) return nullptr;
+    BulkCtl *c = p.free.back();
+    p.free.pop_back();
+    return c;
+}
+
+// `landed`: the event behind a copy that may still be on its way (it changes
+// hands), or null
+void pinned_ctl_give(BulkCtl *c, cudaEvent_t landed)
+{
+    if (!c) return;
+    PinnedCtls &p = pinned_ctls();
+    std::lock_guard<std::mutex> lock(p.mu);
+    if (landed) p.busy.push_back({c, landed});
+    else p.free.push_back(c);
+}
+
 gputx_status read_ctl(gputx_bulk *b)
 {
     gputx_db *db = b->db;
-    CK(cudaMemcpyAsync(&b->host_ctl, b->ctl, sizeof(BulkCtl), cudaMemcpyDeviceToHost, b->stream), "sync");
+    BulkCtl *to = b->pinned_ctl ? b->pinned_ctl : &b->host_ctl;
+    CK(cudaMemcpyAsync(to, b->ctl, sizeof(BulkCtl), cudaMemcpyDeviceToHost, b->stream), "sync");
     CK(cudaStreamSynchronize(b->stream), "sync");
+    if (b->pinned_ctl) b->host_ctl = *b->pinned_ctl;
     return GPUTX_OK;
 }
 
@@ -970,13 +1030,16 @@ gputx_status gputx_submit_bulk(gputx_db *db, const int64_t *ts, const int32_t *t
         if (!e) e = cudaMemcpyAsync(b->params, params, n * params_per_txn * sizeof(int64_t),
                                     cudaMemcpyHostToDevice, b->stream);
     }
-    if (!e) e = cudaMemsetAsync(b->ctl, 0, sizeof(BulkCtl), b->stream);
+    if (!e) e = cudaMemsetAsync(b->status, 0, (size_t)(b->sc.cleared - (char *)b->status), b->stream);
     if (!e && !dc_only(db)) e = clear_outputs(b);   // debit-credit only: by the executor
-    if (!e && n > 0) e = cudaMemsetAsync(b->status, 0, n * sizeof(int32_t), b->stream);
+    b->sort_clear = true;
+    b->scans = 0;
+    b->pinned_ctl = pinned_ctl_take();
     if (!e) e = cudaEventCreate(&b->ev[7]);
     if (e) {
         cudaFreeAsync(b->arena, b->stream);
         cudaEventDestroy(b->ev_in);
+        pinned_ctl_give(b->pinned_ctl, nullptr);
         delete b;
         return cuda_fail(db, e, "bulk upload");
     }
@@ -1031,18 +1094,24 @@ gputx_status run_grouping(gputx_bulk *b, int mode, int part_size, uint32_t *&sk,
 
 // The database-touching tail of a bulk starts after the previous bulk's tail
 // (bulks apply in gputx_execute order); the analysis before it overlaps.
-cudaError_t begin_tail(gputx_bulk *b, bool whole = false)
+// With `dc`, the kernels of the tail take the insert bases from the cursor
+// themselves (launch_dc_rows).
+cudaError_t begin_tail(gputx_bulk *b, bool dc = false)
 {
     cudaError_t e = cudaStreamWaitEvent(b->stream, b->db->last_done, 0);
-    if (e) return e;
-    return launch_begin(b, whole);
+    if (e || dc) return e;
+    return launch_begin(b);
 }
 
-cudaError_t end_tail(gputx_bulk *b)
+cudaError_t end_tail(gputx_bulk *b, bool dc = false)
 {
     gputx_db *db = b->db;
-    cudaError_t e = launch_finish(b);
+    cudaError_t e = dc ? cudaSuccess : launch_finish(b);
     if (!e) e = cudaEventRecord(db->last_done, b->stream);
+    if (!e && b->pinned_ctl) {
+        e = cudaMemcpyAsync(b->pinned_ctl, b->ctl, sizeof(BulkCtl), cudaMemcpyDeviceToHost, b->stream);
+        b->ctl_copied = !e;
+    }
     if (!e) e = cudaEventRecord(b->ev[7], b->stream);
     // callers that order work on the database stream see the bulk as done
     if (!e) e = cudaStreamWaitEvent(db->stream, db->last_done, 0);
@@ -1260,7 +1329,7 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
         if (b->timing) cudaEventRecord(b->ev[1], s);
         if ((st = read_ctl(b))) return st;
         if (b->host_ctl.err) {
-            CK(end_tail(b), "finish");
+            CK(end_tail(b, dc_only(db)), "finish");
             b->strategy_run = run;
             return GPUTX_OK;   // reported by the sync
         }
@@ -1307,7 +1376,8 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
         CK(launch_tpl_reset(b, sk, m), "tpl reset");
     }
     if (b->timing && run != GPUTX_TPL) cudaEventRecord(b->ev[4], s);
-    CK(end_tail(b), "finish");
+    const bool dc_tail = dc_only(db) && (paths || run == GPUTX_SCAN || run == GPUTX_PART || run == GPUTX_PART_RELAXED);
+    CK(end_tail(b, dc_tail), "finish");
     b->strategy_run = run;
     return GPUTX_OK;
 }
@@ -1318,7 +1388,8 @@ gputx_status gputx_sync_bulk(gputx_bulk *b, gputx_exec_stats *stats)
     gputx_db *db = b->db;
     if (!b->executed) return fail(db, GPUTX_ESTATE, "bulk not executed");
     CK(cudaEventSynchronize(b->ev[7]), "sync");
-    CK(cudaMemcpy(&b->host_ctl, b->ctl, sizeof(BulkCtl), cudaMemcpyDeviceToHost), "sync");
+    if (b->ctl_copied) b->host_ctl = *b->pinned_ctl;
+    else CK(cudaMemcpy(&b->host_ctl, b->ctl, sizeof(BulkCtl), cudaMemcpyDeviceToHost), "sync");
     b->synced = true;
     if (stats) {
         memset(stats, 0, sizeof *stats);
@@ -1386,6 +1457,12 @@ void gputx_free_bulk(gputx_bulk *b)
 {
     if (!b) return;
     if (b->arena) cudaFreeAsync(b->arena, b->stream);
+    if (b->ctl_copied && !b->synced) {   // the copy may still be on its way
+        pinned_ctl_give(b->pinned_ctl, b->ev[7]);
+        b->ev[7] = nullptr;
+    } else {
+        pinned_ctl_give(b->pinned_ctl, nullptr);
+    }
     for (int i = 0; i < 8; i++)
         if (b->ev[i]) cudaEventDestroy(b->ev[i]);
     if (b->ev_in) cudaEventDestroy(b->ev_in);

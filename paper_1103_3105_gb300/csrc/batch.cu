@@ -94,10 +94,8 @@ cudaError_t enqueue_pipeline(GraphBulk *g)
         const int64_t parts = (roots + g->part_size - 1) / g->part_size;   // the padding's id
         if ((e = gtx::launch_sort(b, pk, pv, pk2, pv2, b->n, gtx::bits_for((uint64_t)parts)))) return e;
         if (gtx::dc_only(db)) {
-            if ((e = gtx::launch_begin(b, true))) return e;
             if ((e = gtx::launch_dc_ranges(b, pk, pv, 0, false))) return e;
-            if ((e = gtx::launch_dc_rows(b))) return e;
-            return gtx::launch_finish(b);
+            return gtx::launch_dc_rows(b);
         }
         if ((e = gtx::launch_part_heads(b, pk, b->n))) return e;
         if ((e = gtx::launch_gather(b, pv))) return e;

@@ -17,6 +17,14 @@ struct DcOut {
     uint32_t t;
 };
 
+// whether n more history rows fit after the cursor; ERR_CAPACITY if not
+__device__ __forceinline__ bool rows_fit(const InsertBase *cursor, int64_t n, int64_t hist_cap, uint32_t *err)
+{
+    if (*(volatile const int64_t *)&cursor->hist + n <= hist_cap) return true;
+    set_err(err, ERR_CAPACITY);
+    return false;
+}
+
 // a debug build's check of the rows a debit-credit transaction touches and of
 // its index in the bulk (always true in a release build)
 __device__ __forceinline__ bool dbg_dc_rows(const DevDB &db, const DevBulk &b, int64_t a, int64_t tl, int64_t br,

@@ -27,9 +27,12 @@ struct BulkCtl {
     uint32_t hot;          // TPL: some counter has a chain of more than kTplHot operations
     uint32_t chunk;        // relaxed TPL: next chunk to claim (claim counts commit tickets)
     uint32_t front;        // exact depth: chunks of transactions finished
+    uint32_t rows_done;    // debit-credit rows: blocks finished
 };
 
 constexpr uint32_t kTplHot = 128;  // debit-credit TPL: a chain longer than this is served in lock order
+
+constexpr int kScanAreas = 3;      // scans of a submitted bulk whose scratch its submission has cleared
 
 constexpr int kSegMax = 64;        // bulks in one segment of a graph bulk, at most
 
@@ -55,8 +58,9 @@ struct Scratch {
     uint32_t *slot_cf, *slot_ord, *slot_ol;   // n each
     uint32_t *slot_hist;   // n: history rows of debit-credit transactions in mixed databases
     uint32_t *sort_zero;   // a sort's tile counters, digit counts and look-back words, cleared by it at once
-    uint64_t *scan_zero;   // a scan's tile counter and look-back words, likewise
+    uint64_t *scan_zero;   // kScanAreas times a scan's tile counter and look-back words, likewise
     uint64_t *scan_vals;   // 2 x tiles: per-tile values of 64-bit scans
+    char *cleared;         // end of what the submission clears (from `status`)
     // graph bulks that carry a segment of several bulks
     uint32_t *seg_off;     // kSegMax + 1: first transaction of each bulk
     uint32_t *bulk_of;     // n: bulk of each transaction
@@ -130,6 +134,10 @@ struct gputx_bulk {
     bool timing = false;
     cudaEvent_t ev[8] = {};
     gtx::BulkCtl host_ctl{};
+    gtx::BulkCtl *pinned_ctl = nullptr;     // where the control block is copied as the bulk ends (or null)
+    bool ctl_copied = false;                // that copy precedes ev[7]
+    bool sort_clear = false;                // the sort scratch is as its submission cleared it
+    int scans = gtx::kScanAreas;            // scans run so far, of those with a cleared area
     std::vector<uint32_t> level_off_host;   // K-SET level boundaries read back for launch planning
     std::vector<uint32_t> type_cut_host;    // and where the new-orders and payments start in each level
 };
@@ -168,8 +176,7 @@ cudaError_t launch_insert_slots(gputx_bulk *b);
 cudaError_t launch_part_heads(gputx_bulk *b, const uint32_t *skeys, int64_t n);
 cudaError_t launch_tpl_reset(gputx_bulk *b, const uint32_t *skeys, int64_t m);
 cudaError_t launch_gather(gputx_bulk *b, const uint32_t *order);
-// `whole`: the bulk's history rows all fit or the bulk fails (ERR_CAPACITY)
-cudaError_t launch_begin(gputx_bulk *b, bool whole = false);
+cudaError_t launch_begin(gputx_bulk *b);
 cudaError_t launch_finish(gputx_bulk *b);
 
 // exec.cu
@@ -195,8 +202,11 @@ cudaError_t launch_part_scatter(gputx_bulk *b, const uint32_t *off, const uint32
                                 uint32_t *pkeys, uint32_t *order);
 // debit-credit-only bulks: the account updates of transactions (vals >> vshift)
 // grouped by branch or partition (exec_dc.cu), or by account (segmented prefix
-// sums); then the history rows, statuses and teller and branch sums.  `stats`:
-// the groups are the graph's paths, d and w0 are recorded
+// sums); then the history rows, statuses and teller and branch sums.  These take
+// the place of the whole tail, launch_begin and launch_finish included: the
+// bulk's rows start at the database's cursor, which launch_dc_rows moves on, and
+// all fit or nothing runs (ERR_CAPACITY).  `stats`: the groups are the graph's
+// paths, d and w0 are recorded
 cudaError_t launch_dc_ranges(gputx_bulk *b, const uint32_t *keys, const uint32_t *vals, int vshift, bool stats);
 // (the deltas launch_group left in sc.rec_ts)
 cudaError_t launch_scan_exec(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m, bool stats);

@@ -34,6 +34,7 @@ struct RangeArgs {
     DevDB db;
     DevBulk b;
     BulkCtl *ctl;
+    const InsertBase *cursor;
     const uint32_t *keys, *vals;             // sorted by group; transaction = vals >> vshift
     int vshift;
     uint32_t slice;                          // positions per CTA before it follows its last group
@@ -73,7 +74,7 @@ __global__ void __launch_bounds__(kThreads, 4) dc_range_kernel(RangeArgs a)
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const DevBulk &b = a.b;
     const uint32_t n = b.n_live ? *b.n_live : (uint32_t)b.n;
-    if (tid == 0) s_stop = *(volatile uint32_t *)&a.ctl->err;
+    if (tid == 0) s_stop = *(volatile uint32_t *)&a.ctl->err || !rows_fit(a.cursor, n, a.db.hist_cap, &a.ctl->err);
     __syncthreads();
     uint32_t lo, hi;
     if (s_stop || !group_range<kThreads>(a.keys, n, a.slice, &s_min, lo, hi)) return;   // uniform
@@ -237,6 +238,7 @@ cudaError_t launch_dc_ranges(gputx_bulk *b, const uint32_t *keys, const uint32_t
     a.db = b->db->dev;
     a.b = make_dev_bulk(b, GPUTX_CONFLICT_PAPER);
     a.ctl = b->ctl;
+    a.cursor = b->db->d_cursor;
     a.keys = keys;
     a.vals = vals;
     a.vshift = vshift;
