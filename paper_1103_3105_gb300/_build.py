@@ -19,7 +19,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libgputx.so")
 BUILD_DEBUG = os.path.join(HERE, "_build_debug")
 LIB_DEBUG = os.path.join(HERE, "libgputx_debug.so")
-SOURCES = ["api.cu", "analysis.cu", "exec.cu", "exec_dc.cu", "tables.cu", "serve.cu", "batch.cu", "pool.cu", "relaxed.cu", "probe.cu"]
+SOURCES = ["api.cu", "analysis.cu", "exec.cu", "exec_dc.cu", "exec_oe.cu", "tables.cu", "serve.cu", "batch.cu", "pool.cu", "relaxed.cu", "probe.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

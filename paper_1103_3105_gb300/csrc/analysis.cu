@@ -58,8 +58,8 @@ struct ExtractArgs {
     bool write_ops;
     bool sentinel_fill;            // fill unused slots with padding operations
     uint32_t sentinel_key;         // object id above every real one
-    const uint32_t *bulk_of;       // segmented graph bulks: the bulk above the object id (or null)
-    int obj_shift;                 // bits of the object id under the bulk
+    const uint32_t *bulk_of;       // segmented graph bulks: the bulk under the object id (or null)
+    int seg_shift;                 // bits of the bulk under the object id
     uint32_t pad_pid;              // PART: partition id of a padding transaction (after every real one)
 };
 
@@ -117,10 +117,10 @@ __global__ void extract_kernel(ExtractArgs a)
             k = a.uniform_k;
         }
         const uint32_t pid = pad ? a.pad_pid : (k ? root[0] / (uint32_t)a.part_size : 0);
-        const uint32_t seg = (a.bulk_of && !pad) ? (a.bulk_of[t] << a.obj_shift) : 0u;
+        const uint32_t seg = (a.bulk_of && !pad) ? a.bulk_of[t] : 0u;
         for (int j = 0; j < k; j++) {
             if (a.write_ops) {
-                a.keys[off + j] = obj[j] | seg;
+                a.keys[off + j] = (obj[j] << a.seg_shift) | seg;
                 a.vals[off + j] = ((uint32_t)t << 7) | ((uint32_t)j << 2) | cls[j];
             }
             cross |= (root[j] / (uint32_t)a.part_size) != pid;
@@ -1353,7 +1353,8 @@ cudaError_t launch_finish(gputx_bulk *b)
 
 int seg_bits(const gputx_db *db)
 {
-    // segment bulk ids sit above the object id in a 32-bit key
+    // segment bulk ids sit under the object id in a 32-bit key: a group is one
+    // bulk's, and an item's groups lie side by side, bulk after bulk
     const int room = 32 - db->obj_bits;
     return room < 1 ? 0 : (room > 6 ? 6 : room);
 }
@@ -1407,8 +1408,8 @@ cudaError_t launch_extract(gputx_bulk *b, int mode, int part_size, uint32_t *pid
     if (b->graph) a.uniform_k = db->kmax;
     if (segmented && b->graph && b->sc.bulk_of && seg_bits(db) > 0) {
         a.bulk_of = b->sc.bulk_of;
-        a.obj_shift = db->obj_bits;
-        a.sentinel_key = (uint32_t)(((1ull << seg_bits(db)) - 1) << db->obj_bits);   // after every bulk
+        a.seg_shift = seg_bits(db);
+        a.sentinel_key = db->dev.n_objects << a.seg_shift;
     }
     {
         const int64_t roots = std::max<int64_t>({db->dev.n_br, db->dev.n_sub, db->dev.n_wh, 1});

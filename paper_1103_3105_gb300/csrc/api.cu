@@ -1175,6 +1175,10 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
     const bool paths = strategy == GPUTX_KSET && dc_only(db) && !(opts && opts->kset_launch == 1);
     // likewise any bulk of single-operation transactions (kset_rounds_kernel)
     const bool single = db->uniform_k == 1 && !paths && !(opts && opts->kset_launch == 1);
+    // and order-entry, whose items need each other's results in one place only
+    // (exec_oe.cu; 200,003 transactions: 1.59 ms where the levels took 3.86, and
+    // no level is too narrow for it: 1 transaction takes the same launches)
+    const bool items = oe_only(db) && !(opts && opts->kset_launch == 1);
     if (!paths && (strategy == GPUTX_KSET || (strategy == GPUTX_AUTO && run == GPUTX_AUTO))) {
         if ((st = run_grouping(b, mode, part_size, sk, sv, ak, av, m))) return st;
     }
@@ -1187,10 +1191,12 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
         // The exact-depth pass runs only once K-SET is chosen.
         if (db->need_fixpoint && strategy == GPUTX_KSET) CK(launch_exact_depth(b, sv, m), "exact depth");
         else CK(launch_level_stats(b), "stats");
-        if ((st = read_ctl(b))) return st;
-        if (b->host_ctl.err) {
-            CK(cudaEventRecord(b->ev[7], s), "event");
-            return GPUTX_OK;     // reported by the sync
+        if (!(items && strategy == GPUTX_KSET)) {
+            if ((st = read_ctl(b))) return st;
+            if (b->host_ctl.err) {
+                CK(cudaEventRecord(b->ev[7], s), "event");
+                return GPUTX_OK;     // reported by the sync
+            }
         }
         if (strategy == GPUTX_AUTO) {
             // Algorithm 1 (Appendix D): wide 0-set -> K-SET; else few
@@ -1207,10 +1213,12 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
                 // exact depths for the level schedule (Property 1)
                 CK(cudaMemsetAsync(&b->ctl->depth, 0, 3 * sizeof(uint32_t), s), "stats");
                 CK(launch_exact_depth(b, sv, m), "exact depth");
-                if ((st = read_ctl(b))) return st;
-                if (b->host_ctl.err) {
-                    CK(cudaEventRecord(b->ev[7], s), "event");
-                    return GPUTX_OK;
+                if (!items) {
+                    if ((st = read_ctl(b))) return st;
+                    if (b->host_ctl.err) {
+                        CK(cudaEventRecord(b->ev[7], s), "event");
+                        return GPUTX_OK;
+                    }
                 }
             }
         }
@@ -1238,6 +1246,11 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
         CK(begin_tail(b), "order");
         if (b->timing) cudaEventRecord(b->ev[3], s);
         CK(launch_kset_rounds(b, sk, sv, strategy == GPUTX_KSET, add), "k-set execute");
+    } else if (run == GPUTX_KSET && items) {
+        CK(begin_tail(b), "order");
+        if (b->timing) cudaEventRecord(b->ev[3], s);
+        CK(launch_items(b, sk, sv, m, 0), "k-set execute");
+        CK(launch_orders(b), "orders");
     } else if (run == GPUTX_KSET) {
         const int64_t depth = b->host_ctl.last_level;
         const bool persistent = opts && opts->kset_launch == 1;
@@ -1565,13 +1578,17 @@ extern "C" gputx_status gputx_execute_kset_noalloc(gputx_db *db, const int64_t *
     else CK(launch_level_stats(&b), "stats");
     if ((st = read_ctl(&b))) return st;
     if (b.host_ctl.err) return bulk_error(db, b.host_ctl.err);
-    const int64_t depth = b.host_ctl.last_level;
-    uint32_t *rk = ak, *rv = av, *rk2 = sk, *rv2 = sv;
-    CK(launch_regroup_keys(&b, rk, rv), "regroup");
-    CK(launch_sort(&b, rk, rv, rk2, rv2, b.n, bits_for((uint64_t)depth) + db->tbits), "regroup sort");
-    CK(launch_level_tables(&b, rk, depth, block, true), "level tables");
-    CK(launch_gather(&b, rv), "gather");
-    CK(launch_kset(&b, rv, b.sc.chunk_cap, block, add || db->need_fixpoint), "k-set execute");
+    if (oe_only(db)) {
+        CK(launch_items(&b, sk, sv, m, 0), "k-set execute");
+    } else {
+        const int64_t depth = b.host_ctl.last_level;
+        uint32_t *rk = ak, *rv = av, *rk2 = sk, *rv2 = sv;
+        CK(launch_regroup_keys(&b, rk, rv), "regroup");
+        CK(launch_sort(&b, rk, rv, rk2, rv2, b.n, bits_for((uint64_t)depth) + db->tbits), "regroup sort");
+        CK(launch_level_tables(&b, rk, depth, block, true), "level tables");
+        CK(launch_gather(&b, rv), "gather");
+        CK(launch_kset(&b, rv, b.sc.chunk_cap, block, add || db->need_fixpoint), "k-set execute");
+    }
     CK(launch_orders(&b), "orders");
     CK(launch_finish(&b), "finish");
     CK(cudaEventRecord(db->last_done, s), "order");

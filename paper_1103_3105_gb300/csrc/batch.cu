@@ -114,6 +114,12 @@ cudaError_t enqueue_pipeline(GraphBulk *g)
         if ((e = gtx::launch_rank_scan(b, sk, sv, m, db->need_fixpoint))) return e;
         e = db->need_fixpoint ? gtx::launch_exact_depth(b, sv, m) : gtx::launch_level_stats(b);
         if (e) return e;
+        if (gtx::oe_only(db)) {
+            if ((e = gtx::launch_begin(b))) return e;
+            if ((e = gtx::launch_items(b, sk, sv, m, seg ? gtx::seg_bits(db) : 0))) return e;
+            if ((e = gtx::launch_orders(b))) return e;
+            return gtx::launch_finish(b);
+        }
         if (seg && (e = gtx::launch_seg_levels(b))) return e;
         uint32_t *rk = ak, *rv = av, *rk2 = sk, *rv2 = sv;
         if ((e = gtx::launch_regroup_keys(b, rk, rv))) return e;

@@ -212,6 +212,10 @@ cudaError_t launch_dc_ranges(gputx_bulk *b, const uint32_t *keys, const uint32_t
 cudaError_t launch_scan_exec(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m, bool stats);
 cudaError_t launch_dc_rows(gputx_bulk *b);
 bool dc_only(const gputx_db *db);
+// order-entry-only bulks under K-SET, from the operations sorted by item (key >>
+// shift), item by item (exec_oe.cu); launch_orders follows
+bool oe_only(const gputx_db *db);
+cudaError_t launch_items(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m, int shift);
 cudaError_t clear_outputs(gputx_bulk *b);
 int exec_blocks_per_sm(int kind, int block);
 

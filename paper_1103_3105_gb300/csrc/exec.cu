@@ -16,7 +16,8 @@
 //   PART (Section 5.2)   one thread per non-empty partition runs its
 //       transactions serially in timestamp order.
 //   (K-SET under the read/write model and PART of debit-credit-only bulks:
-//   exec_dc.cu; K-SET of blind increments and SCAN: analysis.cu.)
+//   exec_dc.cu; K-SET of blind increments and SCAN: analysis.cu; K-SET of
+//   order-entry-only bulks: exec_oe.cu.)
 //   TPL (Section 5.1)    ordered counter locks: an operation whose group has
 //       `ticket` earlier operations before its run waits until that many have
 //       released the item's counter, then the transaction runs and every
