@@ -296,26 +296,29 @@ struct TicketMode {
 // between two blind increments of the read/write model (CLS_BW): K-SET applies
 // those by atomic additions, so they order nothing.  Order-entry's payments
 // then run beside each other although all of a warehouse's write its total.
-// A finished transaction publishes both in one 64-bit word, so a waiter needs
-// no fence and no second read; a run of several operations is read word by
-// word.
+// A finished transaction publishes both in one 64-bit word with its chunk's tag,
+// so a waiter needs no fence and no second read.
 //
-// What bounds the pass is the longest path, so its hops are made few and cheap.
-// A CTA holds 1,024 consecutive transactions and works in rounds.  In a round a
-// transaction looks at those of the chunk it still waits for, in shared memory,
-// and every kFlowOutside-th round at those of earlier chunks, in L2.  One that
-// waits for a single transaction p knows its depth as max(m, depth(p) + l); if p
-// does too, it takes over p's p (pointer jumping), so a chain through a chunk --
-// the payments of a warehouse -- is one step behind the chunk before in
-// logarithmically many rounds, and in one once that step is known.  (Lanes that
-// each poll by themselves, without rounds: 2,570 us where this takes 1,050;
-// rounds without the jumps: 1,180.)  CTAs far behind the front would only flood
-// L2 with polls: a CTA starts when all but kFlowAhead chunks before its own are
-// finished.  Chunks are claimed in timestamp order, so every transaction waited
-// for belongs to a running CTA: the chain of waits always ends.  Order-entry,
-// 200,003 transactions under R/W (d = 1,442): 1,050 us; one 64-bit word per
-// run, counted off by compare-and-swap by each of its operations, polls in L2
-// only: 2,950.
+// What bounds the pass is the longest path, so its hops are made short.  One
+// cluster runs it: a CTA holds 512 consecutive transactions, its neighbours the
+// chunks before and after, and a CTA's next chunk is the one kFlowCluster
+// further.  A finished transaction stores its word into the shared memory of
+// every CTA of the cluster, where the words of the last kFlowCluster chunks lie in
+// a ring, so waiting is polling one shared-memory word a lane and nothing goes
+// through L2 but what is older.  Warps run by themselves, without barriers: a
+// warp whose transactions are finished costs nothing.  Before that, while the
+// chunks before still run, a transaction that waits for one other, p, knows its
+// depth as max(m, depth(p) + l), and if p does too, it takes over p's p (pointer
+// jumping), so a chain through a chunk -- the payments of a warehouse -- is one
+// hop behind the chunk before.  A CTA waits for earlier transactions only, and
+// all CTAs of a cluster run at the same time: the chain of waits always ends.
+// Order-entry, 200,003 transactions under R/W (d = 1,442, 610 levels): 573 us, 0.9
+// a level; in rounds of a whole chunk with two CTA barriers each and polls in L2,
+// on every SM: 1,050; polls in L2 by each lane alone: 2,950.  A warp works off
+// what its lanes find one pass at a time, so a pass is kept short (lanes that each
+// go on as far as they can: 820) and a chunk small (1,024 transactions: 670, 256:
+// 695); words for the next 2 chunks only, the others' in L2: 813; a cluster of 16:
+// 588.
 
 // per operation: the last operation of the run before its own
 // (kPredNone: none).  Several transactions in that run: kPredRun | the sorted
@@ -346,10 +349,13 @@ __global__ void depth_prep_kernel(const uint32_t *sv, const uint32_t *rid, int64
     pred[slot] = p;
 }
 
-constexpr int kFlowThreads = 1024;
-constexpr uint32_t kFlowAhead = 8;          // unfinished chunks before one that starts
-constexpr uint32_t kFlowOutside = 1;        // rounds from one look at earlier chunks to the next
+constexpr int kFlowThreads = 512, kFlowCluster = 8;
+constexpr int kFlowPush = 7;                // the chunks after a chunk that get its words in shared memory
 constexpr unsigned long long kNotYet = ~0ull;
+
+// a word: tag << 57 | depth << 32 | level (a bulk has at most 2^25 transactions)
+constexpr uint32_t kFlowTags = 128, kFlowMask = (1u << 25) - 1u;
+__device__ __forceinline__ uint32_t flow_tag(uint32_t chunk) { return (chunk + 1) & (kFlowTags - 1); }
 
 __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long *p)
 {
@@ -361,7 +367,7 @@ __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long
 struct FlowArgs {
     const uint32_t *pred, *op_off, *sv, *rid;
     int kslots;
-    unsigned long long *depths;              // per transaction: depth << 32 | level, kNotYet before
+    unsigned long long *depths;              // per transaction: its word, kNotYet before
     uint32_t *level;
     BulkCtl *ctl;
     int64_t n;
@@ -378,164 +384,171 @@ struct FlowNode {
 
 __global__ void __launch_bounds__(kFlowThreads, 1) depth_flow_kernel(FlowArgs a)
 {
-    extern __shared__ __align__(16) uint32_t s_pred[];   // [MAX_OPS][kFlowThreads], then the nodes
+    // [MAX_OPS][kFlowThreads] predecessors, the nodes, the ring of words
+    extern __shared__ __align__(16) uint32_t s_pred[];
     FlowNode *s_node = reinterpret_cast<FlowNode *>(s_pred + MAX_OPS * kFlowThreads);
-    __shared__ uint32_t s_c, s_stop, s_moved, s_late;
-    __shared__ unsigned long long s_depth[kFlowThreads];
+    unsigned long long *s_ring = reinterpret_cast<unsigned long long *>(s_node + kFlowThreads);
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
     BulkCtl *ctl = a.ctl;
-    const uint32_t tid = threadIdx.x;
-    if (blockIdx.x == 0 && tid == 0) ctl->rounds = 1;
-    const int64_t n = a.graph ? (int64_t)ctl->n_live : a.n;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, rank = cl.block_rank();
+    const uint32_t ring = (uint32_t)__cvta_generic_to_shared(s_ring);
+    for (int k = 0; k <= kFlowPush; k++) s_ring[k * kFlowThreads + tid] = 0;
+    if (rank == 0 && tid == 0) ctl->rounds = 1;
+    const bool stop = *(volatile uint32_t *)&ctl->err != 0;   // an earlier launch's: the same in every CTA
+    const uint32_t n = (uint32_t)(a.graph ? (int64_t)ctl->n_live : a.n);
+    cl.sync();
+    if (stop) return;
     uint32_t dmax = 0, lmax = 0, zero = 0;
-    while (true) {
-        if (tid == 0) {
-            s_stop = *(volatile uint32_t *)&ctl->err ? 1u : 0u;
-            s_c = atomicAdd(&ctl->claim, 1u);
-            s_moved = 1;
-            s_late = 0;
-        }
-        s_depth[tid] = kNotYet;
-        s_node[tid].p = kPredNone;
-        __syncthreads();
-        const uint32_t c = s_c;
-        const int64_t start_ = (int64_t)c * kFlowThreads;
-        if (s_stop || start_ >= a.n) break;
-        const uint32_t start = (uint32_t)start_;
-        const int64_t t = start_ + tid;
-        // bit j: the run before operation j's is not known complete, and is a
-        // transaction of this chunk / one of an earlier chunk, or several
-        uint32_t inside = 0, outside = 0;
-        if (t < n) {
-            const int64_t s0 = a.op_off ? (int64_t)a.op_off[t] : t * a.kslots;
-            const int k = a.op_off ? (int)(a.op_off[t + 1] - a.op_off[t]) : a.kslots;
-#pragma unroll
-            for (int j = 0; j < MAX_OPS; j++) {
-                const uint32_t p = j < k ? __ldg(&a.pred[s0 + j]) : kPredNone;
-                if (p == kPredNone) continue;
-                s_pred[j * kFlowThreads + tid] = p;
-                if (!(p & kPredRun) && (p & kPredTxn) >= start) inside |= 1u << j;
-                else outside |= 1u << j;
-            }
-        }
-        if (tid == 0 && c > kFlowAhead) {                  // not yet near the front
-            uint32_t f = ld_relaxed_gpu(&ctl->front);
-            uint64_t t_prog = globaltimer();
-            while (c > f && c - f > kFlowAhead) {
-                if (globaltimer() - t_prog > a.limit_ns || *(volatile uint32_t *)&ctl->err) break;
-                __nanosleep(100);
-                const uint32_t g = ld_relaxed_gpu(&ctl->front);
-                if (g != f) t_prog = globaltimer();
-                f = g;
-            }
-        }
-        __syncthreads();
+    for (uint32_t c = rank; (uint64_t)c * kFlowThreads < n; c += kFlowCluster) {
+        const uint32_t start = c * kFlowThreads, t = start + tid;
         uint32_t dep = 0, lev = 0;
-        auto take = [&](uint32_t word, unsigned long long w) {
-            const uint32_t step = pred_step(word), d = (uint32_t)(w >> 32) + 1u, l = (uint32_t)w + step;
+        auto take = [&](uint32_t hi, uint32_t lo, uint32_t dl, uint32_t ll) {
+            const uint32_t d = (hi & kFlowMask) + dl, l = lo + ll;
             dep = d > dep ? d : dep;
-            if (step) lev = l > lev ? l : lev;
+            if (ll) lev = l > lev ? l : lev;
         };
-        bool done = t >= n;
-        FlowNode me{kPredNone, 0, 0, 0};
-        uint64_t t_prog = globaltimer();                   // thread 0's
-        for (uint32_t round = 0;; round++) {
-            // reads of what the round before left
-            bool moved = false;
-            const bool far = round % kFlowOutside == 0;
-            if (me.p != kPredNone) {
-                unsigned long long w = kNotYet;
-                if (me.p >= start) {
-                    w = s_depth[me.p - start];
-                    const FlowNode o = s_node[me.p - start];
-                    if (w == kNotYet && o.p != kPredNone) {           // jump over p
-                        const uint32_t dl = me.len >> 16, ll = me.len & 0xffffu;
-                        const uint32_t ol = o.len & 0xffffu;
-                        me.dep = o.dep + dl > me.dep ? o.dep + dl : me.dep;
-                        if (ll) me.lev = o.lev + ll > me.lev ? o.lev + ll : me.lev;
-                        me.len = ((dl + (o.len >> 16)) << 16) | (ll && ol ? ll + ol : 0u);
-                        me.p = o.p;
-                        moved = true;
-                    }
-                } else if (far) {
-                    w = ld_relaxed_u64(&a.depths[me.p]);
-                }
-                if (w != kNotYet) {
-                    const uint32_t d = (uint32_t)(w >> 32) + (me.len >> 16), l = (uint32_t)w + (me.len & 0xffffu);
-                    dep = d > me.dep ? d : me.dep;
-                    lev = (me.len & 0xffffu) && l > me.lev ? l : me.lev;
-                    inside = outside = 0;
-                    moved = true;
-                }
-            } else {
-                for (uint32_t b = inside; b; b &= b - 1) {
-                    const int j = __ffs(b) - 1;
-                    const uint32_t p = s_pred[j * kFlowThreads + tid];
-                    const unsigned long long w = s_depth[(p & kPredTxn) - start];
-                    if (w == kNotYet) continue;
-                    take(p, w);
-                    inside &= ~(1u << j);
-                    moved = true;
-                }
-                // up to four at a time, their loads in flight together
-                for (uint32_t b = far ? outside : 0u; b;) {
-                    uint32_t p[4], bit[4];
-                    unsigned long long w[4];
+        // where transaction x's word comes to in this CTA's ring, and its tag
+        auto near_word = [&](uint32_t x) { return c - x / kFlowThreads <= (uint32_t)kFlowPush; };
+        auto ring_word = [&](uint32_t x) {
+            return ring + 8u * ((c - x / kFlowThreads) * kFlowThreads + x % kFlowThreads);
+        };
+        // bit j: the run before operation j's is not known complete, and is one
+        // transaction, or several
+        uint32_t left = 0, runs = 0;
+        if (t < n) {
+            const int64_t s0 = a.op_off ? (int64_t)a.op_off[t] : (int64_t)t * a.kslots;
+            const int k = a.op_off ? (int)(a.op_off[t + 1] - a.op_off[t]) : a.kslots;
+            for (int j0 = 0; j0 < k; j0 += 6) {
+                uint32_t p[6];
+                unsigned long long w[6];
 #pragma unroll
-                    for (int u = 0; u < 4; u++) {
-                        bit[u] = b & (0u - b);
-                        b &= b - 1;
-                        p[u] = bit[u] ? s_pred[(__ffs(bit[u]) - 1) * kFlowThreads + tid] : kPredNone;
-                        w[u] = bit[u] && !(p[u] & kPredRun) ? ld_relaxed_u64(&a.depths[p[u] & kPredTxn]) : kNotYet;
-                    }
+                for (int u = 0; u < 6; u++) p[u] = j0 + u < k ? __ldg(&a.pred[s0 + j0 + u]) : kPredNone;
 #pragma unroll
-                    for (int u = 0; u < 4; u++) {
-                        if (!bit[u]) continue;
-                        if (p[u] & kPredRun) {             // a run of several operations: all of them
-                            const uint32_t q = p[u] & kPredVal, len = (__ldg(&a.rid[q]) & 0x7fffffffu) + 1u;
-                            uint32_t d = 0, l = 0, k = 0;
-                            for (; k < len; k++) {
-                                const uint32_t x = __ldg(&a.sv[q - k]) >> 7;
-                                const unsigned long long v = x >= start ? s_depth[x - start]
-                                                                        : ld_relaxed_u64(&a.depths[x]);
-                                if (v == kNotYet) break;
-                                d = (uint32_t)(v >> 32) > d ? (uint32_t)(v >> 32) : d;
-                                l = (uint32_t)v > l ? (uint32_t)v : l;
-                            }
-                            w[u] = k == len ? ((unsigned long long)d << 32) | l : kNotYet;
-                        }
-                        if (w[u] == kNotYet) continue;
-                        take(p[u], w[u]);
-                        outside &= ~bit[u];
-                        moved = true;
+                for (int u = 0; u < 6; u++)
+                    w[u] = p[u] == kPredNone || (p[u] & kPredRun) ? kNotYet : ld_relaxed_u64(&a.depths[p[u] & kPredTxn]);
+#pragma unroll
+                for (int u = 0; u < 6; u++) {
+                    if (p[u] == kPredNone) continue;
+                    if (w[u] != kNotYet) {
+                        take((uint32_t)(w[u] >> 32), (uint32_t)w[u], 1, pred_step(p[u]));
+                        continue;
                     }
-                }
-                const uint32_t left = inside | outside;
-                if (left && !(left & (left - 1))) {        // one left
-                    const uint32_t p = s_pred[(__ffs(left) - 1) * kFlowThreads + tid];
-                    if (!(p & kPredRun)) me = FlowNode{p & kPredTxn, 0x10000u | pred_step(p), dep, lev};
+                    s_pred[(j0 + u) * kFlowThreads + tid] = p[u];
+                    if (p[u] & kPredRun) runs |= 1u << (j0 + u);
+                    else left |= 1u << (j0 + u);
                 }
             }
-            if (s_late) inside = outside = 0;              // gave up, but publishes: no later waiter hangs
-            __syncthreads();
-            // writes for the next round
-            if (!done && !(inside | outside)) {
-                const unsigned long long w = ((unsigned long long)dep << 32) | lev;
-                s_depth[tid] = w;
-                asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(&a.depths[t]), "l"(w) : "memory");
-                me.p = kPredNone;
-                done = true;
-            } else if (me.p != kPredNone) {
+        }
+        FlowNode me{kPredNone, 0, 0, 0};
+        if (left && !runs && !(left & (left - 1))) {
+            const uint32_t p = s_pred[(__ffs(left) - 1) * kFlowThreads + tid];
+            me = FlowNode{p & kPredTxn, 0x10000u | pred_step(p), dep, lev};
+        }
+        s_node[tid] = me;
+        __syncthreads();
+        while (true) {
+            FlowNode o{kPredNone, 0, 0, 0};
+            if (me.p != kPredNone && me.p >= start) o = s_node[me.p - start];
+            const bool jump = o.p != kPredNone;
+            if (!__syncthreads_or(jump)) break;
+            if (jump) {
+                const uint32_t dl = me.len >> 16, ll = me.len & 0xffffu, ol = o.len & 0xffffu;
+                me.dep = o.dep + dl > me.dep ? o.dep + dl : me.dep;
+                if (ll) me.lev = o.lev + ll > me.lev ? o.lev + ll : me.lev;
+                me.len = ((dl + (o.len >> 16)) << 16) | (ll && ol ? ll + ol : 0u);
+                me.p = o.p;
                 s_node[tid] = me;
             }
-            if (moved) s_moved = 1;
-            if (!__syncthreads_or(!done)) break;
-            if (tid == 0 && round % 64 == 0) {
-                if (s_moved) {
-                    t_prog = globaltimer();
-                    s_moved = 0;
-                } else if (globaltimer() - t_prog > a.limit_ns) {
-                    set_err(&ctl->err, ERR_TIMEOUT);
-                    s_late = 1;
+            __syncthreads();
+        }
+        // what the lane waits for: x, dl and ll edges from it; then `more` earlier
+        // operations of a run, which ends at `end`
+        uint32_t x = start, dl = 1, ll = 1, more = 0, end = 0;
+        bool done = t >= n;
+        auto next = [&]() -> bool {            // false: nothing left
+            if (more | runs) {
+                if (more) {
+                    more--;
+                    end--;
+                } else {
+                    end = s_pred[(__ffs(runs) - 1) * kFlowThreads + tid] & kPredVal;
+                    runs &= runs - 1;
+                    more = __ldg(&a.rid[end]) & 0x7fffffffu;
+                }
+                x = __ldg(&a.sv[end]) >> 7;
+                return true;
+            }
+            if (!left) return false;
+            const uint32_t p = s_pred[(__ffs(left) - 1) * kFlowThreads + tid];
+            left &= left - 1;
+            x = p & kPredTxn;
+            ll = pred_step(p);
+            return true;
+        };
+        auto publish = [&]() {
+            const unsigned long long w = (unsigned long long)(flow_tag(c) << 25 | dep) << 32 | lev;
+            asm volatile("st.relaxed.cluster.shared::cta.u64 [%0], %1;" ::"r"(ring + 8u * tid), "l"(w) : "memory");
+#pragma unroll
+            for (uint32_t r = 1; r <= (uint32_t)kFlowPush; r++) {
+                uint32_t dst;
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                             : "=r"(dst)
+                             : "r"(ring + 8u * (r * kFlowThreads + tid)), "r"((rank + r) % kFlowCluster));
+                asm volatile("st.relaxed.cluster.shared::cluster.u64 [%0], %1;" ::"r"(dst), "l"(w) : "memory");
+            }
+            asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(&a.depths[t]), "l"(w) : "memory");
+            done = true;
+        };
+        if (me.p != kPredNone) {
+            left = 0;
+            x = me.p;
+            dl = me.len >> 16;
+            ll = me.len & 0xffffu;
+            dep = me.dep;
+            lev = me.lev;
+        } else if (!done && !next()) {
+            publish();
+        }
+        // one look a lane and pass; a lane that finds its word goes on to what it
+        // waits for next in the next pass, so the lanes stay together
+        uint64_t t_prog = 0;
+        uint32_t seen = 0;
+        bool near = near_word(x);
+        uint32_t at = near ? ring_word(x) : ring, want = flow_tag(x / kFlowThreads);
+        for (uint32_t spin = 1;; spin++) {
+            unsigned long long w;
+            asm volatile("ld.relaxed.cluster.shared::cta.u64 %0, [%1];" : "=l"(w) : "r"(at) : "memory");
+            uint32_t hi = (uint32_t)(w >> 32), lo = (uint32_t)w;
+            const uint32_t d = ((hi >> 25) - want) & (kFlowTags - 1);
+            bool hit = !done && near && d < kFlowTags / 2;
+            // older than the ring, or overwritten by a later chunk's (that CTA has finished its chunk)
+            const bool far = !done && (near ? hit && d : (spin & 7u) == 0);
+            if (far) {
+                w = ld_relaxed_u64(&a.depths[x]);
+                hi = (uint32_t)(w >> 32);
+                lo = (uint32_t)w;
+                hit = w != kNotYet;
+            }
+            if (__any_sync(kFull, hit)) {
+                if (hit) {
+                    take(hi, lo, dl, ll);
+                    if (!next()) publish();
+                    near = near_word(x);
+                    at = near ? ring_word(x) : ring;
+                    want = flow_tag(x / kFlowThreads);
+                }
+                continue;
+            }
+            if (__all_sync(kFull, done)) break;
+            if ((spin & 1023u) == 0) {         // no chunk finished for the limit: give up, but publish
+                const uint32_t f = ld_relaxed_gpu(&ctl->front);
+                const uint64_t now = globaltimer();
+                if (t_prog == 0 || f != seen) t_prog = now;
+                seen = f;
+                const bool late = now - t_prog > a.limit_ns || *(volatile uint32_t *)&ctl->err;
+                if (__any_sync(kFull, late)) {
+                    if (lane == 0) set_err(&ctl->err, ERR_TIMEOUT);
+                    if (!done) publish();
                 }
             }
         }
@@ -545,17 +558,18 @@ __global__ void __launch_bounds__(kFlowThreads, 1) depth_flow_kernel(FlowArgs a)
             lmax = lev > lmax ? lev : lmax;
             zero += dep == 0;
         }
+        __syncthreads();                       // nobody here waits for this chunk any more
         if (tid == 0) atomicAdd(&ctl->front, 1u);
-        __syncthreads();                                   // s_c, s_late are read until here
     }
-    dmax = __reduce_max_sync(0xffffffffu, dmax);
-    lmax = __reduce_max_sync(0xffffffffu, lmax);
-    zero = __reduce_add_sync(0xffffffffu, zero);
-    if ((tid & 31) == 0) {
+    dmax = __reduce_max_sync(kFull, dmax);
+    lmax = __reduce_max_sync(kFull, lmax);
+    zero = __reduce_add_sync(kFull, zero);
+    if (lane == 0) {
         if (dmax) atomicMax(&ctl->depth, dmax);
         if (lmax) atomicMax(&ctl->last_level, lmax);
         if (zero) atomicAdd(&ctl->w0, zero);
     }
+    cl.sync();                                 // stores into this CTA's ring may still be on their way
 }
 
 // d and w0 (Appendix D structural parameters)
@@ -1620,17 +1634,27 @@ cudaError_t launch_exact_depth(gputx_bulk *b, const uint32_t *sv, int64_t m)
     cudaError_t e;
     if (m > 0 && (e = cudaMemsetAsync(pred, 0xff, (size_t)m * sizeof(uint32_t), s))) return e;
     if ((e = cudaMemsetAsync(a.depths, 0xff, (size_t)b->n * sizeof(unsigned long long), s))) return e;
-    if ((e = cudaMemsetAsync(&b->ctl->claim, 0, sizeof(uint32_t), s))) return e;
     if ((e = cudaMemsetAsync(&b->ctl->front, 0, sizeof(uint32_t), s))) return e;
     if (m > 0) {
         depth_prep_kernel<<<grid_for(m), TB, 0, s>>>(sv, b->sc.rid, m, a.op_off, a.kslots, pred, b->ctl);
         count_launches(1);
     }
-    const int64_t chunks = (b->n + kFlowThreads - 1) / kFlowThreads;
-    const int64_t grid = std::min<int64_t>(b->db->num_sms, chunks);
-    const size_t smem = (sizeof(uint32_t) * MAX_OPS + sizeof(FlowNode)) * kFlowThreads;
+    const size_t smem = (sizeof(uint32_t) * MAX_OPS + sizeof(FlowNode) +
+                         sizeof(unsigned long long) * (kFlowPush + 1)) * kFlowThreads;
     if ((e = cudaFuncSetAttribute(depth_flow_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
-    depth_flow_kernel<<<(unsigned)grid, kFlowThreads, smem, s>>>(a);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kFlowCluster, 1, 1);
+    cfg.blockDim = dim3(kFlowThreads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kFlowCluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if ((e = cudaLaunchKernelEx(&cfg, depth_flow_kernel, a))) return e;
     count_launches(1);
     return cudaGetLastError();
 }

@@ -1,11 +1,12 @@
 """Order-entry under K-SET item by item: items whose operations end at, cross and
 fill a warp's 32 positions, stock rows that wrap in long runs, several bulks in
-one captured segment, and a bulk that overflows the order area.  Against the
-oracle, exactly, and against the executor that walks the levels (kset_launch =
-1)."""
+one captured segment, depths across the chunks of the depth pass, and a bulk that overflows
+the order area.  Against the oracle, exactly, and mixed with the executor that
+walks the levels (kset_launch = 1)."""
 import numpy as np
 import pytest
 
+import oracle
 import paper_1103_3105_gb300 as G
 import workloads as W
 from tests.test_gpu_schemas import check, oe_pair
@@ -39,6 +40,24 @@ def test_hot_items(n, n_wh, mix):
         ost, oout = o.execute(bulk, R=g.width)
         assert np.array_equal(st, ost) and np.array_equal(out, oout), (k, launch)
     check(g, o, st, out, ost, oout, oe=True)
+    g.close()
+
+
+@pytest.mark.parametrize("n,n_wh,mix", [(511, 1, "payments"), (512, 1, "all"), (513, 1, "mixed"), (4097, 2, "orders"),
+                                        (4609, 1, "payments"), (70_000, 3, "all")])
+def test_depths_across_chunks(n, n_wh, mix):
+    """Chunks of 512, a ring of eight, tags that repeat after 128 chunks."""
+    g, o = oe_pair(n_wh, 16, max_bulk=1 << 17)
+    bulk = hot_bulk(n, n_wh, 16, mix, 11 + n)
+    obj, cls, root = o.extract(bulk, G.CONFLICT_PAPER, oracle.MAX_OPS)
+    lv = oracle.levels(obj, cls, o.num_objects())
+    b = g.submit_dict(bulk).execute("kset")
+    stats = b.sync()
+    st, out = b.results()
+    b.free()
+    assert (stats["depth"], stats["w0"], stats["cross"]) == oracle.graph_stats(lv, root)
+    ost, oout = o.execute(bulk, R=g.width)
+    assert np.array_equal(st, ost) and np.array_equal(out, oout)
     g.close()
 
 
