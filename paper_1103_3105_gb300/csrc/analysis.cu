@@ -329,11 +329,14 @@ constexpr uint32_t kPredBlind = 1u << 31, kPredTxn = (1u << 25) - 1u;
 // levels from the predecessor to the transaction (0: it does not order the execution)
 __device__ __forceinline__ uint32_t pred_step(uint32_t p) { return !(p & kPredRun) && (p & kPredBlind) ? 0u : 1u; }
 
+// what stops the depth pass (the executor beside it may set the others)
+constexpr uint32_t kAnalysisErr = ~(uint32_t)(ERR_CAPACITY | ERR_BOUNDS);
+
 __global__ void depth_prep_kernel(const uint32_t *sv, const uint32_t *rid, int64_t m, const uint32_t *op_off,
                                   int kslots, uint32_t *pred, const BulkCtl *ctl)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= m || ctl->err) return;
+    if (i >= m || (ctl->err & kAnalysisErr)) return;
     const uint32_t v = sv[i];
     if (v == OP_SENTINEL) return;
     const uint32_t r = rid[i];
@@ -394,8 +397,11 @@ __global__ void __launch_bounds__(kFlowThreads, 1) depth_flow_kernel(FlowArgs a)
     const uint32_t ring = (uint32_t)__cvta_generic_to_shared(s_ring);
     for (int k = 0; k <= kFlowPush; k++) s_ring[k * kFlowThreads + tid] = 0;
     if (rank == 0 && tid == 0) ctl->rounds = 1;
-    const bool stop = *(volatile uint32_t *)&ctl->err != 0;   // an earlier launch's: the same in every CTA
+    __shared__ uint32_t s_stop;
+    if (tid == 0) s_stop = *(volatile uint32_t *)&ctl->err & kAnalysisErr;
     const uint32_t n = (uint32_t)(a.graph ? (int64_t)ctl->n_live : a.n);
+    cl.sync();
+    const bool stop = *cl.map_shared_rank(&s_stop, 0) != 0;    // the same in every CTA
     cl.sync();
     if (stop) return;
     uint32_t dmax = 0, lmax = 0, zero = 0;
@@ -545,7 +551,7 @@ __global__ void __launch_bounds__(kFlowThreads, 1) depth_flow_kernel(FlowArgs a)
                 const uint64_t now = globaltimer();
                 if (t_prog == 0 || f != seen) t_prog = now;
                 seen = f;
-                const bool late = now - t_prog > a.limit_ns || *(volatile uint32_t *)&ctl->err;
+                const bool late = now - t_prog > a.limit_ns || (*(volatile uint32_t *)&ctl->err & ERR_TIMEOUT);
                 if (__any_sync(kFull, late)) {
                     if (lane == 0) set_err(&ctl->err, ERR_TIMEOUT);
                     if (!done) publish();
@@ -1657,6 +1663,38 @@ cudaError_t launch_exact_depth(gputx_bulk *b, const uint32_t *sv, int64_t m)
     if ((e = cudaLaunchKernelEx(&cfg, depth_flow_kernel, a))) return e;
     count_launches(1);
     return cudaGetLastError();
+}
+
+cudaError_t launch_depths_aside(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m)
+{
+    gputx_db *db = b->db;
+    const cudaStream_t s = b->stream;
+    cudaStream_t side = nullptr;
+    for (int i = 0; i < gputx_db::kPool; i++)
+        if (db->pool[i] == s) side = db->side[i];
+    cudaError_t e = cudaSuccess;
+    if (side) {
+        e = cudaEventRecord(b->ev_in, s);
+        if (!e) e = cudaStreamWaitEvent(side, b->ev_in, 0);
+        if (e) return e;
+        b->stream = side;
+    }
+    e = launch_rank_scan(b, sk, sv, m, true);
+    if (!e) e = launch_exact_depth(b, sv, m);
+    b->stream = s;
+    if (side) {
+        const cudaError_t e2 = cudaEventRecord(b->ev_in, side);
+        b->aside = true;
+        if (!e) e = e2;
+    }
+    return e;
+}
+
+cudaError_t join_depths(gputx_bulk *b)
+{
+    if (!b->aside) return cudaSuccess;
+    b->aside = false;
+    return cudaStreamWaitEvent(b->stream, b->ev_in, 0);
 }
 
 cudaError_t launch_level_stats(gputx_bulk *b)

@@ -327,11 +327,12 @@ void gputx_destroy_db(gputx_db *db)
     if (!db) return;
     if (db->last_done) cudaStreamWaitEvent(db->stream, db->last_done, 0);
     cudaStreamSynchronize(db->stream);
-    for (cudaStream_t ps : db->pool)
-        if (ps) {
-            cudaStreamSynchronize(ps);
-            cudaStreamDestroy(ps);
-        }
+    for (auto *streams : {&db->side, &db->pool})
+        for (cudaStream_t ps : *streams)
+            if (ps) {
+                cudaStreamSynchronize(ps);
+                cudaStreamDestroy(ps);
+            }
     if (db->last_done) cudaEventDestroy(db->last_done);
     for (void *p : db->allocs) cudaFree(p);
     if (db->own_stream) cudaStreamDestroy(db->stream);
@@ -571,6 +572,9 @@ gputx_status gputx_register_types(gputx_db *db, const int32_t *type_ids, int n)
     // levels sorted by (level, type) know where the new-orders are; K-SET then
     // runs them on lane groups and completes orders after the levels
     db->group_oe = db->tbits > 0 && (db->dev.registered >> GPUTX_T_OE_NEW_ORDER & 1u);
+    if (oe_only(db))
+        for (cudaStream_t &ss : db->side)
+            if (!ss) CK(cudaStreamCreateWithFlags(&ss, cudaStreamNonBlocking), "stream");
     return GPUTX_OK;
 }
 
@@ -1108,6 +1112,7 @@ cudaError_t end_tail(gputx_bulk *b, bool dc = false)
     gputx_db *db = b->db;
     cudaError_t e = dc ? cudaSuccess : launch_finish(b);
     if (!e) e = cudaEventRecord(db->last_done, b->stream);
+    if (!e) e = join_depths(b);   // the next bulk's tail need not wait for them
     if (!e && b->pinned_ctl) {
         e = cudaMemcpyAsync(b->pinned_ctl, b->ctl, sizeof(BulkCtl), cudaMemcpyDeviceToHost, b->stream);
         b->ctl_copied = !e;
@@ -1182,8 +1187,20 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
     if (!paths && (strategy == GPUTX_KSET || (strategy == GPUTX_AUTO && run == GPUTX_AUTO))) {
         if ((st = run_grouping(b, mode, part_size, sk, sv, ak, av, m))) return st;
     }
-    if (!paths && !(single && strategy == GPUTX_KSET) &&
-        (strategy == GPUTX_KSET || (strategy == GPUTX_AUTO && run == GPUTX_AUTO))) {
+    // no early return leaves the side stream's work behind
+    struct Joined {
+        gputx_bulk *b;
+        ~Joined() { join_depths(b); }
+    } joined{b};
+    if (items && strategy == GPUTX_KSET && !b->timing) {
+        // the depths are only reported, so they are computed beside the
+        // execution (timing asks for one after the other): 200,003
+        // transactions 1,107 -> 996 us.  The batcher's graphs keep one stream:
+        // there the copies through the host are what a segment waits for
+        // (2,121 and 2,125 us for a stream of 130,001)
+        CK(launch_depths_aside(b, sk, sv, m), "depths");
+    } else if (!paths && !(single && strategy == GPUTX_KSET) &&
+               (strategy == GPUTX_KSET || (strategy == GPUTX_AUTO && run == GPUTX_AUTO))) {
         CK(launch_rank_scan(b, sk, sv, m, db->need_fixpoint), "rank");
         // AUTO decides on the one-pass ranks first: w0 and c are exact there
         // (a transaction is a source exactly when all its operations have

@@ -97,6 +97,9 @@ struct gputx_db {
     // database-touching tail of every bulk after that of its predecessor.
     static constexpr int kPool = 4;
     cudaStream_t pool[kPool] = {};
+    // order-entry: the depths of a bulk on a pool stream are computed on its
+    // side stream, beside the bulk's execution (created with the types)
+    cudaStream_t side[kPool] = {};
     int next_pool = 0;
     cudaEvent_t last_done = nullptr;
     // relaxed PART: per-partition counters and their prefix-scan scratch,
@@ -111,7 +114,8 @@ struct gputx_db {
 struct gputx_bulk {
     gputx_db *db = nullptr;
     cudaStream_t stream = nullptr;          // this bulk's stream (from the database's pool)
-    cudaEvent_t ev_in = nullptr;            // inputs ready on the database stream
+    cudaEvent_t ev_in = nullptr;            // inputs ready on the database stream; later the side stream's fork and join
+    bool aside = false;                     // work on the side stream that the bulk's stream has not waited for
     int64_t n = 0;
     int P = 0, R = 0;
     void *arena = nullptr;
@@ -216,6 +220,10 @@ bool dc_only(const gputx_db *db);
 // shift), item by item (exec_oe.cu); launch_orders follows
 bool oe_only(const gputx_db *db);
 cudaError_t launch_items(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m, int shift);
+// the rank scan and launch_exact_depth on the bulk's side stream; join_depths
+// makes the bulk's own stream wait for them (nothing to do if it has)
+cudaError_t launch_depths_aside(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m);
+cudaError_t join_depths(gputx_bulk *b);
 cudaError_t clear_outputs(gputx_bulk *b);
 int exec_blocks_per_sm(int kind, int block);
 
