@@ -97,7 +97,7 @@ __device__ __forceinline__ ItemOp item_op(const ItemArgs &a, uint64_t i)
 __device__ __forceinline__ void item_load(const ItemArgs &a, ItemOp &o, ItemKind kind)
 {
     const uint32_t t = o.v >> 7;
-    if (!dbg_in(t, a.b.n, a.b.err)) return;
+    if (kind == kItemNone || !dbg_in(t, a.b.n, a.b.err)) return;
     const int64_t *p = a.b.params + (int64_t)t * a.b.P;
     switch (kind) {
     case kItemHouse:
