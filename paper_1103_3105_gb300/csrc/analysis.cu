@@ -300,7 +300,7 @@ struct TicketMode {
 // so a waiter needs no fence and no second read.
 //
 // What bounds the pass is the longest path, so its hops are made short.  One
-// cluster runs it: a CTA holds 512 consecutive transactions, its neighbours the
+// cluster runs it: a CTA holds 1,024 consecutive transactions, its neighbours the
 // chunks before and after, and a CTA's next chunk is the one kFlowCluster
 // further.  A finished transaction stores its word into the shared memory of
 // every CTA of the cluster, where the words of the last kFlowCluster chunks lie in
@@ -312,13 +312,14 @@ struct TicketMode {
 // jumping), so a chain through a chunk -- the payments of a warehouse -- is one
 // hop behind the chunk before.  A CTA waits for earlier transactions only, and
 // all CTAs of a cluster run at the same time: the chain of waits always ends.
-// Order-entry, 200,003 transactions under R/W (d = 1,442, 610 levels): 573 us, 0.9
+// Order-entry, 200,003 transactions under R/W (d = 1,442, 610 levels): 500 us, 0.8
 // a level; in rounds of a whole chunk with two CTA barriers each and polls in L2,
 // on every SM: 1,050; polls in L2 by each lane alone: 2,950.  A warp works off
 // what its lanes find one pass at a time, so a pass is kept short (lanes that each
-// go on as far as they can: 820) and a chunk small (1,024 transactions: 670, 256:
-// 695); words for the next 2 chunks only, the others' in L2: 813; a cluster of 16:
-// 588.
+// went on as far as they could: 820) and what a lane waits for is in timestamp
+// order (in operation order: 670).  Chunks of 512: 535, of 256: 723; words for the
+// next 2 chunks only, the others' in L2: 888 (670 in the same order with 7); a
+// cluster of 16: no faster.
 
 // per operation: the last operation of the run before its own
 // (kPredNone: none).  Several transactions in that run: kPredRun | the sorted
@@ -352,7 +353,7 @@ __global__ void depth_prep_kernel(const uint32_t *sv, const uint32_t *rid, int64
     pred[slot] = p;
 }
 
-constexpr int kFlowThreads = 512, kFlowCluster = 8;
+constexpr int kFlowThreads = 1024, kFlowCluster = 8;
 constexpr int kFlowPush = 7;                // the chunks after a chunk that get its words in shared memory
 constexpr unsigned long long kNotYet = ~0ull;
 
@@ -418,8 +419,10 @@ __global__ void __launch_bounds__(kFlowThreads, 1) depth_flow_kernel(FlowArgs a)
         auto ring_word = [&](uint32_t x) {
             return ring + 8u * ((c - x / kFlowThreads) * kFlowThreads + x % kFlowThreads);
         };
-        // bit j: the run before operation j's is not known complete, and is one
-        // transaction, or several
+        // the runs before its operations that are not known complete: `left` of
+        // one transaction, in timestamp order (the last one's word is the last to
+        // come, and then no other look lies between it and this one's), from the
+        // column's start; `runs` of several, from its end
         uint32_t left = 0, runs = 0;
         if (t < n) {
             const int64_t s0 = a.op_off ? (int64_t)a.op_off[t] : (int64_t)t * a.kslots;
@@ -439,15 +442,23 @@ __global__ void __launch_bounds__(kFlowThreads, 1) depth_flow_kernel(FlowArgs a)
                         take((uint32_t)(w[u] >> 32), (uint32_t)w[u], 1, pred_step(p[u]));
                         continue;
                     }
-                    s_pred[(j0 + u) * kFlowThreads + tid] = p[u];
-                    if (p[u] & kPredRun) runs |= 1u << (j0 + u);
-                    else left |= 1u << (j0 + u);
+                    if (p[u] & kPredRun) {
+                        s_pred[(MAX_OPS - ++runs) * kFlowThreads + tid] = p[u];
+                        continue;
+                    }
+                    uint32_t i = left++;
+                    for (; i > 0; i--) {
+                        const uint32_t o = s_pred[(i - 1) * kFlowThreads + tid];
+                        if ((o & kPredTxn) <= (p[u] & kPredTxn)) break;
+                        s_pred[i * kFlowThreads + tid] = o;
+                    }
+                    s_pred[i * kFlowThreads + tid] = p[u];
                 }
             }
         }
         FlowNode me{kPredNone, 0, 0, 0};
-        if (left && !runs && !(left & (left - 1))) {
-            const uint32_t p = s_pred[(__ffs(left) - 1) * kFlowThreads + tid];
+        if (left == 1 && !runs) {
+            const uint32_t p = s_pred[tid];
             me = FlowNode{p & kPredTxn, 0x10000u | pred_step(p), dep, lev};
         }
         s_node[tid] = me;
@@ -469,7 +480,7 @@ __global__ void __launch_bounds__(kFlowThreads, 1) depth_flow_kernel(FlowArgs a)
         }
         // what the lane waits for: x, dl and ll edges from it; then `more` earlier
         // operations of a run, which ends at `end`
-        uint32_t x = start, dl = 1, ll = 1, more = 0, end = 0;
+        uint32_t x = start, dl = 1, ll = 1, more = 0, end = 0, at_left = tid;
         bool done = t >= n;
         auto next = [&]() -> bool {            // false: nothing left
             if (more | runs) {
@@ -477,16 +488,16 @@ __global__ void __launch_bounds__(kFlowThreads, 1) depth_flow_kernel(FlowArgs a)
                     more--;
                     end--;
                 } else {
-                    end = s_pred[(__ffs(runs) - 1) * kFlowThreads + tid] & kPredVal;
-                    runs &= runs - 1;
+                    end = s_pred[(MAX_OPS - runs--) * kFlowThreads + tid] & kPredVal;
                     more = __ldg(&a.rid[end]) & 0x7fffffffu;
                 }
                 x = __ldg(&a.sv[end]) >> 7;
                 return true;
             }
             if (!left) return false;
-            const uint32_t p = s_pred[(__ffs(left) - 1) * kFlowThreads + tid];
-            left &= left - 1;
+            const uint32_t p = s_pred[at_left];
+            at_left += kFlowThreads;
+            left--;
             x = p & kPredTxn;
             ll = pred_step(p);
             return true;

@@ -43,11 +43,11 @@ def test_hot_items(n, n_wh, mix):
     g.close()
 
 
-@pytest.mark.parametrize("n,n_wh,mix", [(511, 1, "payments"), (512, 1, "all"), (513, 1, "mixed"), (4097, 2, "orders"),
-                                        (4609, 1, "payments"), (70_000, 3, "all")])
+@pytest.mark.parametrize("n,n_wh,mix", [(511, 1, "payments"), (1024, 1, "all"), (1025, 1, "mixed"), (8193, 2, "orders"),
+                                        (9217, 1, "payments"), (140_000, 3, "all")])
 def test_depths_across_chunks(n, n_wh, mix):
-    """Chunks of 512, a ring of eight, tags that repeat after 128 chunks."""
-    g, o = oe_pair(n_wh, 16, max_bulk=1 << 17)
+    """Chunks of 1,024, a ring of eight, tags that repeat after 128 chunks."""
+    g, o = oe_pair(n_wh, 16, max_bulk=1 << 18)
     bulk = hot_bulk(n, n_wh, 16, mix, 11 + n)
     obj, cls, root = o.extract(bulk, G.CONFLICT_PAPER, oracle.MAX_OPS)
     lv = oracle.levels(obj, cls, o.num_objects())
