@@ -379,6 +379,10 @@ gputx_status gputx_create_db(const gputx_schema_desc *schema, const gputx_config
     cudaGetDevice(&dev);
     db->device = dev;
     cudaDeviceGetAttribute(&db->num_sms, cudaDevAttrMultiProcessorCount, dev);
+    int pageable = 0, host_tables = 0;
+    cudaDeviceGetAttribute(&pageable, cudaDevAttrPageableMemoryAccess, dev);
+    cudaDeviceGetAttribute(&host_tables, cudaDevAttrPageableMemoryAccessUsesHostPageTables, dev);
+    db->reads_host = pageable && host_tables;
     if (cuda_stream) {
         db->stream = (cudaStream_t)cuda_stream;
     } else {

@@ -25,6 +25,7 @@
 // tried when that segment had no cross-partition transaction, and a PART
 // segment that turns out to have one runs nothing and is re-run with TPL
 // (Section 5.2's fallback, decided on the device).
+#include <unistd.h>
 #include <algorithm>
 #include <chrono>
 #include <cstring>
@@ -273,11 +274,64 @@ gputx_status get_graph(gputx_batcher *bt, int64_t cap, int strategy, int block, 
     return GPUTX_OK;
 }
 
+// A segment's inputs straight from the caller's arrays (pageable host memory,
+// read over the chip-to-chip link), with the padding's types and what the control
+// block holds of the segment.  Where the GPU reads through the host's page tables
+// this takes the place of the host's copy into pinned staging, which bounded a
+// stream (one core: 700 us for 65,536 order-entry transactions, 10 MB, and 65 for
+// the device's six copies; the kernel: 54).  A stream of 130,001 in two segments,
+// host to host: 2,121 -> 1,223 us.
+struct FetchArgs {
+    const int64_t *ts, *params;
+    const int32_t *type;
+    int64_t *d_ts, *d_params;
+    int32_t *d_type;
+    int64_t n, cap, words;        // words: n x parameters
+    gtx::BulkCtl *ctl;
+    uint32_t *d_seg_off;
+    uint32_t n_seg, seg_off[gtx::kSegMax];
+};
+
+__global__ void __launch_bounds__(256) fetch_kernel(FetchArgs a)
+{
+    const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    constexpr int kAhead = 8;     // loads in flight a thread: a read of the host takes about 1 us
+    for (int64_t i = i0; i < a.words; i += kAhead * step) {
+        int64_t v[kAhead];
+#pragma unroll
+        for (int u = 0; u < kAhead; u++)
+            if (i + u * step < a.words) v[u] = a.params[i + u * step];
+#pragma unroll
+        for (int u = 0; u < kAhead; u++)
+            if (i + u * step < a.words) a.d_params[i + u * step] = v[u];
+    }
+    for (int64_t i = i0; i < a.cap; i += step) {
+        a.d_type[i] = i < a.n ? a.type[i] : -1;
+        if (i < a.n) a.d_ts[i] = a.ts[i];
+    }
+    if (i0 < a.n_seg) a.d_seg_off[i0] = a.seg_off[i0];
+    if (i0 == 0) {
+        a.ctl->n_live = (uint32_t)a.n;
+        a.ctl->n_seg = a.n_seg;
+    }
+}
+
+// reads a word of each page of [p, p + bytes): memory that is not there faults
+// here, in the caller's thread as the copy into staging would, and not on the GPU
+void touch_pages(const void *p, size_t bytes)
+{
+    static const size_t page = (size_t)sysconf(_SC_PAGESIZE);
+    const volatile char *c = (const volatile char *)p;
+    for (size_t i = 0; i < bytes; i += page) (void)c[i];
+    if (bytes) (void)c[bytes - 1];
+}
+
 // One segment of n <= cap transactions through a graph: n_seg bulks whose
 // first transactions (relative to the segment) are seg_off[0..n_seg-1].  The
-// host copies the inputs into the pinned staging `st`; the device copies them
-// in, replays the graph and copies the results and the control block back
-// into `st`, then records g->done.  Nothing here waits for the device.
+// device fetches the inputs (fetch_kernel), or the host copies them into the
+// pinned staging `st` and the device from there; it replays the graph and copies
+// the results and the control block back into `st`, then records g->done.  Nothing
+// here waits for the device; the inputs stay in place until g->done.
 gputx_status enqueue_segment(gputx_batcher *bt, GraphBulk *g, Staging &st, const int64_t *ts, const int32_t *type,
                              const int64_t *params, int64_t n, const uint32_t *seg_off, uint32_t n_seg)
 {
@@ -285,26 +339,54 @@ gputx_status enqueue_segment(gputx_batcher *bt, GraphBulk *g, Staging &st, const
     gputx_bulk *b = g->b;
     cudaStream_t s = b->stream;
     const int64_t cap = g->cap;
-    std::memcpy(st.ts, ts, sizeof(int64_t) * n);
-    std::memcpy(st.type, type, sizeof(int32_t) * n);
-    std::memcpy(st.params, params, sizeof(int64_t) * n * g->P);
-    st.ctl_words[0] = (uint32_t)n;
-    st.ctl_words[1] = n_seg;
-    std::memcpy(st.ctl_words + 2, seg_off, sizeof(uint32_t) * n_seg);
+    if (db->reads_host) {
+        touch_pages(ts, sizeof(int64_t) * n);
+        touch_pages(type, sizeof(int32_t) * n);
+        touch_pages(params, sizeof(int64_t) * n * g->P);
+    } else {
+        std::memcpy(st.ts, ts, sizeof(int64_t) * n);
+        std::memcpy(st.type, type, sizeof(int32_t) * n);
+        std::memcpy(st.params, params, sizeof(int64_t) * n * g->P);
+        st.ctl_words[0] = (uint32_t)n;
+        st.ctl_words[1] = n_seg;
+        std::memcpy(st.ctl_words + 2, seg_off, sizeof(uint32_t) * n_seg);
+    }
+    // the inputs come in while the segment before runs: only this graph's
+    // buffers are written, and its last replay is on the same stream
+    CKB(cudaMemsetAsync(b->ctl, 0, sizeof(gtx::BulkCtl), s), "reset");
+    if (db->reads_host) {
+        FetchArgs a;
+        a.ts = ts;
+        a.params = params;
+        a.type = type;
+        a.d_ts = b->ts;
+        a.d_params = b->params;
+        a.d_type = b->type;
+        a.n = n;
+        a.cap = cap;
+        a.words = n * g->P;
+        a.ctl = b->ctl;
+        a.d_seg_off = b->sc.seg_off;
+        a.n_seg = n_seg;
+        std::memcpy(a.seg_off, seg_off, sizeof(uint32_t) * n_seg);
+        fetch_kernel<<<(unsigned)std::min<int64_t>((cap + 255) / 256, (int64_t)db->num_sms * 8), 256, 0, s>>>(a);
+        gtx::count_launches(1);
+        CKB(cudaGetLastError(), "inputs");
+    } else {
+        CKB(cudaMemcpyAsync(&b->ctl->n_live, &st.ctl_words[0], sizeof(uint32_t), cudaMemcpyHostToDevice, s), "inputs");
+        CKB(cudaMemcpyAsync(&b->ctl->n_seg, &st.ctl_words[1], sizeof(uint32_t), cudaMemcpyHostToDevice, s), "inputs");
+        CKB(cudaMemcpyAsync(b->sc.seg_off, st.ctl_words + 2, sizeof(uint32_t) * n_seg, cudaMemcpyHostToDevice, s),
+            "inputs");
+        CKB(cudaMemcpyAsync(b->ts, st.ts, sizeof(int64_t) * n, cudaMemcpyHostToDevice, s), "inputs");
+        CKB(cudaMemcpyAsync(b->type, st.type, sizeof(int32_t) * n, cudaMemcpyHostToDevice, s), "inputs");
+        CKB(cudaMemcpyAsync(b->params, st.params, sizeof(int64_t) * n * g->P, cudaMemcpyHostToDevice, s), "inputs");
+        if (n < cap) CKB(cudaMemsetAsync(b->type + n, 0xff, sizeof(int32_t) * (cap - n), s), "inputs");
+    }
+    CKB(cudaMemsetAsync(b->out, 0, sizeof(int64_t) * cap * b->R, s), "inputs");
     // earlier work on the database stream (loads, other bulks) comes first
     CKB(cudaEventRecord(b->ev_in, db->stream), "order");
     CKB(cudaStreamWaitEvent(s, b->ev_in, 0), "order");
     CKB(cudaStreamWaitEvent(s, db->last_done, 0), "order");
-    CKB(cudaMemsetAsync(b->ctl, 0, sizeof(gtx::BulkCtl), s), "reset");
-    CKB(cudaMemcpyAsync(&b->ctl->n_live, &st.ctl_words[0], sizeof(uint32_t), cudaMemcpyHostToDevice, s), "inputs");
-    CKB(cudaMemcpyAsync(&b->ctl->n_seg, &st.ctl_words[1], sizeof(uint32_t), cudaMemcpyHostToDevice, s), "inputs");
-    CKB(cudaMemcpyAsync(b->sc.seg_off, st.ctl_words + 2, sizeof(uint32_t) * n_seg, cudaMemcpyHostToDevice, s),
-        "inputs");
-    CKB(cudaMemcpyAsync(b->ts, st.ts, sizeof(int64_t) * n, cudaMemcpyHostToDevice, s), "inputs");
-    CKB(cudaMemcpyAsync(b->type, st.type, sizeof(int32_t) * n, cudaMemcpyHostToDevice, s), "inputs");
-    CKB(cudaMemcpyAsync(b->params, st.params, sizeof(int64_t) * n * g->P, cudaMemcpyHostToDevice, s), "inputs");
-    if (n < cap) CKB(cudaMemsetAsync(b->type + n, 0xff, sizeof(int32_t) * (cap - n), s), "inputs");
-    CKB(cudaMemsetAsync(b->out, 0, sizeof(int64_t) * cap * b->R, s), "inputs");
     CKB(cudaEventRecord(g->e0, s), "event");
     CKB(cudaGraphLaunch(g->exec, s), "graph launch");
     CKB(cudaEventRecord(g->e1, s), "event");
@@ -536,8 +618,10 @@ gputx_status gputx_batcher_run_bulks(gputx_batcher *bt, const int64_t *ts, const
         if ((st = get_graph(bt, size, strategy, block, sync ? 0 : buf, &g))) break;
         if ((st = ensure_staging(bt, bt->stage[buf], size))) break;
         if ((st = enqueue_segment(bt, g, bt->stage[buf], ts + first_txn, type + first_txn, params + first_txn * P, k,
-                                  seg_off.data(), (uint32_t)seg_off.size())))
+                                  seg_off.data(), (uint32_t)seg_off.size()))) {
+            cudaStreamSynchronize(g->b->stream);   // nothing reads the caller's arrays after the call
             break;
+        }
         InFlight cur;
         cur.valid = true;
         cur.first = first;

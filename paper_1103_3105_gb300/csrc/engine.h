@@ -80,6 +80,7 @@ struct gputx_db {
     bool own_stream = false;
     int device = 0;
     int num_sms = 0;
+    bool reads_host = false;               // kernels can read any host memory through the host's page tables
     std::string last_error;
     std::vector<void *> allocs;
     gtx::InsertBase *d_cursor = nullptr;   // device insert cursors
