@@ -47,19 +47,20 @@ METRIC = "txns/sec on 1 GB300 per strategy & bulk size vs plain path; p50/p99 la
 EXEC_BYTES_PER_TXN = 32 + 64 + 0 + 40 + 12
 L2_FLUSH_BYTES = 256 << 20
 # the executor kernel that dominates each headline configuration
-DOMINANT_KERNEL = {("kset", "paper"): "kset_narrow_dc_kernel", ("kset", "add"): "kset_level_kernel",
-                   ("part_relaxed", "paper"): "part_dc_kernel", ("tpl_relaxed", "paper"): "tpl_relaxed_kernel",
-                   ("tpl_relaxed", "add"): "tpl_relaxed_kernel",
-                   ("part", "paper"): "part_dc_kernel", ("part", "add"): "part_dc_kernel",
+DOMINANT_KERNEL = {("kset", "paper"): "dc_range_kernel", ("kset", "add"): "acct_scan_kernel",
+                   ("part_relaxed", "paper"): "dc_range_kernel", ("part_relaxed", "add"): "dc_range_kernel",
+                   ("tpl_relaxed", "paper"): "tpl_relaxed_kernel", ("tpl_relaxed", "add"): "tpl_relaxed_kernel",
+                   ("part", "paper"): "dc_range_kernel", ("part", "add"): "dc_range_kernel",
                    ("tpl", "paper"): "tpl_dc_kernel", ("tpl", "add"): "tpl_dc_kernel",
-                   ("scan", "paper"): "seg64_scan_kernel", ("scan", "add"): "seg64_scan_kernel"}
-# DRAM bytes (read + write) of the dominant kernel's launches for one bulk
-# (the narrow runner's segments: the main run and the narrow tail) from one
-# ncu capture at this configuration, keyed by (strategy, mode, bulk log2);
-# each entry holds the digest of the kernel and launch-planner sources it was
-# taken on, and is reported as null once those sources change
-TRAFFIC = {("kset", "paper", 22): {"bytes": 341127168 + 361984 + 290942208, "digest": "3472c3d645ba694a"}}
-KERNEL_SOURCES = ("common.cuh", "fastdiv.h", "engine.h", "dc.cuh", "levels.cuh", "exec_dc.cu", "exec.cu")
+                   ("scan", "paper"): "acct_scan_kernel", ("scan", "add"): "acct_scan_kernel"}
+# DRAM bytes (read + write) of the executor's launches for one bulk (account
+# updates, then history rows and sums) from one ncu capture at this
+# configuration, keyed by (strategy, mode, bulk log2); each entry holds the
+# digest of the executor's sources it was taken on, and is reported as null once
+# those sources change
+TRAFFIC = {("kset", "paper", 22): {"bytes": 325240000 + 98550000 + 100770000 + 124180000,
+                                   "digest": "ebc7f2f22626cc9f"}}
+KERNEL_SOURCES = ("common.cuh", "fastdiv.h", "engine.h", "dc.cuh", "ranges.cuh", "exec_dc.cu", "analysis.cu")
 
 
 def kernel_digest():
@@ -331,33 +332,6 @@ def run_engine(args, rank, world, local_rank):
         return
     peak, peak_kind = measured_peak_hbm()
     ex = statistics.median(exec_ms)
-    # the latency roofline of the level chain: the bare skeleton of a level
-    # (updates of cells another SM updated at the previous level, stores,
-    # cluster barrier) in the narrow runner's launch shape, with the
-    # executor's traffic and with the minimum
-    latency = None
-    if args.strategy == "kset" and stats and stats["depth"] > 0:
-        levels = stats["depth"] + 1
-        def probe(*shape, **kw):   # a floor: the best of three launches
-            return min(G.gputx_probe_level_chain(levels, 16, 64, *shape, **kw) for _ in range(3))
-        # the runner's own shape: the account's fetch-and-add before the
-        # barrier's release; after it, 9 fire-and-forget writes (teller and
-        # branch additions, history row, outputs), stores in the probe
-        floor_dc = probe(0, 1, 9, rmw=1)
-        floor_min = probe(0, 1, 0, rmw=1)
-        # the same with the fetch-and-add on random cells of a table the size
-        # of the 10M accounts, prefetched two levels ahead like the runner's
-        floor_rand = probe(0, 1, 9, rmw=2)
-        # the same level applying its updates as loads then stores
-        floor_ld_st = probe(3, 3, 7)
-        measured = ex * 1e6 / levels
-        latency = {"levels": levels, "measured_ns_per_level": measured,
-                   "floor_ns_per_level": floor_dc, "floor_ns_per_level_min": floor_min,
-                   "floor_ns_per_level_load_store": floor_ld_st, "frac": floor_dc / measured,
-                   "floor_ns_per_level_random_cells": floor_rand, "frac_random_cells": floor_rand / measured,
-                   "probe": "cluster 16 x 64 threads; per thread and level 1 fetch-and-add on a cell another "
-                            "CTA updated at the previous level, barrier arrive (release), 9 stores, "
-                            "barrier wait (acquire); best of 3 launches"}
     # L2 atomic throughput (random cells of a 10M-cell table, the 10,000
     # tellers, the 1,000 branches), beside the atomics the executor issues
     atomics = None
@@ -365,13 +339,13 @@ def run_engine(args, rank, world, local_rank):
         atomics = {f"{kind}_{name}_gops": G.gputx_probe_atomics(cells, fetch)
                    for name, cells in (("accounts", ACCOUNTS), ("tellers", TELLERS), ("branches", BRANCHES))
                    for kind, fetch in (("red", 0), ("fetch_add", 1))}
-        # K-SET R/W: fetch-and-add + 2 reductions (narrow runner); K-SET ADD:
-        # teller and branch reductions; TPL: one counter release per lock
-        # (the branch, or the account under ADD) + the 2 reductions under ADD
-        per_txn = {("kset", "paper"): 3, ("kset", "add"): 2, ("tpl", "paper"): 1,
-                   ("tpl", "add"): 3}[(args.strategy, args.mode)]
-        atomics["executor_gops"] = n * per_txn / (ex / 1e3) / 1e9
-        atomics["executor_atomics_per_txn"] = per_txn
+        # TPL: one counter release per lock (the branch, or the account under
+        # ADD) + the 2 reductions under ADD; K-SET's executors hold each item's
+        # updates in one CTA and issue next to none
+        if args.strategy == "tpl":
+            per_txn = {"paper": 1, "add": 3}[args.mode]
+            atomics["executor_gops"] = n * per_txn / (ex / 1e3) / 1e9
+            atomics["executor_atomics_per_txn"] = per_txn
     achieved = n * EXEC_BYTES_PER_TXN / (ex / 1e3) / 1e9
     l2_bytes = int(getattr(torch.cuda.get_device_properties(dev), "L2_cache_size", 0))
     clocks = clk.summary()
@@ -403,20 +377,13 @@ def run_engine(args, rank, world, local_rank):
                      "bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,
                      "peak_source": peak_kind, "bytes_per_txn": EXEC_BYTES_PER_TXN,
-                     "txn_per_launch_set": n, "kernel_ms": ex,
-                     # the level chain, not bandwidth, bounds K-SET on a deep graph
-                     "levels": levels, "ns_per_level": ex * 1e6 / levels if levels else None},
+                     "txn_per_launch_set": n, "kernel_ms": ex, "levels": levels},
         "clocks": {k: clocks[k] for k in ("sm_mhz", "sm_max_mhz", "reasons", "samples")},
     }
-    if latency is not None:
-        line["latency_roofline"] = {k: latency[k] for k in ("levels", "measured_ns_per_level",
-                                                             "floor_ns_per_level", "frac",
-                                                             "floor_ns_per_level_random_cells",
-                                                             "frac_random_cells")}
     if args.cpu_baseline:
         line["cpu_baseline"] = cpu_baseline(args, bulks)
     # everything else goes to the detail file; stdout ends with the compact headline
-    detail = {"headline": line, "latency_roofline": latency, "atomics": atomics,
+    detail = {"headline": line, "atomics": atomics,
               "phases_ms": {"execute": ex, "op_sort": statistics.median(sort_ms),
                             "analysis": stats["ms_analysis"] if stats else None},
               "graph": {"depth": stats["depth"], "w0": stats["w0"], "cross": stats["cross"]} if stats else None,

@@ -49,8 +49,17 @@ typedef enum {
 } gputx_status;
 
 typedef enum {
-    GPUTX_KSET = 0,       /* Section 5.3: k-sets level by level */
-    GPUTX_PART = 1,       /* Section 5.2: one thread per partition */
+    GPUTX_KSET = 0,       /* Section 5.3: an item's k-th run of operations
+                           * after its earlier ones.  Where a transaction
+                           * waits for one item's earlier runs only (every
+                           * registered type is debit-credit, or has one
+                           * operation, or is order-entry) the items run side
+                           * by side, else the k-sets level by level.  A
+                           * debit-credit-only bulk whose history rows do not
+                           * all fit fails with ECAPACITY and writes nothing,
+                           * under PART and PART_RELAXED as well; history rows
+                           * are in timestamp order. */
+    GPUTX_PART = 1,       /* Section 5.2: a partition's transactions serially */
     GPUTX_TPL = 2,        /* Section 5.1: ordered counter locks */
     GPUTX_AUTO = 3,       /* Algorithm 1 over the measured d, w0, c.  The
                            * decision reads the one-pass ranks of Section 4.2
@@ -180,12 +189,15 @@ typedef struct {
     int32_t block_threads;    /* 0 = database default */
     int32_t part_size;        /* 0 = database default */
     int32_t timing;           /* 1 = record per-phase CUDA events in stats */
-    int32_t kset_launch;      /* K-SET launch shape: 0 = per-level plan (wide
-                                 levels on the whole grid, runs of narrow levels
-                                 on one thread-block cluster), 1 = one persistent
-                                 launch with per-level counters (no host sync
-                                 after the analysis) */
-    int32_t narrow_max;       /* widest level run on one cluster; 0 = 16384 */
+    int32_t kset_launch;      /* K-SET launch shape: 0 = items side by side
+                                 where that can be done (gputx_strategy), else a
+                                 per-level plan (wide levels on the whole grid,
+                                 runs of narrow levels on one thread-block
+                                 cluster), 1 = levels, in one persistent launch
+                                 with per-level counters (no host sync after the
+                                 analysis) */
+    int32_t narrow_max;       /* per-level plan: widest level (in lanes) run on
+                                 one cluster; 0 = 8192 */
 } gputx_exec_opts;
 
 typedef struct gputx_db gputx_db;
@@ -327,8 +339,8 @@ unsigned long long gputx_launch_count(void);
  *
  * ts[n], type[n], params[n x params_per_txn] are DEVICE arrays; status[n]
  * (int32) and values[n x gputx_output_width(db)] (int64) are DEVICE arrays
- * the caller owns and the call fills.  The bulk runs with K-SET (one
- * persistent launch per level run) under conflict_mode on the database's
+ * the caller owns and the call fills.  The bulk runs with K-SET (order-entry
+ * item by item, else one persistent launch) under conflict_mode on the database's
  * stream, and the call returns after it finished.  Results and the database
  * are the same as gputx_submit_bulk + gputx_execute(GPUTX_KSET) +
  * gputx_read_results would produce.
@@ -338,7 +350,7 @@ unsigned long long gputx_launch_count(void);
  * until the process exits; the call allocates nothing (no cudaMalloc,
  * cudaFree or allocating library routine).  A bulk whose working set does
  * not fit returns EINVAL before any work is enqueued (for debit-credit
- * about 300,000 transactions fit; multi-item order-entry bulks fewer).
+ * more than 300,000 transactions fit; multi-item order-entry bulks fewer).
  * The first call on a device looks up the array's device address with that
  * device current; make that first call before any stream capture.  Every
  * call shares the one array and each clears what must start at zero, so
@@ -358,8 +370,8 @@ gputx_status gputx_execute_kset_noalloc(gputx_db *db, const int64_t *ts, const i
 /* A stream of transactions (uneven sizes, mixed types) runs as consecutive
  * bulks of one size.  For each (bulk size, strategy, block shape) a
  * fixed-capacity bulk's whole pipeline -- extraction, grouping sort, ranks,
- * the exact-depth pass on the device, regrouping and one persistent K-SET launch
- * (or the TPL kernel) -- is captured once in a CUDA graph and replayed for
+ * the exact-depth pass on the device, then order-entry's items side by side or
+ * regrouping and one persistent K-SET launch (or the TPL kernel) -- is captured once in a CUDA graph and replayed for
  * every bulk of that shape, shorter bulks padded with inactive transactions.
  * With tune = 1 the stream's own first bulks run under different
  * configurations, seeded by Algorithm 1 (Appendix D) on the first bulk's
@@ -405,8 +417,9 @@ gputx_status gputx_batcher_create(gputx_db *db, const gputx_batch_config *cfg, g
  * a bulk above the capacity is cut into pieces, each its own bulk.  Under
  * K-SET each bulk (piece) keeps its own dependency graph and k-sets
  * (Definition 1 per bulk, bulks in order); TPL and PART run a segment in
- * timestamp order.  EINVAL on bad offsets; device errors as for
- * gputx_sync_bulk. */
+ * timestamp order.  The arrays are read until the call returns, by the GPU itself
+ * where it reads through the host's page tables.  EINVAL on bad offsets; device
+ * errors as for gputx_sync_bulk. */
 gputx_status gputx_batcher_run_bulks(gputx_batcher *bt, const int64_t *ts, const int32_t *type,
                                      const int64_t *params, const int64_t *bulk_off, size_t n_bulks,
                                      int32_t *status, int64_t *values);
@@ -524,7 +537,7 @@ gputx_status gputx_probe_level_chain(int levels, int cluster_size, int threads, 
 
 /* Throughput of 64-bit atomic additions performed at L2, the operation TPL's
  * counters, the ADD class's blind increments (Section 5.1's workload under
- * the blind-increment refinement) and the debit-credit level runners rely on.
+ * the blind-increment refinement) and the ordered locks rely on.
  * A grid of (SMs x 8) CTAs of 256 threads each adds 1 to 64 cells drawn
  * uniformly from a table of n_cells (1 .. 2^32) 8-byte cells: reductions
  * (fetch = 0) or fetch-and-adds whose results are used (fetch = 1).  The

@@ -243,8 +243,9 @@ __device__ __forceinline__ LaneRecord lane_record(const DevBulk &b, const LevelL
 // records come into L1 three and into registers two levels ahead, its rows into
 // L2 and its insert slots into registers one level ahead; order rows, lines,
 // index entries and the order-statuses' sums are left to launch_orders, and the
-// payments' totals follow the barrier's arrival.  Order-entry, 200,003
-// transactions, 317 a level: 3.5 us a level; 7.3 when the records were
+// payments' totals follow the barrier's arrival.  200,003 order-entry
+// transactions (which run item by item unless other schemas' share the database),
+// 317 a level: 3.5 us a level; 7.3 when the records were
 // loaded during the level before and the procedures ran whole (of it 3.0
 // without any procedure, 1.2 the index entry's compare-and-swap).
 template <bool CLUSTER, int MAXT>
