@@ -5,8 +5,8 @@ Workload (debit-credit at scale): 1,000 branches, 10,000 tellers, 10,000,000
 accounts with int64 balances; bulks of 2^22 transactions (account uniform or
 Zipf(theta) then scrambled, delta uniform in [-99999, 99999]).  One step = one
 bulk through the whole path: bulk hand-over, basic-operation extraction,
-grouping sort, ranks and depths, (level, type) regrouping, execution, results
-left on the device.  The headline is the plain per-bulk K-SET path with the
+grouping sort, execution in dependency order with the graph's d and w0 recorded,
+results left on the device.  The headline is the plain per-bulk K-SET path with the
 paper's read/write conflict model; a bounded sweep reports every strategy,
 conflict model, skew and bulk size beside it.
 
