@@ -6,14 +6,16 @@
 // most the segment capacity; a bulk larger than that is cut into pieces)
 // that goes through ONE replay of a captured CUDA graph.  The graph holds
 // the whole pipeline for a fixed capacity -- extraction, grouping sort,
-// ranks, the device-side exact-depth pass, (level, type) regrouping and one
-// persistent executor launch -- and reads the segment's bulk boundaries from
-// a device descriptor array, so no host synchronisation happens inside it.
+// ranks, the device-side exact-depth pass, then order-entry's items or (level,
+// type) regrouping and one persistent executor launch -- and reads the segment's
+// bulk boundaries from a device descriptor array, so no host synchronisation
+// happens inside it.
 // For K-SET every bulk keeps its own dependency graph: the bulk's index sits
-// above the object id in the grouping key, each bulk's levels are numbered
-// after those of the bulks before it, and the persistent executor walks the
-// levels of the whole segment in that order with per-level counters (bulk
-// by bulk, level by level).  TPL and PART need no boundary: their order is
+// under the object id in the grouping key, so an item's operations of all bulks
+// lie in order side by side.  Item by item they are one chain; by levels, each
+// bulk's levels are numbered after those of the bulks before it, and the
+// persistent executor walks the levels of the whole segment in that order with
+// per-level counters (bulk by bulk, level by level).  TPL and PART need no boundary: their order is
 // the timestamp order, which runs across bulks.  Shorter segments are padded
 // with inactive transactions.
 //
