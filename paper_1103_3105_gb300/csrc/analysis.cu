@@ -242,10 +242,9 @@ struct RankMode {
 };
 
 // TPL tickets: number of operations of the group before this operation's run
-// (Section 5.1 key values, read with ticket semantics).  A ticket of at least
-// `hot_ticket` raises `hot`: some counter carries a chain that long, which
-// picks the order the debit-credit executor hands transactions out in (the flag
-// is written once, by the first such ticket seen).
+// (Section 5.1 key values, read with ticket semantics).  `hot` becomes the
+// largest last ticket of a group if that is at least `hot_ticket`: the longest
+// chain, which picks how the debit-credit executor hands transactions out.
 struct TicketMode {
     const uint32_t *sk, *sv;
     uint32_t *lock_key, *lock_ticket;
@@ -255,6 +254,7 @@ struct TicketMode {
     uint32_t hot_ticket;
     uint32_t n_objects;   // a debug build checks every lock key against it
     uint32_t *err;
+    int64_t m;
     __device__ uint64_t element(int64_t i) const
     {
         const uint32_t k = sk[i], v = sv[i];
@@ -276,7 +276,7 @@ struct TicketMode {
         if (!dbg_in(sk[i], n_objects, err)) return;
         lock_key[slot] = sk[i];
         lock_ticket[slot] = tk;
-        if (tk >= hot_ticket && !*(volatile uint32_t *)hot) *hot = 1u;
+        if (tk >= hot_ticket && (i + 1 >= m || sk[i + 1] != sk[i]) && tk > *(volatile uint32_t *)hot) atomicMax(hot, tk);
     }
 };
 
@@ -1621,7 +1621,7 @@ cudaError_t launch_ticket_scan(gputx_bulk *b, const uint32_t *sk, const uint32_t
     const bool fixed = b->db->uniform_k || b->graph;
     TicketMode tm{sk, sv, b->sc.lock_key, b->sc.lock_ticket, fixed ? nullptr : b->sc.op_off,
                   b->graph ? b->db->kmax : b->db->uniform_k, &b->ctl->hot,
-                  kTplHot, b->db->dev.n_objects, &b->ctl->err};
+                  kTplHot, b->db->dev.n_objects, &b->ctl->err, m};
     cudaError_t e = cudaMemsetAsync(&b->ctl->hot, 0, sizeof(uint32_t), b->stream);
     if (e) return e;
     return run_scan(b, tm, m);

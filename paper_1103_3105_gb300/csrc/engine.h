@@ -24,13 +24,15 @@ struct BulkCtl {
     InsertBase total;      // inserts this bulk reserves
     uint32_t rounds;       // exact-depth passes run (the dataflow pass: 1)
     uint32_t n_seg;        // segmented graph bulks: bulks in this segment (0 = one)
-    uint32_t hot;          // TPL: some counter has a chain of more than kTplHot operations
+    uint32_t hot;          // TPL: operations before the last of the longest chain, if kTplHot at least (else 0)
     uint32_t chunk;        // relaxed TPL: next chunk to claim (claim counts commit tickets)
     uint32_t front;        // exact depth: chunks of transactions finished
     uint32_t rows_done;    // debit-credit rows: blocks finished
 };
 
 constexpr uint32_t kTplHot = 128;  // debit-credit TPL: a chain longer than this is served in lock order
+
+constexpr int kTplMany = 64;       // and where the bulk is this many times as long, a warp takes a run of them
 
 constexpr int kScanAreas = 3;      // scans of a submitted bulk whose scratch its submission has cleared
 

@@ -620,6 +620,7 @@ struct TplArgs {
     bool orders;         // new-orders are registered: launch_orders completes them and the order-statuses
     LockSlots slot;      // item -> its counter in `done`
     const uint32_t *sk, *sv;   // debit-credit: the operations sorted by lock
+    int steps;           // tpl_dc_kernel in lock order: times 32 positions a warp takes
 };
 
 // releases of the lanes with `rel` (every lane of the warp calls it): lanes
@@ -818,12 +819,20 @@ __global__ void __launch_bounds__(512) tpl_kernel(TplArgs a)
 // itself.  They are consecutive in timestamp order, or, once the ticket scan has
 // found a chain of more than kTplHot operations, consecutive in the operations
 // sorted by lock: a lock's queue then changes hands once per 32 transactions
-// instead of once per transaction.  Either way a transaction waits for ones
-// handed out before it only.  What bounds a long chain is its hand-offs, about
+// instead of once per transaction.  Where the longest chain is a small part of the
+// bulk (kTplMany), a warp takes a run of 32s side by side, so many that the grid
+// holds the whole bulk and all chains move at once: with 32 a warp, 2^20
+// transactions had 148 of 1,000 chains at work.  The end of a chain that began in
+// an earlier run comes last in its warp's, as nothing waits for it.  A chain that
+// is a large part of the bulk is better off with 32 a warp: the next warp is ready
+// while the last one writes its rows (Zipf 0.99, one chain of a 16th of 200,003: 680
+// against 800 us a bulk).  Always a transaction waits for ones handed out before
+// it, or earlier in its warp's run, only.  What bounds a long chain is its hand-offs, about
 // 2 us each through L2; in lock order the signatures and outputs are scattered,
 // which costs about 50 us per 2^20, hence the line.  1,000 branches, 2^20
-// transactions (chains of 1,050): 360 us, 1,900 in timestamp order; Zipf 0.99
-// accounts, 200,003: 490 us, 5,500 with CTA-wide groups in timestamp order.
+// transactions (chains of 1,050): 145 us, 360 with 32 a warp, 1,900 in timestamp
+// order; Zipf 0.99 accounts, 200,003: 490 us, 5,500 with CTA-wide groups in
+// timestamp order.
 //
 // __match_any_sync groups the lanes that need the same counter.  Every
 // operation here is a write and no other transaction's operation on that item
@@ -841,126 +850,166 @@ __global__ void __launch_bounds__(512) tpl_kernel(TplArgs a)
 // behind one far back in its chain.  A warp in which no two lanes share a
 // counter needs none of this: there each lane waits on its own counter and runs
 // as soon as it is granted.
-__global__ void tpl_dc_kernel(TplArgs a)
+__global__ void __launch_bounds__(1024) tpl_dc_kernel(TplArgs a)
 {
     __shared__ uint32_t s_c, s_stop;
     const int64_t n = a.b.n;
     const int64_t hb = a.ctl->base.hist;
     const uint32_t lane = threadIdx.x & 31;
-    const bool by_lock = a.ctl->hot != 0;
+    const bool by_lock = a.ctl->hot != 0, many = by_lock && (int64_t)a.ctl->hot * kTplMany <= n;
     while (true) {
         if (threadIdx.x == 0) {
             s_stop = *(volatile uint32_t *)&a.ctl->err ? 1u : 0u;
             s_c = atomicAdd(&a.ctl->claim, 1u);
         }
         __syncthreads();
-        const int64_t start = (int64_t)s_c * blockDim.x;
+        // in lock order a warp takes `steps` times 32 positions side by side
+        const int steps = many ? a.steps : 1;
+        const int64_t start = (int64_t)s_c * blockDim.x * steps;
         if (s_stop || start >= n) break;
-        const int64_t i = start + threadIdx.x;
-        const bool live = i < n;
-        const int64_t t = live && by_lock ? (int64_t)(__ldg(&a.sv[i]) >> 7) : i;
-        DcRecord r{};
-        uint32_t key = 0xFFFFFFE0u | lane, tk = 0;   // a key of its own for an idle lane
-        bool rows_ok = true;   // a debug build's check of the record's rows
-        if (live) {
-            r.a = (uint32_t)__ldg(&a.b.params[t * a.b.P]);
-            r.delta = __ldg(&a.b.params[t * a.b.P + 1]);
-            r.ts = __ldg(&a.b.ts[t]);
-            r.t = (uint32_t)t;
-            r.tl = a.db.div_tel.div(r.a);
-            r.br = a.db.div_br.div(r.a);
-            rows_ok = dbg_dc_rows(a.db, a.b, r.a, r.tl, r.br, r.t);
-            if (rows_ok) prefetch_l2(&a.db.acc_bal[r.a]);
-            key = a.slot(by_lock ? __ldg(&a.sk[i]) : a.lock_key[t]);
-            tk = a.lock_ticket[t];
+        // the warp's positions [lo, hi); those before `head` end a queue that began
+        // in an earlier warp's: they come last, as nothing waits for them and what
+        // follows them waits for no other warp
+        const int64_t lo = min(n, start + (int64_t)(threadIdx.x & ~31u) * steps);
+        const int64_t hi = min(n, lo + 32 * (int64_t)steps);
+        int64_t head = lo;
+        if (steps > 1) {
+            head = hi;
+            for (int64_t p = lo; p < hi; p += 32) {
+                const int64_t q = p + lane;
+                const uint32_t m = __ballot_sync(kFull, q < hi && (q == 0 || __ldg(&a.sk[q]) != __ldg(&a.sk[q - 1])));
+                if (m) {
+                    head = p + __ffs(m) - 1;
+                    break;
+                }
+            }
+            if (head == hi) head = lo;
         }
-        const uint32_t grp = __match_any_sync(kFull, key);
-        if (!__any_sync(kFull, live && __popc(grp) > 1)) {
-            // no two lanes of the warp share a counter: each waits on its own,
-            // without the warp's lockstep rounds
+        const int after = (int)((hi - head + 31) / 32), total = after + (int)((head - lo + 31) / 32);
+        auto place = [&](int step) { return (step < after ? head + 32 * step : lo + 32 * (step - after)) + lane; };
+        auto there = [&](int step) { return step < total && place(step) < (step < after ? hi : head); };
+        // a step's record, loaded while the step before runs
+        DcRecord ahead{};
+        uint32_t ahead_key = 0, ahead_tk = 0;
+        auto txn_at = [&](int step) {
+            return !there(step) ? 0u : by_lock ? __ldg(&a.sv[place(step)]) >> 7 : (uint32_t)place(step);
+        };
+        auto load = [&](int step, uint32_t t) {
+            if (!there(step)) return;
+            ahead.a = (uint32_t)__ldg(&a.b.params[(int64_t)t * a.b.P]);
+            ahead.delta = __ldg(&a.b.params[(int64_t)t * a.b.P + 1]);
+            ahead.ts = __ldg(&a.b.ts[t]);
+            ahead.t = t;
+            ahead_key = by_lock ? __ldg(&a.sk[place(step)]) : a.lock_key[t];
+            ahead_tk = a.lock_ticket[t];
+        };
+        uint32_t t1 = txn_at(1);
+        load(0, txn_at(0));
+        for (int step = 0; step < total; step++) {
+            const bool live = there(step);
+            DcRecord r = ahead;
+            const int64_t t = live ? (int64_t)r.t : 0;
+            uint32_t key = 0xFFFFFFE0u | lane, tk = 0;   // a key of its own for an idle lane
+            bool rows_ok = true;   // a debug build's check of the record's rows
             if (live) {
-                const bool ok = !tk || wait_at_least(&a.done[key], tk, a.spin_limit_ns, 500);
-                if (!ok) set_err(&a.ctl->err, ERR_TIMEOUT);
-                DcOut o;
-                const bool pend = ok && dc_account_rmw(a.db, a.b, r, hb + t, o);
-                red_release_add(&a.done[key], 1u);
-                if (pend) dc_finish_rmw(a.db, a.b, o);
+                r.tl = a.db.div_tel.div(r.a);
+                r.br = a.db.div_br.div(r.a);
+                rows_ok = dbg_dc_rows(a.db, a.b, r.a, r.tl, r.br, r.t);
+                if (rows_ok) prefetch_l2(&a.db.acc_bal[r.a]);
+                key = a.slot(ahead_key);
+                tk = ahead_tk;
             }
-        } else {
-            const uint32_t leader = __ffs(grp) - 1;
-            const uint32_t need = __shfl_sync(kFull, tk, leader);   // the group's first ticket
-            bool pending = live;
-            uint64_t t_prog = globaltimer(), t_next = 0;   // t_next: when the group polls next
-            uint32_t idle = 0, seen = 0;
-            while (__any_sync(kFull, pending)) {
-                const uint64_t now = globaltimer();
-                uint32_t v = need ? seen : need;
-                if (pending && lane == leader && need && now >= t_next) {
-                    v = seen = ld_acquire(&a.done[key]);
-                    // missing `gap` releases take at least that many hand-offs
-                    // (in lock order: a hand-off releases a warp's 32)
-                    const uint32_t gap = v >= need ? 0 : by_lock ? (need - v + 31) / 32 : need - v;
-                    t_next = now + (gap > 1 ? (uint64_t)(gap > 64 ? 64 : gap) * 500 : 0);
-                }
-                v = __shfl_sync(kFull, v, leader);
-                bool ready = pending && v >= need;
-                bool failed = false;
-                if (!__any_sync(kFull, ready)) {
-                    if (now - t_prog > a.spin_limit_ns) {
-                        // no group made progress within the limit: give up, but
-                        // release, so no later waiter hangs on these counters
-                        failed = ready = pending;
-                        if (failed && lane == leader) set_err(&a.ctl->err, ERR_TIMEOUT);
-                    } else {
-                        // sleep until the first group is due to poll
-                        const uint32_t due = (pending && lane == leader)
-                                                 ? (t_next > now ? (uint32_t)min(t_next - now, (uint64_t)32000) : 0u)
-                                                 : kFull;
-                        const uint32_t d = __reduce_min_sync(kFull, due);
-                        if (d > 0 && d != kFull) __nanosleep(d);
-                        else if (++idle > 64) __nanosleep(32);
-                        continue;
-                    }
-                }
-                // the lanes of `ready` groups run now; the leader's acquire
-                // orders the members' accesses after the previous holder's
-                __syncwarp();
-                const int64_t slot = hb + t;
-                const bool run = ready && !failed && rows_ok && slot < a.db.hist_cap;
-                if (ready && !failed && rows_ok && !run) {      // history full: not executed
-                    set_err(a.b.err, ERR_CAPACITY);
-                    a.b.status[r.t] = 3;
-                }
-                // the account: one fetch-and-add per distinct account
-                const uint32_t am = __match_any_sync(kFull, run ? r.a : (0xFFFFFFE0u | lane));
-                int64_t pre = r.delta, tot = r.delta;
-                if (__any_sync(kFull, run && __popc(am) > 1)) group_sum(am, r.delta, pre, tot);
-                const uint32_t al = __ffs(am) - 1;
-                int64_t old = 0;
-                if (run && lane == al)
-                    old = (int64_t)atomicAdd((unsigned long long *)&a.db.acc_bal[r.a], (unsigned long long)tot);
-                old = __shfl_sync(kFull, old, al);
-                __syncwarp();
-                // one release per group: every member's update precedes it
-                if (ready && lane == leader) red_release_add(&a.done[key], (uint32_t)__popc(grp));
-                warp_add(run, r.tl, (unsigned long long *)&a.db.tel_bal[r.tl], r.delta);
-                warp_add(run, r.br, (unsigned long long *)&a.db.br_bal[r.br], r.delta);
-                if (run) {
+            load(step + 1, t1);
+            t1 = txn_at(step + 2);
+            const uint32_t grp = __match_any_sync(kFull, key);
+            if (!__any_sync(kFull, live && __popc(grp) > 1)) {
+                // no two lanes of the warp share a counter: each waits on its own,
+                // without the warp's lockstep rounds
+                if (live) {
+                    const bool ok = !tk || wait_at_least(&a.done[key], tk, a.spin_limit_ns, 500);
+                    if (!ok) set_err(&a.ctl->err, ERR_TIMEOUT);
                     DcOut o;
-                    o.slot = slot;
-                    o.ts = r.ts;
-                    o.delta = r.delta;
-                    o.na = wrap_add(old, pre);
-                    o.a = r.a;
-                    o.tl = r.tl;
-                    o.br = r.br;
-                    o.t = r.t;
-                    dc_finish(a.db, a.b, o);
+                    const bool pend = ok && dc_account_rmw(a.db, a.b, r, hb + t, o);
+                    red_release_add(&a.done[key], 1u);
+                    if (pend) dc_finish_rmw(a.db, a.b, o);
                 }
-                pending = pending && !ready;
-                t_prog = globaltimer();
-                idle = 0;
+            } else {
+                const uint32_t leader = __ffs(grp) - 1;
+                const uint32_t need = __shfl_sync(kFull, tk, leader);   // the group's first ticket
+                bool pending = live;
+                uint64_t t_prog = globaltimer(), t_next = 0;   // t_next: when the group polls next
+                uint32_t idle = 0, seen = 0;
+                while (__any_sync(kFull, pending)) {
+                    const uint64_t now = globaltimer();
+                    uint32_t v = need ? seen : need;
+                    if (pending && lane == leader && need && now >= t_next) {
+                        v = seen = ld_acquire(&a.done[key]);
+                        // missing `gap` releases take at least that many hand-offs
+                        // (in lock order: a hand-off releases a warp's 32)
+                        const uint32_t gap = v >= need ? 0 : by_lock ? (need - v + 31) / 32 : need - v;
+                        t_next = now + (gap > 1 ? (uint64_t)(gap > 64 ? 64 : gap) * 500 : 0);
+                    }
+                    v = __shfl_sync(kFull, v, leader);
+                    bool ready = pending && v >= need;
+                    bool failed = false;
+                    if (!__any_sync(kFull, ready)) {
+                        if (now - t_prog > a.spin_limit_ns) {
+                            // no group made progress within the limit: give up, but
+                            // release, so no later waiter hangs on these counters
+                            failed = ready = pending;
+                            if (failed && lane == leader) set_err(&a.ctl->err, ERR_TIMEOUT);
+                        } else {
+                            // sleep until the first group is due to poll
+                            const uint32_t due = (pending && lane == leader)
+                                                     ? (t_next > now ? (uint32_t)min(t_next - now, (uint64_t)32000) : 0u)
+                                                     : kFull;
+                            const uint32_t d = __reduce_min_sync(kFull, due);
+                            if (d > 0 && d != kFull) __nanosleep(d);
+                            else if (++idle > 64) __nanosleep(32);
+                            continue;
+                        }
+                    }
+                    // the lanes of `ready` groups run now; the leader's acquire
+                    // orders the members' accesses after the previous holder's
+                    __syncwarp();
+                    const int64_t slot = hb + t;
+                    const bool run = ready && !failed && rows_ok && slot < a.db.hist_cap;
+                    if (ready && !failed && rows_ok && !run) {      // history full: not executed
+                        set_err(a.b.err, ERR_CAPACITY);
+                        a.b.status[r.t] = 3;
+                    }
+                    // the account: one fetch-and-add per distinct account
+                    const uint32_t am = __match_any_sync(kFull, run ? r.a : (0xFFFFFFE0u | lane));
+                    int64_t pre = r.delta, tot = r.delta;
+                    if (__any_sync(kFull, run && __popc(am) > 1)) group_sum(am, r.delta, pre, tot);
+                    const uint32_t al = __ffs(am) - 1;
+                    int64_t old = 0;
+                    if (run && lane == al)
+                        old = (int64_t)atomicAdd((unsigned long long *)&a.db.acc_bal[r.a], (unsigned long long)tot);
+                    old = __shfl_sync(kFull, old, al);
+                    __syncwarp();
+                    // one release per group: every member's update precedes it
+                    if (ready && lane == leader) red_release_add(&a.done[key], (uint32_t)__popc(grp));
+                    warp_add(run, r.tl, (unsigned long long *)&a.db.tel_bal[r.tl], r.delta);
+                    warp_add(run, r.br, (unsigned long long *)&a.db.br_bal[r.br], r.delta);
+                    if (run) {
+                        DcOut o;
+                        o.slot = slot;
+                        o.ts = r.ts;
+                        o.delta = r.delta;
+                        o.na = wrap_add(old, pre);
+                        o.a = r.a;
+                        o.tl = r.tl;
+                        o.br = r.br;
+                        o.t = r.t;
+                        dc_finish(a.db, a.b, o);
+                    }
+                    pending = pending && !ready;
+                    t_prog = globaltimer();
+                    idle = 0;
+                }
             }
+            if (there(step + 1)) prefetch_l2(&a.db.acc_bal[ahead.a]);
         }
         __syncthreads();
     }
@@ -1259,6 +1308,8 @@ cudaError_t launch_tpl(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, in
     if (grid > chunks) grid = chunks;
     a.sk = sk;
     a.sv = sv;
+    // lock order: as many positions a warp as let the grid hold the whole bulk
+    a.steps = (int)((b->n + grid * block - 1) / (grid * block));
     if (dc) tpl_dc_kernel<<<(unsigned)grid, block, 0, b->stream>>>(a);
     else tpl_kernel<<<(unsigned)grid, block, 0, b->stream>>>(a);
     count_launches(1);

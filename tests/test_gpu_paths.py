@@ -104,3 +104,31 @@ def test_tpl_in_lock_order(n, pattern, mode):
         np.add.at(want, acct // 100, bulk["params"][:, 1])
     assert np.array_equal(g.read(G.TBL_DC_BRANCH)[:, 0], want)
     g.close()
+
+
+@pytest.mark.parametrize("n,n_br,block", [(150_000, 300, 0), (200_003, 1000, 0), (300_000, 70, 0), (300_000, 60, 1024),
+                                          (160_001, 1, 0)])
+def test_lock_order_in_runs(n, n_br, block):
+    """More transactions than the grid holds 32 a warp: runs of several, chains
+    that end in one, cross several or are too long a part of the bulk.  The
+    balance after each transaction against its account's deltas summed up."""
+    n_acc = 1000 * n_br
+    bulk = W.dc_bulk(n, n_acc, 0.0, seed=n + n_br)
+    g = G.Database(dc=(n_br, 10 * n_br, n_acc), history_capacity=n, max_bulk=n)
+    g.register(G.DC_TYPES)
+    b = g.submit_dict(bulk).execute("tpl", block_threads=block)
+    b.sync()
+    st, out = b.results()
+    b.free()
+    acc, delta = bulk["params"][:, 0], bulk["params"][:, 1]
+    order = np.argsort(acc, kind="stable")
+    run = np.cumsum(delta[order])
+    first = np.searchsorted(acc[order], acc[order])
+    expect = np.empty(n, np.int64)
+    expect[order] = run - (run - delta[order])[first]
+    want = np.zeros(n_acc, np.int64)
+    np.add.at(want, acc, delta)
+    assert not st.any() and np.array_equal(out[:, 0], expect)
+    assert np.array_equal(g.read(G.TBL_DC_ACCOUNT)[:, 0], want)
+    assert np.array_equal(g.read(G.TBL_DC_BRANCH)[:, 0], want.reshape(n_br, 1000).sum(1))
+    g.close()
