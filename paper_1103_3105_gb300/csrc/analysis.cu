@@ -17,6 +17,10 @@ namespace {
 
 constexpr int TB = 256;  // threads per block of the simple map kernels
 
+// what stops the rank scan and the depth pass: errors of the analysis.  The
+// others are the executor's, which may run beside them (launch_depths_aside).
+constexpr uint32_t kAnalysisErr = ~(uint32_t)(ERR_CAPACITY | ERR_BOUNDS);
+
 inline unsigned grid_for(int64_t n, int block = TB)
 {
     int64_t g = (n + block - 1) / block;
@@ -330,11 +334,8 @@ constexpr uint32_t kPredBlind = 1u << 31, kPredTxn = (1u << 25) - 1u;
 // levels from the predecessor to the transaction (0: it does not order the execution)
 __device__ __forceinline__ uint32_t pred_step(uint32_t p) { return !(p & kPredRun) && (p & kPredBlind) ? 0u : 1u; }
 
-// what stops the depth pass (the executor beside it may set the others)
-constexpr uint32_t kAnalysisErr = ~(uint32_t)(ERR_CAPACITY | ERR_BOUNDS);
-
 __global__ void depth_prep_kernel(const uint32_t *sv, const uint32_t *rid, int64_t m, const uint32_t *op_off,
-                                  int kslots, uint32_t *pred, const BulkCtl *ctl)
+                                  int kslots, uint32_t *pred, BulkCtl *ctl)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= m || (ctl->err & kAnalysisErr)) return;
@@ -346,6 +347,7 @@ __global__ void depth_prep_kernel(const uint32_t *sv, const uint32_t *rid, int64
     uint32_t p = kPredNone;
     if (!(r & 0x80000000u)) {
         const int64_t q = i - r - 1;                       // the run before ends here
+        if (!dbg_in(q, m, &ctl->err)) return;
         const uint32_t w = sv[q];
         p = (rid[q] & 0x7fffffffu) ? (kPredRun | (uint32_t)q) : (w >> 7);
         if (!(p & kPredRun) && (v & 3u) == CLS_BW && (w & 3u) == CLS_BW) p |= kPredBlind;
@@ -849,7 +851,7 @@ cudaError_t scan_scratch(gputx_bulk *b, int64_t tiles, uint64_t *&z)
     return cudaMemsetAsync(z, 0, (1 + tiles) * sizeof(uint64_t), b->stream);
 }
 
-template <class Mode> cudaError_t run_scan(gputx_bulk *b, const Mode &mode, int64_t count)
+template <class Mode> cudaError_t run_scan(gputx_bulk *b, const Mode &mode, int64_t count, uint32_t stop = ~0u)
 {
     if (count <= 0) return cudaSuccess;
     const int64_t tiles = (count + SCAN_TILE - 1) / SCAN_TILE;
@@ -858,7 +860,7 @@ template <class Mode> cudaError_t run_scan(gputx_bulk *b, const Mode &mode, int6
     const cudaError_t e = scan_scratch(b, tiles, z);
     if (e) return e;
     dualseg_scan_kernel<Mode><<<(unsigned)tiles, SCAN_THREADS, 0, s>>>(
-        mode, count, z + 1, (uint32_t *)z, &b->ctl->err,
+        mode, count, z + 1, (uint32_t *)z, &b->ctl->err, stop,
         (uint64_t)b->db->cfg.spin_limit_ns);
     count_launches(1);
     return cudaGetLastError();
@@ -1351,7 +1353,7 @@ cudaError_t launch_part_offsets(gputx_bulk *b, const uint32_t *cnt, uint32_t *of
     if (!e) e = cudaMemsetAsync(tile_ctr, 0, sizeof(uint32_t), b->stream);
     if (e) return e;
     dualseg_scan_kernel<OffsetMode><<<(unsigned)tiles, SCAN_THREADS, 0, b->stream>>>(
-        om, parts, status, tile_ctr, &b->ctl->err, (uint64_t)b->db->cfg.spin_limit_ns);
+        om, parts, status, tile_ctr, &b->ctl->err, ~0u, (uint64_t)b->db->cfg.spin_limit_ns);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -1613,7 +1615,7 @@ cudaError_t launch_rank_scan(gputx_bulk *b, const uint32_t *sk, const uint32_t *
     cudaError_t e = cudaMemsetAsync(b->sc.level, 0, b->n * sizeof(uint32_t), b->stream);
     if (e) return e;
     RankMode rm{sk, sv, b->sc.level, want_rid ? b->sc.rid : nullptr};
-    return run_scan(b, rm, m);
+    return run_scan(b, rm, m, kAnalysisErr);
 }
 
 cudaError_t launch_ticket_scan(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m)
