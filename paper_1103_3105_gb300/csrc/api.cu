@@ -1271,7 +1271,7 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
         CK(begin_tail(b), "order");
         if (b->timing) cudaEventRecord(b->ev[3], s);
         CK(launch_items(b, sk, sv, m, 0), "k-set execute");
-        CK(launch_orders(b), "orders");
+        CK(launch_orders(b, true), "orders");
     } else if (run == GPUTX_KSET) {
         const int64_t depth = b->host_ctl.last_level;
         const bool persistent = opts && opts->kset_launch == 1;
@@ -1285,7 +1285,7 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
             CK(begin_tail(b), "order");
             if (b->timing) cudaEventRecord(b->ev[3], s);
             CK(launch_kset(b, rv, b->sc.chunk_cap, block, add || db->need_fixpoint), "k-set execute");
-            CK(launch_orders(b), "orders");
+            CK(launch_orders(b, false), "orders");
         } else if (b->n > 0) {
             // plan launches from the level widths
             b->level_off_host.resize((size_t)depth + 2);
@@ -1306,7 +1306,7 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
                 CK(launch_kset_levels(b, b->level_off_host.data(), depth, narrow, add || db->need_fixpoint,
                                       b->sc.type_cut ? b->type_cut_host.data() : nullptr),
                    "k-set execute");
-                CK(launch_orders(b), "orders");
+                CK(launch_orders(b, false), "orders");
             }
         } else {
             CK(begin_tail(b), "order");   // empty bulk
@@ -1405,7 +1405,7 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
         CK(begin_tail(b), "order");
         if (b->timing) cudaEventRecord(b->ev[3], s);
         CK(launch_tpl(b, sk, sv, block, add), "tpl execute");
-        CK(launch_orders(b), "orders");
+        CK(launch_orders(b, false), "orders");
         if (b->timing) cudaEventRecord(b->ev[4], s);
         CK(launch_tpl_reset(b, sk, m), "tpl reset");
     }
@@ -1610,7 +1610,7 @@ extern "C" gputx_status gputx_execute_kset_noalloc(gputx_db *db, const int64_t *
         CK(launch_gather(&b, rv), "gather");
         CK(launch_kset(&b, rv, b.sc.chunk_cap, block, add || db->need_fixpoint), "k-set execute");
     }
-    CK(launch_orders(&b), "orders");
+    CK(launch_orders(&b, oe_only(db)), "orders");
     CK(launch_finish(&b), "finish");
     CK(cudaEventRecord(db->last_done, s), "order");
     if ((st = read_ctl(&b))) return st;

@@ -120,7 +120,7 @@ cudaError_t enqueue_pipeline(GraphBulk *g)
         if (gtx::oe_only(db)) {
             if ((e = gtx::launch_begin(b))) return e;
             if ((e = gtx::launch_items(b, sk, sv, m, seg ? gtx::seg_bits(db) : 0))) return e;
-            if ((e = gtx::launch_orders(b))) return e;
+            if ((e = gtx::launch_orders(b, true))) return e;
             return gtx::launch_finish(b);
         }
         if (seg && (e = gtx::launch_seg_levels(b))) return e;
@@ -132,12 +132,12 @@ cudaError_t enqueue_pipeline(GraphBulk *g)
         if ((e = gtx::launch_gather(b, rv))) return e;
         if ((e = gtx::launch_begin(b))) return e;
         if ((e = gtx::launch_kset(b, rv, b->sc.chunk_cap, g->block, add || db->need_fixpoint))) return e;
-        if ((e = gtx::launch_orders(b))) return e;
+        if ((e = gtx::launch_orders(b, false))) return e;
     } else {
         if ((e = gtx::launch_ticket_scan(b, sk, sv, m))) return e;
         if ((e = gtx::launch_begin(b))) return e;
         if ((e = gtx::launch_tpl(b, sk, sv, g->block, add))) return e;
-        if ((e = gtx::launch_orders(b))) return e;
+        if ((e = gtx::launch_orders(b, false))) return e;
         if ((e = gtx::launch_tpl_reset(b, sk, m))) return e;
     }
     return gtx::launch_finish(b);

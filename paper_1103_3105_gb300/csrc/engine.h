@@ -194,8 +194,9 @@ cudaError_t launch_kset_levels(gputx_bulk *b, const uint32_t *level_off_host, in
 cudaError_t launch_kset_rounds(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, bool stats, bool atomic_add);
 cudaError_t launch_part(gputx_bulk *b, const uint32_t *pkeys, int block, int64_t max_parts);
 cudaError_t launch_tpl(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int block, bool atomic_add);
-// after K-SET's levels, after TPL: the rows of the new orders, then what the order-statuses read of them
-cudaError_t launch_orders(gputx_bulk *b);
+// after K-SET's levels, after TPL, after the items: the rows of the new orders,
+// then what the order-statuses read of them.  `decided`: launch_items preceded
+cudaError_t launch_orders(gputx_bulk *b, bool decided);
 // a conflict-free bulk (a 0-set) in one launch
 cudaError_t launch_independent(gputx_bulk *b, bool atomic_add);
 // relaxed timestamps (Appendix G)

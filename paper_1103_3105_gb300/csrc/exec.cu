@@ -150,8 +150,11 @@ __device__ __forceinline__ void exec_lane(const DevDB &db, const DevBulk &b, con
 
 // The second parts of a bulk's new-orders (orders = true: order rows, lines,
 // index entries, outputs), then of its order-statuses, 16 lanes a transaction
-// in timestamp order, so slots and outputs are written side by side.
-__global__ void __launch_bounds__(256) orders_kernel(DevDB db, DevBulk b, const BulkCtl *ctl, bool orders)
+// in timestamp order, so slots and outputs are written side by side.  Only
+// transactions whose first part ran have a second one: an order that never ran
+// has an insert slot all the same, which may lie past the area.  `decided`: every
+// new-order with status 0 ran (order_status_kernel set it).
+__global__ void __launch_bounds__(256) orders_kernel(DevDB db, DevBulk b, const BulkCtl *ctl, bool orders, bool decided)
 {
     if (ctl->err & ~(uint32_t)ERR_CAPACITY) return;
     const int64_t n = b.n_live ? (int64_t)*b.n_live : b.n;
@@ -160,6 +163,7 @@ __global__ void __launch_bounds__(256) orders_kernel(DevDB db, DevBulk b, const 
     for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kGroup; t < n; t += stride) {
         const int32_t type = __ldg(&b.type[t]);
         if (type != (orders ? GPUTX_T_OE_NEW_ORDER : GPUTX_T_OE_ORDER_STATUS) || b.status[t] != 0) continue;
+        if (!decided && b.out[t * b.R + (orders ? 2 : 1)] == 0) continue;
         const TxnView v = view_of(b, (uint32_t)t, 0);
         if (orders) {
             NewOrderPart o;
@@ -1251,16 +1255,16 @@ cudaError_t launch_kset_rounds(gputx_bulk *b, const uint32_t *sk, const uint32_t
     return cudaGetLastError();
 }
 
-cudaError_t launch_orders(gputx_bulk *b)
+cudaError_t launch_orders(gputx_bulk *b, bool decided)
 {
     gputx_db *db = b->db;
     if (b->n == 0 || !(db->dev.registered >> GPUTX_T_OE_NEW_ORDER & 1u)) return cudaSuccess;
     const DevBulk d = make_dev_bulk(b, GPUTX_CONFLICT_PAPER);
     const unsigned grid = (unsigned)std::min<int64_t>((b->n * kGroup + 255) / 256, (int64_t)db->num_sms * 8);
-    orders_kernel<<<grid, 256, 0, b->stream>>>(db->dev, d, b->ctl, true);
+    orders_kernel<<<grid, 256, 0, b->stream>>>(db->dev, d, b->ctl, true, decided);
     count_launches(1);
     if (db->dev.registered >> GPUTX_T_OE_ORDER_STATUS & 1u) {
-        orders_kernel<<<grid, 256, 0, b->stream>>>(db->dev, d, b->ctl, false);
+        orders_kernel<<<grid, 256, 0, b->stream>>>(db->dev, d, b->ctl, false, decided);
         count_launches(1);
     }
     return cudaGetLastError();

@@ -952,15 +952,19 @@ __device__ __forceinline__ int64_t new_order_params(const DevBulk &b, const TxnV
 }
 
 // the first part of a new-order whose second runs after the levels: it finds
-// the order's id in the first output (a status other than 0 tells it to stay
-// away)
+// the order's id in the first output and its line count in the third.  A status
+// other than 0 tells it to stay away, and so does a count of 0 (an order has one
+// line at least): once an error stops the executor, orders that it never came to
+// still have the status 0 that the bulk began with.
 __device__ __forceinline__ void new_order_first(const DevDB &db, const DevBulk &b, const TxnView &v, uint32_t gl,
                                                 int64_t p2, int64_t p3, int64_t line, int64_t os, int64_t ls)
 {
     NewOrderPart o;
     new_order_state(db, b, v, gl, p2, p3, line, os, ls, o);
     if (o.run && gl == 0) {
-        b.out[(int64_t)v.t * b.R] = o.o_id;
+        int64_t *out = b.out + (int64_t)v.t * b.R;
+        out[0] = o.o_id;
+        out[2] = o.cnt;
         b.status[v.t] = 0;
     }
 }
@@ -1016,12 +1020,15 @@ __device__ __forceinline__ void new_order_first_lane(const DevDB &db, const DevB
     __stcg(&db.d_next_o_id[d], o_id + 1);
     __stcg(&db.c_last_o_id[c], o_id);
     stg_cg(&db.c_last_slot[c], (uint32_t)oslot);
-    b.out[(int64_t)v.t * b.R] = o_id;
+    int64_t *out = b.out + (int64_t)v.t * b.R;
+    out[0] = o_id;
+    out[2] = cnt;
     b.status[v.t] = 0;
 }
 
 // an order-status in two parts: the customer's balance and last order, then
-// the order's count and amounts (the order's slot waits in the third output)
+// the order's count and amounts (the order's slot waits in the third output; an
+// order id of 0 is one without a second part, or one that never ran)
 __device__ __forceinline__ void order_status_first(const DevDB &db, const DevBulk &b, const TxnView &v, int64_t p2)
 {
     if (kDebug && !valid_txn(db, v.type, v.p, b.P)) {
