@@ -418,8 +418,8 @@ gputx_status gputx_batcher_create(gputx_db *db, const gputx_batch_config *cfg, g
  * K-SET each bulk (piece) keeps its own dependency graph and k-sets
  * (Definition 1 per bulk, bulks in order); TPL and PART run a segment in
  * timestamp order.  The arrays are read until the call returns, by the GPU itself
- * where it reads through the host's page tables.  EINVAL on bad offsets; device
- * errors as for gputx_sync_bulk. */
+ * where it reads through the host's page tables and they are aligned to their
+ * elements.  EINVAL on bad offsets; device errors as for gputx_sync_bulk. */
 gputx_status gputx_batcher_run_bulks(gputx_batcher *bt, const int64_t *ts, const int32_t *type,
                                      const int64_t *params, const int64_t *bulk_off, size_t n_bulks,
                                      int32_t *status, int64_t *values);

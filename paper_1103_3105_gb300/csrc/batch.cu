@@ -328,6 +328,14 @@ void touch_pages(const void *p, size_t bytes)
     if (bytes) (void)c[bytes - 1];
 }
 
+// whether fetch_kernel's loads may take these arrays: addresses that are
+// multiples of the elements' sizes (memory that the caller packed by bytes need
+// not be)
+bool word_aligned(const int64_t *ts, const int32_t *type, const int64_t *params)
+{
+    return ((uintptr_t)ts | (uintptr_t)params) % sizeof(int64_t) == 0 && (uintptr_t)type % sizeof(int32_t) == 0;
+}
+
 // One segment of n <= cap transactions through a graph: n_seg bulks whose
 // first transactions (relative to the segment) are seg_off[0..n_seg-1].  The
 // device fetches the inputs (fetch_kernel), or the host copies them into the
@@ -341,7 +349,8 @@ gputx_status enqueue_segment(gputx_batcher *bt, GraphBulk *g, Staging &st, const
     gputx_bulk *b = g->b;
     cudaStream_t s = b->stream;
     const int64_t cap = g->cap;
-    if (db->reads_host) {
+    const bool fetch = db->reads_host && word_aligned(ts, type, params);
+    if (fetch) {
         touch_pages(ts, sizeof(int64_t) * n);
         touch_pages(type, sizeof(int32_t) * n);
         touch_pages(params, sizeof(int64_t) * n * g->P);
@@ -356,7 +365,7 @@ gputx_status enqueue_segment(gputx_batcher *bt, GraphBulk *g, Staging &st, const
     // the inputs come in while the segment before runs: only this graph's
     // buffers are written, and its last replay is on the same stream
     CKB(cudaMemsetAsync(b->ctl, 0, sizeof(gtx::BulkCtl), s), "reset");
-    if (db->reads_host) {
+    if (fetch) {
         FetchArgs a;
         a.ts = ts;
         a.params = params;
