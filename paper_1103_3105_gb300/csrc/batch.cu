@@ -342,8 +342,8 @@ bool word_aligned(const int64_t *ts, const int32_t *type, const int64_t *params)
 // pinned staging `st` and the device from there; it replays the graph and copies
 // the results and the control block back into `st`, then records g->done.  Nothing
 // here waits for the device; the inputs stay in place until g->done.
-gputx_status enqueue_segment(gputx_batcher *bt, GraphBulk *g, Staging &st, const int64_t *ts, const int32_t *type,
-                             const int64_t *params, int64_t n, const uint32_t *seg_off, uint32_t n_seg)
+gputx_status enqueue_steps(gputx_batcher *bt, GraphBulk *g, Staging &st, const int64_t *ts, const int32_t *type,
+                           const int64_t *params, int64_t n, const uint32_t *seg_off, uint32_t n_seg)
 {
     gputx_db *db = bt->db;
     gputx_bulk *b = g->b;
@@ -408,6 +408,16 @@ gputx_status enqueue_segment(gputx_batcher *bt, GraphBulk *g, Staging &st, const
     CKB(cudaMemcpyAsync(st.ctl, b->ctl, sizeof(gtx::BulkCtl), cudaMemcpyDeviceToHost, s), "results");
     CKB(cudaEventRecord(g->done, s), "event");
     return GPUTX_OK;
+}
+
+// enqueue_steps; where a step fails, what is on its way has ended on return (no
+// kernel reads the caller's arrays after the call)
+gputx_status enqueue_segment(gputx_batcher *bt, GraphBulk *g, Staging &st, const int64_t *ts, const int32_t *type,
+                             const int64_t *params, int64_t n, const uint32_t *seg_off, uint32_t n_seg)
+{
+    const gputx_status r = enqueue_steps(bt, g, st, ts, type, params, n, seg_off, n_seg);
+    if (r) cudaStreamSynchronize(g->b->stream);
+    return r;
 }
 
 // Waits for a segment enqueued by enqueue_segment, copies its results to the
@@ -629,10 +639,8 @@ gputx_status gputx_batcher_run_bulks(gputx_batcher *bt, const int64_t *ts, const
         if ((st = get_graph(bt, size, strategy, block, sync ? 0 : buf, &g))) break;
         if ((st = ensure_staging(bt, bt->stage[buf], size))) break;
         if ((st = enqueue_segment(bt, g, bt->stage[buf], ts + first_txn, type + first_txn, params + first_txn * P, k,
-                                  seg_off.data(), (uint32_t)seg_off.size()))) {
-            cudaStreamSynchronize(g->b->stream);   // nothing reads the caller's arrays after the call
+                                  seg_off.data(), (uint32_t)seg_off.size())))
             break;
-        }
         InFlight cur;
         cur.valid = true;
         cur.first = first;
