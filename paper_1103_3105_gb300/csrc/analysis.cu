@@ -300,8 +300,8 @@ struct TicketMode {
 // between two blind increments of the read/write model (CLS_BW): K-SET applies
 // those by atomic additions, so they order nothing.  Order-entry's payments
 // then run beside each other although all of a warehouse's write its total.
-// A finished transaction publishes both in one 64-bit word with its chunk's tag,
-// so a waiter needs no fence and no second read.
+// A finished transaction publishes both in one 64-bit word with its chunk's lap
+// (below), so a waiter needs no fence and no second read.
 //
 // What bounds the pass is the longest path, so its hops are made short.  One
 // cluster runs it: a CTA holds 1,024 consecutive transactions, its neighbours the
@@ -359,9 +359,14 @@ constexpr int kFlowThreads = 1024, kFlowCluster = 8;
 constexpr int kFlowPush = 7;                // the chunks after a chunk that get its words in shared memory
 constexpr unsigned long long kNotYet = ~0ull;
 
-// a word: tag << 57 | depth << 32 | level (a bulk has at most 2^25 transactions)
-constexpr uint32_t kFlowTags = 128, kFlowMask = (1u << 25) - 1u;
-__device__ __forceinline__ uint32_t flow_tag(uint32_t chunk) { return (chunk + 1) & (kFlowTags - 1); }
+// A word: lap << 50 | depth << 25 | level (a bulk has at most 2^25 transactions).
+// A place in the ring takes the words of one CTA, whose chunks lie kFlowCluster
+// apart, so the lap (from 1, at most 2^12 + 1) says which chunk's word it holds:
+// nothing keeps the CTAs of the cluster in step, and one may be any number of laps
+// ahead of another.
+constexpr uint32_t kFlowBits = 25, kFlowMask = (1u << kFlowBits) - 1u;
+__device__ __forceinline__ uint32_t flow_lap(uint32_t chunk) { return chunk / kFlowCluster + 1; }
+__device__ __forceinline__ uint32_t word_lap(unsigned long long w) { return (uint32_t)(w >> (2 * kFlowBits)); }
 
 __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long *p)
 {
@@ -411,12 +416,12 @@ __global__ void __launch_bounds__(kFlowThreads, 1) depth_flow_kernel(FlowArgs a)
     for (uint32_t c = rank; (uint64_t)c * kFlowThreads < n; c += kFlowCluster) {
         const uint32_t start = c * kFlowThreads, t = start + tid;
         uint32_t dep = 0, lev = 0;
-        auto take = [&](uint32_t hi, uint32_t lo, uint32_t dl, uint32_t ll) {
-            const uint32_t d = (hi & kFlowMask) + dl, l = lo + ll;
+        auto take = [&](unsigned long long w, uint32_t dl, uint32_t ll) {
+            const uint32_t d = ((uint32_t)(w >> kFlowBits) & kFlowMask) + dl, l = ((uint32_t)w & kFlowMask) + ll;
             dep = d > dep ? d : dep;
             if (ll) lev = l > lev ? l : lev;
         };
-        // where transaction x's word comes to in this CTA's ring, and its tag
+        // where transaction x's word comes to in this CTA's ring
         auto near_word = [&](uint32_t x) { return c - x / kFlowThreads <= (uint32_t)kFlowPush; };
         auto ring_word = [&](uint32_t x) {
             return ring + 8u * ((c - x / kFlowThreads) * kFlowThreads + x % kFlowThreads);
@@ -441,7 +446,7 @@ __global__ void __launch_bounds__(kFlowThreads, 1) depth_flow_kernel(FlowArgs a)
                 for (int u = 0; u < 6; u++) {
                     if (p[u] == kPredNone) continue;
                     if (w[u] != kNotYet) {
-                        take((uint32_t)(w[u] >> 32), (uint32_t)w[u], 1, pred_step(p[u]));
+                        take(w[u], 1, pred_step(p[u]));
                         continue;
                     }
                     if (p[u] & kPredRun) {
@@ -505,7 +510,8 @@ __global__ void __launch_bounds__(kFlowThreads, 1) depth_flow_kernel(FlowArgs a)
             return true;
         };
         auto publish = [&]() {
-            const unsigned long long w = (unsigned long long)(flow_tag(c) << 25 | dep) << 32 | lev;
+            const unsigned long long w =
+                (unsigned long long)flow_lap(c) << (2 * kFlowBits) | (unsigned long long)dep << kFlowBits | lev;
             asm volatile("st.relaxed.cluster.shared::cta.u64 [%0], %1;" ::"r"(ring + 8u * tid), "l"(w) : "memory");
 #pragma unroll
             for (uint32_t r = 1; r <= (uint32_t)kFlowPush; r++) {
@@ -533,28 +539,25 @@ __global__ void __launch_bounds__(kFlowThreads, 1) depth_flow_kernel(FlowArgs a)
         uint64_t t_prog = 0;
         uint32_t seen = 0;
         bool near = near_word(x);
-        uint32_t at = near ? ring_word(x) : ring, want = flow_tag(x / kFlowThreads);
+        uint32_t at = near ? ring_word(x) : ring, want = flow_lap(x / kFlowThreads);
         for (uint32_t spin = 1;; spin++) {
             unsigned long long w;
             asm volatile("ld.relaxed.cluster.shared::cta.u64 %0, [%1];" : "=l"(w) : "r"(at) : "memory");
-            uint32_t hi = (uint32_t)(w >> 32), lo = (uint32_t)w;
-            const uint32_t d = ((hi >> 25) - want) & (kFlowTags - 1);
-            bool hit = !done && near && d < kFlowTags / 2;
+            const uint32_t lap = word_lap(w);
+            bool hit = !done && near && lap >= want;
             // older than the ring, or overwritten by a later chunk's (that CTA has finished its chunk)
-            const bool far = !done && (near ? hit && d : (spin & 7u) == 0);
+            const bool far = !done && (near ? hit && lap != want : (spin & 7u) == 0);
             if (far) {
                 w = ld_relaxed_u64(&a.depths[x]);
-                hi = (uint32_t)(w >> 32);
-                lo = (uint32_t)w;
                 hit = w != kNotYet;
             }
             if (__any_sync(kFull, hit)) {
                 if (hit) {
-                    take(hi, lo, dl, ll);
+                    take(w, dl, ll);
                     if (!next()) publish();
                     near = near_word(x);
                     at = near ? ring_word(x) : ring;
-                    want = flow_tag(x / kFlowThreads);
+                    want = flow_lap(x / kFlowThreads);
                 }
                 continue;
             }
