@@ -176,8 +176,12 @@ typedef struct {
     int32_t fallback;         /* 1 when PART fell back to TPL (Section 5.2) */
     int64_t n;                /* transactions */
     int64_t n_ops;            /* basic operations extracted */
-    int64_t depth;            /* d: depth of the T-dependency graph */
-    int64_t w0;               /* size of the 0-set */
+    int64_t depth;            /* d: depth of the T-dependency graph; -1 where it is
+                               * computed beside the execution (order-entry alone
+                               * under K-SET, without timing) and a wait of that
+                               * ran out: the bulk is applied in full, and neither
+                               * d nor w0 is known */
+    int64_t w0;               /* size of the 0-set; -1 as for d */
     int64_t cross;            /* c: cross-partition transactions */
     int64_t fixpoint_rounds;  /* exact-depth passes after the one-pass ranks
                                * (1 when they ran, 0 when skipped) */

@@ -20,6 +20,10 @@ constexpr int TB = 256;  // threads per block of the simple map kernels
 // what stops the rank scan and the depth pass: errors of the analysis.  The
 // others are the executor's, which may run beside them (launch_depths_aside).
 constexpr uint32_t kAnalysisErr = ~(uint32_t)(ERR_CAPACITY | ERR_BOUNDS);
+__device__ __forceinline__ uint32_t analysis_errors(const BulkCtl *ctl)
+{
+    return *(const volatile uint32_t *)&ctl->err & kAnalysisErr | *(const volatile uint32_t *)&ctl->depth_err;
+}
 
 inline unsigned grid_for(int64_t n, int block = TB)
 {
@@ -338,7 +342,7 @@ __global__ void depth_prep_kernel(const uint32_t *sv, const uint32_t *rid, int64
                                   int kslots, uint32_t *pred, BulkCtl *ctl)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= m || (ctl->err & kAnalysisErr)) return;
+    if (i >= m || analysis_errors(ctl)) return;
     const uint32_t v = sv[i];
     if (v == OP_SENTINEL) return;
     const uint32_t r = rid[i];
@@ -381,6 +385,7 @@ struct FlowArgs {
     unsigned long long *depths;              // per transaction: its word, kNotYet before
     uint32_t *level;
     BulkCtl *ctl;
+    uint32_t *err;
     int64_t n;
     bool graph;                              // transactions from n_live on are padding
     uint64_t limit_ns;
@@ -406,7 +411,7 @@ __global__ void __launch_bounds__(kFlowThreads, 1) depth_flow_kernel(FlowArgs a)
     for (int k = 0; k <= kFlowPush; k++) s_ring[k * kFlowThreads + tid] = 0;
     if (rank == 0 && tid == 0) ctl->rounds = 1;
     __shared__ uint32_t s_stop;
-    if (tid == 0) s_stop = *(volatile uint32_t *)&ctl->err & kAnalysisErr;
+    if (tid == 0) s_stop = analysis_errors(ctl);
     const uint32_t n = (uint32_t)(a.graph ? (int64_t)ctl->n_live : a.n);
     cl.sync();
     const bool stop = *cl.map_shared_rank(&s_stop, 0) != 0;    // the same in every CTA
@@ -567,9 +572,9 @@ __global__ void __launch_bounds__(kFlowThreads, 1) depth_flow_kernel(FlowArgs a)
                 const uint64_t now = globaltimer();
                 if (t_prog == 0 || f != seen) t_prog = now;
                 seen = f;
-                const bool late = now - t_prog > a.limit_ns || (*(volatile uint32_t *)&ctl->err & ERR_TIMEOUT);
+                const bool late = now - t_prog > a.limit_ns || (*(volatile uint32_t *)a.err & ERR_TIMEOUT);
                 if (__any_sync(kFull, late)) {
-                    if (lane == 0) set_err(&ctl->err, ERR_TIMEOUT);
+                    if (lane == 0) set_err(a.err, ERR_TIMEOUT);
                     if (!done) publish();
                 }
             }
@@ -854,7 +859,11 @@ cudaError_t scan_scratch(gputx_bulk *b, int64_t tiles, uint64_t *&z)
     return cudaMemsetAsync(z, 0, (1 + tiles) * sizeof(uint64_t), b->stream);
 }
 
-template <class Mode> cudaError_t run_scan(gputx_bulk *b, const Mode &mode, int64_t count, uint32_t stop = ~0u)
+// where the rank scan and the depth pass note that a wait ran out
+uint32_t *analysis_err(gputx_bulk *b, bool aside) { return aside ? &b->ctl->depth_err : &b->ctl->err; }
+
+template <class Mode>
+cudaError_t run_scan(gputx_bulk *b, const Mode &mode, int64_t count, uint32_t stop = ~0u, bool aside = false)
 {
     if (count <= 0) return cudaSuccess;
     const int64_t tiles = (count + SCAN_TILE - 1) / SCAN_TILE;
@@ -863,7 +872,7 @@ template <class Mode> cudaError_t run_scan(gputx_bulk *b, const Mode &mode, int6
     const cudaError_t e = scan_scratch(b, tiles, z);
     if (e) return e;
     dualseg_scan_kernel<Mode><<<(unsigned)tiles, SCAN_THREADS, 0, s>>>(
-        mode, count, z + 1, (uint32_t *)z, &b->ctl->err, stop,
+        mode, count, z + 1, (uint32_t *)z, analysis_err(b, aside), &b->ctl->err, stop,
         (uint64_t)b->db->cfg.spin_limit_ns);
     count_launches(1);
     return cudaGetLastError();
@@ -1356,7 +1365,7 @@ cudaError_t launch_part_offsets(gputx_bulk *b, const uint32_t *cnt, uint32_t *of
     if (!e) e = cudaMemsetAsync(tile_ctr, 0, sizeof(uint32_t), b->stream);
     if (e) return e;
     dualseg_scan_kernel<OffsetMode><<<(unsigned)tiles, SCAN_THREADS, 0, b->stream>>>(
-        om, parts, status, tile_ctr, &b->ctl->err, ~0u, (uint64_t)b->db->cfg.spin_limit_ns);
+        om, parts, status, tile_ctr, &b->ctl->err, &b->ctl->err, ~0u, (uint64_t)b->db->cfg.spin_limit_ns);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -1613,12 +1622,13 @@ cudaError_t launch_group(gputx_bulk *b, int mode, int part_size, bool by_part, u
     return launch_sort_passes(b, keys, vals, keys_alt, vals_alt, n, bits, a.hist != nullptr);
 }
 
-cudaError_t launch_rank_scan(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m, bool want_rid)
+cudaError_t launch_rank_scan(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m, bool want_rid,
+                             bool aside)
 {
     cudaError_t e = cudaMemsetAsync(b->sc.level, 0, b->n * sizeof(uint32_t), b->stream);
     if (e) return e;
     RankMode rm{sk, sv, b->sc.level, want_rid ? b->sc.rid : nullptr};
-    return run_scan(b, rm, m, kAnalysisErr);
+    return run_scan(b, rm, m, kAnalysisErr, aside);
 }
 
 cudaError_t launch_ticket_scan(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m)
@@ -1633,7 +1643,7 @@ cudaError_t launch_ticket_scan(gputx_bulk *b, const uint32_t *sk, const uint32_t
 }
 
 // exact depths after the one-pass ranks (A1): the dataflow pass
-cudaError_t launch_exact_depth(gputx_bulk *b, const uint32_t *sv, int64_t m)
+cudaError_t launch_exact_depth(gputx_bulk *b, const uint32_t *sv, int64_t m, bool aside)
 {
     if (b->n == 0) return cudaSuccess;
     if (m >= (int64_t)kPredVal) return cudaErrorInvalidValue;
@@ -1650,6 +1660,7 @@ cudaError_t launch_exact_depth(gputx_bulk *b, const uint32_t *sv, int64_t m)
     a.depths = b->sc.depths;
     a.level = b->sc.level;
     a.ctl = b->ctl;
+    a.err = analysis_err(b, aside);
     a.n = b->n;
     a.graph = b->graph;
     a.limit_ns = (uint64_t)b->db->cfg.spin_limit_ns;
@@ -1695,8 +1706,8 @@ cudaError_t launch_depths_aside(gputx_bulk *b, const uint32_t *sk, const uint32_
         if (e) return e;
         b->stream = side;
     }
-    e = launch_rank_scan(b, sk, sv, m, true);
-    if (!e) e = launch_exact_depth(b, sv, m);
+    e = launch_rank_scan(b, sk, sv, m, true, true);
+    if (!e) e = launch_exact_depth(b, sv, m, true);
     b->stream = s;
     if (side) {
         const cudaError_t e2 = cudaEventRecord(b->ev_in, side);

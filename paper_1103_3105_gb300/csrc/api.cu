@@ -1431,8 +1431,8 @@ gputx_status gputx_sync_bulk(gputx_bulk *b, gputx_exec_stats *stats)
         stats->fallback = b->fallback;
         stats->n = b->n;
         stats->n_ops = b->sc.m_cap;
-        stats->depth = b->host_ctl.depth;
-        stats->w0 = b->host_ctl.w0;
+        stats->depth = b->host_ctl.depth_err ? -1 : (int64_t)b->host_ctl.depth;
+        stats->w0 = b->host_ctl.depth_err ? -1 : (int64_t)b->host_ctl.w0;
         stats->cross = b->host_ctl.cross;
         stats->fixpoint_rounds = b->host_ctl.rounds;
         if (b->timing) {

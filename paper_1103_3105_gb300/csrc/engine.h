@@ -28,6 +28,7 @@ struct BulkCtl {
     uint32_t chunk;        // relaxed TPL: next chunk to claim (claim counts commit tickets)
     uint32_t front;        // exact depth: chunks of transactions finished
     uint32_t rows_done;    // debit-credit rows: blocks finished
+    uint32_t depth_err;    // launch_depths_aside: its ERR_* bits, which the execution beside it does not read
 };
 
 constexpr uint32_t kTplHot = 128;  // debit-credit TPL: a chain longer than this is served in lock order
@@ -171,10 +172,12 @@ cudaError_t launch_group(gputx_bulk *b, int mode, int part_size, bool by_part, u
                          uint32_t *&keys_alt, uint32_t *&vals_alt, int bits, int64_t *deltas = nullptr);
 cudaError_t launch_sort(gputx_bulk *b, uint32_t *&keys, uint32_t *&vals, uint32_t *&keys_alt,
                         uint32_t *&vals_alt, int64_t count, int bits);
-cudaError_t launch_rank_scan(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m, bool want_rid);
+// `aside`: a wait that runs out is noted in depth_err, not in err
+cudaError_t launch_rank_scan(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m, bool want_rid,
+                             bool aside = false);
 cudaError_t launch_ticket_scan(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m);
 // d, w0 and the level array, exact; the rank scan's rid precedes it
-cudaError_t launch_exact_depth(gputx_bulk *b, const uint32_t *sv, int64_t m);
+cudaError_t launch_exact_depth(gputx_bulk *b, const uint32_t *sv, int64_t m, bool aside = false);
 // d, w0 of the one-pass ranks
 cudaError_t launch_level_stats(gputx_bulk *b);
 cudaError_t launch_regroup_keys(gputx_bulk *b, uint32_t *keys, uint32_t *vals);
@@ -224,8 +227,10 @@ bool dc_only(const gputx_db *db);
 // shift), item by item (exec_oe.cu); launch_orders follows
 bool oe_only(const gputx_db *db);
 cudaError_t launch_items(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m, int shift);
-// the rank scan and launch_exact_depth on the bulk's side stream; join_depths
-// makes the bulk's own stream wait for them (nothing to do if it has)
+// the rank scan and launch_exact_depth on the bulk's side stream, beside its
+// execution, which needs neither: if a wait of theirs runs out, the bulk is
+// applied all the same and the depths are reported as unknown.  join_depths makes
+// the bulk's own stream wait for them (nothing to do if it has)
 cudaError_t launch_depths_aside(gputx_bulk *b, const uint32_t *sk, const uint32_t *sv, int64_t m);
 cudaError_t join_depths(gputx_bulk *b);
 cudaError_t clear_outputs(gputx_bulk *b);

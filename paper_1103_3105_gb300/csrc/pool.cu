@@ -232,7 +232,7 @@ cudaError_t pool_scan(gputx_bulk *b, const Mode &mode, int64_t count)
     cudaError_t e = cudaMemsetAsync(b->sc.scan_zero, 0, (1 + tiles) * sizeof(uint64_t), b->stream);
     if (e) return e;
     dualseg_scan_kernel<Mode><<<(unsigned)tiles, SCAN_THREADS, 0, b->stream>>>(
-        mode, count, b->sc.scan_zero + 1, (uint32_t *)b->sc.scan_zero, &b->ctl->err, ~0u,
+        mode, count, b->sc.scan_zero + 1, (uint32_t *)b->sc.scan_zero, &b->ctl->err, &b->ctl->err, ~0u,
         (uint64_t)b->db->cfg.spin_limit_ns);
     count_launches(1);
     return cudaGetLastError();

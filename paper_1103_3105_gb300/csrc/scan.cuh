@@ -124,15 +124,16 @@ __device__ __forceinline__ uint64_t lookback_prefix(uint64_t *status, uint32_t t
 // Generic single-pass scan of a DualSeg state over [0, count).  Mode
 // provides `uint64_t element(int64_t i)` and `void output(int64_t i,
 // uint64_t inclusive)`; elements are produced and consumed in blocked order
-// (thread t owns SCAN_ITEMS consecutive elements).  `stop`: the error bits that
-// make it do nothing.  They are bits that only earlier work on its stream sets,
-// or that the scan itself sets when it gives up: a bit that something running
-// beside the scan may set would leave the tiles not yet started without their
-// outputs.
+// (thread t owns SCAN_ITEMS consecutive elements).  `err`: where the scan notes
+// that it gave up; `before`: the errors of the steps before it (the same word, but
+// for a scan beside an executor); `stop`: the bits of both that make it do
+// nothing.  They are bits that only earlier work on its stream sets, or that the
+// scan itself sets when it gives up: a bit that something running beside the scan
+// may set would leave the tiles not yet started without their outputs.
 template <class Mode>
 __global__ void __launch_bounds__(SCAN_THREADS)
-dualseg_scan_kernel(Mode mode, int64_t count, uint64_t *status, uint32_t *tile_ctr, uint32_t *err, uint32_t stop,
-                    uint64_t spin_limit_ns)
+dualseg_scan_kernel(Mode mode, int64_t count, uint64_t *status, uint32_t *tile_ctr, uint32_t *err,
+                    const uint32_t *before, uint32_t stop, uint64_t spin_limit_ns)
 {
     __shared__ uint32_t s_tile;
     __shared__ uint64_t s_warp[SCAN_THREADS / 32];
@@ -141,7 +142,7 @@ dualseg_scan_kernel(Mode mode, int64_t count, uint64_t *status, uint32_t *tile_c
     // an earlier step failed: consume nothing (a block that returns here has
     // not taken a tile id, so no look-back waits on it); decided once per block
     if (threadIdx.x == 0) {
-        s_abort = *(volatile uint32_t *)err & stop;
+        s_abort = (*(volatile uint32_t *)err | *(const volatile uint32_t *)before) & stop;
         if (!s_abort) s_tile = atomicAdd(tile_ctr, 1u);
     }
     __syncthreads();

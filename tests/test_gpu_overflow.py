@@ -1,6 +1,6 @@
-"""Order-entry bulks that overflow the order area: the call reports ECAPACITY,
-orders beyond the area leave no trace, and what is reported of the graph is
-exact."""
+"""Order-entry bulks that do not end well: the order area overflows, or a wait
+of the depth pass runs out.  The call says so, orders beyond the area leave no
+trace, and what is reported of the graph is exact or unknown."""
 import ctypes as C
 
 import numpy as np
@@ -9,7 +9,8 @@ import pytest
 import oracle
 import paper_1103_3105_gb300 as G
 import workloads as W
-from tests.test_gpu_schemas import oe_pair
+from tests._helpers import gpu_logical_state, oracle_logical_state, states_equal
+from tests.test_gpu_schemas import check, oe_pair
 
 pytestmark = pytest.mark.gpu
 
@@ -73,4 +74,30 @@ def test_orders_that_never_ran(strategy, launch, types, batch):
     expect = [(d << 32) | i for d in range(10 * n_wh) for i in range(first[d], after[d])]
     assert np.array_equal(np.sort(keys[used]), np.array(expect, np.uint64))
     assert rows[used].max() < fit and len(np.unique(rows[used])) == used.sum()
+    g.close()
+
+
+@pytest.mark.parametrize("timing", [0, 1])
+def test_depths_that_give_up(timing):
+    """A 1 ns wait limit makes the depth pass give up in a chain of 680 orders
+    (one tile for every scan and sort, so that nothing else waits).  Beside the
+    execution that costs the depths alone; before it (timing) the bulk fails and
+    nothing runs."""
+    n, n_wh, n_items = 680, 1, 10
+    g, o = oe_pair(n_wh, n_items, spin_limit_ns=1)
+    params = np.zeros((n, W.OE_PARAMS), np.int64)
+    params[:, 3], params[:, 4] = 1, 3 | 2 << 40
+    bulk = {"ts": np.arange(n, dtype=np.int64), "type": np.full(n, G.T_OE_NEW_ORDER, np.int32), "params": params,
+            "P": W.OE_PARAMS}
+    b = g.submit_dict(bulk).execute("kset", timing=bool(timing))
+    status, stats = sync(b)
+    if timing:
+        assert status == G.ETIMEOUT
+        assert states_equal(gpu_logical_state(g, oe=True), oracle_logical_state(o))
+    else:
+        assert (status, stats.depth, stats.w0) == (G.OK, -1, -1)
+        st, out = b.results()
+        ost, oout = o.execute(bulk, R=g.width)
+        check(g, o, st, out, ost, oout, oe=True)
+    b.free()
     g.close()
