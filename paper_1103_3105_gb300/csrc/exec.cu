@@ -1258,12 +1258,18 @@ cudaError_t launch_kset_rounds(gputx_bulk *b, const uint32_t *sk, const uint32_t
 cudaError_t launch_orders(gputx_bulk *b, bool decided)
 {
     gputx_db *db = b->db;
-    if (b->n == 0 || !(db->dev.registered >> GPUTX_T_OE_NEW_ORDER & 1u)) return cudaSuccess;
+    // without new-orders registered the levels and TPL run order-statuses whole;
+    // the items never do
+    const bool made = db->dev.registered >> GPUTX_T_OE_NEW_ORDER & 1u;
+    const bool read = (made || decided) && (db->dev.registered >> GPUTX_T_OE_ORDER_STATUS & 1u);
+    if (b->n == 0 || !(made || read)) return cudaSuccess;
     const DevBulk d = make_dev_bulk(b, GPUTX_CONFLICT_PAPER);
     const unsigned grid = (unsigned)std::min<int64_t>((b->n * kGroup + 255) / 256, (int64_t)db->num_sms * 8);
-    orders_kernel<<<grid, 256, 0, b->stream>>>(db->dev, d, b->ctl, true, decided);
-    count_launches(1);
-    if (db->dev.registered >> GPUTX_T_OE_ORDER_STATUS & 1u) {
+    if (made) {
+        orders_kernel<<<grid, 256, 0, b->stream>>>(db->dev, d, b->ctl, true, decided);
+        count_launches(1);
+    }
+    if (read) {
         orders_kernel<<<grid, 256, 0, b->stream>>>(db->dev, d, b->ctl, false, decided);
         count_launches(1);
     }
