@@ -1363,6 +1363,7 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
         if (b->timing) cudaEventRecord(b->ev[1], s);
         if ((st = read_ctl(b))) return st;
         if (b->host_ctl.err) {
+            if (dc_only(db)) CK(clear_outputs(b), "clear");   // the executor would have
             CK(end_tail(b, dc_only(db)), "finish");
             b->strategy_run = run;
             return GPUTX_OK;   // reported by the sync
