@@ -1297,13 +1297,15 @@ cudaError_t launch_dc_rows(gputx_bulk *b)
     // block per SM
     const int64_t cells = db->dev.n_tel + db->dev.n_br;
     const size_t smem = (size_t)cells * sizeof(unsigned long long);
-    const bool local = smem <= (200u << 10) && b->n >= 4 * cells;
+    constexpr unsigned kMaxCells = 200u << 10;
+    const bool local = smem <= kMaxCells && b->n >= 4 * cells;
     const int threads = 1024;
     int64_t grid = (b->n + threads - 1) / threads;
     if (grid > (int64_t)db->num_sms) grid = db->num_sms;
     if (local && smem > (48u << 10)) {
+        // always the same limit: another thread's database may need more than this one
         const cudaError_t e = cudaFuncSetAttribute(dc_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)smem);
+                                                   (int)kMaxCells);
         if (e) return e;
     }
     DcRowsArgs a;
