@@ -22,7 +22,7 @@ constexpr int TB = 256;  // threads per block of the simple map kernels
 constexpr uint32_t kAnalysisErr = ~(uint32_t)(ERR_CAPACITY | ERR_BOUNDS);
 __device__ __forceinline__ uint32_t analysis_errors(const BulkCtl *ctl)
 {
-    return *(const volatile uint32_t *)&ctl->err & kAnalysisErr | *(const volatile uint32_t *)&ctl->depth_err;
+    return (ctl->err & kAnalysisErr) | ctl->depth_err;
 }
 
 inline unsigned grid_for(int64_t n, int block = TB)
