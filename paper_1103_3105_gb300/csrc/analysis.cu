@@ -370,7 +370,7 @@ constexpr unsigned long long kNotYet = ~0ull;
 // ahead of another.
 constexpr uint32_t kFlowBits = 25, kFlowMask = (1u << kFlowBits) - 1u;
 __device__ __forceinline__ uint32_t flow_lap(uint32_t chunk) { return chunk / kFlowCluster + 1; }
-__device__ __forceinline__ uint32_t word_lap(unsigned long long w) { return (uint32_t)(w >> (2 * kFlowBits)); }
+constexpr int32_t kLapStep = 1 << (2 * kFlowBits - 32);   // a lap in a word's upper half
 
 __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long *p)
 {
@@ -543,16 +543,25 @@ __global__ void __launch_bounds__(kFlowThreads, 1) depth_flow_kernel(FlowArgs a)
         // waits for next in the next pass, so the lanes stay together
         uint64_t t_prog = 0;
         uint32_t seen = 0;
-        bool near = near_word(x);
-        uint32_t at = near ? ring_word(x) : ring, want = flow_lap(x / kFlowThreads);
+        // where it looks, and the least upper half of a word there that ends the wait
+        // (none for a lane that is done or whose word is in L2 only)
+        bool l2;
+        uint32_t at;
+        int32_t want;
+        auto aim = [&]() {
+            const bool near = near_word(x) && !done;
+            l2 = !near && !done;
+            at = near ? ring_word(x) : ring;
+            want = near ? (int32_t)flow_lap(x / kFlowThreads) * kLapStep : INT32_MAX;
+        };
+        aim();
         for (uint32_t spin = 1;; spin++) {
             unsigned long long w;
             asm volatile("ld.relaxed.cluster.shared::cta.u64 %0, [%1];" : "=l"(w) : "r"(at) : "memory");
-            const uint32_t lap = word_lap(w);
-            bool hit = !done && near && lap >= want;
+            const int32_t ahead = (int32_t)(w >> 32) - want;
+            bool hit = ahead >= 0;
             // older than the ring, or overwritten by a later chunk's (that CTA has finished its chunk)
-            const bool far = !done && (near ? hit && lap != want : (spin & 7u) == 0);
-            if (far) {
+            if (ahead >= kLapStep || (l2 && (spin & 7u) == 0)) {
                 w = ld_relaxed_u64(&a.depths[x]);
                 hit = w != kNotYet;
             }
@@ -560,9 +569,7 @@ __global__ void __launch_bounds__(kFlowThreads, 1) depth_flow_kernel(FlowArgs a)
                 if (hit) {
                     take(w, dl, ll);
                     if (!next()) publish();
-                    near = near_word(x);
-                    at = near ? ring_word(x) : ring;
-                    want = flow_lap(x / kFlowThreads);
+                    aim();
                 }
                 continue;
             }
@@ -576,6 +583,7 @@ __global__ void __launch_bounds__(kFlowThreads, 1) depth_flow_kernel(FlowArgs a)
                 if (__any_sync(kFull, late)) {
                     if (lane == 0) set_err(a.err, ERR_TIMEOUT);
                     if (!done) publish();
+                    aim();
                 }
             }
         }
