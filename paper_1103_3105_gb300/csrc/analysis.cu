@@ -1177,9 +1177,15 @@ __device__ __forceinline__ void warp_add_cell(bool on, uint32_t key, unsigned lo
 // in 51 us).  With `local` the sums gather in shared memory first (one slot per
 // teller and branch) and each block adds its non-zero sums once: the
 // same-address atomics on the few branch rows would otherwise serialise in L2.
-// With `few` cells even the shared-memory atomics collide, and a warp adds up
-// what its lanes have for one cell first (4 branches, 4,096 transactions: 4.9
-// us, 14.7 without).
+// With `few` cells (64 branches at most) even the shared-memory atomics collide,
+// and a warp adds up what its lanes have for one cell first.  That guards against
+// 64-bit additions in shared memory as compare-and-swap loops, which the compiler
+// makes of them where it can tell the address space: 4 branches, 4,096
+// transactions 42 us, 2^20 258, all of one account 308 (with the warps' sums 5.2,
+// 16, 16).  In the code below the address is generic and the additions are single
+// instructions, and the warps' sums are not worth their shuffles on either side of
+// the line: 4 branches at 2^20 16.0 us against 12.9 without, 64 20.9 against 13.2,
+// 128 21.8 against 13.0.
 struct DcRowsArgs {
     DevDB db;
     DevBulk b;

@@ -1284,7 +1284,7 @@ gputx_status gputx_execute(gputx_db *db, gputx_bulk *b, int strategy, const gput
             CK(launch_gather(b, rv), "gather");
             CK(begin_tail(b), "order");
             if (b->timing) cudaEventRecord(b->ev[3], s);
-            CK(launch_kset(b, rv, b->sc.chunk_cap, block, add || db->need_fixpoint), "k-set execute");
+            CK(launch_kset(b, b->sc.chunk_cap, block, add || db->need_fixpoint), "k-set execute");
             CK(launch_orders(b, false), "orders");
         } else if (b->n > 0) {
             // plan launches from the level widths
@@ -1609,7 +1609,7 @@ extern "C" gputx_status gputx_execute_kset_noalloc(gputx_db *db, const int64_t *
         CK(launch_sort(&b, rk, rv, rk2, rv2, b.n, bits_for((uint64_t)depth) + db->tbits), "regroup sort");
         CK(launch_level_tables(&b, rk, depth, block, true), "level tables");
         CK(launch_gather(&b, rv), "gather");
-        CK(launch_kset(&b, rv, b.sc.chunk_cap, block, add || db->need_fixpoint), "k-set execute");
+        CK(launch_kset(&b, b.sc.chunk_cap, block, add || db->need_fixpoint), "k-set execute");
     }
     CK(launch_orders(&b, oe_only(db)), "orders");
     CK(launch_finish(&b), "finish");

@@ -131,7 +131,7 @@ cudaError_t enqueue_pipeline(GraphBulk *g)
         if ((e = gtx::launch_level_tables(b, rk, 0, g->block, true))) return e;
         if ((e = gtx::launch_gather(b, rv))) return e;
         if ((e = gtx::launch_begin(b))) return e;
-        if ((e = gtx::launch_kset(b, rv, b->sc.chunk_cap, g->block, add || db->need_fixpoint))) return e;
+        if ((e = gtx::launch_kset(b, b->sc.chunk_cap, g->block, add || db->need_fixpoint))) return e;
         if ((e = gtx::launch_orders(b, false))) return e;
     } else {
         if ((e = gtx::launch_ticket_scan(b, sk, sv, m))) return e;

@@ -33,7 +33,12 @@ struct BulkCtl {
 
 constexpr uint32_t kTplHot = 128;  // debit-credit TPL: a chain longer than this is served in lock order
 
-constexpr int kTplMany = 64;       // and where the bulk is this many times as long, a warp takes a run of them
+// and where the bulk is this many times as long, a warp takes a run of 32s.  At
+// 200,003 transactions, two 32s a warp, that line is where both are the same (16
+// chains 858 us in runs, 834 with one 32; 32 445 / 447; 64 235 / 241; 128 133 /
+// 135); at 2^20, seven a warp, runs are faster on both sides of it (16 chains 6.0
+// ms against 12.3, 64 1.57 / 3.61, 256 0.42 / 1.04)
+constexpr int kTplMany = 64;
 
 constexpr int kScanAreas = 3;      // scans of a submitted bulk whose scratch its submission has cleared
 
@@ -190,7 +195,7 @@ cudaError_t launch_begin(gputx_bulk *b);
 cudaError_t launch_finish(gputx_bulk *b);
 
 // exec.cu
-cudaError_t launch_kset(gputx_bulk *b, const uint32_t *order, int64_t nchunks, int block, bool atomic_add);
+cudaError_t launch_kset(gputx_bulk *b, int64_t nchunks, int block, bool atomic_add);
 cudaError_t launch_kset_levels(gputx_bulk *b, const uint32_t *level_off_host, int64_t depth, int narrow_max,
                                bool atomic_add, const uint32_t *type_cut_host = nullptr);
 // single-operation bulks, from the sorted operations: item by item, run by run

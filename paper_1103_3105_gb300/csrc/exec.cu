@@ -54,10 +54,9 @@ struct KsetArgs {
     DevDB db;
     DevBulk b;
     BulkCtl *ctl;
-    const uint32_t *order, *level_off, *chunk_off, *chunk_level;
+    const uint32_t *level_off, *chunk_off, *chunk_level;
     const uint32_t *type_cut;   // per level, where the new-orders and payments start (or null)
     uint32_t *done;
-    int64_t levels;
     uint64_t spin_limit_ns;
     bool orders;                // new-orders are registered (launch_orders follows)
     bool atomic_add;
@@ -1102,7 +1101,7 @@ int exec_blocks_per_sm(int kind, int block)
     return nb < 1 ? 1 : nb;
 }
 
-cudaError_t launch_kset(gputx_bulk *b, const uint32_t *order, int64_t nchunks, int block, bool atomic_add)
+cudaError_t launch_kset(gputx_bulk *b, int64_t nchunks, int block, bool atomic_add)
 {
     gputx_db *db = b->db;
     if (b->n == 0 || nchunks == 0) return cudaSuccess;
@@ -1110,13 +1109,11 @@ cudaError_t launch_kset(gputx_bulk *b, const uint32_t *order, int64_t nchunks, i
     a.db = db->dev;
     a.b = make_dev_bulk(b, atomic_add ? GPUTX_CONFLICT_ADD : GPUTX_CONFLICT_PAPER);
     a.ctl = b->ctl;
-    a.order = order;
     a.level_off = b->sc.level_off;
     a.chunk_off = b->sc.chunk_off;
     a.chunk_level = b->sc.chunk_level;
     a.type_cut = b->sc.type_cut;
     a.done = b->sc.done;
-    a.levels = 0;
     a.orders = db->dev.registered >> GPUTX_T_OE_NEW_ORDER & 1u;
     a.spin_limit_ns = (uint64_t)db->cfg.spin_limit_ns;
     a.atomic_add = atomic_add;
