@@ -58,8 +58,8 @@ DOMINANT_KERNEL = {("kset", "paper"): "dc_range_kernel", ("kset", "add"): "acct_
 # configuration, keyed by (strategy, mode, bulk log2); each entry holds the
 # digest of the executor's sources it was taken on, and is reported as null once
 # those sources change
-TRAFFIC = {("kset", "paper", 22): {"bytes": 325240000 + 98550000 + 100770000 + 124180000,
-                                   "digest": "e1847de4ef3fee20"}}
+TRAFFIC = {("kset", "paper", 22): {"bytes": 325010000 + 98490000 + 100770000 + 124200000,
+                                   "digest": "97fa5babe499a806"}}
 KERNEL_SOURCES = ("common.cuh", "fastdiv.h", "engine.h", "dc.cuh", "ranges.cuh", "exec_dc.cu", "analysis.cu")
 
 
